@@ -2,19 +2,22 @@
 
 Argument marshalling only: tensors are checked (device, dtype, contiguity,
 shape) and passed as raw device pointers; every step of the path runs in the
-library's kernels.
+library's kernels.  The calls made once per step go through the native half of
+the binding (``csrc/esa_native.cpp``); creation, weights and diagnostics go
+through ctypes.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib.machinery
+import importlib.util
 import os
 from dataclasses import dataclass
-from typing import Optional, Sequence
 
 import numpy as np
 import torch
 
-from .build import LIB_PATH
+from .build import LIB_PATH, NATIVE_PATH
 
 STATUS_NAMES = {
     0: "ESA_OK", 1: "ESA_ERR_INVALID_ARG", 2: "ESA_ERR_SHAPE", 3: "ESA_ERR_CAPACITY",
@@ -141,20 +144,24 @@ def load_library():
     return lib
 
 
-def _ptr(t: Optional[torch.Tensor]):
-    return 0 if t is None else t.data_ptr()
+_native = None
 
 
-def _check(t: torch.Tensor, name: str, dtype, shape=None):
-    # kept cheap: it runs for every tensor of every call
-    if not t.is_cuda:
-        raise TypeError(f"{name} must be a CUDA tensor")
-    if t.dtype != dtype:
-        raise TypeError(f"{name} must have dtype {dtype}, got {t.dtype}")
-    if not t.is_contiguous():
-        raise ValueError(f"{name} must be contiguous")
-    if shape is not None and t.shape != shape:
-        raise ValueError(f"{name} must have shape {tuple(shape)}, got {tuple(t.shape)}")
+def load_native():
+    """The native half of this binding (``csrc/esa_native.cpp``): tensor checks and argument passing of the
+    calls that are made once per step.  Loaded after the library it is linked against."""
+    global _native
+    if _native is None:
+        load_library()
+        if not os.path.exists(NATIVE_PATH):
+            raise RuntimeError(f"{NATIVE_PATH} is missing: build it with `python -m paper_2502_14477_b200.build`.")
+        loader = importlib.machinery.ExtensionFileLoader("_esa_native", NATIVE_PATH)
+        spec = importlib.util.spec_from_file_location("_esa_native", NATIVE_PATH, loader=loader)
+        mod = importlib.util.module_from_spec(spec)
+        loader.exec_module(mod)
+        mod.set_error(EsaError)
+        _native = mod
+    return _native
 
 
 def _stream_ptr(stream) -> int:
@@ -179,10 +186,13 @@ class Esa:
         if st != 0:
             raise EsaError(st, "esa_create")
         self._h = h
+        self._n = load_native().Ctx(h.value, cfg)
 
     # ------------------------------------------------------------------ admin
     def close(self):
         if getattr(self, "_h", None) is not None and self._h.value:
+            if getattr(self, "_n", None) is not None:
+                self._n.drop()
             self.lib.esa_destroy(self._h)
             self._h = C.c_void_p()
 
@@ -220,157 +230,33 @@ class Esa:
         if st != 0:
             raise EsaError(st, "esa_set_compressors")
 
-    @staticmethod
-    def _nprev(n_prev: Sequence[int], B: int):
-        """Host int64[B] for the C call (a ctypes array: cheaper to build than a numpy one)."""
-        if len(n_prev) != B:
-            raise ValueError("n_prev must have one entry per sequence")
-        return (C.c_int64 * B)(*[int(x) for x in n_prev])
-
     # ------------------------------------------------------------ entry points
+    # n_prev: one integer per sequence.  stream: None (torch's current stream), a stream object or a raw handle.
     def append_kv(self, K_new, V_new, K_cache, V_cache, n_prev, stream=None, sync=False):
-        c = self.cfg
-        B, n_new = K_new.shape[0], K_new.shape[1]
-        _check(K_new, "K_new", torch.bfloat16, (B, n_new, c.n_kv_heads, c.head_dim))
-        _check(V_new, "V_new", torch.bfloat16, (B, n_new, c.n_kv_heads, c.head_dim))
-        _check(K_cache, "K_cache", torch.bfloat16, (B, c.max_tokens, c.n_kv_heads, c.head_dim))
-        _check(V_cache, "V_cache", torch.bfloat16, (B, c.max_tokens, c.n_kv_heads, c.head_dim))
-        npv = self._nprev(n_prev, B)
-        if sync:
-            st = self.lib.esa_append_kv(self._h, B, _ptr(K_new), _ptr(V_new), n_new, _ptr(K_cache),
-                                        _ptr(V_cache), npv)
-        else:
-            st = self.lib.esa_append_kv_async(self._h, B, _ptr(K_new), _ptr(V_new), n_new, _ptr(K_cache),
-                                              _ptr(V_cache), npv,
-                                              _stream_ptr(stream))
-        if st != 0:
-            raise EsaError(st, "esa_append_kv")
+        self._n.append_kv(K_new, V_new, K_cache, V_cache, n_prev, stream, sync)
 
     def compress_keys(self, K_new, kc_cache, n_prev, stream=None, sync=False):
-        c = self.cfg
-        B, n_new = K_new.shape[0], K_new.shape[1]
-        _check(K_new, "K_new", torch.bfloat16, (B, n_new, c.n_kv_heads, c.head_dim))
-        _check(kc_cache, "kc_cache", torch.bfloat16, (B, c.max_tokens, c.d_c))
-        npv = self._nprev(n_prev, B)
-        if sync:
-            st = self.lib.esa_compress_keys(self._h, B, _ptr(K_new), n_new, _ptr(kc_cache),
-                                            npv)
-        else:
-            st = self.lib.esa_compress_keys_async(self._h, B, _ptr(K_new), n_new, _ptr(kc_cache),
-                                                  npv, _stream_ptr(stream))
-        if st != 0:
-            raise EsaError(st, "esa_compress_keys")
+        self._n.compress_keys(K_new, kc_cache, n_prev, stream, sync)
 
     def select(self, Q_cur, kc_cache, n_prev, idx_out, n_sel_out, stream=None, sync=False):
-        c = self.cfg
-        B, l_C = Q_cur.shape[0], Q_cur.shape[1]
-        _check(Q_cur, "Q_cur", torch.bfloat16, (B, l_C, c.n_q_heads, c.head_dim))
-        _check(kc_cache, "kc_cache", torch.bfloat16, (B, c.max_tokens, c.d_c))
-        _check(idx_out, "idx_out", torch.int32, (B, c.top_k))
-        _check(n_sel_out, "n_sel_out", torch.int32, (B,))
-        npv = self._nprev(n_prev, B)
-        if sync:
-            st = self.lib.esa_select(self._h, B, _ptr(Q_cur), l_C, _ptr(kc_cache),
-                                     npv, _ptr(idx_out), _ptr(n_sel_out))
-        else:
-            st = self.lib.esa_select_async(self._h, B, _ptr(Q_cur), l_C, _ptr(kc_cache),
-                                           npv, _ptr(idx_out), _ptr(n_sel_out),
-                                           _stream_ptr(stream))
-        if st != 0:
-            raise EsaError(st, "esa_select")
+        self._n.select(Q_cur, kc_cache, n_prev, idx_out, n_sel_out, stream, sync)
 
     def select_full(self, Q_cur, K_cache, n_prev, idx_out, n_sel_out, per_head=False, stream=None, sync=False):
         """``esa_select_full``: selection on full-dimension scores (Eq. 3) or the per-head vote."""
-        c = self.cfg
-        B, l_C = Q_cur.shape[0], Q_cur.shape[1]
-        _check(Q_cur, "Q_cur", torch.bfloat16, (B, l_C, c.n_q_heads, c.head_dim))
-        _check(K_cache, "K_cache", torch.bfloat16, (B, c.max_tokens, c.n_kv_heads, c.head_dim))
-        _check(idx_out, "idx_out", torch.int32, (B, c.top_k))
-        _check(n_sel_out, "n_sel_out", torch.int32, (B,))
-        npv = self._nprev(n_prev, B)
-        mode = 1 if per_head else 0
-        if sync:
-            st = self.lib.esa_select_full(self._h, B, _ptr(Q_cur), l_C, _ptr(K_cache), npv, mode, _ptr(idx_out),
-                                          _ptr(n_sel_out))
-        else:
-            st = self.lib.esa_select_full_async(self._h, B, _ptr(Q_cur), l_C, _ptr(K_cache), npv, mode, _ptr(idx_out),
-                                                _ptr(n_sel_out), _stream_ptr(stream))
-        if st != 0:
-            raise EsaError(st, "esa_select_full")
+        self._n.select_full(Q_cur, K_cache, n_prev, per_head, idx_out, n_sel_out, stream, sync)
 
     def attend(self, Q_cur, K_cache, V_cache, n_prev, idx, n_sel, O, stream=None, sync=False):
-        c = self.cfg
-        B, l_C = Q_cur.shape[0], Q_cur.shape[1]
-        _check(Q_cur, "Q_cur", torch.bfloat16, (B, l_C, c.n_q_heads, c.head_dim))
-        _check(K_cache, "K_cache", torch.bfloat16, (B, c.max_tokens, c.n_kv_heads, c.head_dim))
-        _check(V_cache, "V_cache", torch.bfloat16, (B, c.max_tokens, c.n_kv_heads, c.head_dim))
-        _check(idx, "idx", torch.int32, (B, c.top_k))
-        _check(n_sel, "n_sel", torch.int32, (B,))
-        _check(O, "O", torch.bfloat16, (B, l_C, c.n_q_heads, c.head_dim))
-        npv = self._nprev(n_prev, B)
-        if sync:
-            st = self.lib.esa_attend(self._h, B, _ptr(Q_cur), l_C, _ptr(K_cache), _ptr(V_cache),
-                                     npv, _ptr(idx), _ptr(n_sel), _ptr(O))
-        else:
-            st = self.lib.esa_attend_async(self._h, B, _ptr(Q_cur), l_C, _ptr(K_cache), _ptr(V_cache),
-                                           npv, _ptr(idx), _ptr(n_sel), _ptr(O),
-                                           _stream_ptr(stream))
-        if st != 0:
-            raise EsaError(st, "esa_attend")
+        self._n.attend(Q_cur, K_cache, V_cache, n_prev, idx, n_sel, O, stream, sync)
 
     def attend_two_position(self, Q_cur, Q_far, K_cache, K_far_cache, V_cache, n_prev, idx, n_sel, O, stream=None,
                             sync=False):
         """``esa_attend_two_position``: Q_far / K_far_cache (either may be None) are read for I and M_k."""
-        c = self.cfg
-        B, l_C = Q_cur.shape[0], Q_cur.shape[1]
-        _check(Q_cur, "Q_cur", torch.bfloat16, (B, l_C, c.n_q_heads, c.head_dim))
-        if Q_far is not None:
-            _check(Q_far, "Q_far", torch.bfloat16, (B, l_C, c.n_q_heads, c.head_dim))
-        _check(K_cache, "K_cache", torch.bfloat16, (B, c.max_tokens, c.n_kv_heads, c.head_dim))
-        if K_far_cache is not None:
-            _check(K_far_cache, "K_far_cache", torch.bfloat16, (B, c.max_tokens, c.n_kv_heads, c.head_dim))
-        _check(V_cache, "V_cache", torch.bfloat16, (B, c.max_tokens, c.n_kv_heads, c.head_dim))
-        _check(idx, "idx", torch.int32, (B, c.top_k))
-        _check(n_sel, "n_sel", torch.int32, (B,))
-        _check(O, "O", torch.bfloat16, (B, l_C, c.n_q_heads, c.head_dim))
-        npv = self._nprev(n_prev, B)
-        if sync:
-            st = self.lib.esa_attend_two_position(self._h, B, _ptr(Q_cur), _ptr(Q_far), l_C, _ptr(K_cache),
-                                                  _ptr(K_far_cache), _ptr(V_cache), npv, _ptr(idx), _ptr(n_sel), _ptr(O))
-        else:
-            st = self.lib.esa_attend_two_position_async(self._h, B, _ptr(Q_cur), _ptr(Q_far), l_C, _ptr(K_cache),
-                                                        _ptr(K_far_cache), _ptr(V_cache), npv, _ptr(idx), _ptr(n_sel),
-                                                        _ptr(O), _stream_ptr(stream))
-        if st != 0:
-            raise EsaError(st, "esa_attend_two_position")
+        self._n.attend_two_position(Q_cur, Q_far, K_cache, K_far_cache, V_cache, n_prev, idx, n_sel, O, stream, sync)
 
     def attend_host_kv(self, Q_cur, K_host, V_host, n_prev, idx, n_sel, K_stage, V_stage, O, stream=None, sync=False):
         """``esa_attend_host_kv``: K_host / V_host are pinned host tensors [B, max_tokens, H_G, d]; K_stage / V_stage
         device scratch [B, stage_rows, H_G, d]."""
-        c = self.cfg
-        B, l_C = Q_cur.shape[0], Q_cur.shape[1]
-        _check(Q_cur, "Q_cur", torch.bfloat16, (B, l_C, c.n_q_heads, c.head_dim))
-        for t, name in ((K_host, "K_host"), (V_host, "V_host")):
-            if t.is_cuda or not t.is_pinned():
-                raise TypeError(f"{name} must be a pinned host tensor")
-            if t.dtype != torch.bfloat16 or not t.is_contiguous() or t.shape != (B, c.max_tokens, c.n_kv_heads, c.head_dim):
-                raise ValueError(f"{name} must be contiguous bf16 [B, max_tokens, H_G, d]")
-        stage_rows = K_stage.shape[1]
-        _check(K_stage, "K_stage", torch.bfloat16, (B, stage_rows, c.n_kv_heads, c.head_dim))
-        _check(V_stage, "V_stage", torch.bfloat16, (B, stage_rows, c.n_kv_heads, c.head_dim))
-        _check(idx, "idx", torch.int32, (B, c.top_k))
-        _check(n_sel, "n_sel", torch.int32, (B,))
-        _check(O, "O", torch.bfloat16, (B, l_C, c.n_q_heads, c.head_dim))
-        npv = self._nprev(n_prev, B)
-        if sync:
-            st = self.lib.esa_attend_host_kv(self._h, B, _ptr(Q_cur), l_C, K_host.data_ptr(), V_host.data_ptr(), npv, _ptr(idx),
-                                             _ptr(n_sel), _ptr(K_stage), _ptr(V_stage), stage_rows, _ptr(O))
-        else:
-            st = self.lib.esa_attend_host_kv_async(self._h, B, _ptr(Q_cur), l_C, K_host.data_ptr(), V_host.data_ptr(), npv,
-                                                   _ptr(idx), _ptr(n_sel), _ptr(K_stage), _ptr(V_stage), stage_rows, _ptr(O),
-                                                   _stream_ptr(stream))
-        if st != 0:
-            raise EsaError(st, "esa_attend_host_kv")
+        self._n.attend_host_kv(Q_cur, K_host, V_host, n_prev, idx, n_sel, K_stage, V_stage, O, stream, sync)
 
     def read_pooled_scores(self, b: int, n: int, stream=None) -> np.ndarray:
         out = np.empty(n, dtype=np.float32)
@@ -421,9 +307,12 @@ class EsaFit:
         if st != 0:
             raise EsaError(st, "esa_fit_create")
         self._h = h
+        self._n = load_native().Fit(h.value, cfg)
 
     def close(self):
         if getattr(self, "_h", None) is not None and self._h.value:
+            if getattr(self, "_n", None) is not None:
+                self._n.drop()
             self.lib.esa_fit_destroy(self._h)
             self._h = C.c_void_p()
 
@@ -453,15 +342,7 @@ class EsaFit:
         return out
 
     def step(self, Q_batch, K_batch, loss_out=None, stream=None):
-        c = self.cfg
-        n = Q_batch.shape[0]
-        _check(Q_batch, "Q_batch", torch.bfloat16, (n, c.n_q_heads, c.head_dim))
-        _check(K_batch, "K_batch", torch.bfloat16, (n, c.n_kv_heads, c.head_dim))
-        if loss_out is not None:
-            _check(loss_out, "loss_out", torch.float32, (1,))
-        st = self.lib.esa_fit_step_async(self._h, _ptr(Q_batch), _ptr(K_batch), n, _ptr(loss_out), _stream_ptr(stream))
-        if st != 0:
-            raise EsaError(st, "esa_fit_step_async")
+        self._n.step(Q_batch, K_batch, loss_out, stream)
 
 
 def attend_noalloc(cfg: EsaConfig, Q_cur, K_cache, V_cache, n_prev, idx, n_sel, O, stream=None):
@@ -469,17 +350,4 @@ def attend_noalloc(cfg: EsaConfig, Q_cur, K_cache, V_cache, n_prev, idx, n_sel, 
     any device allocation -- the split partials live in a fixed array inside the library.  For
     callers that must not allocate once running (see ``include/esa.h``).  Calls on one device
     share that array and must be ordered with respect to each other."""
-    lib = load_library()
-    B, l_C = Q_cur.shape[0], Q_cur.shape[1]
-    _check(Q_cur, "Q_cur", torch.bfloat16, (B, l_C, cfg.n_q_heads, cfg.head_dim))
-    _check(K_cache, "K_cache", torch.bfloat16, (B, cfg.max_tokens, cfg.n_kv_heads, cfg.head_dim))
-    _check(V_cache, "V_cache", torch.bfloat16, (B, cfg.max_tokens, cfg.n_kv_heads, cfg.head_dim))
-    _check(idx, "idx", torch.int32, (B, cfg.top_k))
-    _check(n_sel, "n_sel", torch.int32, (B,))
-    _check(O, "O", torch.bfloat16, (B, l_C, cfg.n_q_heads, cfg.head_dim))
-    npv = Esa._nprev(n_prev, B)
-    c = cfg.to_c()
-    st = lib.esa_attend_noalloc(C.byref(c), B, _ptr(Q_cur), l_C, _ptr(K_cache), _ptr(V_cache),
-                                npv, _ptr(idx), _ptr(n_sel), _ptr(O), _stream_ptr(stream))
-    if st != 0:
-        raise EsaError(st, "esa_attend_noalloc")
+    load_native().attend_noalloc(cfg, Q_cur, K_cache, V_cache, n_prev, idx, n_sel, O, stream)

@@ -1,14 +1,18 @@
-"""Builds the C-ABI CUDA library in-tree with nvcc for sm_100a."""
+"""Builds the C-ABI CUDA library in-tree with nvcc for sm_100a, and the native half of the Python binding
+(a small extension module linked against it and against the installed torch) with g++."""
 from __future__ import annotations
 
 import glob
 import os
 import shutil
 import subprocess
+import sysconfig
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libesa_b200.so")
+NATIVE_SRC = os.path.join(CSRC, "esa_native.cpp")
+NATIVE_PATH = os.path.join(PKG_DIR, "_esa_native.so")
 INCLUDE_DIR = os.path.join(os.path.dirname(PKG_DIR), "include")
 
 
@@ -28,31 +32,57 @@ def _deps():
         glob.glob(os.path.join(INCLUDE_DIR, "*.h"))
 
 
-def is_stale() -> bool:
-    if not os.path.exists(LIB_PATH):
+def _stale(target: str, deps) -> bool:
+    if not os.path.exists(target):
         return True
-    t = os.path.getmtime(LIB_PATH)
-    return any(os.path.getmtime(f) > t for f in _deps())
+    t = os.path.getmtime(target)
+    return any(os.path.getmtime(f) > t for f in deps)
+
+
+def is_stale() -> bool:
+    return _stale(LIB_PATH, _deps()) or _stale(NATIVE_PATH, [NATIVE_SRC, LIB_PATH])
+
+
+def _run(cmd) -> str:
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        raise RuntimeError(f"{os.path.basename(cmd[0])} failed:\n" + res.stdout + res.stderr)
+    return res.stderr
+
+
+def _build_native() -> None:
+    import torch
+    tdir = os.path.dirname(torch.__file__)
+    cuda_inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_nvcc()))), "include")
+    _run([
+        os.environ.get("CXX") or "g++", "-shared", "-fPIC", "-std=c++17", "-O2",
+        f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+        "-I", sysconfig.get_paths()["include"], "-I", os.path.join(tdir, "include"),
+        "-I", os.path.join(tdir, "include", "torch", "csrc", "api", "include"), "-I", cuda_inc,
+        "-o", NATIVE_PATH, NATIVE_SRC,
+        "-L", os.path.join(tdir, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python",
+        "-L", PKG_DIR, "-l:" + os.path.basename(LIB_PATH), "-Wl,-rpath,$ORIGIN",
+    ])
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ into one shared library (sm_100a only)."""
+    """Compile every .cu under csrc/ into one shared library (sm_100a only), and the binding's native module."""
     if not force and not is_stale():
         return LIB_PATH
-    cmd = [
-        _nvcc(), "-shared", "-Xcompiler", "-fPIC", "-std=c++17", "-O3", "-lineinfo", "--threads", "8",
-        "-gencode", "arch=compute_100a,code=sm_100a",
-        "-I", INCLUDE_DIR, "-I", CSRC,
-        "-o", LIB_PATH,
-    ] + sources() + ["-lcuda"]
-    if verbose:
-        cmd.insert(1, "-Xptxas")
-        cmd.insert(2, "-v")
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if res.returncode != 0:
-        raise RuntimeError("nvcc failed:\n" + res.stdout + res.stderr)
-    if verbose:
-        print(res.stderr)
+    if force or _stale(LIB_PATH, _deps()):
+        cmd = [
+            _nvcc(), "-shared", "-Xcompiler", "-fPIC", "-std=c++17", "-O3", "-lineinfo", "--threads", "8",
+            "-gencode", "arch=compute_100a,code=sm_100a",
+            "-I", INCLUDE_DIR, "-I", CSRC,
+            "-o", LIB_PATH,
+        ] + sources() + ["-lcuda"]
+        if verbose:
+            cmd.insert(1, "-Xptxas")
+            cmd.insert(2, "-v")
+        log = _run(cmd)
+        if verbose:
+            print(log)
+    _build_native()
     return LIB_PATH
 
 

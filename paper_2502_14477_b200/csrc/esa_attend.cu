@@ -689,10 +689,11 @@ template <int D, int G, bool TWO>
 static cudaError_t launch_decode_t(esa_ctx* ctx, AttendParams& p, int B, int n_att_max, cudaStream_t st) {
     constexpr int smem = DEC_WARPS * DEC_STAGES * 2 * DEC_ROWS * D * 2;
     static_assert(smem >= (2 * DEC_WARPS * 8 + DEC_WARPS * 8 * D) * 4, "the warp merge reuses the rings");
-    cudaError_t e = cudaFuncSetAttribute(attend_decode_kernel<D, G, TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    static KernelMemo memo;
+    cudaError_t e = allow_smem(attend_decode_kernel<D, G, TWO>, ctx->device, smem, memo);
     if (e != cudaSuccess) return e;
     int per_sm = 1;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, attend_decode_kernel<D, G, TWO>, DEC_WARPS * 32, smem);
+    e = resident_per_sm(attend_decode_kernel<D, G, TWO>, ctx->device, DEC_WARPS * 32, smem, memo, &per_sm);
     if (e != cudaSuccess) return e;
     const int iters = (n_att_max + DEC_ROWS - 1) / DEC_ROWS;
     // one wave of CTAs, each warp with at least a few iterations
@@ -728,13 +729,14 @@ static cudaError_t launch_attend_t(esa_ctx* ctx, AttendParams& p, int B, int n_a
     const int R = p.l_C * p.G;
     const int row_tiles = (R + BM - 1) / BM;
     constexpr int smem = ((TWO ? 2 : 1) * BM + 4 * BN) * (D / 8) * 16;
-    cudaError_t e = cudaFuncSetAttribute(attend_kernel<D, NW, BN, TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    static KernelMemo memo;
+    cudaError_t e = allow_smem(attend_kernel<D, NW, BN, TWO>, ctx->device, smem, memo);
     if (e != cudaSuccess) return e;
     int nsplit = 1;
     if (R <= kAttSplitRows && row_tiles == 1) {
         // split the key list so that one wave of CTAs fills the machine (never a second, short wave)
         int per_sm = 1;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, attend_kernel<D, NW, BN, TWO>, NW * 32, smem);
+        e = resident_per_sm(attend_kernel<D, NW, BN, TWO>, ctx->device, NW * 32, smem, memo, &per_sm);
         if (e != cudaSuccess) return e;
         const int ctas = p.HG * B;
         const int n_tiles = (n_att_max + BN - 1) / BN;
@@ -835,13 +837,14 @@ NoAllocDevice g_noalloc_dev[kNoAllocMaxDevices];
 std::mutex g_noalloc_mutex;      // host threads may make a device's first call together
 
 template <int D, int NW, int BN>
-cudaError_t launch_noalloc_t(const NoAllocDevice& dev, AttendParams& p, int B, int n_att_max, cudaStream_t st) {
+cudaError_t launch_noalloc_t(const NoAllocDevice& dev, int device, AttendParams& p, int B, int n_att_max, cudaStream_t st) {
     const int R = p.l_C * p.G;
     constexpr int smem = (NW * 16 + 4 * BN) * (D / 8) * 16;
-    cudaError_t e = cudaFuncSetAttribute(attend_kernel<D, NW, BN, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    static KernelMemo memo;
+    cudaError_t e = allow_smem(attend_kernel<D, NW, BN, false>, device, smem, memo);
     if (e != cudaSuccess) return e;
     int per_sm = 1;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, attend_kernel<D, NW, BN, false>, NW * 32, smem);
+    e = resident_per_sm(attend_kernel<D, NW, BN, false>, device, NW * 32, smem, memo, &per_sm);
     if (e != cudaSuccess) return e;
     const int n_tiles = (n_att_max + BN - 1) / BN;
     int nsplit = (per_sm * dev.num_sms) / (p.HG * B);
@@ -925,9 +928,9 @@ extern "C" esa_status esa_attend_noalloc(const esa_config* cfg, int32_t B, const
     p.meta = meta;
     cudaStream_t st = (cudaStream_t)stream;
     cudaError_t e;
-    if (D == 128) e = R <= 16 ? launch_noalloc_t<128, 1, 32>(dev, p, B, n_att_max, st)
-                              : launch_noalloc_t<128, 4, 64>(dev, p, B, n_att_max, st);
-    else e = R <= 16 ? launch_noalloc_t<64, 1, 32>(dev, p, B, n_att_max, st)
-                     : launch_noalloc_t<64, 4, 64>(dev, p, B, n_att_max, st);
+    if (D == 128) e = R <= 16 ? launch_noalloc_t<128, 1, 32>(dev, device, p, B, n_att_max, st)
+                              : launch_noalloc_t<128, 4, 64>(dev, device, p, B, n_att_max, st);
+    else e = R <= 16 ? launch_noalloc_t<64, 1, 32>(dev, device, p, B, n_att_max, st)
+                     : launch_noalloc_t<64, 4, 64>(dev, device, p, B, n_att_max, st);
     return e == cudaSuccess ? ESA_OK : ESA_ERR_CUDA;
 }

@@ -930,7 +930,8 @@ template <int D, bool PAIR>
 static cudaError_t launch_tc_kernel(esa_ctx* ctx, const CUtensorMap& qmap, const CUtensorMap& qgmap, const TcAttendParams& p,
                                     dim3 grid, cudaStream_t st, bool probe_only) {
     constexpr int smem = 2 * 128 * D * 2 + 2 * TC_STAGES * TC_BN * D * 2 + 1024;
-    cudaError_t e = cudaFuncSetAttribute(attend_tc_kernel<D, PAIR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    static KernelMemo memo;
+    cudaError_t e = allow_smem(attend_tc_kernel<D, PAIR>, ctx->device, smem, memo);
     if (e != cudaSuccess) return e;
     // the in-kernel register split assumes the launch allocation it was sized for
     static int regs_checked = 0;

@@ -135,7 +135,8 @@ static cudaError_t launch_compress_t(esa_ctx* ctx, const __nv_bfloat16* X, int r
     while (nsplit < 8 && (nk_total % (nsplit * 2)) == 0 && row_tiles * nsplit < 2 * ctx->num_sms) nsplit *= 2;
     const int kslice = d_in / nsplit;
     constexpr int smem = 2 * (CP_BM + DC) * (CP_BK / 8) * 16 + CP_BM * DC * 4;
-    cudaError_t e = cudaFuncSetAttribute(compress_kernel<DC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    static KernelMemo memo;
+    cudaError_t e = allow_smem(compress_kernel<DC>, ctx->device, smem, memo);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(row_tiles, nsplit);

@@ -191,14 +191,17 @@ cudaError_t launch_t(esa_ctx* ctx, const __nv_bfloat16* X, int rows, int rows_pe
     constexpr int smem_stage = (CT_ROWS + DC) * CT_KCHUNK * 2;
     constexpr int smem_part = CT_ROWS * (DC + 4) * 4;
     constexpr int smem = (CT_STAGES * smem_stage > smem_part ? CT_STAGES * smem_stage : smem_part) + 1024;
-    cudaError_t e = cudaFuncSetAttribute(compress_tc_kernel<DC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(compress_tc_kernel<DC>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    static KernelMemo memo;
+    cudaError_t e = allow_smem(compress_tc_kernel<DC>, ctx->device, smem, memo);
     if (e != cudaSuccess) return e;
     // a cluster of 16 is beyond the portable size: use it only where the device can place one
-    static int max_split = 0;
+    static std::atomic<int> max_splits[64];
+    const int slot = ctx->device & 63;
+    int max_split = max_splits[slot].load(std::memory_order_relaxed);
     if (!max_split) {
         max_split = 8;
+        e = cudaFuncSetAttribute(compress_tc_kernel<DC>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        if (e != cudaSuccess) return e;
         cudaLaunchConfig_t probe = {};
         probe.gridDim = dim3(1, CT_MAX_SPLIT);
         probe.blockDim = dim3(CT_THREADS);
@@ -215,6 +218,7 @@ cudaError_t launch_t(esa_ctx* ctx, const __nv_bfloat16* X, int rows, int rows_pe
             max_split = CT_MAX_SPLIT;
         else
             cudaGetLastError();
+        max_splits[slot].store(max_split, std::memory_order_relaxed);
     }
     while (nsplit > max_split) nsplit /= 2;
     CompressTcParams p;

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <vector>
 
 #include "../../include/esa.h"
@@ -28,6 +29,29 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
+// Facts about a kernel that hold for the life of the process are asked of the runtime once per device, not at every
+// launch (a step of a small model is bound by what its launches cost the host).  `memo`: a static of the launching function.
+struct KernelMemo {
+    std::atomic<uint64_t> smem_set{0};      // devices whose dynamic shared-memory limit has been raised
+    std::atomic<int> per_sm[64] = {};       // resident CTAs per SM, 0 = not asked yet
+};
+template <typename F>
+cudaError_t allow_smem(F* kernel, int device, int bytes, KernelMemo& memo) {
+    const uint64_t bit = device >= 0 && device < 64 ? uint64_t(1) << device : 0;
+    if (memo.smem_set.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) memo.smem_set.fetch_or(bit, std::memory_order_release);
+    return e;
+}
+template <typename F>
+cudaError_t resident_per_sm(F* kernel, int device, int threads, int smem, KernelMemo& memo, int* out) {
+    const bool known = device >= 0 && device < 64;
+    if (known && (*out = memo.per_sm[device].load(std::memory_order_relaxed)) > 0) return cudaSuccess;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, kernel, threads, smem);
+    if (e == cudaSuccess && known) memo.per_sm[device].store(*out, std::memory_order_relaxed);
+    return e;
 }
 
 constexpr int kAttMaxSplits = 64;     // split-KV factor of the attention kernel (small chunks)
@@ -53,6 +77,26 @@ struct ProfRec {
     cudaEvent_t a, b;
 };
 
+// TMA descriptor of a row-major bf16 matrix [rows, cols] (cols a multiple of 64), read in boxes of
+// box_rows x 64 columns with the 128-byte swizzle.  False when the driver entry point is missing
+// or refuses the shape.
+bool make_tensor_map_bf16(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
+
+// A descriptor kept with the matrix it was made for (column count and box never change for one user of it).
+struct CachedMap {
+    CUtensorMap map;
+    const void* base = nullptr;
+    uint64_t rows = 0;
+    bool matches(const void* b, uint64_t r) const { return base == b && rows == r; }
+    bool encode(const void* b, uint64_t r, uint64_t cols, uint32_t box_rows) {
+        base = nullptr;
+        if (!make_tensor_map_bf16(&map, b, r, cols, box_rows)) return false;
+        base = b;
+        rows = r;
+        return true;
+    }
+};
+
 }  // namespace esa
 
 struct esa_ctx {
@@ -67,6 +111,7 @@ struct esa_ctx {
     __nv_bfloat16* Wk;   // [dc, dG]
     CUtensorMap wq_map, wk_map;   // TMA descriptors of Wq / Wk (valid when has_wmaps)
     bool has_wmaps;
+    esa::CachedMap kc_map, qc_map;   // descriptors of the compressed-key cache and of Qc used by the last scoring
     float* bq;           // [dc]
     float* bk;           // [dc]
     __nv_bfloat16* Qc;   // [max_batch * max_chunk, dc]
@@ -189,11 +234,6 @@ cudaError_t launch_attend_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* 
                              const __nv_bfloat16* K, const __nv_bfloat16* Kg, const __nv_bfloat16* V, const SeqMeta& meta,
                              const int32_t* idx, const int32_t* n_sel, __nv_bfloat16* O,
                              int n_att_max, cudaStream_t st, int* nsplit_out, int64_t cache_rows = 0, bool staged = false);
-
-// TMA descriptor of a row-major bf16 matrix [rows, cols] (cols a multiple of 64), read in boxes of
-// box_rows x 64 columns with the 128-byte swizzle.  False when the driver entry point is missing
-// or refuses the shape.
-bool make_tensor_map_bf16(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
 
 // TMA descriptor of the query tensor [n_queries, H, D] for the attention kernel (group size G must
 // divide 128).

@@ -376,9 +376,10 @@ static cudaError_t launch_score_t(esa_ctx* ctx, int B, int l_C, const __nv_bfloa
     if (gx > n_tiles) gx = n_tiles;
     if (gx < 1) gx = 1;
     constexpr int smem = (SC_BN + SC_STAGES * SC_BM) * (DC / 8) * 16 + 8 * SC_BN * 4;
-    e = cudaFuncSetAttribute(score_pass_kernel<DC, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    static KernelMemo memo1, memo2;
+    e = allow_smem(score_pass_kernel<DC, 1>, ctx->device, smem, memo1);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(score_pass_kernel<DC, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    e = allow_smem(score_pass_kernel<DC, 2>, ctx->device, smem, memo2);
     if (e != cudaSuccess) return e;
     dim3 grid(gx, qblocks, B);
     ProfScope prof(ctx, KC_SCORE_MMA, st);

@@ -431,9 +431,13 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
 template <int DC>
 cudaError_t launch_t(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache, const SeqMeta& meta, int max_lM,
                      cudaStream_t st, bool* pooled_ready) {
-    CUtensorMap kmap, qmap;
-    if (!make_tensor_map_bf16(&kmap, kc_cache, (uint64_t)B * ctx->cfg.max_tokens, DC, 128)) return cudaErrorNotSupported;
-    if (!make_tensor_map_bf16(&qmap, ctx->Qc, (uint64_t)B * l_C, DC, 128)) return cudaErrorNotSupported;
+    // the descriptors of the last call serve again while the caller keeps its cache and chunk size
+    if (!ctx->kc_map.matches(kc_cache, (uint64_t)B * ctx->cfg.max_tokens) &&
+        !ctx->kc_map.encode(kc_cache, (uint64_t)B * ctx->cfg.max_tokens, DC, 128))
+        return cudaErrorNotSupported;
+    if (!ctx->qc_map.matches(ctx->Qc, (uint64_t)B * l_C) && !ctx->qc_map.encode(ctx->Qc, (uint64_t)B * l_C, DC, 128))
+        return cudaErrorNotSupported;
+    const CUtensorMap &kmap = ctx->kc_map.map, &qmap = ctx->qc_map.map;
     ScoreTcParams p;
     p.rkey = ctx->rkey; p.skey = ctx->skey; p.pkey = ctx->pkey; p.ghist0 = ctx->ghist0; p.status = ctx->status;
     p.max_tokens = ctx->cfg.max_tokens; p.l_C = l_C; p.eps = ctx->cfg.eps; p.meta = meta;
@@ -441,9 +445,10 @@ cudaError_t launch_t(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache
     p.q_groups = q_groups;
     using C1 = ScoreCfg<DC, 1>;
     using C2 = ScoreCfg<DC, 2>;
-    cudaError_t e = cudaFuncSetAttribute(score_tc_kernel<DC, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, C1::SMEM);
+    static KernelMemo memo1, memo2;
+    cudaError_t e = allow_smem(score_tc_kernel<DC, 1>, ctx->device, C1::SMEM, memo1);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(score_tc_kernel<DC, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, C2::SMEM);
+    e = allow_smem(score_tc_kernel<DC, 2>, ctx->device, C2::SMEM, memo2);
     if (e != cudaSuccess) return e;
     const int n_tiles = (max_lM + ST_KEYS - 1) / ST_KEYS;
     int per_seq = ctx->num_sms / (q_groups * B);

@@ -548,7 +548,8 @@ cudaError_t launch_select(esa_ctx* ctx, int B, bool mapped, const SeqMeta& meta,
     p.max_tokens = ctx->cfg.max_tokens; p.slice_stride = ctx->sel_slice_stride; p.top_k = ctx->cfg.top_k;
     p.mapped = mapped ? 1 : 0; p.l_C = 1; p.meta = meta;     // (mapped mode reads rkey[b]: one query per sequence)
     constexpr size_t smem = (size_t)(SEL_MAX_SLICES_SMEM + 2 * SEL_STAGE_CAP) * 4;
-    e = cudaFuncSetAttribute(select_topk_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static KernelMemo memo;
+    e = allow_smem(select_topk_kernel, ctx->device, (int)smem, memo);
     if (e != cudaSuccess) return e;
     ProfScope prof(ctx, KC_SELECT_TOPK, st);
     e = launch_pdl(select_topk_kernel, dim3(n_slices, B), dim3(SEL_THREADS), smem, st, p);
