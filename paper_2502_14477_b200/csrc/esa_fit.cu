@@ -1,16 +1,27 @@
 // Eq. 7: fitting the two linear compressors f_q(q) = W_q q + b_q and f_k(k) = W_k k + b_k so that
 // f_q(q_c) . f_k(k_m) reproduces the full-dimension score q_c k_m^T (Eq. 3) of every query-key pair
 // of a batch (mean squared error over the n x n pairs), with Adam.  An offline, per-layer step
-// (Section 4.1: learning rate 5e-4, batches of 128 pairs, 10 epochs over 50k pairs): a few small
-// products per step, bound by launch latency and fp32 arithmetic, kept in fp32 throughout so that
-// thousands of steps stay close to a double-precision run.
+// (Section 4.1: learning rate 5e-4, batches of 128 pairs, 10 epochs over 50k pairs) of fp32 accuracy,
+// so that thousands of steps stay close to a double-precision run.
 //
 // One step (n pairs; Q [n, H, d] and K [n, H_G, d] bf16 on the device):
-//   Qf = heads of each GQA group summed            T  = Qf K^T            (Eq. 3 for all pairs)
+//   T  = sum over heads of Q_h K_g(h)^T            (Eq. 3 for all pairs)
 //   A  = Q W_q^T + b_q      Bm = K W_k^T + b_k     E  = A Bm^T - T        loss = mean(E^2)
 //   dP = 2 E / n^2          dA = dP Bm             dBm = dP^T A
 //   dW_q = dA^T Q   db_q = column sums of dA       dW_k = dBm^T K   db_k = column sums of dBm
 //   Adam update of W_q, b_q, W_k, b_k
+//
+// The work of a batch of 128 pairs is 0.4 GFLOP and the 16 MB of parameters and moments live in L2, so a step is
+// bound by its chain of dependent launches and by the latency inside each.  It is three launches
+// (fit_forward_kernel, fit_pairs_kernel, fit_update_kernel) chained with programmatic dependent launch; 28 us on the
+// Llama-3-8B shape (forward 10, pairs 5, update 8, the rest boundaries), where 17 launches of generic fp32 product
+// kernels took 202 us.
+// The long products have one bf16 operand (the batch), so they run on mma.sync with the fp32 operand cut into three
+// bf16 pieces (w = w1 + w2 + w3, 24 significant bits): every product is exact and the sums are fp32, as with fp32
+// multiply-adds.  The tensor core truncates when it adds, so its sums are kept short (64 terms) and added up in fp32
+// registers, smallest pieces first.
+#include <cooperative_groups.h>
+
 #include <cmath>
 #include <new>
 
@@ -28,14 +39,524 @@ struct esa_fit {
     float* m1;                    // Adam first moments
     float* m2;                    // Adam second moments
     float *Qf, *T, *A, *Bm, *dP, *dA, *dBm;
-    float* part;                  // partial sums of split reductions
+    __nv_bfloat16 *dA3, *dBm3;    // [3][n, dc]: gradients of A and Bm as bf16 pieces
+    float* loss_part;             // per-band partial losses
+    float* part;                  // partial sums of split reductions (generic kernels)
     float* loss_acc;              // one float
     int64_t launches;
 };
 
+namespace cg = cooperative_groups;
+
 namespace esa {
 namespace {
 
+__device__ __forceinline__ void split3(float lo, float hi, uint32_t (&w)[3]) {
+    // (lo, hi) as three packed bf16 pairs whose sum is exact to 24 bits
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        w[i] = pack_bf16(lo, hi);
+        lo -= __uint_as_float(w[i] << 16);
+        hi -= __uint_as_float(w[i] & 0xffff0000u);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Launch 1: A, Bm and T.  A job is one 32 x 32 output tile of one of the three products; the reduction dimension is
+// dealt out to the 8 CTAs of a cluster (64 columns a chunk, four chunks in flight), whose partial tiles are added
+// through distributed shared memory in rank order.  The tiles are this small because the jobs of A hold two thirds of
+// the tensor-core work: 128 CTAs of them for 128 pairs, d' = 128, where 64 x 32 tiles leave it to 64 SMs.
+// ---------------------------------------------------------------------------
+constexpr int FF_M = 32, FF_N = 32, FF_K = 64, FF_STAGES = 4, FF_CLUSTER = 8, FF_THREADS = 256;
+constexpr int FF_XBYTES = FF_M * FF_K * 2;
+constexpr int FF_YROW = (FF_K + 8) * 4;          // fp32 row stride: 8 rows x 4 column pairs of 8 bytes hit all banks
+constexpr int FF_YROW16 = (FF_K + 8) * 2;        // the same for bf16 rows
+constexpr int FF_YBYTES = FF_N * FF_YROW;
+constexpr int FF_SMEM = FF_STAGES * (FF_XBYTES + FF_YBYTES);
+
+struct FitParams {
+    const __nv_bfloat16 *Q, *K;
+    float *Wq, *bq, *Wk, *bk;
+    float *m1, *m2;              // moments, laid out like [Wq | bq | Wk | bk]
+    float *A, *Bm, *T;           // [n, dc], [n, dc], [n, n]
+    __nv_bfloat16 *dA, *dBm;     // [3][n, dc]: the pieces of the gradients of A and Bm
+    float* loss_part;            // one value per band of FP_R pairs
+    float* loss_out;             // may be null
+    int n, dc, dH, dG, d, G;
+    float lr, beta1, beta2, eps, ic1, ic2;     // ic: 1 / (1 - beta^step)
+};
+
+__global__ void __launch_bounds__(FF_THREADS, 3) fit_forward_kernel(FitParams p) {
+    extern __shared__ __align__(128) uint8_t ff_smem[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int rank = blockIdx.x;                             // rank in the cluster
+    const int row_tiles = (p.n + FF_M - 1) / FF_M, dc_tiles = (p.dc + FF_N - 1) / FF_N, pair_tiles = (p.n + FF_N - 1) / FF_N;
+    // jobs: A tiles (the dearest first), Bm tiles, T tiles
+    int job = blockIdx.y, kind = 0, cols = dc_tiles;
+    if (job >= row_tiles * dc_tiles) {
+        job -= row_tiles * dc_tiles;
+        kind = 1;
+        if (job >= row_tiles * dc_tiles) {
+            job -= row_tiles * dc_tiles;
+            kind = 2;
+            cols = pair_tiles;
+        }
+    }
+    const int r0 = (job / cols) * FF_M, c0 = (job % cols) * FF_N;
+    const __nv_bfloat16* X = kind == 1 ? p.K : p.Q;
+    const int kdim = kind == 1 ? p.dG : p.dH;                // columns of X, all reduced over
+    const float* Y = kind == 0 ? p.Wq : p.Wk;                // fp32 operand of A and Bm
+    const int n_cols = kind == 2 ? p.n : p.dc;
+    const int chunks = (kdim + FF_K - 1) / FF_K;
+    const int per = (chunks + FF_CLUSTER - 1) / FF_CLUSTER;
+    const int ch0 = min(chunks, rank * per), ch1 = min(chunks, ch0 + per);
+
+    pdl_wait();
+    pdl_launch_dependents();
+    auto load = [&](int ch) {
+        if (ch < ch1) {
+            uint8_t* sx = ff_smem + ((ch - ch0) % FF_STAGES) * (FF_XBYTES + FF_YBYTES);
+            uint8_t* sy = sx + FF_XBYTES;
+            const int k0 = ch * FF_K;
+            static_assert(FF_M * (FF_K / 8) == FF_THREADS && FF_N * (FF_K / 8) == FF_THREADS, "one 16-byte copy of bf16 rows per thread");
+            {
+                const int r = tid / (FF_K / 8), c = tid % (FF_K / 8), k = k0 + c * 8;
+                const bool ok = r0 + r < p.n && k < kdim;
+                cp_async16(reinterpret_cast<uint4*>(sx) + swz<FF_K / 8>(r, c), X + (ok ? (int64_t)(r0 + r) * kdim + k : 0), ok ? 16 : 0);
+            }
+            if (kind == 2) {
+                // row m of K, the column of the head's group (a 16-byte chunk stays inside a head)
+                const int r = tid / (FF_K / 8), c = tid % (FF_K / 8), k = k0 + c * 8;
+                const bool ok = c0 + r < p.n && k < kdim;
+                const int g = k / p.d / p.G;
+                cp_async16(sy + r * FF_YROW16 + c * 16, p.K + (ok ? (int64_t)(c0 + r) * p.dG + g * p.d + k % p.d : 0), ok ? 16 : 0);
+            } else {
+#pragma unroll
+                for (int i = tid; i < FF_N * (FF_K / 4); i += FF_THREADS) {
+                    const int r = i / (FF_K / 4), c = i % (FF_K / 4), k = k0 + c * 4;
+                    const bool ok = c0 + r < p.dc && k < kdim;
+                    cp_async16(sy + r * FF_YROW + c * 16, Y + (ok ? (int64_t)(c0 + r) * kdim + k : 0), ok ? 16 : 0);
+                }
+            }
+        }
+        cp_async_commit();
+    };
+#pragma unroll
+    for (int s = 0; s < FF_STAGES - 1; ++s) load(ch0 + s);
+
+    // warps: 4 groups of 8 columns x 2 halves of a chunk's reduction (every weight is cut into pieces by one warp)
+    constexpr int KQ = FF_THREADS / 128;
+    const int wn = (warp & 3) * 8, kh = (warp >> 2) * (FF_K / 16 / KQ);
+    float sum[FF_M / 16][4];
+#pragma unroll
+    for (int m = 0; m < FF_M / 16; ++m)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) sum[m][e] = 0.f;
+    for (int ch = ch0; ch < ch1; ++ch) {
+        cp_async_wait<FF_STAGES - 2>();
+        __syncthreads();                                     // chunk ch has landed; everybody is done with chunk ch - 1
+        load(ch + FF_STAGES - 1);
+        const uint8_t* sx = ff_smem + ((ch - ch0) % FF_STAGES) * (FF_XBYTES + FF_YBYTES);
+        const uint8_t* sy = sx + FF_XBYTES;
+        float acc[3][FF_M / 16][4];
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+#pragma unroll
+            for (int m = 0; m < FF_M / 16; ++m)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) acc[q][m][e] = 0.f;
+#pragma unroll
+        for (int kk = 0; kk < FF_K / 16 / KQ; ++kk) {
+            const int ks = kh + kk;
+            uint32_t a[FF_M / 16][4];
+#pragma unroll
+            for (int m = 0; m < FF_M / 16; ++m) load_a_frag<FF_K / 8>(a[m], reinterpret_cast<const uint4*>(sx), m * 16, ks * 2, lane);
+            const int row = wn + (lane >> 2), k = ks * 16 + (lane & 3) * 2;
+            if (kind == 2) {
+                const uint32_t b0 = *reinterpret_cast<const uint32_t*>(sy + row * FF_YROW16 + k * 2);
+                const uint32_t b1 = *reinterpret_cast<const uint32_t*>(sy + row * FF_YROW16 + (k + 8) * 2);
+#pragma unroll
+                for (int m = 0; m < FF_M / 16; ++m) mma_bf16_16816(acc[0][m], a[m], b0, b1);
+            } else {
+                const float2 f0 = *reinterpret_cast<const float2*>(sy + row * FF_YROW + k * 4);
+                const float2 f1 = *reinterpret_cast<const float2*>(sy + row * FF_YROW + (k + 8) * 4);
+                uint32_t b0[3], b1[3];
+                split3(f0.x, f0.y, b0);
+                split3(f1.x, f1.y, b1);
+#pragma unroll
+                for (int q = 0; q < 3; ++q)
+#pragma unroll
+                    for (int m = 0; m < FF_M / 16; ++m) mma_bf16_16816(acc[q][m], a[m], b0[q], b1[q]);
+            }
+        }
+#pragma unroll
+        for (int m = 0; m < FF_M / 16; ++m)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) sum[m][e] += (acc[2][m][e] + acc[1][m][e]) + acc[0][m][e];
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+    float* part = reinterpret_cast<float*>(ff_smem);         // [KQ][FF_M][FF_N]
+#pragma unroll
+    for (int m = 0; m < FF_M / 16; ++m) {
+        float* dst = part + (warp >> 2) * (FF_M * FF_N) + (m * 16 + (lane >> 2)) * FF_N + wn + (lane & 3) * 2;
+        *reinterpret_cast<float2*>(dst) = make_float2(sum[m][0], sum[m][1]);
+        *reinterpret_cast<float2*>(dst + 8 * FF_N) = make_float2(sum[m][2], sum[m][3]);
+    }
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();
+    // a thread adds one half of an element over the ranks; the halves meet through shared memory
+    constexpr int FF_BAND = FF_M * FF_N / FF_CLUSTER;        // elements this CTA adds up
+    static_assert(FF_BAND * KQ == FF_THREADS, "one half of an element per thread");
+    __shared__ float half[KQ][FF_BAND];
+    {
+        const int e = rank * FF_BAND + tid % FF_BAND, kq = tid / FF_BAND;
+        float v[FF_CLUSTER];
+#pragma unroll
+        for (int j = 0; j < FF_CLUSTER; ++j) v[j] = cluster.map_shared_rank(part, j)[kq * (FF_M * FF_N) + e];
+        float s = 0.f;
+#pragma unroll
+        for (int j = 0; j < FF_CLUSTER; ++j) s += v[j];
+        half[kq][tid % FF_BAND] = s;
+    }
+    __syncthreads();
+    if (tid < FF_BAND) {
+        const int e = rank * FF_BAND + tid, r = r0 + e / FF_N, c = c0 + e % FF_N;
+        const float s = half[0][tid] + half[1][tid];
+        if (r < p.n && c < n_cols) {
+            if (kind == 0) p.A[(int64_t)r * p.dc + c] = s + p.bq[c];
+            else if (kind == 1) p.Bm[(int64_t)r * p.dc + c] = s + p.bk[c];
+            else p.T[(int64_t)r * p.n + c] = s;
+        }
+    }
+    cluster.sync();          // shared memory stays alive until every remote read is done
+}
+
+// ---------------------------------------------------------------------------
+// Launch 2: the n x n part.  A CTA owns FP_R pairs: side 0 takes rows of A (E row by row, its share of the loss,
+// the rows of dA), side 1 rows of Bm (E^T, the rows of dBm), each against the whole other matrix, FP_C rows of it
+// at a time in shared memory.  Two pairs a CTA (128 CTAs for 128 pairs) and four threads per column, each a quarter
+// of the reduction: with four pairs and two threads the kernel took 9 us of mostly waiting warps.  The result leaves
+// as three bf16 pieces, ready for the next launch's tensor-core operand.
+// ---------------------------------------------------------------------------
+constexpr int FP_R = 2, FP_C = 128, FP_DC = 128, FP_Q = 4, FP_THREADS = FP_Q * FP_C;
+constexpr int FP_SMEM = (FP_C * (FP_DC + 4) + FP_R * FP_DC + (1 + FP_Q) * FP_C * FP_R) * 4;
+
+__global__ void __launch_bounds__(FP_THREADS) fit_pairs_kernel(FitParams p) {
+    extern __shared__ __align__(128) float fp_smem[];
+    float* sY = fp_smem;                                     // [FP_C][dc + 4]
+    float* sX = sY + FP_C * (FP_DC + 4);                     // [FP_R][dc]
+    float2* sP = reinterpret_cast<float2*>(sX + FP_R * FP_DC);   // [FP_C] dP of the two pairs
+    float2* sE = sP + FP_C;                                  // [FP_Q][FP_C] quarters of the sums
+    __shared__ float red[FP_C / 32];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int side = blockIdx.y, r0 = blockIdx.x * FP_R;
+    const int n = p.n, dc = p.dc, ldy = dc + 4, q4 = dc / 4;
+    const int col = tid % FP_C, quarter = tid / FP_C;        // E column / dX column; quarter of the reduction
+    const float inv = 1.f / ((float)n * (float)n);
+    pdl_wait();
+    pdl_launch_dependents();
+    const float* X = side == 0 ? p.A : p.Bm;
+    const float* Y = side == 0 ? p.Bm : p.A;
+    if (tid < FP_R * 32 && lane < q4) {
+        const bool ok = r0 + tid / 32 < n;
+        cp_async16(sX + (tid / 32) * dc + lane * 4, X + (ok ? (int64_t)(r0 + tid / 32) * dc + lane * 4 : 0), ok ? 16 : 0);
+    }
+    float2 dx = make_float2(0.f, 0.f);
+    float loss = 0.f;
+    for (int m0 = 0; m0 < n; m0 += FP_C) {
+        if (lane < q4) {                                     // a warp takes a row: dc / 4 <= 32 pieces of 16 bytes
+#pragma unroll
+            for (int r = tid >> 5; r < FP_C; r += FP_THREADS / 32) {
+                const bool ok = m0 + r < n;
+                cp_async16(sY + r * ldy + lane * 4, Y + (ok ? (int64_t)(m0 + r) * dc + lane * 4 : 0), ok ? 16 : 0);
+            }
+        }
+        cp_async_commit();
+        const int m = m0 + col;
+        float t[FP_R] = {0.f, 0.f};
+        if (quarter == 0 && m < n) {
+#pragma unroll
+            for (int r = 0; r < FP_R; ++r)
+                if (r0 + r < n) t[r] = __ldcg(p.T + (side == 0 ? (int64_t)(r0 + r) * n + m : (int64_t)m * n + r0 + r));
+        }
+        cp_async_wait<0>();
+        __syncthreads();
+        float2 e = make_float2(0.f, 0.f);
+        {
+            const float4* y = reinterpret_cast<const float4*>(sY + col * ldy) + quarter * (q4 / FP_Q);
+            const float4* x = reinterpret_cast<const float4*>(sX) + quarter * (q4 / FP_Q);
+#pragma unroll 8
+            for (int c = 0; c < q4 / FP_Q; ++c) {
+                const float4 b = y[c], a0 = x[c], a1 = x[q4 + c];
+                e.x = fmaf(a0.x, b.x, e.x); e.y = fmaf(a1.x, b.x, e.y);
+                e.x = fmaf(a0.y, b.y, e.x); e.y = fmaf(a1.y, b.y, e.y);
+                e.x = fmaf(a0.z, b.z, e.x); e.y = fmaf(a1.z, b.z, e.y);
+                e.x = fmaf(a0.w, b.w, e.x); e.y = fmaf(a1.w, b.w, e.y);
+            }
+        }
+        sE[quarter * FP_C + col] = e;
+        __syncthreads();
+        if (quarter == 0) {
+            const float2 e1 = sE[FP_C + col], e2 = sE[2 * FP_C + col], e3 = sE[3 * FP_C + col];
+            const float v0 = (m < n && r0 < n) ? ((e.x + e1.x) + (e2.x + e3.x)) - t[0] : 0.f;
+            const float v1 = (m < n && r0 + 1 < n) ? ((e.y + e1.y) + (e2.y + e3.y)) - t[1] : 0.f;
+            loss += v0 * v0 + v1 * v1;
+            sP[col] = make_float2(2.f * v0 * inv, 2.f * v1 * inv);
+        }
+        __syncthreads();
+        if (col < dc) {
+            const float* y = sY + quarter * (FP_C / FP_Q) * ldy + col;
+            const float2* q = sP + quarter * (FP_C / FP_Q);
+#pragma unroll 8
+            for (int i = 0; i < FP_C / FP_Q; ++i) {
+                const float b = y[i * ldy];
+                const float2 a = q[i];
+                dx.x = fmaf(a.x, b, dx.x);
+                dx.y = fmaf(a.y, b, dx.y);
+            }
+        }
+        __syncthreads();
+    }
+    sE[quarter * FP_C + col] = dx;
+    if (side == 0 && quarter == 0) {
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+        if (lane == 0) red[tid >> 5] = loss;
+    }
+    __syncthreads();
+    if (quarter < FP_R && col < dc && r0 + quarter < n) {    // quarters 0 and 1 write one pair's row each
+        const float* e = reinterpret_cast<const float*>(sE) + 2 * col + quarter;
+        float v = (e[0] + e[2 * FP_C]) + (e[4 * FP_C] + e[6 * FP_C]);
+        __nv_bfloat16* out = side == 0 ? p.dA : p.dBm;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            const __nv_bfloat16 w = __float2bfloat16_rn(v);
+            out[((int64_t)i * n + r0 + quarter) * dc + col] = w;
+            v -= __bfloat162float(w);
+        }
+    }
+    if (side == 0 && tid == 0) p.loss_part[blockIdx.x] = ((red[0] + red[1]) + (red[2] + red[3])) * inv;
+}
+
+// ---------------------------------------------------------------------------
+// Launch 3: gradients and Adam.  A CTA owns a FU_J x FU_N tile of W_q or W_k: its gradient, reduced over the pairs,
+// stays in the accumulators and the update is applied from there, so gradients never go to memory.  Tiles of 32 x 128
+// read the least (6 bytes per feature and pair in pieces, 2 per column and pair: 56 KB a CTA for 128 pairs, against
+// 104 KB for 128 x 32, which took 10 us where this takes 6) and update whole 512-byte row segments.  The parameters
+// and moments of the tile are requested first: they were last written by the launch before the last but one.  The
+// last two CTAs do the biases, and add up the loss.
+// ---------------------------------------------------------------------------
+constexpr int FU_J = 32, FU_N = 128, FU_C = 64, FU_DC = 128, FU_STAGES = 2, FU_THREADS = 512;
+constexpr int FU_PBYTES = FU_C * FU_J * 2;                  // one piece of FU_C gradient rows
+constexpr int FU_STAGE = 3 * FU_PBYTES + FU_C * FU_N * 2;
+constexpr int FU_SMEM = FU_STAGES * FU_STAGE;
+
+__device__ __forceinline__ void adam(float& w, float& a, float& b, float gr, const FitParams& p) {
+    a = p.beta1 * a + (1.f - p.beta1) * gr;
+    b = p.beta2 * b + (1.f - p.beta2) * gr * gr;
+    w -= p.lr * (a * p.ic1) / (sqrtf(b * p.ic2) + p.eps);
+}
+
+__global__ void __launch_bounds__(FU_THREADS, 2) fit_update_kernel(FitParams p) {
+    extern __shared__ __align__(128) uint8_t fu_smem[];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n = p.n, dc = p.dc, jt = (dc + FU_J - 1) / FU_J;
+    const int q_ctas = (p.dH + FU_N - 1) / FU_N * jt, k_ctas = (p.dG + FU_N - 1) / FU_N * jt;
+    int cta = blockIdx.x;
+    if (cta >= q_ctas + k_ctas) {
+        // ---- bias of one side: column sums of its gradient rows; threads = 32 groups of rows x 16 chunks of 8 columns
+        const int side = cta - q_ctas - k_ctas;
+        float(*sum)[FU_DC] = reinterpret_cast<float(*)[FU_DC]>(fu_smem);
+        pdl_wait();
+        pdl_launch_dependents();
+        const __nv_bfloat16* src = side == 0 ? p.dA : p.dBm;
+        const int c8 = (tid & 15) * 8, grp = tid >> 4;
+        float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (c8 < dc) {
+#pragma unroll 4
+            for (int r = grp; r < n; r += FU_THREADS / 16) {
+                uint4 w[3];
+#pragma unroll
+                for (int i = 0; i < 3; ++i) w[i] = __ldcg(reinterpret_cast<const uint4*>(src + ((int64_t)i * n + r) * dc + c8));
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 x = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(&w[0])[j]);
+                    const float2 y = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(&w[1])[j]);
+                    const float2 z = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(&w[2])[j]);
+                    v[2 * j] += (z.x + y.x) + x.x;
+                    v[2 * j + 1] += (z.y + y.y) + x.y;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) sum[grp][c8 + j] = v[j];
+        }
+        __syncthreads();
+        if (tid < dc) {
+            float g = 0.f;
+#pragma unroll
+            for (int i = 0; i < FU_THREADS / 16; ++i) g += sum[i][tid];
+            float* b = side == 0 ? p.bq : p.bk;
+            const int64_t off = b - p.Wq + tid;
+            float a1 = p.m1[off], a2 = p.m2[off], w = b[tid];
+            adam(w, a1, a2, g, p);
+            b[tid] = w; p.m1[off] = a1; p.m2[off] = a2;
+        }
+        if (side == 0 && warp == 7 && p.loss_out) {
+            const int bands = (n + FP_R - 1) / FP_R;
+            float s = 0.f;
+            for (int i = lane; i < bands; i += 32) s += __ldcg(p.loss_part + i);
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (lane == 0) *p.loss_out = s;
+        }
+        return;
+    }
+    const bool qs = cta < q_ctas;
+    if (!qs) cta -= q_ctas;
+    const int ld = qs ? p.dH : p.dG, i0 = cta / jt * FU_N, jb = cta % jt * FU_J;
+    const __nv_bfloat16* X = qs ? p.Q : p.K;
+    const __nv_bfloat16* D = qs ? p.dA : p.dBm;
+    float* W = qs ? p.Wq : p.Wk;
+    const int64_t base = W - p.Wq;
+
+    // this thread's elements of the tile: rows jb + warp + 16 u, four columns
+    const int jr = jb + warp, ic = lane * 4;
+    const bool col_ok = i0 + ic < ld;
+    float4 w[FU_J / 16], a1[FU_J / 16], a2[FU_J / 16];
+#pragma unroll
+    for (int u = 0; u < FU_J / 16; ++u) {
+        const bool ok = col_ok && jr + 16 * u < dc;
+        const int64_t off = base + (ok ? (int64_t)(jr + 16 * u) * ld + i0 + ic : 0);
+        w[u] = __ldcg(reinterpret_cast<const float4*>(p.Wq + off));
+        a1[u] = __ldcg(reinterpret_cast<const float4*>(p.m1 + off));
+        a2[u] = __ldcg(reinterpret_cast<const float4*>(p.m2 + off));
+    }
+    pdl_wait();
+    pdl_launch_dependents();
+    auto load = [&](int c0) {
+        if (c0 < n) {
+            uint8_t* st = fu_smem + ((c0 / FU_C) % FU_STAGES) * FU_STAGE;
+#pragma unroll
+            for (int i = tid; i < 3 * FU_C * (FU_J / 8); i += FU_THREADS) {
+                const int q = i / (FU_C * (FU_J / 8)), r = i / (FU_J / 8) % FU_C, c = i % (FU_J / 8);
+                const bool ok = c0 + r < n && jb + c * 8 < dc;
+                cp_async16(reinterpret_cast<uint4*>(st + q * FU_PBYTES) + swz<FU_J / 8>(r, c),
+                           D + (ok ? ((int64_t)q * n + c0 + r) * dc + jb + c * 8 : 0), ok ? 16 : 0);
+            }
+#pragma unroll
+            for (int i = tid; i < FU_C * (FU_N / 8); i += FU_THREADS) {
+                const int r = i / (FU_N / 8), c = i % (FU_N / 8);
+                const bool ok = c0 + r < n && i0 + c * 8 < ld;
+                cp_async16(reinterpret_cast<uint4*>(st + 3 * FU_PBYTES) + swz<FU_N / 8>(r, c),
+                           X + (ok ? (int64_t)(c0 + r) * ld + i0 + c * 8 : 0), ok ? 16 : 0);
+            }
+        }
+        cp_async_commit();
+    };
+    // warps: 2 groups of 16 features x 8 of 16 columns
+    const int wj = (warp & 1) * 16, wi = (warp >> 1) * 16;
+    float g[2][4];
+#pragma unroll
+    for (int nb = 0; nb < 2; ++nb)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) g[nb][e] = 0.f;
+    load(0);
+    for (int c0 = 0; c0 < n; c0 += FU_C) {
+        load(c0 + FU_C);
+        cp_async_wait<1>();
+        __syncthreads();
+        const uint8_t* st = fu_smem + ((c0 / FU_C) % FU_STAGES) * FU_STAGE;
+        {
+            const uint4* tx = reinterpret_cast<const uint4*>(st + 3 * FU_PBYTES);
+#pragma unroll
+            for (int q = 2; q >= 0; --q) {
+                float acc[2][4];
+#pragma unroll
+                for (int nb = 0; nb < 2; ++nb)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) acc[nb][e] = 0.f;
+#pragma unroll
+                for (int ks = 0; ks < FU_C / 16; ++ks) {
+                    uint32_t b[4];
+                    load_b_frag_kn<FU_N / 8>(b, tx, ks * 16, wi / 8, lane);
+                    // A = transposed rows of the gradient: 16 features x 16 pairs
+                    uint32_t a[4];
+                    const int r = ks * 16 + (lane & 7) + ((lane >> 4) & 1) * 8, c = wj / 8 + ((lane >> 3) & 1);
+                    ldmatrix_x4_trans(a, reinterpret_cast<const uint4*>(st + q * FU_PBYTES) + swz<FU_J / 8>(r, c));
+                    mma_bf16_16816(acc[0], a, b[0], b[1]);
+                    mma_bf16_16816(acc[1], a, b[2], b[3]);
+                }
+#pragma unroll
+                for (int nb = 0; nb < 2; ++nb)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) g[nb][e] += acc[nb][e];
+            }
+        }
+        __syncthreads();
+    }
+    cp_async_wait<0>();
+    // gradient tile -> shared memory (the stages are idle), row stride FU_N + 4
+    float* sg = reinterpret_cast<float*>(fu_smem);
+    {
+#pragma unroll
+        for (int nb = 0; nb < 2; ++nb) {
+            float* d = sg + (wj + (lane >> 2)) * (FU_N + 4) + wi + nb * 8 + (lane & 3) * 2;
+            *reinterpret_cast<float2*>(d) = make_float2(g[nb][0], g[nb][1]);
+            *reinterpret_cast<float2*>(d + 8 * (FU_N + 4)) = make_float2(g[nb][2], g[nb][3]);
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < FU_J / 16; ++u) {
+        if (!col_ok || jr + 16 * u >= dc) continue;
+        const int64_t off = base + (int64_t)(jr + 16 * u) * ld + i0 + ic;
+        const float4 gr = *reinterpret_cast<const float4*>(sg + (warp + 16 * u) * (FU_N + 4) + ic);
+        adam(w[u].x, a1[u].x, a2[u].x, gr.x, p);
+        adam(w[u].y, a1[u].y, a2[u].y, gr.y, p);
+        adam(w[u].z, a1[u].z, a2[u].z, gr.z, p);
+        adam(w[u].w, a1[u].w, a2[u].w, gr.w, p);
+        *reinterpret_cast<float4*>(p.Wq + off) = w[u];
+        *reinterpret_cast<float4*>(p.m1 + off) = a1[u];
+        *reinterpret_cast<float4*>(p.m2 + off) = a2[u];
+    }
+}
+
+cudaError_t launch_fit_step(int device, const FitParams& p, cudaStream_t st) {
+    static KernelMemo memo1, memo2, memo3;
+    cudaError_t e = allow_smem(fit_forward_kernel, device, FF_SMEM, memo1);
+    if (e == cudaSuccess) e = allow_smem(fit_pairs_kernel, device, FP_SMEM, memo2);
+    if (e == cudaSuccess) e = allow_smem(fit_update_kernel, device, FU_SMEM, memo3);
+    if (e != cudaSuccess) return e;
+    const int row_tiles = (p.n + FF_M - 1) / FF_M, dc_tiles = (p.dc + FF_N - 1) / FF_N, pair_tiles = (p.n + FF_N - 1) / FF_N;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(FF_CLUSTER, row_tiles * (2 * dc_tiles + pair_tiles));
+    cfg.blockDim = dim3(FF_THREADS);
+    cfg.dynamicSmemBytes = FF_SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = FF_CLUSTER;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    e = cudaLaunchKernelEx(&cfg, fit_forward_kernel, p);
+    if (e == cudaSuccess) e = launch_pdl(fit_pairs_kernel, dim3((p.n + FP_R - 1) / FP_R, 2), dim3(FP_THREADS), FP_SMEM, st, p);
+    if (e == cudaSuccess)
+        e = launch_pdl(fit_update_kernel, dim3(((p.dH + FU_N - 1) / FU_N + (p.dG + FU_N - 1) / FU_N) * ((p.dc + FU_J - 1) / FU_J) + 2), dim3(FU_THREADS), FU_SMEM, st, p);
+    return e;
+}
+
+// The kernels above want d' a multiple of 16 up to 128 (what the selection kernels take) and head dimensions that are
+// multiples of 16 (16-byte copies); other shapes run on the generic fp32 product kernel below.
+bool fit_is_fast(int d, int dc) { return d % 16 == 0 && dc % 16 == 0 && dc <= FP_DC; }
+
+// ---------------------------------------------------------------------------
+// Any shape.
+// ---------------------------------------------------------------------------
 constexpr int GT = 64;            // output tile of the generic product kernel
 constexpr int GK = 16;
 
@@ -215,7 +736,8 @@ esa_status esa_fit_create(const esa_config* cfg, int32_t batch, float lr, esa_fi
     f->n_params = (size_t)f->dc * f->dH + f->dc + (size_t)f->dc * f->dG + f->dc;
     const size_t n = batch, dc = f->dc;
     const size_t part_floats = 32 * (n * n > n * dc ? n * n : n * dc);
-    const size_t floats = 4 * f->n_params + n * f->dG + 2 * n * n + 4 * n * dc + part_floats + 64;
+    const size_t piece_floats = (3 * n * dc + 1) / 2 + 4;      // 3 n dc bf16 values, rounded up
+    const size_t floats = 4 * f->n_params + n * f->dG + 2 * n * n + 4 * n * dc + part_floats + 2 * piece_floats + n + 128;
     if (cudaGetDevice(&f->device) != cudaSuccess || cudaMalloc(&f->base, floats * sizeof(float)) != cudaSuccess) {
         cudaGetLastError();
         delete f;
@@ -223,14 +745,20 @@ esa_status esa_fit_create(const esa_config* cfg, int32_t batch, float lr, esa_fi
     }
     float* p = reinterpret_cast<float*>(f->base);
     f->params = p; p += f->n_params;
-    f->grads = p; p += f->n_params;
     f->m1 = p; p += f->n_params;
     f->m2 = p; p += f->n_params;
+    f->A = p; p += n * dc;
+    f->Bm = p; p += n * dc;
+    auto align16 = [&](float* q) { return q + (4 - (q - reinterpret_cast<float*>(f->base)) % 4) % 4; };
+    p = align16(p);
+    f->dA3 = reinterpret_cast<__nv_bfloat16*>(p); p += piece_floats;
+    p = align16(p);
+    f->dBm3 = reinterpret_cast<__nv_bfloat16*>(p); p += piece_floats;
+    f->loss_part = p; p += n;
+    f->grads = p; p += f->n_params;
     f->Qf = p; p += n * f->dG;
     f->T = p; p += n * n;
     f->dP = p; p += n * n;
-    f->A = p; p += n * dc;
-    f->Bm = p; p += n * dc;
     f->dA = p; p += n * dc;
     f->dBm = p; p += n * dc;
     f->part = p; p += part_floats;
@@ -263,7 +791,7 @@ esa_status esa_fit_set_weights(esa_fit* f, const float* Wq, const float* bq, con
     size_t owq, obq, owk, obk;
     fit_offsets(f, &owq, &obq, &owk, &obk);
     // parameters, and a fresh optimiser state
-    if (cudaMemset(f->params, 0, 4 * f->n_params * sizeof(float)) != cudaSuccess) return ESA_ERR_CUDA;
+    if (cudaMemset(f->params, 0, 3 * f->n_params * sizeof(float)) != cudaSuccess) return ESA_ERR_CUDA;
     if (cudaMemcpy(f->params + owq, Wq, sizeof(float) * f->dc * f->dH, cudaMemcpyHostToDevice) != cudaSuccess) return ESA_ERR_CUDA;
     if (cudaMemcpy(f->params + owk, Wk, sizeof(float) * f->dc * f->dG, cudaMemcpyHostToDevice) != cudaSuccess) return ESA_ERR_CUDA;
     if (bq && cudaMemcpy(f->params + obq, bq, sizeof(float) * f->dc, cudaMemcpyHostToDevice) != cudaSuccess) return ESA_ERR_CUDA;
@@ -294,6 +822,18 @@ esa_status esa_fit_step_async(esa_fit* f, const void* Q_batch, const void* K_bat
     fit_offsets(f, &owq, &obq, &owk, &obk);
     float *Wq = f->params + owq, *bq = f->params + obq, *Wk = f->params + owk, *bk = f->params + obk;
     const int dc = f->dc, dH = f->dH, dG = f->dG;
+    if (fit_is_fast(f->d, dc) && ((reinterpret_cast<uintptr_t>(Q) | reinterpret_cast<uintptr_t>(K)) & 15) == 0) {
+        FitParams p;
+        p.Q = Q; p.K = K; p.Wq = Wq; p.bq = bq; p.Wk = Wk; p.bk = bk; p.m1 = f->m1; p.m2 = f->m2;
+        p.A = f->A; p.Bm = f->Bm; p.T = f->T; p.dA = f->dA3; p.dBm = f->dBm3; p.loss_part = f->loss_part; p.loss_out = loss_out;
+        p.n = n; p.dc = dc; p.dH = dH; p.dG = dG; p.d = f->d; p.G = f->H / f->HG;
+        p.lr = f->lr; p.beta1 = f->beta1; p.beta2 = f->beta2; p.eps = f->eps;
+        f->step += 1;
+        p.ic1 = 1.f / (1.f - std::pow(f->beta1, (float)f->step));
+        p.ic2 = 1.f / (1.f - std::pow(f->beta2, (float)f->step));
+        f->launches += 3;
+        return launch_fit_step(f->device, p, st) == cudaSuccess ? ESA_OK : ESA_ERR_CUDA;
+    }
     // targets (Eq. 3 for every pair)
     fit_fold_kernel<<<(unsigned)(((int64_t)n * dG + 255) / 256), 256, 0, st>>>(Q, f->Qf, n, f->H, f->HG, f->d);
     int launches = 5;                                  // fold, loss, two column sums, Adam

@@ -55,6 +55,22 @@ def test_fit_steps_follow_the_oracle(name, n, steps):
         assert d.max() <= 2.5 * lr, f"{key}: largest difference {d.max():.3e}"
 
 
+@pytest.mark.parametrize("kw,n,steps", [
+    (dict(), 1, 4), (dict(), 33, 4), (dict(), 130, 3),                     # tiles of 32 pairs and features, 64 and 128 pairs a pass
+    (dict(H=28, H_G=4, d=128, d_c=128), 257, 2), (dict(d_c=16), 64, 3), (dict(d_c=80), 96, 3),
+    (dict(d_c=24), 40, 3), (dict(d=24, H=4, H_G=2), 40, 3)])               # (the generic kernels)
+def test_fit_steps_at_tile_edges(kw, n, steps):
+    """Sizes around the tiles of the fitting kernels, against the oracle within the tolerance of the test above."""
+    cfg = syn.get_config("c1").with_(**kw)
+    losses, got, want = _run(cfg, n, steps, 5e-4, seed=5)
+    for it, (a, b) in enumerate(losses):
+        assert abs(a - b) <= 2e-4 * abs(b), f"loss of step {it}: {a} against {b}"
+    for key in want:
+        d = np.abs(got[key].astype(np.float64) - want[key])
+        assert (d > 2e-6 + 1e-4 * np.abs(want[key])).mean() <= 2e-3, key
+        assert d.max() <= 2.5 * 5e-4, key
+
+
 def test_fitting_lowers_the_loss_and_raises_the_recall_of_the_selection():
     """A short fit on the mixture workload: the loss falls, and the selection made with the fitted
     compressors recovers more of the full-dimension selection (Fig. 3's recall) than the one made
