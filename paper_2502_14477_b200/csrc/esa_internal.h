@@ -199,6 +199,9 @@ cudaError_t launch_score(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_c
 cudaError_t launch_score_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache,
                             const SeqMeta& meta, int max_lM, cudaStream_t st, bool* pooled_ready);
 
+cudaError_t launch_score_tc_heads(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* K, const SeqMeta& meta,
+                                  int max_lM, cudaStream_t st);
+
 // Eq. 8 (unless pooled_ready) + Eq. 2 -> idx_out / n_sel_out.  mapped: ctx->pkey holds the pooled RAW scores of a
 // single query per sequence and ctx->rkey[b] its maximum (the decode scoring kernel's output).
 cudaError_t launch_select(esa_ctx* ctx, int B, bool mapped, const SeqMeta& meta, int max_lM, bool pooled_ready,

@@ -32,6 +32,8 @@
 //
 // Chunks of more than 512 queries run as groups of 512 (grid.y); pass 2 then combines the
 // groups by an atomic maximum on the unpooled scores and the pooling is left to a later kernel.
+// The per-head vote of Section 4.3 is the same with one group per head: the operands are then the
+// head's columns of the uncompressed queries and keys (d in the place of d').
 //
 // Warp roles: warp 0 issues the TMA loads, warps 1-2 issue the MMAs (converged, lane 0 leads;
 // pass 2 uses warp 1 only), warps 3-10 run the epilogue: two groups of four warps (one TMEM lane
@@ -55,15 +57,18 @@ constexpr int ST_ONES_BYTES = ST_KEYS * 32;    // ninth k-step, key side: 128 ro
 constexpr int ST_RT_BYTES = ST_QCAP * 32;      // ninth k-step, query side: 512 rows x 16 bf16
 
 struct ScoreTcParams {
-    uint32_t* rkey;     // [B, l_C] ordered keys of r_c
-    uint32_t* skey;     // [B, max_tokens] ordered keys of s_m (index = m - i_end); used when q_groups > 1
-    uint32_t* pkey;     // [B, max_tokens] ordered keys of s'_m; written when q_groups == 1
+    uint32_t* rkey;     // [B, heads, l_C] ordered keys of r_c
+    uint32_t* skey;     // [B, max_tokens] ordered keys of s_m (index = m - i_end); used when !pool
+    uint32_t* pkey;     // [B, max_tokens] ordered keys of s'_m; written when pool
     uint32_t* ghist0;   // [B, ST_BINS] histogram of the top 11 bits of pkey; zeroed by pass 1
     int* status;
     int64_t max_tokens;
     int l_C;
     int eps;
-    int q_groups;       // groups of up to ST_QCAP queries (gridDim.y)
+    int groups;         // gridDim.y: heads x groups of up to ST_QCAP queries
+    int heads;          // 1 (compressed scores), or H: every head scores by itself (Section 4.3's vote)
+    int G;              // heads > 1: query heads per key/value head
+    int pool;           // pass 2 pools and writes pkey and ghist0 (one group per sequence), else skey
     SeqMeta meta;
 };
 
@@ -128,13 +133,21 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
     const int tid = threadIdx.x, lane = tid & 31;
     const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
     const int b = blockIdx.z;
-    const int q0 = blockIdx.y * ST_QCAP;
+    int q0 = blockIdx.y * ST_QCAP, qx = 0, kx = 0;
+    uint32_t* rkey = p.rkey + (int64_t)b * p.heads * p.l_C;
+    if (p.heads > 1) {                                     // this head's columns, its row maxima
+        const int head = blockIdx.y % p.heads;
+        q0 = blockIdx.y / p.heads * ST_QCAP;
+        qx = head * DC;
+        kx = head / p.G * DC;
+        rkey += (int64_t)head * p.l_C;
+    }
     const int nq = min(ST_QCAP, p.l_C - q0);
     const int NU = (nq + UNIT - 1) / UNIT;                 // items per key tile
     const int i_end = p.meta.i_end[b];
     const int l_M = p.meta.m_end[b] - i_end;
     const int eps = p.eps;
-    const bool fused = PASS == 2 && p.q_groups == 1;
+    const bool fused = PASS == 2 && p.pool;
 
     // ---- this CTA's keys: local tile lt covers keys [key_first + 128 lt, + 128); its items are
     // w = 0 .. n_items - 1 with (tile, unit) = divmod(w + woff, NU)
@@ -204,7 +217,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
                 mbar_arrive_expect_tx(bar(C::B_FULL + s), TILE_BYTES);
 #pragma unroll
                 for (int blk = 0; blk < NBLK; ++blk)
-                    tma_load_2d(smem_u32(sK + s * TILE_BYTES + blk * (ST_KEYS * 128)), &kmap, blk * 64,
+                    tma_load_2d(smem_u32(sK + s * TILE_BYTES + blk * (ST_KEYS * 128)), &kmap, kx + blk * 64,
                                 (int)(row_base + key_first + (int64_t)lt * ST_KEYS), bar(C::B_FULL + s));
             };
             const int first = min(n_ltiles, STAGES);
@@ -217,7 +230,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
                 for (int blk = 0; blk < NBLK; ++blk)
 #pragma unroll
                     for (int r0 = 0; r0 < UNIT; r0 += 128)
-                        tma_load_2d(smem_u32(sQ + blk * (ST_QCAP * 128) + (u * UNIT + r0) * 128), &qmap, blk * 64,
+                        tma_load_2d(smem_u32(sQ + blk * (ST_QCAP * 128) + (u * UNIT + r0) * 128), &qmap, qx + blk * 64,
                                     b * p.l_C + q0 + u * UNIT + r0, bar(C::B_QFULL + u));
             }
             for (int lt = first; lt < n_ltiles; ++lt) load_tile(lt);
@@ -298,7 +311,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
             for (int i = e256; i < ST_QCAP; i += ST_EPI) {
                 uint32_t w01 = 0x0000ff80u, w2 = 0u;       // (-inf, 0), (0, 0)
                 if (i < nq) {
-                    const float r = key_to_f32(p.rkey[(int64_t)b * p.l_C + q0 + i]);
+                    const float r = key_to_f32(rkey[q0 + i]);
                     const __nv_bfloat16 r1 = __float2bfloat16_rn(r);
                     const float d1 = r - __bfloat162float(r1);
                     const __nv_bfloat16 r2 = __float2bfloat16_rn(d1);
@@ -328,7 +341,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
                 tmem_ld32(tbase + buf * ACC_COLS + c0, v);
                 tmem_ld32(tbase + buf * ACC_COLS + c0 + 32, v + 32);
                 // (groups of queries: group 0 zeroes the words the groups of pass 2 combine into)
-                if (p.q_groups > 1 && blockIdx.y == 0 && eg == 0 && key0 + et < l_M)
+                if (!p.pool && blockIdx.y == 0 && eg == 0 && key0 + et < l_M)
                     p.skey[(int64_t)b * p.max_tokens + key0 + et] = 0u;
                 tmem_wait_ld();
                 tc_fence_before_sync();
@@ -405,7 +418,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
         }
         if (PASS == 1) {
             const int qb = q0 + et;
-            uint32_t* rk = p.rkey + (int64_t)b * p.l_C;
+            uint32_t* rk = rkey;
             if (qb < p.l_C && rm0 > -INFINITY) atomicMax(rk + qb, f32_to_key(rm0));
             if (qb + 128 < p.l_C && rm1 > -INFINITY) atomicMax(rk + qb + 128, f32_to_key(rm1));
             if (qb + 256 < p.l_C && rm2 > -INFINITY) atomicMax(rk + qb + 256, f32_to_key(rm2));
@@ -428,21 +441,12 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
     if (warp == 1) tmem_dealloc(tmem, 512);
 }
 
+// p: groups, heads, rkey and skey set by the caller; the descriptors cover its operands.
 template <int DC>
-cudaError_t launch_t(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache, const SeqMeta& meta, int max_lM,
-                     cudaStream_t st, bool* pooled_ready) {
-    // the descriptors of the last call serve again while the caller keeps its cache and chunk size
-    if (!ctx->kc_map.matches(kc_cache, (uint64_t)B * ctx->cfg.max_tokens) &&
-        !ctx->kc_map.encode(kc_cache, (uint64_t)B * ctx->cfg.max_tokens, DC, 128))
-        return cudaErrorNotSupported;
-    if (!ctx->qc_map.matches(ctx->Qc, (uint64_t)B * l_C) && !ctx->qc_map.encode(ctx->Qc, (uint64_t)B * l_C, DC, 128))
-        return cudaErrorNotSupported;
-    const CUtensorMap &kmap = ctx->kc_map.map, &qmap = ctx->qc_map.map;
-    ScoreTcParams p;
-    p.rkey = ctx->rkey; p.skey = ctx->skey; p.pkey = ctx->pkey; p.ghist0 = ctx->ghist0; p.status = ctx->status;
+cudaError_t launch_t(esa_ctx* ctx, int B, int l_C, const CUtensorMap& kmap, const CUtensorMap& qmap, ScoreTcParams& p, const SeqMeta& meta,
+                     int max_lM, cudaStream_t st) {
+    p.skey = ctx->skey; p.pkey = ctx->pkey; p.ghist0 = ctx->ghist0; p.status = ctx->status;
     p.max_tokens = ctx->cfg.max_tokens; p.l_C = l_C; p.eps = ctx->cfg.eps; p.meta = meta;
-    const int q_groups = (l_C + ST_QCAP - 1) / ST_QCAP;
-    p.q_groups = q_groups;
     using C1 = ScoreCfg<DC, 1>;
     using C2 = ScoreCfg<DC, 2>;
     static KernelMemo memo1, memo2;
@@ -451,7 +455,7 @@ cudaError_t launch_t(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache
     e = allow_smem(score_tc_kernel<DC, 2>, ctx->device, C2::SMEM, memo2);
     if (e != cudaSuccess) return e;
     const int n_tiles = (max_lM + ST_KEYS - 1) / ST_KEYS;
-    int per_seq = ctx->num_sms / (q_groups * B);
+    int per_seq = ctx->num_sms / (p.groups * B);
     if (per_seq < 1) per_seq = 1;
     // pass 1: items of 128 queries x 128 keys
     const int nq = l_C < ST_QCAP ? l_C : ST_QCAP;
@@ -461,7 +465,7 @@ cudaError_t launch_t(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache
     if (gx1 < 1) gx1 = 1;
     {
         ProfScope prof(ctx, KC_SCORE_PASS1, st);
-        e = launch_pdl(score_tc_kernel<DC, 1>, dim3(gx1, q_groups, B), dim3(ST_THREADS), C1::SMEM, st, kmap, qmap, p);
+        e = launch_pdl(score_tc_kernel<DC, 1>, dim3(gx1, p.groups, B), dim3(ST_THREADS), C1::SMEM, st, kmap, qmap, p);
     }
     if (e != cudaSuccess) return e;
     // pass 2: whole tiles (every query of a group) per CTA
@@ -470,11 +474,10 @@ cudaError_t launch_t(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache
     if (gx2 < 1) gx2 = 1;
     {
         ProfScope prof(ctx, KC_SCORE_PASS2, st);
-        e = launch_pdl(score_tc_kernel<DC, 2>, dim3(gx2, q_groups, B), dim3(ST_THREADS), C2::SMEM, st, kmap, qmap, p);
+        e = launch_pdl(score_tc_kernel<DC, 2>, dim3(gx2, p.groups, B), dim3(ST_THREADS), C2::SMEM, st, kmap, qmap, p);
     }
     if (e != cudaSuccess) return e;
     ctx->launches += 2;
-    *pooled_ready = q_groups == 1;
     return cudaGetLastError();
 }
 
@@ -486,10 +489,32 @@ cudaError_t launch_t(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache
 // Returns cudaErrorNotSupported when this path does not cover the shape.
 cudaError_t launch_score_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache, const SeqMeta& meta,
                             int max_lM, cudaStream_t st, bool* pooled_ready) {
-    if (l_C < 64) return cudaErrorNotSupported;
-    if (ctx->dc == 128) return launch_t<128>(ctx, B, l_C, kc_cache, meta, max_lM, st, pooled_ready);
-    if (ctx->dc == 64) return launch_t<64>(ctx, B, l_C, kc_cache, meta, max_lM, st, pooled_ready);
-    return cudaErrorNotSupported;
+    if (l_C < 64 || (ctx->dc != 64 && ctx->dc != 128)) return cudaErrorNotSupported;
+    // the descriptors of the last call serve again while the caller keeps its cache and chunk size
+    const uint64_t k_rows = (uint64_t)B * ctx->cfg.max_tokens, q_rows = (uint64_t)B * l_C;
+    if (!ctx->kc_map.matches(kc_cache, k_rows) && !ctx->kc_map.encode(kc_cache, k_rows, ctx->dc, ST_KEYS)) return cudaErrorNotSupported;
+    if (!ctx->qc_map.matches(ctx->Qc, q_rows) && !ctx->qc_map.encode(ctx->Qc, q_rows, ctx->dc, 128)) return cudaErrorNotSupported;
+    ScoreTcParams p;
+    p.rkey = ctx->rkey;
+    p.groups = (l_C + ST_QCAP - 1) / ST_QCAP; p.heads = 1; p.G = 1; p.pool = p.groups == 1 ? 1 : 0;
+    *pooled_ready = p.pool != 0;
+    return ctx->dc == 128 ? launch_t<128>(ctx, B, l_C, ctx->kc_map.map, ctx->qc_map.map, p, meta, max_lM, st)
+                          : launch_t<64>(ctx, B, l_C, ctx->kc_map.map, ctx->qc_map.map, p, meta, max_lM, st);
+}
+
+// The per-head vote: every head's own scores (uncompressed queries and keys), the maximum over the heads in ctx->skey,
+// unpooled.  ctx->rkey_heads must be zeroed; ctx->ghist0 is zero afterwards.
+cudaError_t launch_score_tc_heads(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* K, const SeqMeta& meta,
+                                  int max_lM, cudaStream_t st) {
+    CUtensorMap kmap, qmap;
+    if (!make_tensor_map_bf16(&kmap, K, (uint64_t)B * ctx->cfg.max_tokens, ctx->dG, ST_KEYS) ||
+        !make_tensor_map_bf16(&qmap, Q, (uint64_t)B * l_C, ctx->dH, 128))
+        return cudaErrorInvalidValue;
+    ScoreTcParams p;
+    p.rkey = ctx->rkey_heads;
+    p.groups = ctx->H * ((l_C + ST_QCAP - 1) / ST_QCAP); p.heads = ctx->H; p.G = ctx->G; p.pool = 0;
+    return ctx->d == 128 ? launch_t<128>(ctx, B, l_C, kmap, qmap, p, meta, max_lM, st)
+                         : launch_t<64>(ctx, B, l_C, kmap, qmap, p, meta, max_lM, st);
 }
 
 }  // namespace esa

@@ -447,6 +447,15 @@ def test_select_full_llama_shape(per_head):
     _select_full_case(syn.get_config("c2"), 9000, 1, per_head)
 
 
+@pytest.mark.parametrize("per_head", [False, True])
+@pytest.mark.parametrize("H,H_G,d,t,l_C", [(28, 4, 128, 2600, 257), (28, 4, 128, 1410, 3), (4, 4, 128, 3000, 129), (6, 3, 64, 2200, 64),
+                                           (1, 1, 64, 2200, 100)])
+def test_select_full_at_tile_edges(H, H_G, d, t, l_C, per_head):
+    """Groups of 7, 1 and 2 heads (folded and unfolded queries), chunks around the 64/128/256-row tiles, ragged key tiles."""
+    cfg = syn.get_config("c1").with_(H=H, H_G=H_G, d=d, l_I=16, l_L=512, k=300)
+    _select_full_case(cfg, t, l_C, per_head)
+
+
 def test_recall_of_the_compressed_selection_against_the_full_dimension_one():
     """Fig. 3's metric on the mixture-with-needles workload: the share of the full-dimension
     selection (Eq. 3) that the compressed selection (Eq. 6) also picks.  The kernels' recall equals
