@@ -57,11 +57,11 @@ Layout make_layout(const esa_config* c) {
     size_t rows = (size_t)c->max_chunk * G;
     if (rows > (size_t)kAttSplitRows) rows = kAttSplitRows;
     L.att_elems = (size_t)c->max_batch * c->n_kv_heads * kAttMaxSplits * rows * (c->head_dim + 2);
-    // prefill-sized chunks: room for one sequence's key list split kAttPrefillSplits ways
-    const size_t big = (size_t)c->n_kv_heads * kAttPrefillSplits * (c->max_chunk * G + 1) * (c->head_dim + 2);
+    // prefill-sized chunks: room for one sequence's key list split kAttPrefillParts ways
+    const size_t big = (size_t)c->n_kv_heads * kAttPrefillParts * (c->max_chunk * G + 1) * (c->head_dim + 2);
     if ((size_t)c->max_chunk * G > (size_t)kAttSplitRows && big > L.att_elems) L.att_elems = big;
     L.att = take(4 * L.att_elems);
-    L.att_count_elems = (size_t)c->max_batch * c->n_kv_heads * ((c->max_chunk * G + 255) / 256);
+    L.att_count_elems = (size_t)c->max_batch * c->n_kv_heads;
     L.att_count = take(4 * L.att_count_elems);
     L.status = take(256);
     L.total = off;
@@ -544,8 +544,8 @@ const char* esa_kernel_class_name(int32_t cls) {
         "compress_tc_kernel", "compress_gemv_kernel", "compress_kernel", "append_kv_kernel", "score_tc_kernel<.,1>",
         "score_tc_kernel<.,2>", "score_pass_kernel<.,1>+<.,2>", "score_decode_kernel", "score_full_kernel<.,1>+<.,2>",
         "pool_hist_kernel",
-        "select_topk_kernel", "select_all_kernel", "attend_tc_kernel", "attend_decode_kernel", "attend_kernel",
-        "attend_merge_kernel", "gather_kv_kernel"};
+        "select_topk_kernel", "select_all_kernel", "attend_tc_kernel", "attend_decode_kernel",
+        "attend_tc_merge_kernel", "gather_kv_kernel"};
     return cls >= 0 && cls < KC_COUNT ? names[cls] : "";
 }
 

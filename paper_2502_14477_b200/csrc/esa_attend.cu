@@ -15,11 +15,8 @@
 // that share it.  Flash-style online softmax in the exp2 domain, bf16 operands, fp32
 // scores and accumulators.
 //
-// This file holds the kernels for small chunks: a generic split-KV mma.sync kernel
-// (up to 64 rows per key/value head), the streaming kernel for decode (one query per
-// sequence), the kernel that merges the partial (O, m, l) triples of key-list splits -- the
-// same algebra as Algorithm 1's merge -- and the entry point that needs no allocation.
-// Prefill-sized chunks run in esa_attend_tc.cu.
+// This file holds the streaming kernel for decode (one query per sequence), the choice between it and the tcgen05
+// kernel of esa_attend_tc.cu (every other chunk), and the entry point that needs no allocation.
 #include <mutex>
 
 #include "esa_internal.h"
@@ -46,330 +43,6 @@ struct AttendParams {
     float scale_log2;         // softmax scale * log2(e)
     SeqMeta meta;
 };
-
-// layout of the split-KV partial buffer, per (b, kvh, split): R rows x (D + 2) floats
-// (unnormalised O row, running max m in the exp2 domain, running sum l)
-
-// TWO: the list entries of I and M_k (the first n_glob) take their logits from Qg and Kg, the entries
-// of L and C from Q and K; both score tiles are formed and each key column keeps the one that applies.
-template <int D, int NW, int BN, bool TWO>
-__global__ void __launch_bounds__(NW * 32)
-attend_kernel(AttendParams p) {
-    constexpr int CH = D / 8;
-    constexpr int BM = NW * 16;
-    constexpr int NT = NW * 32;
-    extern __shared__ uint4 smem[];
-    uint4* sQ = smem;                         // [BM][CH]
-    uint4* sK = sQ + BM * CH;                 // 2 x [BN][CH]
-    uint4* sV = sK + 2 * BN * CH;             // 2 x [BN][CH]
-    uint4* sQg = sV + 2 * BN * CH;            // [BM][CH] (TWO)
-
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int row0 = blockIdx.x * BM;
-    const int kvh = blockIdx.y;
-    const int b = blockIdx.z / p.nsplit;
-    const int split = blockIdx.z % p.nsplit;
-    const int G = p.G;
-    const int R = p.l_C * G;
-
-    const int t = p.meta.t[b], i_end = p.meta.i_end[b], m_end = p.meta.m_end[b];
-    int n_sel = p.n_sel[b];
-    n_sel = max(0, min(n_sel, min(p.top_k, m_end - i_end)));
-    const int n_glob = i_end + n_sel;                  // entries before L
-    const int n_att = n_glob + (t - m_end) + p.l_C;
-    const int c_first = n_att - p.l_C;                 // list position of the chunk's first key
-
-    // keys this row tile can see: up to the chunk key of its last query
-    const int r_last = min(R, row0 + BM) - 1;
-    const int j_end = c_first + r_last / G + 1;
-    const int n_tiles = (j_end + BN - 1) / BN;
-    const int per = (n_tiles + p.nsplit - 1) / p.nsplit;
-    const int tile_begin = split * per;
-    const int tile_end = min(n_tiles, tile_begin + per);
-
-    const __nv_bfloat16* Kb = p.K + ((int64_t)b * p.max_tokens * p.HG + kvh) * D;
-    const __nv_bfloat16* Kgb = p.Kg + ((int64_t)b * p.max_tokens * p.HG + kvh) * D;
-    const __nv_bfloat16* Vb = p.V + ((int64_t)b * p.max_tokens * p.HG + kvh) * D;
-    const int32_t* idx = p.idx + (int64_t)b * p.top_k;
-    const int64_t tok_stride = (int64_t)p.HG * D;
-
-    int bad_idx = 0;
-    auto load_kv = [&](int st, int tile) {
-        uint4* dk = sK + st * BN * CH;
-        uint4* dv = sV + st * BN * CH;
-        for (int i = tid; i < BN * CH; i += NT) {
-            int r = i / CH, c = i % CH;
-            int j = tile * BN + r;
-            bool ok = j < n_att;
-            int pos = 0;
-            if (ok) {
-                if (p.staged) pos = j;
-                else if (j < i_end) pos = j;
-                else if (j < n_glob) pos = clamp_selected(__ldg(idx + (j - i_end)), i_end, m_end, bad_idx);
-                else pos = m_end + (j - n_glob);
-            }
-            const int64_t off = (int64_t)pos * tok_stride + c * 8;
-            cp_async16(&dk[swz<CH>(r, c)], ((TWO && j < n_glob) ? Kgb : Kb) + off, ok ? 16 : 0);
-            cp_async16(&dv[swz<CH>(r, c)], Vb + off, ok ? 16 : 0);
-        }
-    };
-
-    // Q tile -> smem (rows past R are zero)
-    for (int i = tid; i < BM * CH; i += NT) {
-        int r = i / CH, c = i % CH;
-        int row = row0 + r;
-        bool ok = row < R;
-        int cq = ok ? row / G : 0, g = ok ? row % G : 0;
-        const int64_t qoff = (((int64_t)b * p.l_C + cq) * p.H + kvh * G + g) * D + c * 8;
-        cp_async16(&sQ[swz<CH>(r, c)], p.Q + qoff, ok ? 16 : 0);
-        if (TWO) cp_async16(&sQg[swz<CH>(r, c)], p.Qg + qoff, ok ? 16 : 0);
-    }
-    if (tile_begin < tile_end) load_kv(0, tile_begin);
-    cp_async_commit();
-
-    float o_acc[D / 8][4];
-#pragma unroll
-    for (int i = 0; i < D / 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) o_acc[i][j] = 0.f;
-    float m_run[2] = {-INFINITY, -INFINITY};
-    float l_run[2] = {0.f, 0.f};
-
-    // this thread's two rows and their causal limits (first invisible list position)
-    const int r_lo = row0 + warp * 16 + (lane >> 2);
-    const int lim_lo = c_first + min(r_lo / G, p.l_C - 1) + 1;
-    const int lim_hi = c_first + min((r_lo + 8) / G, p.l_C - 1) + 1;
-    const int warp_min_lim = c_first + min((row0 + warp * 16) / G, p.l_C - 1) + 1;
-
-    uint32_t qf[D / 16][4];
-    uint32_t qfg[TWO ? D / 16 : 1][4];
-    bool q_loaded = false;
-
-    for (int tile = tile_begin; tile < tile_end; ++tile) {
-        const int st = (tile - tile_begin) & 1;
-        if (tile + 1 < tile_end) {
-            load_kv(st ^ 1, tile + 1);
-            cp_async_commit();
-            cp_async_wait<1>();
-        } else {
-            cp_async_wait<0>();
-        }
-        __syncthreads();
-        if (!q_loaded) {
-#pragma unroll
-            for (int ks = 0; ks < D / 16; ++ks) load_a_frag<CH>(qf[ks], sQ, warp * 16, ks * 2, lane);
-            if (TWO) {
-#pragma unroll
-                for (int ks = 0; ks < D / 16; ++ks) load_a_frag<CH>(qfg[ks], sQg, warp * 16, ks * 2, lane);
-            }
-            q_loaded = true;
-        }
-        const uint4* tk = sK + st * BN * CH;
-        const uint4* tv = sV + st * BN * CH;
-
-        // S = Q K^T
-        float s[BN / 8][4];
-#pragma unroll
-        for (int i = 0; i < BN / 8; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
-#pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks) {
-#pragma unroll
-            for (int nb = 0; nb < BN / 16; ++nb) {
-                uint32_t kb[4];
-                load_b_frag_nk<CH>(kb, tk, nb * 16, ks * 2, lane);
-                mma_bf16_16816(s[2 * nb], qf[ks], kb[0], kb[1]);
-                mma_bf16_16816(s[2 * nb + 1], qf[ks], kb[2], kb[3]);
-            }
-        }
-        const int j0 = tile * BN;
-        if (TWO && j0 < n_glob) {
-            // some key columns of this tile belong to I or M_k: their logits come from Qg (the tile holds Kg rows there)
-            float sg[BN / 8][4];
-#pragma unroll
-            for (int i = 0; i < BN / 8; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) sg[i][j] = 0.f;
-#pragma unroll
-            for (int ks = 0; ks < D / 16; ++ks) {
-#pragma unroll
-                for (int nb = 0; nb < BN / 16; ++nb) {
-                    uint32_t kb[4];
-                    load_b_frag_nk<CH>(kb, tk, nb * 16, ks * 2, lane);
-                    mma_bf16_16816(sg[2 * nb], qfg[ks], kb[0], kb[1]);
-                    mma_bf16_16816(sg[2 * nb + 1], qfg[ks], kb[2], kb[3]);
-                }
-            }
-#pragma unroll
-            for (int nb = 0; nb < BN / 8; ++nb)
-#pragma unroll
-                for (int e = 0; e < 2; ++e)
-                    if (j0 + nb * 8 + (lane & 3) * 2 + e < n_glob) {
-                        s[nb][e] = sg[nb][e];
-                        s[nb][2 + e] = sg[nb][2 + e];
-                    }
-        }
-
-        // scale, mask (causal inside C and the ragged tail), online softmax
-        const bool need_mask = j0 + BN > warp_min_lim;
-        float mx_lo = -INFINITY, mx_hi = -INFINITY;
-#pragma unroll
-        for (int nb = 0; nb < BN / 8; ++nb) {
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                float a = s[nb][e] * p.scale_log2, c2 = s[nb][2 + e] * p.scale_log2;
-                if (need_mask) {
-                    int j = j0 + nb * 8 + (lane & 3) * 2 + e;
-                    if (j >= lim_lo) a = -INFINITY;
-                    if (j >= lim_hi) c2 = -INFINITY;
-                }
-                s[nb][e] = a;
-                s[nb][2 + e] = c2;
-                mx_lo = fmaxf(mx_lo, a);
-                mx_hi = fmaxf(mx_hi, c2);
-            }
-        }
-        mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 1));
-        mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 2));
-        mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 1));
-        mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 2));
-        const float mn_lo = fmaxf(m_run[0], mx_lo), mn_hi = fmaxf(m_run[1], mx_hi);
-        const float ms_lo = (mn_lo == -INFINITY) ? 0.f : mn_lo;   // a fully masked row stays empty
-        const float ms_hi = (mn_hi == -INFINITY) ? 0.f : mn_hi;
-        const float al_lo = fast_exp2(m_run[0] - ms_lo), al_hi = fast_exp2(m_run[1] - ms_hi);
-        m_run[0] = mn_lo;
-        m_run[1] = mn_hi;
-        float sum_lo = 0.f, sum_hi = 0.f;
-        uint32_t pf[BN / 16][4];
-#pragma unroll
-        for (int nb = 0; nb < BN / 8; ++nb) {
-            float p0 = fast_exp2(s[nb][0] - ms_lo), p1 = fast_exp2(s[nb][1] - ms_lo);
-            float p2 = fast_exp2(s[nb][2] - ms_hi), p3 = fast_exp2(s[nb][3] - ms_hi);
-            sum_lo += p0 + p1;
-            sum_hi += p2 + p3;
-            pf[nb >> 1][(nb & 1) * 2] = pack_bf16(p0, p1);
-            pf[nb >> 1][(nb & 1) * 2 + 1] = pack_bf16(p2, p3);
-        }
-        l_run[0] = l_run[0] * al_lo + sum_lo;
-        l_run[1] = l_run[1] * al_hi + sum_hi;
-#pragma unroll
-        for (int nb = 0; nb < D / 8; ++nb) {
-            o_acc[nb][0] *= al_lo;
-            o_acc[nb][1] *= al_lo;
-            o_acc[nb][2] *= al_hi;
-            o_acc[nb][3] *= al_hi;
-        }
-        // O += P V
-#pragma unroll
-        for (int kk = 0; kk < BN / 16; ++kk) {
-#pragma unroll
-            for (int dp = 0; dp < D / 16; ++dp) {
-                uint32_t vb[4];
-                load_b_frag_kn<CH>(vb, tv, kk * 16, dp * 2, lane);
-                mma_bf16_16816(o_acc[2 * dp], pf[kk], vb[0], vb[1]);
-                mma_bf16_16816(o_acc[2 * dp + 1], pf[kk], vb[2], vb[3]);
-            }
-        }
-        __syncthreads();
-    }
-    cp_async_wait<0>();
-    if (bad_idx && p.status) atomicExch(p.status, kStatusBadIndex);
-
-    l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 1);
-    l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 2);
-    l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], 1);
-    l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], 2);
-
-#pragma unroll
-    for (int half = 0; half < 2; ++half) {
-        const int row = r_lo + half * 8;
-        if (row >= R) continue;
-        if (p.nsplit == 1) {
-            const float inv = 1.f / l_run[half];
-            const int cq = row / G, g = row % G;
-            __nv_bfloat16* dst = p.O + (((int64_t)b * p.l_C + cq) * p.H + kvh * G + g) * D;
-#pragma unroll
-            for (int nb = 0; nb < D / 8; ++nb) {
-                int col = nb * 8 + (lane & 3) * 2;
-                *reinterpret_cast<uint32_t*>(dst + col) =
-                    pack_bf16(o_acc[nb][half * 2] * inv, o_acc[nb][half * 2 + 1] * inv);
-            }
-        } else {
-            float* dst = p.part + ((((int64_t)b * p.HG + kvh) * p.nsplit + split) * R + row) * (D + 2);
-#pragma unroll
-            for (int nb = 0; nb < D / 8; ++nb) {
-                int col = nb * 8 + (lane & 3) * 2;
-                *reinterpret_cast<float2*>(dst + col) = make_float2(o_acc[nb][half * 2], o_acc[nb][half * 2 + 1]);
-            }
-            if ((lane & 3) == 0) {
-                dst[D] = m_run[half];
-                dst[D + 1] = l_run[half];
-            }
-        }
-    }
-}
-
-// Merge of the split-KV partials (Algorithm 1's merge generalised to nsplit parts):
-// O = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s with M = max_s m_s.
-// One warp per output row: each lane owns D / 32 consecutive columns, so a part's row is one
-// coalesced read and the result one coalesced bf16 write.
-// Combines the nsplit parts of one row (Algorithm 1's merge of (O, m, l)) and writes the bf16 row.
-// `base` points at the row's slot in part 0, parts are `sstride` floats apart.  Loads go to L2
-// (the parts may have been written by other SMs a moment ago).
-template <int D>
-__device__ __forceinline__ void merge_row(const float* base, int64_t sstride, int nsplit, int lane, __nv_bfloat16* dst_row) {
-    constexpr int PER = D / 32;                  // columns per lane: 2 or 4
-    // parts are taken four at a time so that their loads are in flight together
-    float M = -INFINITY;
-    for (int s = 0; s < nsplit; ++s) M = fmaxf(M, __ldcg(base + s * sstride + D));
-    float den = 0.f;
-    float acc[PER];
-#pragma unroll
-    for (int i = 0; i < PER; ++i) acc[i] = 0.f;
-    for (int s0 = 0; s0 < nsplit; s0 += 4) {
-        float mm[4], ll[4];
-        float2 v[4][PER / 2];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const bool in = s0 + j < nsplit;
-            const float* ps = base + (in ? s0 + j : 0) * sstride;
-            mm[j] = in ? __ldcg(ps + D) : -INFINITY;
-            ll[j] = __ldcg(ps + D + 1);
-#pragma unroll
-            for (int i = 0; i < PER / 2; ++i) v[j][i] = __ldcg(reinterpret_cast<const float2*>(ps + lane * PER + 2 * i));
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            if (mm[j] == -INFINITY) continue;        // an empty or absent part (uniform over the warp)
-            const float w = fast_exp2(mm[j] - M);
-            den += w * ll[j];
-#pragma unroll
-            for (int i = 0; i < PER / 2; ++i) {
-                acc[2 * i] += w * v[j][i].x;
-                acc[2 * i + 1] += w * v[j][i].y;
-            }
-        }
-    }
-    const float inv = 1.f / den;
-#pragma unroll
-    for (int i = 0; i < PER; i += 2)
-        *reinterpret_cast<uint32_t*>(dst_row + lane * PER + i) = pack_bf16(acc[i] * inv, acc[i + 1] * inv);
-}
-
-template <int D>
-__global__ void __launch_bounds__(256) attend_merge_kernel(AttendParams p) {
-    pdl_wait();
-    pdl_launch_dependents();
-    const int R = p.l_C * p.G;
-    const int lane = threadIdx.x & 31;
-    const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int kvh = blockIdx.y, b = blockIdx.z;
-    if (row >= R) return;
-    const float* base = p.part + (((int64_t)b * p.HG + kvh) * p.nsplit * R + row) * (D + 2);
-    const int cq = row / p.G, g = row % p.G;
-    merge_row<D>(base, (int64_t)R * (D + 2), p.nsplit, lane, p.O + (((int64_t)b * p.l_C + cq) * p.H + kvh * p.G + g) * D);
-}
 
 // ---------------------------------------------------------------------------
 // Decode (one query per sequence): the step is bound by reading the gathered K/V rows, so the
@@ -679,7 +352,7 @@ attend_decode_kernel(AttendParams p) {
             __threadfence();
             for (int g = warp; g < G; g += DEC_WARPS) {
                 const float* base = p.part + (((int64_t)b * p.HG + kvh) * p.nsplit * G + g) * (D + 2);
-                merge_row<D>(base, (int64_t)G * (D + 2), p.nsplit, lane, p.O + ((int64_t)b * p.H + kvh * G + g) * D);
+                merge_row<D>(base, base + D, (int64_t)G * (D + 2), p.nsplit, lane, p.O + ((int64_t)b * p.H + kvh * G + g) * D);
             }
         }
     }
@@ -723,64 +396,6 @@ static cudaError_t launch_decode(esa_ctx* ctx, AttendParams& p, int B, int n_att
     return cudaErrorNotSupported;
 }
 
-template <int D, int NW, int BN, bool TWO>
-static cudaError_t launch_attend_t(esa_ctx* ctx, AttendParams& p, int B, int n_att_max, cudaStream_t st) {
-    constexpr int BM = NW * 16;
-    const int R = p.l_C * p.G;
-    const int row_tiles = (R + BM - 1) / BM;
-    constexpr int smem = ((TWO ? 2 : 1) * BM + 4 * BN) * (D / 8) * 16;
-    static KernelMemo memo;
-    cudaError_t e = allow_smem(attend_kernel<D, NW, BN, TWO>, ctx->device, smem, memo);
-    if (e != cudaSuccess) return e;
-    int nsplit = 1;
-    if (R <= kAttSplitRows && row_tiles == 1) {
-        // split the key list so that one wave of CTAs fills the machine (never a second, short wave)
-        int per_sm = 1;
-        e = resident_per_sm(attend_kernel<D, NW, BN, TWO>, ctx->device, NW * 32, smem, memo, &per_sm);
-        if (e != cudaSuccess) return e;
-        const int ctas = p.HG * B;
-        const int n_tiles = (n_att_max + BN - 1) / BN;
-        nsplit = (per_sm * ctx->num_sms) / ctas;
-        if (nsplit > kAttMaxSplits) nsplit = kAttMaxSplits;
-        if (nsplit > n_tiles) nsplit = n_tiles;
-        while (nsplit > 1 && (size_t)B * p.HG * nsplit * R * (D + 2) > ctx->att_part_elems) --nsplit;
-        if (nsplit < 1) nsplit = 1;
-    }
-    p.nsplit = nsplit;
-    {
-        ProfScope prof(ctx, KC_ATTEND_SMALL, st);
-        attend_kernel<D, NW, BN, TWO><<<dim3(row_tiles, p.HG, B * nsplit), NW * 32, smem, st>>>(p);
-    }
-    ctx->launches += 1;
-    if (nsplit > 1) {
-        ProfScope prof(ctx, KC_ATTEND_MERGE, st);
-        attend_merge_kernel<D><<<dim3((R + 7) / 8, p.HG, B), 256, 0, st>>>(p);
-        ctx->launches += 1;
-    }
-    return cudaGetLastError();
-}
-
-template <bool TWO>
-static cudaError_t launch_small(esa_ctx* ctx, AttendParams& p, int B, int l_C, int n_att_max, cudaStream_t st) {
-    const int R = l_C * ctx->G;
-    if (l_C == 1) {
-        // decode: streaming kernel for the usual group sizes
-        cudaError_t e = ctx->d == 128 ? launch_decode<128, TWO>(ctx, p, B, n_att_max, st)
-                                      : launch_decode<64, TWO>(ctx, p, B, n_att_max, st);
-        if (e != cudaErrorNotSupported) return e;
-    }
-    if (ctx->d == 128) {
-        if (R <= 16) return launch_attend_t<128, 1, 32, TWO>(ctx, p, B, n_att_max, st);
-        if (R <= 64) return launch_attend_t<128, 4, 64, TWO>(ctx, p, B, n_att_max, st);
-        return launch_attend_t<128, 8, 64, TWO>(ctx, p, B, n_att_max, st);
-    } else if (ctx->d == 64) {
-        if (R <= 16) return launch_attend_t<64, 1, 32, TWO>(ctx, p, B, n_att_max, st);
-        if (R <= 64) return launch_attend_t<64, 4, 64, TWO>(ctx, p, B, n_att_max, st);
-        return launch_attend_t<64, 8, 64, TWO>(ctx, p, B, n_att_max, st);
-    }
-    return cudaErrorInvalidValue;
-}
-
 // Qg / Kg: queries and key cache used against I and M_k (Section 3.2); null = Q / K.
 cudaError_t launch_attend(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* Qg,
                           const __nv_bfloat16* K, const __nv_bfloat16* Kg, const __nv_bfloat16* V, const SeqMeta& meta,
@@ -803,14 +418,18 @@ cudaError_t launch_attend(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, 
         int n = meta.i_end[b] + (lM < ctx->cfg.top_k ? lM : ctx->cfg.top_k) + (meta.t[b] - meta.m_end[b]) + l_C;
         if (n > n_att_max) n_att_max = n;
     }
-    const int R = l_C * ctx->G;
-    if (R > kAttSplitRows) {
-        // prefill-sized chunks: tcgen05 kernel (a split key list is merged inside it)
-        int nsplit = 1;
-        return launch_attend_tc(ctx, B, l_C, Q, two ? p.Qg : nullptr, K, two ? p.Kg : nullptr, V, meta, idx, n_sel, O, n_att_max, st,
-                                &nsplit, cache_rows, staged);
+    if (l_C == 1) {
+        // decode: streaming kernel for the usual group sizes
+        cudaError_t e;
+        if (ctx->d == 128) e = two ? launch_decode<128, true>(ctx, p, B, n_att_max, st) : launch_decode<128, false>(ctx, p, B, n_att_max, st);
+        else e = two ? launch_decode<64, true>(ctx, p, B, n_att_max, st) : launch_decode<64, false>(ctx, p, B, n_att_max, st);
+        if (e != cudaErrorNotSupported) return e;
     }
-    return two ? launch_small<true>(ctx, p, B, l_C, n_att_max, st) : launch_small<false>(ctx, p, B, l_C, n_att_max, st);
+    // Any other chunk: tcgen05 kernel.  Few rows leave most of its 128-row tile empty, but the key list is then split far
+    // enough that the products do not matter: 3 queries (12 rows a head) over 7400 keys 39 -> 22 us, 8 queries 32 -> 21 us
+    // against a split mma.sync kernel.
+    return launch_attend_tc(ctx, B, l_C, Q, two ? p.Qg : nullptr, K, two ? p.Kg : nullptr, V, meta, idx, n_sel, O, n_att_max, st,
+                            cache_rows, staged);
 }
 
 // ---------------------------------------------------------------------------
@@ -824,39 +443,23 @@ namespace {
 // the same call, so nothing has to be cleared between calls.
 constexpr size_t kNoAllocPartFloats = size_t(2) << 20;
 static __device__ __align__(256) float g_noalloc_part[kNoAllocPartFloats];
+// Arrival counters of the decode kernel's merge (zero between launches; a call of B * H_G units needs four parts of at
+// least 66 floats each in the array above) and a status word nobody reads.
+constexpr int kNoAllocUnits = 8192;
+static __device__ int g_noalloc_count[kNoAllocUnits + 1];
+static_assert(kNoAllocUnits * size_t(4 * 66) > kNoAllocPartFloats, "more units than the partials have room for");
 
 constexpr int kNoAllocMaxDevices = 64;
 constexpr int kNoAllocMinSplits = 4;      // a call must be able to split its key list at least this far
 
 struct NoAllocDevice {
     float* part;      // device address of g_noalloc_part on this device (the symbol itself is not one)
+    int* count;       // of g_noalloc_count
     int num_sms;
     bool ready;
 };
 NoAllocDevice g_noalloc_dev[kNoAllocMaxDevices];
 std::mutex g_noalloc_mutex;      // host threads may make a device's first call together
-
-template <int D, int NW, int BN>
-cudaError_t launch_noalloc_t(const NoAllocDevice& dev, int device, AttendParams& p, int B, int n_att_max, cudaStream_t st) {
-    const int R = p.l_C * p.G;
-    constexpr int smem = (NW * 16 + 4 * BN) * (D / 8) * 16;
-    static KernelMemo memo;
-    cudaError_t e = allow_smem(attend_kernel<D, NW, BN, false>, device, smem, memo);
-    if (e != cudaSuccess) return e;
-    int per_sm = 1;
-    e = resident_per_sm(attend_kernel<D, NW, BN, false>, device, NW * 32, smem, memo, &per_sm);
-    if (e != cudaSuccess) return e;
-    const int n_tiles = (n_att_max + BN - 1) / BN;
-    int nsplit = (per_sm * dev.num_sms) / (p.HG * B);
-    if (nsplit > kAttMaxSplits) nsplit = kAttMaxSplits;
-    if (nsplit > n_tiles) nsplit = n_tiles;
-    while (nsplit > 1 && (size_t)B * p.HG * nsplit * R * (D + 2) > kNoAllocPartFloats) --nsplit;
-    if (nsplit < 1) nsplit = 1;
-    p.nsplit = nsplit;
-    attend_kernel<D, NW, BN, false><<<dim3(1, p.HG, B * nsplit), NW * 32, smem, st>>>(p);
-    if (nsplit > 1) attend_merge_kernel<D><<<dim3((R + 7) / 8, p.HG, B), 256, 0, st>>>(p);
-    return cudaGetLastError();
-}
 
 }  // namespace
 }  // namespace esa
@@ -880,7 +483,6 @@ extern "C" esa_status esa_attend_noalloc(const esa_config* cfg, int32_t B, const
     if ((size_t)B * cfg->n_kv_heads * kNoAllocMinSplits * (size_t)R * (D + 2) > kNoAllocPartFloats) return ESA_ERR_CAPACITY;
 
     SeqMeta meta;
-    int n_att_max = 0;
     for (int b = 0; b < B; ++b) {
         const int64_t t = n_prev[b];
         if (t < 0) return ESA_ERR_INVALID_ARG;
@@ -889,9 +491,6 @@ extern "C" esa_status esa_attend_noalloc(const esa_config* cfg, int32_t B, const
         int64_t m_end = t - cfg->l_local;
         if (m_end < i_end) m_end = i_end;
         meta.t[b] = (int)t; meta.i_end[b] = (int)i_end; meta.m_end[b] = (int)m_end;
-        const int64_t lM = m_end - i_end;
-        const int64_t n = i_end + (lM < cfg->top_k ? lM : cfg->top_k) + (t - m_end) + l_C;
-        if (n > n_att_max) n_att_max = (int)n;
     }
     for (int b = B; b < kMaxBatch; ++b) meta.t[b] = meta.i_end[b] = meta.m_end[b] = 0;
 
@@ -903,8 +502,9 @@ extern "C" esa_status esa_attend_noalloc(const esa_config* cfg, int32_t B, const
     std::unique_lock<std::mutex> lock(g_noalloc_mutex);
     NoAllocDevice& dev = g_noalloc_dev[device];
     if (!dev.ready) {
-        void* ptr = nullptr;
-        if (cudaGetSymbolAddress(&ptr, g_noalloc_part) != cudaSuccess || !ptr) {
+        void *ptr = nullptr, *cnt = nullptr;
+        if (cudaGetSymbolAddress(&ptr, g_noalloc_part) != cudaSuccess || !ptr ||
+            cudaGetSymbolAddress(&cnt, g_noalloc_count) != cudaSuccess || !cnt) {
             cudaGetLastError();
             return ESA_ERR_CUDA;
         }
@@ -912,25 +512,22 @@ extern "C" esa_status esa_attend_noalloc(const esa_config* cfg, int32_t B, const
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || sms <= 0)
             return ESA_ERR_CUDA;
         dev.part = static_cast<float*>(ptr);
+        dev.count = static_cast<int*>(cnt);
         dev.num_sms = sms;
         dev.ready = true;
     }
     lock.unlock();
 
-    AttendParams p;
-    p.Q = (const __nv_bfloat16*)Q_cur; p.K = (const __nv_bfloat16*)K_cache; p.V = (const __nv_bfloat16*)V_cache;
-    p.Qg = p.Q; p.Kg = p.K;
-    p.O = (__nv_bfloat16*)O; p.idx = idx; p.n_sel = n_sel; p.part = dev.part; p.unit_count = nullptr; p.status = nullptr; p.staged = 0; p.early = 0;
-    p.max_tokens = cfg->max_tokens; p.l_C = l_C; p.H = cfg->n_q_heads; p.HG = cfg->n_kv_heads; p.G = G;
-    p.top_k = cfg->top_k; p.nsplit = 1;
-    const float scale = cfg->softmax_scale > 0.f ? cfg->softmax_scale : 1.0f / sqrtf((float)D);
-    p.scale_log2 = scale * 1.4426950408889634f;
-    p.meta = meta;
-    cudaStream_t st = (cudaStream_t)stream;
-    cudaError_t e;
-    if (D == 128) e = R <= 16 ? launch_noalloc_t<128, 1, 32>(dev, device, p, B, n_att_max, st)
-                              : launch_noalloc_t<128, 4, 64>(dev, device, p, B, n_att_max, st);
-    else e = R <= 16 ? launch_noalloc_t<64, 1, 32>(dev, device, p, B, n_att_max, st)
-                     : launch_noalloc_t<64, 4, 64>(dev, device, p, B, n_att_max, st);
+    // the ordinary launch path, on a context that owns nothing
+    esa_ctx c = {};
+    c.cfg = *cfg;
+    c.device = device; c.num_sms = dev.num_sms;
+    c.H = cfg->n_q_heads; c.HG = cfg->n_kv_heads; c.d = D; c.dH = c.H * D; c.dG = c.HG * D; c.G = G;
+    c.scale = cfg->softmax_scale > 0.f ? cfg->softmax_scale : 1.0f / sqrtf((float)D);
+    c.att_part = dev.part; c.att_part_elems = kNoAllocPartFloats;
+    c.att_count = dev.count; c.att_count_elems = kNoAllocUnits;
+    c.status = dev.count + kNoAllocUnits;
+    const cudaError_t e = launch_attend(&c, B, l_C, (const __nv_bfloat16*)Q_cur, nullptr, (const __nv_bfloat16*)K_cache, nullptr,
+                                        (const __nv_bfloat16*)V_cache, meta, idx, n_sel, (__nv_bfloat16*)O, (cudaStream_t)stream);
     return e == cudaSuccess ? ESA_OK : ESA_ERR_CUDA;
 }

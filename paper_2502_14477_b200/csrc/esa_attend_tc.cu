@@ -1,6 +1,6 @@
 // Eq. 1 / Algorithm 1 for prefill-sized chunks on the 5th-generation tensor cores.
 //
-// Same computation as the split kernel in esa_attend.cu (one softmax over the key list
+// Same computation as the decode kernel in esa_attend.cu (one softmax over the key list
 // I u M_k u L u C, C causal), organised for tcgen05:
 //
 //   * A CTA owns 256 rows (row = query c * G + head-in-group g) of one key/value head: two
@@ -32,8 +32,8 @@
 //     bf16 (P) carry the range.
 //   * A long key list can be split across CTAs (blockIdx.z); a two-way split runs as CTA pairs that exchange
 //     halves of their partial (O, m, l) through distributed shared memory (PAIR, below); otherwise the partials
-//     go to the context's scratch through coalesced stores, and the CTA that finishes a unit last merges
-//     them with its own accumulator (an arrival counter per unit decides; nobody waits).
+//     go to the context's scratch through coalesced stores and a second launch merges them, a warp per row (on all
+//     SMs: the last CTA of a unit merging four parts by itself took 15 us).
 //   * A call that follows the selection of its step (p.early) takes the attended set as two lists: I then L,
 //     whose rows are older than the chunk and do not depend on the selection, before the kernel's wait for the
 //     preceding kernel, and M_k then C after it.  Every role runs the two phases in turn; the selection kernel
@@ -68,7 +68,6 @@ constexpr int TC_PRODUCERS = TC_PRODUCER_WARPS * 32;
 constexpr int TC_REGS_LAUNCH = 128;
 constexpr int TC_REGS_SOFTMAX = 168;
 constexpr int TC_REGS_OTHER = 88;
-static_assert(kAttPrefillSplits == 4, "the in-kernel merge selects among four weights");
 static_assert(8 * TC_REGS_SOFTMAX + 8 * TC_REGS_OTHER <= 16 * TC_REGS_LAUNCH,
               "register split exceeds the CTA's launch allocation: setmaxnreg.inc would never return");
 constexpr float kSumLimit = 1.8446744e19f;   // 2^64: a tile whose sum of 2^(score - m) reaches this has its maximum looked up
@@ -88,7 +87,6 @@ struct TcAttendParams {
     int l_C, H, HG, G, top_k;
     int nsplit;
     int Rp;             // rows of a scratch part (R rounded up to even: 16-byte aligned parts)
-    int* unit_count;    // arrivals per (sequence, key/value head, row tile); returns to 0 after each launch
     int q_tma;          // Q tiles arrive by TMA (one arrival) instead of cp.async (one per producer thread)
     int staged;         // the caches hold the attended list itself: row j = list entry j
     int early;          // the rows of I and L are attended ahead of the wait for the preceding kernel (never with staged or two)
@@ -201,7 +199,9 @@ __device__ __forceinline__ void store_half_rows(const float* acc, float4* stage,
 // (Measured for the 128 KB of a partial: loads from the other CTA's shared memory 9 us, one 16-byte store per
 // lane and row 6 us, bulk copies 3.5 us.)  A second cluster barrier keeps each sender's shared memory alive until
 // its copies have landed.
-template <int D, bool PAIR>
+// NQT: Q tiles of a CTA that hold rows.  One for chunks of at most 128 rows per key/value head: the second tile's
+// products and softmax would only be in the way.
+template <int D, bool PAIR, int NQT>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap qgmap, TcAttendParams p) {
     constexpr int STAGES = TC_STAGES;
@@ -219,7 +219,6 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
     __shared__ uint64_t bars[BAR_COUNT];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
-    __shared__ int merge_ticket;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int warp_u = __shfl_sync(0xffffffffu, warp, 0);     // provably warp-uniform copy
@@ -322,6 +321,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
     if (warp_u < TC_SOFTMAX_WARPS) {
         // ------------------------------------------------------------ softmax, one row per thread
         const int qt = warp_u >> 2;                      // Q tile of this warpgroup
+        const bool active = qt < NQT;
         const int lane_base = (warp_u & 3) * 32;         // TMEM lanes this warp may touch
         const int row = row0 + qt * 128 + lane_base + lane;
         const uint32_t tS = tmem_addr(tmem, lane_base, qt * 128);
@@ -338,7 +338,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
         // early list)
         const int lim = phase == 0 ? e_len : min(part_hi, c_first + min(row / G, p.l_C - 1) + 1);
         const int lim_min = phase == 0 ? e_len : min(part_hi, c_first + min((row0 + qt * 128) / G, p.l_C - 1) + 1);
-        for (int j = j_first; j < j_last; ++j) {            // j counts halves: tile j >> 1, half j & 1
+        for (int j = j_first; active && j < j_last; ++j) {  // j counts halves: tile j >> 1, half j & 1
             const int T = j >> 1, u = j & 1;
             const int key0 = key_first + (j - j_first) * TC_HALF;
             if (u == 0) {
@@ -427,13 +427,14 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
 
         // ---- epilogue: O / l  (or the unnormalised partial for the split merge)
         // (BAR_O_READY completes exactly once.)
-        if (n_tiles > 0) {
+        if (n_tiles > 0 && active) {
             mbar_wait(bar(BAR_O_READY + qt), 0, wc);
             tc_fence_after_sync();
         }
         const bool row_ok = row < R;
         const int cq = row_ok ? row / G : 0, g = row_ok ? row % G : 0;
         if (p.nsplit == 1) {
+            if (active) {
             const float inv = 1.f / l_run;
             __nv_bfloat16* dst = p.O + (((int64_t)b * p.l_C + cq) * p.H + kvh * G + g) * D;
 #pragma unroll
@@ -452,6 +453,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
                         *reinterpret_cast<uint4*>(dst + c0 + q4 * 8) = w;
                     }
                 }
+            }
             }
         } else if (PAIR) {
             // ---- key list split in two, the two CTAs in one cluster (see the comment above the kernel).
@@ -478,7 +480,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
             if (tid == 0) mbar_arrive_expect_tx(bar(BAR_PAIR), HALF_BYTES + ML_BYTES);
             {
                 float4* prow = reinterpret_cast<float4*>(park) + (size_t)rl * NCELL;
-                if (n_tiles > 0) {
+                if (n_tiles > 0 && active) {
 #pragma unroll
                     for (int c0 = 0; c0 < DH; c0 += 32) {
                         uint32_t o[32];
@@ -507,7 +509,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
             }
             mbar_wait(bar(BAR_PAIR), 0, wc);
             cluster_arrive();                                // the partner's copies have landed here: it may go once it has them too
-            {
+            if (active) {
                 float4* stage = reinterpret_cast<float4*>(wslot);
                 const int wrow0 = row0 + qt * 128 + lane_base;
                 const int64_t own_off = (((int64_t)b * p.l_C + cq) * p.H + kvh * G + g) * D;
@@ -569,166 +571,43 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
             }
             cluster_wait();
         } else {
-            // ---- split key list.  Every CTA leaves its partial (O, m, l) in the scratch; the CTA that
-            // finishes a (sequence, head, row tile) unit last combines the others' partials with its own,
-            // which is still in tensor memory, and writes the rows of O: no CTA waits for another one.
+            // ---- split key list: the partial (O, m, l) goes to the scratch, the merge is a launch of its own.
             // Scratch of part s: O rows [Rp][D] fp32, then (m, l) pairs [Rp][2].
             constexpr int DH = D / 2;                  // columns handled per round
             constexpr int NC = DH / 4;                 // float4 per staged row: 16 or 8
             const int Rp = p.Rp;
-            float* unit_base = p.part + (((int64_t)b * p.HG + kvh) * p.nsplit) * (int64_t)Rp * (D + 2);
-            const int64_t part_stride = (int64_t)Rp * (D + 2);
-            float* myO = unit_base + split * part_stride;
+            float* myO = p.part + ((((int64_t)b * p.HG + kvh) * p.nsplit) + split) * (int64_t)Rp * (D + 2);
             // Staging for coalesced traffic: this warp's quarter of its own Q tile, 32 rows x DH fp32.
             // Free by now: O_READY covers every Q K^T of the tile.  16-byte cells are XOR-swizzled by
             // the row so that row-per-lane and row-per-half-warp accesses are both conflict-free.
             float4* stage = reinterpret_cast<float4*>(sQ + qt * Q_TILE_BYTES + (warp_u & 3) * (Q_TILE_BYTES / 4));
             const int wrow0 = row0 + qt * 128 + lane_base;        // first row of this warp
-            int* cnt = p.unit_count + ((int64_t)b * p.HG + kvh) * gridDim.x + blockIdx.x;
-            // When every other CTA of the unit has arrived already, this one merges straight from its
-            // tensor memory and publishes nothing.
-            asm volatile("bar.sync 1, 256;\n" ::: "memory");
-            if (tid == 0) {
-                const bool all_in = atomicAdd(cnt, 0) == p.nsplit - 1;
-                if (all_in) *cnt = 0;                              // ready for the next launch
-                merge_ticket = all_in ? p.nsplit - 1 : -1;
-            }
-            asm volatile("bar.sync 1, 256;\n" ::: "memory");
-            if (merge_ticket != p.nsplit - 1) {
-                if (n_tiles > 0) {
-#pragma unroll 1
-                    for (int h = 0; h < 2; ++h) {
-#pragma unroll
-                        for (int cc = 0; cc < DH; cc += 32) {
-                            uint32_t o[32];
-                            tmem_ld32(tO + h * DH + cc, o);
-                            tmem_wait_ld();
-#pragma unroll
-                            for (int q4 = 0; q4 < 8; ++q4)
-                                stage[lane * NC + ((cc / 4 + q4) ^ (lane & (NC - 1)))] =
-                                    make_float4(__uint_as_float(o[4 * q4]), __uint_as_float(o[4 * q4 + 1]),
-                                                __uint_as_float(o[4 * q4 + 2]), __uint_as_float(o[4 * q4 + 3]));
-                        }
-                        __syncwarp();
-#pragma unroll 4
-                        for (int it = 0; it < NC; ++it) {
-                            const int e = it * 32 + lane, rr = e / NC, c = e % NC;
-                            const float4 val = stage[rr * NC + (c ^ (rr & (NC - 1)))];
-                            if (wrow0 + rr < R)
-                                __stcg(reinterpret_cast<float4*>(myO + (int64_t)(wrow0 + rr) * D + h * DH) + c, val);
-                        }
-                        __syncwarp();
-                    }
-                }
-                if (row_ok) __stcg(reinterpret_cast<float2*>(myO + (int64_t)Rp * D) + row, make_float2(m_run, l_run));   // m = -inf: empty part
-                __threadfence();
-                asm volatile("bar.sync 1, 256;\n" ::: "memory");
-                if (tid == 0) {
-                    const int ticket = atomicAdd(cnt, 1);
-                    if (ticket == p.nsplit - 1) *cnt = 0;
-                    merge_ticket = ticket;
-                }
-                asm volatile("bar.sync 1, 256;\n" ::: "memory");
-            }
-            if (merge_ticket == p.nsplit - 1) {
-                __threadfence();
-                // The other parts' rows arrive through a ring of two shared-memory buffers per warp
-                // (16-byte cp.async, all copies of a buffer in flight together), in the order
-                // (column half, part).  The K/V stages serve as the ring: both warpgroups have passed
-                // their O_READY before the arrival barrier above, so no MMA reads them any more.
-                const int64_t own_off = (((int64_t)b * p.l_C + cq) * p.H + kvh * G + g) * D;     // this lane's row of O, in elements
-                const uint32_t own_lo = (uint32_t)own_off, own_hi = (uint32_t)(own_off >> 32);
-                constexpr int RING_BYTES = 2 * STAGES * KV_TILE_BYTES;
-                static_assert(RING_BYTES / 8 >= 2 * 32 * (D / 8) * 16, "two buffers of 32 rows x D/2 floats per warp");
-                float4* ring = reinterpret_cast<float4*>(sK + warp_u * (RING_BYTES / 8));
-                const int n_other = p.nsplit - 1, n_pairs = 2 * n_other;
-                auto other = [&](int i) { const int s = i % n_other; return s + (s >= split ? 1 : 0); };
-                auto issue = [&](int i) {
-                    const int h = i / n_other;
-                    const float* srcO = unit_base + other(i) * part_stride + h * DH;
-                    float4* buf = ring + (i & 1) * (32 * NC);
-#pragma unroll
-                    for (int it = 0; it < NC; ++it) {
-                        const int e = it * 32 + lane, rr = e / NC, c = e % NC;
-                        const bool ok = wrow0 + rr < R;
-                        cp_async16(buf + rr * NC + (c ^ (rr & (NC - 1))), srcO + (int64_t)(ok ? wrow0 + rr : 0) * D + c * 4,
-                                   ok ? 16 : 0);
-                    }
-                    cp_async_commit();
-                };
-                issue(0);
-                if (n_pairs > 1) issue(1);
-                // weights of the parts in the log2 domain (Algorithm 1's merge of (O, m, l))
-                float w[kAttPrefillSplits];
-                float m_max = m_run;
-                float2 ml[kAttPrefillSplits];
-#pragma unroll
-                for (int s = 0; s < kAttPrefillSplits; ++s) {
-                    ml[s] = make_float2(-INFINITY, 0.f);
-                    if (s < p.nsplit && s != split && row_ok)
-                        ml[s] = __ldcg(reinterpret_cast<const float2*>(unit_base + s * part_stride + (int64_t)Rp * D) + row);
-                    if (s == split) ml[s] = make_float2(m_run, l_run);
-                    m_max = fmaxf(m_max, ml[s].x);
-                }
-                float den = 0.f;
-#pragma unroll
-                for (int s = 0; s < kAttPrefillSplits; ++s) {
-                    w[s] = (ml[s].x == -INFINITY) ? 0.f : fast_exp2(ml[s].x - m_max);
-                    den += w[s] * ml[s].y;
-                }
-                const float inv = 1.f / den;
-                auto pick = [&](int s) { return s == 0 ? w[0] : s == 1 ? w[1] : s == 2 ? w[2] : w[3]; };   // no dynamic register indexing
+            if (n_tiles > 0 && wrow0 < R) {
 #pragma unroll 1
                 for (int h = 0; h < 2; ++h) {
-                    // The parts are added in split order whichever CTA happens to merge (its own part comes
-                    // from tensor memory, the others from the ring), so the result does not depend on the
-                    // order of arrival: the same bits as a merge pass over all parts.
-                    float acc[DH];
 #pragma unroll
-                    for (int i = 0; i < DH; ++i) acc[i] = 0.f;
-                    auto add_own = [&]() {
-                        const float wo = pick(split) * inv;       // 0 when this CTA's own part is empty
+                    for (int cc = 0; cc < DH; cc += 32) {
+                        uint32_t o[32];
+                        tmem_ld32(tO + h * DH + cc, o);
+                        tmem_wait_ld();
 #pragma unroll
-                        for (int cc = 0; cc < DH; cc += 16) {
-                            uint32_t o[16];
-                            tmem_ld16(tO + h * DH + cc, o);
-                            tmem_wait_ld();
-                            if (wo != 0.f) {
-#pragma unroll
-                                for (int i = 0; i < 16; ++i) acc[cc + i] = fmaf(wo, __uint_as_float(o[i]), acc[cc + i]);
-                            }
-                        }
-                    };
-                    int k = 0;                                    // index among the other parts
-#pragma unroll 1
-                    for (int sp = 0; sp < p.nsplit; ++sp) {
-                        if (sp == split) {
-                            add_own();
-                            continue;
-                        }
-                        const int i = h * n_other + k;
-                        ++k;
-                        if (i + 1 < n_pairs) cp_async_wait<1>();
-                        else cp_async_wait<0>();
-                        __syncwarp();
-                        const float4* buf = ring + (i & 1) * (32 * NC);
-                        const float ws = pick(sp) * inv;
-#pragma unroll
-                        for (int c = 0; c < NC; ++c) {
-                            const float4 val = buf[lane * NC + (c ^ (lane & (NC - 1)))];
-                            if (ws != 0.f) {                     // an empty part may hold anything
-                                acc[4 * c] = fmaf(ws, val.x, acc[4 * c]);
-                                acc[4 * c + 1] = fmaf(ws, val.y, acc[4 * c + 1]);
-                                acc[4 * c + 2] = fmaf(ws, val.z, acc[4 * c + 2]);
-                                acc[4 * c + 3] = fmaf(ws, val.w, acc[4 * c + 3]);
-                            }
-                        }
-                        __syncwarp();
-                        if (i + 2 < n_pairs) issue(i + 2);
+                        for (int q4 = 0; q4 < 8; ++q4)
+                            stage[lane * NC + ((cc / 4 + q4) ^ (lane & (NC - 1)))] =
+                                make_float4(__uint_as_float(o[4 * q4]), __uint_as_float(o[4 * q4 + 1]),
+                                            __uint_as_float(o[4 * q4 + 2]), __uint_as_float(o[4 * q4 + 3]));
                     }
-                    store_half_rows<D / 2>(acc, stage, lane, wrow0, R, own_lo, own_hi, p.O + h * DH);
+                    __syncwarp();
+#pragma unroll 4
+                    for (int it = 0; it < NC; ++it) {
+                        const int e = it * 32 + lane, rr = e / NC, c = e % NC;
+                        const float4 val = stage[rr * NC + (c ^ (rr & (NC - 1)))];
+                        if (wrow0 + rr < R)
+                            __stcg(reinterpret_cast<float4*>(myO + (int64_t)(wrow0 + rr) * D + h * DH) + c, val);
+                    }
+                    __syncwarp();
                 }
             }
+            if (row_ok) __stcg(reinterpret_cast<float2*>(myO + (int64_t)Rp * D) + row, make_float2(m_run, l_run));   // m = -inf: empty part
         }
     } else if (warp_u < TC_MMA_WARP) {
         // ------------------------------------------------------------ producers: Q, then K/V tiles
@@ -874,8 +753,10 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
         tc_fence_after_sync();
         issue_qk(0, 0);
         umma_commit(bar(BAR_S_READY + 0), lead);
-        issue_qk(1, 0);
-        umma_commit(bar(BAR_S_READY + 1), lead);
+        if (NQT == 2) {
+            issue_qk(1, 0);
+            umma_commit(bar(BAR_S_READY + 1), lead);
+        }
         umma_commit(bar(BAR_K_EMPTY + 0), lead);
         for (int T = 0; !planned || T < n_tiles; ++T) {
             const int s = T % STAGES;
@@ -888,7 +769,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
             mbar_wait(bar(BAR_V_FULL + s), (T / STAGES) & 1, wc);
             fence_async_smem();
 #pragma unroll
-            for (int qt = 0; qt < 2; ++qt) {
+            for (int qt = 0; qt < NQT; ++qt) {
                 mbar_wait(bar(BAR_P_READY + qt * 2 + 0), T & 1, wc);
                 tc_fence_after_sync();
                 issue_pv(qt, s, 0, T > 0);
@@ -902,11 +783,11 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
                 issue_pv(qt, s, 1, 1);
                 umma_commit(bar(BAR_PV_DONE + qt), lead);
                 if (!more) umma_commit(bar(BAR_O_READY + qt), lead);
-                if (qt == 1) umma_commit(bar(BAR_V_EMPTY + s), lead);
+                if (qt == NQT - 1) umma_commit(bar(BAR_V_EMPTY + s), lead);
                 if (more) {
                     issue_qk(qt, sn);         // overwrites S and P of this tile after the P V products above, in issue order
                     umma_commit(bar(BAR_S_READY + qt), lead);
-                    if (qt == 1) umma_commit(bar(BAR_K_EMPTY + sn), lead);
+                    if (qt == NQT - 1) umma_commit(bar(BAR_K_EMPTY + sn), lead);
                 }
             }
         }
@@ -926,18 +807,18 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
 
 }  // namespace
 
-template <int D, bool PAIR>
+template <int D, bool PAIR, int NQT>
 static cudaError_t launch_tc_kernel(esa_ctx* ctx, const CUtensorMap& qmap, const CUtensorMap& qgmap, const TcAttendParams& p,
                                     dim3 grid, cudaStream_t st, bool probe_only) {
     constexpr int smem = 2 * 128 * D * 2 + 2 * TC_STAGES * TC_BN * D * 2 + 1024;
     static KernelMemo memo;
-    cudaError_t e = allow_smem(attend_tc_kernel<D, PAIR>, ctx->device, smem, memo);
+    cudaError_t e = allow_smem(attend_tc_kernel<D, PAIR, NQT>, ctx->device, smem, memo);
     if (e != cudaSuccess) return e;
     // the in-kernel register split assumes the launch allocation it was sized for
     static int regs_checked = 0;
     if (!regs_checked) {
         cudaFuncAttributes fa;
-        e = cudaFuncGetAttributes(&fa, attend_tc_kernel<D, PAIR>);
+        e = cudaFuncGetAttributes(&fa, attend_tc_kernel<D, PAIR, NQT>);
         if (e != cudaSuccess) return e;
         if (fa.numRegs != TC_REGS_LAUNCH) return cudaErrorInvalidConfiguration;
         regs_checked = 1;
@@ -959,42 +840,58 @@ static cudaError_t launch_tc_kernel(esa_ctx* ctx, const CUtensorMap& qmap, const
     if (probe_only) {
         // can the device place a pair of these CTAs at all?
         int n_clusters = 0;
-        e = cudaOccupancyMaxActiveClusters(&n_clusters, attend_tc_kernel<D, PAIR>, &cfg);
+        e = cudaOccupancyMaxActiveClusters(&n_clusters, attend_tc_kernel<D, PAIR, NQT>, &cfg);
         if (e != cudaSuccess) return e;
         return n_clusters > 0 ? cudaSuccess : cudaErrorNotSupported;
     }
-    return cudaLaunchKernelEx(&cfg, attend_tc_kernel<D, PAIR>, qmap, qgmap, p);
+    return cudaLaunchKernelEx(&cfg, attend_tc_kernel<D, PAIR, NQT>, qmap, qgmap, p);
 }
 
+// Merge of a key list split more than two ways: a warp per row.
 template <int D>
-static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_max, cudaStream_t st, int* nsplit_out) {
+__global__ void __launch_bounds__(256) attend_tc_merge_kernel(const float* part, int nsplit, int Rp, int R, int G, int HG, int H, int l_C,
+                                                              __nv_bfloat16* O) {
+    pdl_wait();
+    pdl_launch_dependents();
+    const int lane = threadIdx.x & 31, row = blockIdx.x * 8 + (threadIdx.x >> 5);
+    const int kvh = blockIdx.y, b = blockIdx.z;
+    if (row >= R) return;
+    const float* unit = part + ((int64_t)b * HG + kvh) * nsplit * (int64_t)Rp * (D + 2);
+    merge_row<D>(unit + (int64_t)row * D, unit + (int64_t)Rp * D + 2 * row, (int64_t)Rp * (D + 2), nsplit, lane,
+                 O + (((int64_t)b * l_C + row / G) * H + kvh * G + row % G) * D);
+}
+
+template <int D, int NQT>
+static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_max, cudaStream_t st) {
     const int R = p.l_C * p.G;
     const int row_tiles = (R + TC_ROWS - 1) / TC_ROWS;
     p.Rp = (R + 1) & ~1;
-    if ((size_t)B * p.HG * row_tiles > ctx->att_count_elems) return cudaErrorNotSupported;
-    // Split the key list when that fills the machine better: cost model = waves x tiles per CTA
-    // (+ half a tile-equivalent of fixed work per CTA), one CTA per SM.  Two-position attention needs an even
-    // number of splits (one group per part); its longer part sets the tiles per CTA.
+    // Split the key list when that fills the machine better.  Cost in us, fitted to measured sweeps: 1.55 per 128-key tile
+    // of the longest CTA and 7 for its start and end, per wave (one CTA per SM); 7.5 for a pair's exchange or a merge
+    // launch, whose traffic (4 TB/s) counts; and 6 when the grid leaves the merge launch no SMs to start on meanwhile
+    // (37 queries, 8 units over 6300 keys: 41 us with 3 parts, 23 with 9, 21 with 14, 32 with 18).  Two-position
+    // attention needs an even number of splits (one group per part); its longer part sets the tiles per CTA.
     const int ctas = row_tiles * p.HG * B;
     const int n_tiles = (n_att_max + TC_BN - 1) / TC_BN;
     int i_end_max = 0;
     for (int b = 0; b < B; ++b) i_end_max = max(i_end_max, p.meta.i_end[b]);
     const int far_tiles = min(n_tiles, (i_end_max + p.top_k + TC_BN - 1) / TC_BN);
     const int step = p.two ? 2 : 1;
+    const double merge_bytes = (double)B * p.HG * p.Rp * (D + 2) * 4;      // per part
     int best = 0;
     double best_cost = 1e30;
     for (int ns = step; ns <= kAttPrefillSplits && (ns <= n_tiles || best == 0); ns += step) {
-        if ((size_t)B * p.HG * ns * p.Rp * (D + 2) > ctx->att_part_elems) break;
+        if (ns > 2 && (size_t)B * p.HG * ns * p.Rp * (D + 2) > ctx->att_part_elems) break;      // (pairs use no scratch)
         const int grp = p.two ? ns / 2 : ns;
         const int longest = p.two ? max(far_tiles, n_tiles - far_tiles + 1) : n_tiles;
         const int per = (longest + grp - 1) / grp;
         const int waves = (ctas * ns + ctx->num_sms - 1) / ctx->num_sms;
-        const double cost = (double)waves * (per + 0.5) + (ns > 1 ? 0.25 * ns : 0.0);
+        const double join = ns == 1 ? 0.0 : ns == 2 ? 7.5 : 7.5 + ns * merge_bytes / 4e6 + (ctas * ns * 8 > ctx->num_sms * 7 ? 6.0 : 0.0);
+        const double cost = waves * (1.55 * per + 7.0) + join;
         if (cost < best_cost - 1e-9) { best_cost = cost; best = ns; }
     }
     if (best == 0) return cudaErrorNotSupported;
     p.nsplit = best;
-    *nsplit_out = best;
     CUtensorMap qmap, qgmap;
     p.q_tma = make_tensor_map_q(&qmap, p.Q, (uint64_t)B * p.l_C, p.H, D, p.G) ? 1 : 0;
     if (p.q_tma && p.two) p.q_tma = make_tensor_map_q(&qgmap, p.Qg, (uint64_t)B * p.l_C, p.H, D, p.G) ? 1 : 0;
@@ -1003,25 +900,32 @@ static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_m
     const dim3 grid(row_tiles, p.HG, B * best);
     // a two-way split runs as CTA pairs that merge through distributed shared memory, where the device can place pairs
     static int pair_ok = -1;                                 // per instantiation; probed once
-    if (best == 2 && pair_ok < 0) pair_ok = launch_tc_kernel<D, true>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess ? 1 : 0;
-    ProfScope prof(ctx, KC_ATTEND_TC, st);
-    cudaError_t e = (best == 2 && pair_ok == 1) ? launch_tc_kernel<D, true>(ctx, qmap, qgmap, p, grid, st, false)
-                                                : launch_tc_kernel<D, false>(ctx, qmap, qgmap, p, grid, st, false);
+    if (best == 2 && pair_ok < 0) pair_ok = launch_tc_kernel<D, true, NQT>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess ? 1 : 0;
+    const bool pair = best == 2 && pair_ok == 1;
+    if (best == 2 && !pair && (size_t)B * p.HG * 2 * p.Rp * (D + 2) > ctx->att_part_elems) return cudaErrorNotSupported;
+    cudaError_t e;
+    {
+        ProfScope prof(ctx, KC_ATTEND_TC, st);
+        e = pair ? launch_tc_kernel<D, true, NQT>(ctx, qmap, qgmap, p, grid, st, false)
+                 : launch_tc_kernel<D, false, NQT>(ctx, qmap, qgmap, p, grid, st, false);
+    }
+    ctx->launches += 1;
+    if (e != cudaSuccess || best == 1 || pair) return e;
+    ProfScope prof(ctx, KC_ATTEND_MERGE, st);
+    e = launch_pdl(attend_tc_merge_kernel<D>, dim3((R + 7) / 8, p.HG, B), dim3(256), 0, st, (const float*)p.part, p.nsplit, p.Rp, R, p.G,
+                   p.HG, p.H, p.l_C, p.O);
     ctx->launches += 1;
     return e;
 }
 
-// Returns cudaErrorNotSupported when this path does not cover the shape (the caller then
-// uses the split kernel); nsplit_out reports how many ways the key list was split (merged in-kernel).
 cudaError_t launch_attend_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* Qg,
                              const __nv_bfloat16* K, const __nv_bfloat16* Kg, const __nv_bfloat16* V, const SeqMeta& meta,
                              const int32_t* idx, const int32_t* n_sel, __nv_bfloat16* O, int n_att_max, cudaStream_t st,
-                             int* nsplit_out, int64_t cache_rows, bool staged) {
+                             int64_t cache_rows, bool staged) {
     const bool two = Qg != nullptr || Kg != nullptr;
     TcAttendParams p;
     p.Q = Q; p.K = K; p.Qg = Qg ? Qg : Q; p.Kg = Kg ? Kg : K;
     p.V = V; p.O = O; p.idx = idx; p.n_sel = n_sel; p.part = ctx->att_part; p.status = ctx->status;
-    p.unit_count = ctx->att_count;
     p.staged = staged ? 1 : 0;
     p.two = two ? 1 : 0;
     p.early = ctx->attend_early && !two && !staged ? 1 : 0;
@@ -1029,8 +933,9 @@ cudaError_t launch_attend_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* 
     p.top_k = ctx->cfg.top_k; p.nsplit = 1;
     p.scale_log2 = ctx->scale * 1.4426950408889634f;
     p.meta = meta;
-    if (ctx->d == 128) return launch_tc<128>(ctx, p, B, n_att_max, st, nsplit_out);
-    if (ctx->d == 64) return launch_tc<64>(ctx, p, B, n_att_max, st, nsplit_out);
+    const bool one = l_C * ctx->G <= 128;
+    if (ctx->d == 128) return one ? launch_tc<128, 1>(ctx, p, B, n_att_max, st) : launch_tc<128, 2>(ctx, p, B, n_att_max, st);
+    if (ctx->d == 64) return one ? launch_tc<64, 1>(ctx, p, B, n_att_max, st) : launch_tc<64, 2>(ctx, p, B, n_att_max, st);
     return cudaErrorNotSupported;
 }
 

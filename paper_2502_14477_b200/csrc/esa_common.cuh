@@ -114,6 +114,61 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
+// Combines the nsplit partial results (O, m, l) of one row of a split key list -- Algorithm 1's merge -- and writes the
+// bf16 row: O = sum_s 2^(m_s - M) O_s / sum_s 2^(m_s - M) l_s with M = max_s m_s.  One warp; lane i owns D / 32
+// columns.  o: the row in part 0, ml: its (m, l) pair, parts `stride` floats apart (rows and pairs 8-byte aligned), nsplit <= 64.  The weights are
+// formed with one part per lane and the rows are read sixteen parts at a time, so that a merge is a few round trips to L2
+// however many parts there are (with four at a time, and the maximum searched part by part, 37 parts took 9 us).
+// Loads bypass L1: the parts may have been written by other SMs a moment ago.
+template <int D>
+__device__ __forceinline__ void merge_row(const float* o, const float* ml, int64_t stride, int nsplit, int lane, __nv_bfloat16* dst_row) {
+    constexpr int PER = D / 32, BATCH = 16;
+    float2 v[BATCH][PER / 2];
+    auto load = [&](int s0) {
+#pragma unroll
+        for (int j = 0; j < BATCH; ++j) {
+            const float* src = o + (int64_t)(s0 + j) * stride + lane * PER;
+#pragma unroll
+            for (int i = 0; i < PER / 2; ++i)
+                v[j][i] = s0 + j < nsplit ? __ldcg(reinterpret_cast<const float2*>(src + 2 * i)) : make_float2(0.f, 0.f);
+        }
+    };
+    load(0);
+    float2 a = make_float2(-INFINITY, 0.f), c = a;
+    if (lane < nsplit) a = __ldcg(reinterpret_cast<const float2*>(ml + lane * stride));
+    if (lane + 32 < nsplit) c = __ldcg(reinterpret_cast<const float2*>(ml + (lane + 32) * stride));
+    float M = fmaxf(a.x, c.x);
+#pragma unroll
+    for (int i = 16; i >= 1; i >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, i));
+    // (a part without keys has m = -inf: weight 0, and its row may hold anything)
+    const float w_a = a.x == -INFINITY ? 0.f : fast_exp2(a.x - M), w_b = c.x == -INFINITY ? 0.f : fast_exp2(c.x - M);
+    float den = w_a * a.y + w_b * c.y;
+#pragma unroll
+    for (int i = 16; i >= 1; i >>= 1) den += __shfl_xor_sync(0xffffffffu, den, i);
+    float acc[PER];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) acc[i] = 0.f;
+    for (int s0 = 0; s0 < nsplit; s0 += BATCH) {
+        if (s0 > 0) load(s0);
+#pragma unroll
+        for (int j = 0; j < BATCH; ++j) {
+            const int s = s0 + j;
+            const float w = __shfl_sync(0xffffffffu, s < 32 ? w_a : w_b, s & 31);
+            if (s < nsplit && w != 0.f) {
+#pragma unroll
+                for (int i = 0; i < PER / 2; ++i) {
+                    acc[2 * i] = fmaf(w, v[j][i].x, acc[2 * i]);
+                    acc[2 * i + 1] = fmaf(w, v[j][i].y, acc[2 * i + 1]);
+                }
+            }
+        }
+    }
+    const float inv = 1.f / den;
+#pragma unroll
+    for (int i = 0; i < PER; i += 2)
+        *reinterpret_cast<uint32_t*>(dst_row + lane * PER + i) = pack_bf16(acc[i] * inv, acc[i + 1] * inv);
+}
+
 // A-operand fragment (16 rows x 16 k) of a K-major tile: row0 = first row, kc = first
 // 16-byte chunk of the k-step.
 template <int ROW_CHUNKS>

@@ -269,7 +269,7 @@ static EncodeTiledFn encode_fn() {
 
 bool make_tensor_map_bf16(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows) {
     EncodeTiledFn fn = encode_fn();
-    if (!fn || cols % 64 || box_rows == 0 || box_rows > 256 || (reinterpret_cast<uintptr_t>(base) & 15)) return false;
+    if (!fn || (cols % 64 && cols != 32) || box_rows == 0 || box_rows > 256 || (reinterpret_cast<uintptr_t>(base) & 15)) return false;
     cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
     cuuint32_t box[2] = {64, box_rows};

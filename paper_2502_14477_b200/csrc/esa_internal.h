@@ -54,9 +54,10 @@ cudaError_t resident_per_sm(F* kernel, int device, int threads, int smem, Kernel
     return e;
 }
 
-constexpr int kAttMaxSplits = 64;     // split-KV factor of the attention kernel (small chunks)
-constexpr int kAttSplitRows = 64;     // split-KV is used only when l_C * (H/H_G) <= this
-constexpr int kAttPrefillSplits = 4; // largest split of a prefill-sized chunk's key list
+constexpr int kAttMaxSplits = 64;     // largest key-list split of the decode kernel
+constexpr int kAttSplitRows = 64;     // rows per key/value head for which the scratch holds kAttMaxSplits parts
+constexpr int kAttPrefillSplits = 32; // largest split of a prefill-sized chunk's key list
+constexpr int kAttPrefillParts = 4;  // ... of a full-sized chunk of one sequence (sizes the scratch)
 constexpr int kCompressGemvRows = 16;   // at most this many input rows (B * n_new): compression runs as a GEMV
 constexpr int kCompressMaxRows = 4096;
 
@@ -69,7 +70,7 @@ struct RowMap {
 // Kernel classes of the per-kernel timing facility (esa_set_profiling / esa_read_profile).
 enum KernelClass {
     KC_COMPRESS_TC = 0, KC_COMPRESS_GEMV, KC_COMPRESS_MMA, KC_APPEND_KV, KC_SCORE_PASS1, KC_SCORE_PASS2, KC_SCORE_MMA,
-    KC_SCORE_DECODE, KC_SCORE_FULL, KC_POOL_HIST, KC_SELECT_TOPK, KC_SELECT_ALL, KC_ATTEND_TC, KC_ATTEND_DECODE, KC_ATTEND_SMALL,
+    KC_SCORE_DECODE, KC_SCORE_FULL, KC_POOL_HIST, KC_SELECT_TOPK, KC_SELECT_ALL, KC_ATTEND_TC, KC_ATTEND_DECODE,
     KC_ATTEND_MERGE, KC_GATHER_KV, KC_COUNT
 };
 struct ProfRec {
@@ -77,8 +78,8 @@ struct ProfRec {
     cudaEvent_t a, b;
 };
 
-// TMA descriptor of a row-major bf16 matrix [rows, cols] (cols a multiple of 64), read in boxes of
-// box_rows x 64 columns with the 128-byte swizzle.  False when the driver entry point is missing
+// TMA descriptor of a row-major bf16 matrix [rows, cols] (cols a multiple of 64, or 32: the box then reads zeros past
+// the row), read in boxes of box_rows x 64 columns with the 128-byte swizzle.  False when the driver entry point is missing
 // or refuses the shape.
 bool make_tensor_map_bf16(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
 
@@ -136,7 +137,7 @@ struct esa_ctx {
     bool attend_early;   // set around the launch of an armed attention call
     float* att_part;     // split-KV partial outputs + (m, l)
     size_t att_part_elems;
-    int* att_count;      // arrival counters of the split prefill attention, one per (sequence, kv head, row tile); 0 between launches
+    int* att_count;      // arrival counters of the decode attention's in-kernel merge, one per (sequence, kv head); 0 between launches
     size_t att_count_elems;
     int* status;         // device status word
     int64_t launches;
@@ -194,7 +195,7 @@ cudaError_t launch_score(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_c
                          const SeqMeta& meta, int max_lM, bool rkey_cleared, bool ghist_cleared, cudaStream_t st,
                          bool* pooled_ready);
 
-// The same for chunks of >= 64 queries and d' in {64, 128} on tcgen05 with TMA-fed tiles; expects
+// The same on tcgen05 with TMA-fed tiles; expects
 // ctx->rkey zeroed (pass 1 clears what pass 2 accumulates into).  cudaErrorNotSupported when the shape is not covered.
 cudaError_t launch_score_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache,
                             const SeqMeta& meta, int max_lM, cudaStream_t st, bool* pooled_ready);
@@ -230,13 +231,13 @@ cudaError_t launch_gather_kv(esa_ctx* ctx, int B, int l_C, const void* K_host, c
                              const int32_t* idx, const int32_t* n_sel, void* K_stage, void* V_stage, int64_t stage_rows,
                              cudaStream_t st);
 
-// Prefill-sized chunks (l_C * H/H_G > kAttSplitRows) on tcgen05; *nsplit_out reports the number of
-// key-list splits (their partials pass through ctx->att_part and are merged inside the kernel).
+// Chunks on tcgen05 (the partials of a key list split more than two ways
+// pass through ctx->att_part and are merged by a second launch).
 // Qg / Kg non-null: two-position attention (both given then).
 cudaError_t launch_attend_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* Qg,
                              const __nv_bfloat16* K, const __nv_bfloat16* Kg, const __nv_bfloat16* V, const SeqMeta& meta,
                              const int32_t* idx, const int32_t* n_sel, __nv_bfloat16* O,
-                             int n_att_max, cudaStream_t st, int* nsplit_out, int64_t cache_rows = 0, bool staged = false);
+                             int n_att_max, cudaStream_t st, int64_t cache_rows = 0, bool staged = false);
 
 // TMA descriptor of the query tensor [n_queries, H, D] for the attention kernel (group size G must
 // divide 128).
@@ -257,11 +258,11 @@ cudaError_t launch_compress_tc(esa_ctx* ctx, const __nv_bfloat16* X, int B, int 
                                int64_t dst_seq_stride, const RowMap& map, uint32_t* zero_words, int zero_count,
                                cudaStream_t st, bool small_grid = false);
 
-// True when launch_score takes the tcgen05 path for this call.
-inline bool score_uses_tc(const esa_ctx* ctx, int B, int l_C) {
-    return l_C >= 64 && (ctx->dc == 64 || ctx->dc == 128) &&
-           (int64_t)B * ctx->cfg.max_tokens < (int64_t(1) << 31);
-}
+// True when launch_score takes the tcgen05 path for this call: every chunk (row numbers are 32-bit TMA coordinates).
+// For a handful of queries most of a 128-row tile is padding, but the passes are bound by the stream of keys and their
+// own latency, and pooling and the first radix digit come with the second pass: 37 queries after 50021 tokens, select
+// 51 -> 32 us against the mma.sync kernels with their memsets and pooling launch.
+inline bool score_uses_tc(const esa_ctx* ctx, int B) { return (int64_t)B * ctx->cfg.max_tokens < (int64_t(1) << 31); }
 
 cudaError_t launch_append_kv(esa_ctx* ctx, int B, const __nv_bfloat16* K_new,
                              const __nv_bfloat16* V_new, int n_new, __nv_bfloat16* K_cache,

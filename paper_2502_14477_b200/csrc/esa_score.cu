@@ -355,8 +355,9 @@ static cudaError_t launch_score_t(esa_ctx* ctx, int B, int l_C, const __nv_bfloa
         *pooled_ready = true;
         return e;
     }
-    // prefill-sized chunks with d' of 64 or 128: tcgen05 + TMA kernels (they clear what they accumulate into)
-    if (score_uses_tc(ctx, B, l_C)) {
+    // tcgen05 + TMA kernels (they clear what they accumulate into); the mma.sync kernels above remain for caches of
+    // 2^31 rows and more, which TMA coordinates do not reach
+    if (score_uses_tc(ctx, B)) {
         e = launch_score_tc(ctx, B, l_C, kc_cache, meta, max_lM, st, pooled_ready);
         if (e != cudaErrorNotSupported) return e;
         cudaGetLastError();

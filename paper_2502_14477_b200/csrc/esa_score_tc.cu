@@ -1,4 +1,4 @@
-// Eq. 6 + Eq. 4 (+ Eq. 8) for prefill-sized chunks on the 5th-generation tensor cores.
+// Eq. 6 + Eq. 4 (+ Eq. 8) for chunks of two queries or more on the 5th-generation tensor cores.
 //
 //   S[c, m] = q'_c . k'_m          r_c = max_m S[c, m]          s_m = max_c ( S[c, m] - r_c )
 //   s'_j = max of s over [j - eps, j + eps] clipped to M
@@ -483,13 +483,12 @@ cudaError_t launch_t(esa_ctx* ctx, int B, int l_C, const CUtensorMap& kmap, cons
 
 }  // namespace
 
-// Both scoring passes for chunks of at least 64 queries and d' of 64 or 128; rkey must be zeroed.
+// Both scoring passes; rkey must be zeroed.  d' = 32 runs as 64 with the upper half of every row read as zeros.
 // *pooled_ready: ctx->pkey and ctx->ghist0 hold the pooled keys and their first-digit histogram
 // (else ctx->skey holds the unpooled keys and ghist0 is zero).
 // Returns cudaErrorNotSupported when this path does not cover the shape.
 cudaError_t launch_score_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache, const SeqMeta& meta,
                             int max_lM, cudaStream_t st, bool* pooled_ready) {
-    if (l_C < 64 || (ctx->dc != 64 && ctx->dc != 128)) return cudaErrorNotSupported;
     // the descriptors of the last call serve again while the caller keeps its cache and chunk size
     const uint64_t k_rows = (uint64_t)B * ctx->cfg.max_tokens, q_rows = (uint64_t)B * l_C;
     if (!ctx->kc_map.matches(kc_cache, k_rows) && !ctx->kc_map.encode(kc_cache, k_rows, ctx->dc, ST_KEYS)) return cudaErrorNotSupported;
