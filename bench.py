@@ -125,7 +125,7 @@ def kernel_rooflines(prof: dict, sampled, cfg, peaks):
 
     tensor("attend_tc_kernel", sum(attend_flops(cfg, t, l_C) for t, l_C in sampled))
     tensor("score_tc_kernel<.,1>", sc, "one pass: (2 d' + 1) l_C l_M flops per launch")
-    tensor("score_tc_kernel<.,2>", sc, "second pass over the same products (the method counts one), with Eq. 4, Eq. 8 and the first radix digit in the epilogue")
+    tensor("score_tc_kernel<.,2>", sc, "second pass over the same products (the method counts one), with Eq. 4 and Eq. 8 in the epilogue")
     tensor("compress_tc_kernel", sum(compress_flops(cfg, l_C) for t, l_C in sampled),
            "both compressions of a chunk (keys on the side stream, queries ahead of the scoring); latency-bound launches")
     if "score_tc_kernel<.,1>" in out and "score_tc_kernel<.,2>" in out:
@@ -584,7 +584,7 @@ def time_extensions(peaks):
         pr = timed(lambda: ctx.select_full(Q, K, [t], idx, n_sel, per_head=per_head), key)
         us = pr["score_full_kernel<.,1>+<.,2>"]
         out[key] = {"score_us_per_call": us, "achieved_tflops": fl_full / us * 1e-6, "frac_burst": fl_full / us * 1e-6 / peaks["tflops_burst"],
-                    "pool_hist_us": pr.get("pool_hist_kernel"), "select_topk_us": pr.get("select_topk_kernel"),
+                    "pool_us": pr.get("pool_kernel"), "select_topk_us": pr.get("select_topk_kernel"),
                     "note": "mma.sync kernels (both passes timed together); flops = 2 passes x 2 d_H l_C l_M"}
     idx[0] = (torch.sort(torch.randperm(l_M, device="cuda", generator=g)[: cfg.k])[0] + i_end).to(torch.int32)
     n_sel[0] = cfg.k

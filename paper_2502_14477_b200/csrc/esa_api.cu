@@ -29,8 +29,8 @@ bool config_ok(const esa_config* c) {
 size_t align_up(size_t x) { return (x + 255) & ~size_t(255); }
 
 struct Layout {
-    size_t wq, wk, bq, bk, qc, rkey, rkey_heads, skey, pkey, ghist0, ghist1, cidx, slice_cnt, ticket, att, att_count, status, total;
-    size_t att_elems, att_count_elems, slice_stride;
+    size_t wq, wk, bq, bk, qc, rkey, rkey_heads, skey, pkey, att, att_count, status, total;
+    size_t att_elems, att_count_elems;
 };
 
 Layout make_layout(const esa_config* c) {
@@ -47,12 +47,6 @@ Layout make_layout(const esa_config* c) {
     L.rkey_heads = take(4 * (size_t)c->max_batch * c->max_chunk * c->n_q_heads);
     L.skey = take(4 * (size_t)c->max_batch * c->max_tokens);
     L.pkey = take(4 * (size_t)c->max_batch * c->max_tokens);
-    L.ghist0 = take(4 * (size_t)c->max_batch * 2048);
-    L.ghist1 = take(4 * (size_t)c->max_batch * 2048);
-    L.cidx = take(4 * (size_t)c->max_batch * c->max_tokens);
-    L.slice_stride = ((size_t)c->max_tokens + 4095) / 4096;
-    L.slice_cnt = take(4 * (size_t)c->max_batch * L.slice_stride);
-    L.ticket = take(4 * (size_t)c->max_batch);
     const size_t G = c->n_q_heads / c->n_kv_heads;
     size_t rows = (size_t)c->max_chunk * G;
     if (rows > (size_t)kAttSplitRows) rows = kAttSplitRows;
@@ -176,12 +170,6 @@ esa_status esa_create(const esa_config* cfg, esa_ctx** out) {
     c->rkey_heads = reinterpret_cast<uint32_t*>(base + L.rkey_heads);
     c->skey = reinterpret_cast<uint32_t*>(base + L.skey);
     c->pkey = reinterpret_cast<uint32_t*>(base + L.pkey);
-    c->ghist0 = reinterpret_cast<uint32_t*>(base + L.ghist0);
-    c->ghist1 = reinterpret_cast<uint32_t*>(base + L.ghist1);
-    c->cidx = reinterpret_cast<int32_t*>(base + L.cidx);
-    c->sel_slice_cnt = reinterpret_cast<int*>(base + L.slice_cnt);
-    c->sel_ticket = reinterpret_cast<int*>(base + L.ticket);
-    c->sel_slice_stride = (int)L.slice_stride;
     c->last_decode = false;
     c->sel_armed = false;
     c->sel_stream = nullptr;
@@ -192,8 +180,6 @@ esa_status esa_create(const esa_config* cfg, esa_ctx** out) {
     c->att_count_elems = L.att_count_elems;
     c->status = reinterpret_cast<int*>(base + L.status);
     if (cudaMemset(c->status, 0, 256) != cudaSuccess ||
-        cudaMemset(c->sel_ticket, 0, 4 * (size_t)cfg->max_batch) != cudaSuccess ||
-        cudaMemset(c->ghist1, 0, 4 * (size_t)cfg->max_batch * 2048) != cudaSuccess ||
         cudaMemset(c->att_count, 0, 4 * L.att_count_elems) != cudaSuccess) {
         cudaFree(base);
         delete c;
@@ -279,7 +265,7 @@ esa_status esa_compress_keys_async(esa_ctx* ctx, int32_t B, const void* K_new, i
     if (B * n_new <= kCompressGemvRows) {
         cudaError_t e = launch_compress_gemv(ctx, (const __nv_bfloat16*)K_new, B, n_new, ctx->dG, ctx->Wk,
                                              ctx->has_bk ? ctx->bk : nullptr, (__nv_bfloat16*)kc_cache,
-                                             ctx->cfg.max_tokens, map, nullptr, 0, nullptr, 0, (cudaStream_t)stream);
+                                             ctx->cfg.max_tokens, map, nullptr, 0, (cudaStream_t)stream);
         if (e != cudaErrorNotSupported) return from_cuda(e);
         cudaGetLastError();
     }
@@ -336,14 +322,11 @@ esa_status esa_select_async(esa_ctx* ctx, int32_t B, const void* Q_cur, int32_t 
     RowMap zero;
     for (int b = 0; b < kMaxBatch; ++b) zero.row0[b] = 0;
     e = cudaErrorNotSupported;
-    bool rkey_cleared = false, ghist_cleared = false;
+    bool rkey_cleared = false;
     if (B * l_C <= kCompressGemvRows) {
-        // (with one query per sequence the scoring kernel also accumulates first-digit histograms: cleared here too)
         e = launch_compress_gemv(ctx, (const __nv_bfloat16*)Q_cur, B, l_C, ctx->dH, ctx->Wq,
-                                 ctx->has_bq ? ctx->bq : nullptr, ctx->Qc, l_C, zero, ctx->rkey, B * l_C,
-                                 l_C == 1 ? ctx->ghist0 : nullptr, B * 2048, st);
+                                 ctx->has_bq ? ctx->bq : nullptr, ctx->Qc, l_C, zero, ctx->rkey, B * l_C, st);
         rkey_cleared = e == cudaSuccess;
-        ghist_cleared = rkey_cleared && l_C == 1;
     }
     if (e == cudaErrorNotSupported && ctx->has_wmaps) {
         // the compression kernel also clears the row-maximum words that the scoring pass accumulates into
@@ -363,8 +346,7 @@ esa_status esa_select_async(esa_ctx* ctx, int32_t B, const void* Q_cur, int32_t 
         if (meta.m_end[b] - meta.i_end[b] <= ctx->cfg.top_k) smeta.m_end[b] = smeta.i_end[b];
     ctx->last_decode = l_C == 1;
     bool pooled_ready = false;
-    e = launch_score(ctx, B, l_C, (const __nv_bfloat16*)kc_cache, smeta, max_lM, rkey_cleared, ghist_cleared, st,
-                     &pooled_ready);
+    e = launch_score(ctx, B, l_C, (const __nv_bfloat16*)kc_cache, smeta, max_lM, rkey_cleared, st, &pooled_ready);
     if (e != cudaSuccess) return ESA_ERR_CUDA;
     e = launch_select(ctx, B, l_C == 1, smeta, max_lM, pooled_ready, idx_out, n_sel_out, st);
     if (e == cudaSuccess) arm_attention(ctx, st);
@@ -514,7 +496,7 @@ esa_status esa_read_pooled_scores(esa_ctx* ctx, int32_t b, float* dst_host, int6
     if (n > ctx->last_lM[b]) return ESA_ERR_CAPACITY;
     if (n == 0) return ESA_OK;
     cudaStream_t st = (cudaStream_t)stream;
-    // the candidate-key buffer of this sequence is free again after the selection: stage there
+    // the unpooled keys of this sequence are no longer needed after the selection: stage there
     float* tmp = reinterpret_cast<float*>(ctx->skey + (int64_t)b * ctx->cfg.max_tokens);
     if (launch_read_pooled(ctx, b, tmp, n, st) != cudaSuccess) return ESA_ERR_CUDA;
     if (cudaMemcpyAsync(dst_host, tmp, 4 * (size_t)n, cudaMemcpyDeviceToHost, st) != cudaSuccess) return ESA_ERR_CUDA;
@@ -543,7 +525,7 @@ const char* esa_kernel_class_name(int32_t cls) {
     static const char* names[KC_COUNT] = {
         "compress_tc_kernel", "compress_gemv_kernel", "compress_kernel", "append_kv_kernel", "score_tc_kernel<.,1>",
         "score_tc_kernel<.,2>", "score_pass_kernel<.,1>+<.,2>", "score_decode_kernel", "score_full_kernel<.,1>+<.,2>",
-        "pool_hist_kernel",
+        "pool_kernel",
         "select_topk_kernel", "select_all_kernel", "attend_tc_kernel", "attend_decode_kernel",
         "attend_tc_merge_kernel", "gather_kv_kernel"};
     return cls >= 0 && cls < KC_COUNT ? names[cls] : "";
@@ -590,8 +572,6 @@ esa_status esa_last_device_status(esa_ctx* ctx, void* stream) {
         if (cudaMemsetAsync(ctx->status, 0, sizeof(int), st) != cudaSuccess) return ESA_ERR_CUDA;
         // a kernel that gave up may have left arrival counters of the in-kernel merges behind
         if (cudaMemsetAsync(ctx->att_count, 0, sizeof(int) * ctx->att_count_elems, st) != cudaSuccess) return ESA_ERR_CUDA;
-        if (cudaMemsetAsync(ctx->sel_ticket, 0, sizeof(int) * ctx->cfg.max_batch, st) != cudaSuccess) return ESA_ERR_CUDA;
-        if (cudaMemsetAsync(ctx->ghist1, 0, sizeof(uint32_t) * ctx->cfg.max_batch * 2048, st) != cudaSuccess) return ESA_ERR_CUDA;
         return (esa_status)h;
     }
     return ESA_OK;

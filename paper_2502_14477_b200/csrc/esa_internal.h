@@ -70,7 +70,7 @@ struct RowMap {
 // Kernel classes of the per-kernel timing facility (esa_set_profiling / esa_read_profile).
 enum KernelClass {
     KC_COMPRESS_TC = 0, KC_COMPRESS_GEMV, KC_COMPRESS_MMA, KC_APPEND_KV, KC_SCORE_PASS1, KC_SCORE_PASS2, KC_SCORE_MMA,
-    KC_SCORE_DECODE, KC_SCORE_FULL, KC_POOL_HIST, KC_SELECT_TOPK, KC_SELECT_ALL, KC_ATTEND_TC, KC_ATTEND_DECODE,
+    KC_SCORE_DECODE, KC_SCORE_FULL, KC_POOL, KC_SELECT_TOPK, KC_SELECT_ALL, KC_ATTEND_TC, KC_ATTEND_DECODE,
     KC_ATTEND_MERGE, KC_GATHER_KV, KC_COUNT
 };
 struct ProfRec {
@@ -118,15 +118,8 @@ struct esa_ctx {
     __nv_bfloat16* Qc;   // [max_batch * max_chunk, dc]
     uint32_t* rkey;      // [max_batch * max_chunk] ordered keys of the row maxima r_c
     uint32_t* rkey_heads;  // [max_batch, H, max_chunk] row maxima of the full-dimension / per-head scoring variants
-    uint32_t* skey;      // [max_batch, max_tokens] unpooled aggregated scores (ordered keys) of the scoring paths that do not pool;
-                         // afterwards the selection's candidate keys
+    uint32_t* skey;      // [max_batch, max_tokens] unpooled aggregated scores (ordered keys) of the scoring paths that do not pool
     uint32_t* pkey;      // [max_batch, max_tokens] pooled scores s' as ordered keys (l_C = 1: of the pooled raw scores, r not yet subtracted)
-    uint32_t* ghist0;    // [max_batch, 2048] histograms of pkey's top 11 bits (first radix digit)
-    uint32_t* ghist1;    // [max_batch, 2048] second-digit histograms of the selection kernel; 0 between launches
-    int32_t* cidx;       // [max_batch, max_tokens] positions of the selection's candidates
-    int* sel_slice_cnt;  // [max_batch, sel_slice_stride] candidates per slice of the selection kernel (sized for 4096-token slices, the kernel uses larger ones)
-    int* sel_ticket;     // [max_batch] arrival tickets of the selection kernel; 0 between launches
-    int sel_slice_stride;
     bool last_decode;    // the last selection ran with l_C = 1 (pkey holds raw pooled scores)
     // The attention kernels may read cache rows older than the chunk ahead of their wait for the preceding kernel
     // only when the work ahead of them in the stream is known not to write such rows: a selection enqueued through
@@ -187,13 +180,11 @@ cudaError_t launch_compress(esa_ctx* ctx, const __nv_bfloat16* X, int B, int row
                             int64_t dst_seq_stride, const RowMap& map, cudaStream_t st);
 
 // Eq. 6 + Eq. 4: fills ctx->skey (and ctx->rkey) for the middle tokens of every sequence.
-// l_C = 1: fills ctx->pkey (pooled raw scores), ctx->ghist0 and ctx->rkey instead.
-// rkey_cleared / ghist_cleared: the caller's compression kernel has already zeroed ctx->rkey / ctx->ghist0 for this call.
-// *pooled_ready: ctx->pkey and ctx->ghist0 hold the pooled keys and their first-digit histogram; otherwise
-// ctx->skey holds unpooled keys and ctx->ghist0 is zero.
+// l_C = 1: fills ctx->pkey (pooled raw scores) and ctx->rkey instead.
+// rkey_cleared: the caller's compression kernel has already zeroed ctx->rkey for this call.
+// *pooled_ready: ctx->pkey holds the pooled keys; otherwise ctx->skey holds unpooled keys.
 cudaError_t launch_score(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache,
-                         const SeqMeta& meta, int max_lM, bool rkey_cleared, bool ghist_cleared, cudaStream_t st,
-                         bool* pooled_ready);
+                         const SeqMeta& meta, int max_lM, bool rkey_cleared, cudaStream_t st, bool* pooled_ready);
 
 // The same on tcgen05 with TMA-fed tiles; expects
 // ctx->rkey zeroed (pass 1 clears what pass 2 accumulates into).  cudaErrorNotSupported when the shape is not covered.
@@ -209,7 +200,7 @@ cudaError_t launch_select(esa_ctx* ctx, int B, bool mapped, const SeqMeta& meta,
                           int32_t* idx_out, int32_t* n_sel_out, cudaStream_t st);
 
 // Eq. 3 + Eq. 4 on the uncompressed queries and keys (per_head: the per-head vote of Section 4.3): unpooled keys to
-// ctx->skey, ctx->ghist0 zeroed.
+// ctx->skey.
 cudaError_t launch_score_full(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* K, const SeqMeta& meta,
                               int max_lM, bool per_head, cudaStream_t st);
 
@@ -246,11 +237,11 @@ bool make_tensor_map_q(CUtensorMap* map, const void* base, uint64_t n_queries, i
 // Eq. 5 on tcgen05 for d' in {64, 128} and d_in a multiple of 128.  X is [rows, d_in] contiguous.
 // cudaErrorNotSupported when the shape is not covered (the caller then uses the mma.sync kernel).
 // Compression of a handful of rows (B * rows_per_seq <= kCompressGemvRows) as a GEMV; optionally clears
-// zero_count words at zero_words (one CTA) and zero2_count words at zero2_words (spread over the grid).  cudaErrorNotSupported when the shape is not covered.
+// zero_count words at zero_words.  cudaErrorNotSupported when the shape is not covered.
 cudaError_t launch_compress_gemv(esa_ctx* ctx, const __nv_bfloat16* X, int B, int rows_per_seq, int d_in,
                                  const __nv_bfloat16* W, const float* bias, __nv_bfloat16* dst,
                                  int64_t dst_seq_stride, const RowMap& map, uint32_t* zero_words, int zero_count,
-                                 uint32_t* zero2_words, int zero2_count, cudaStream_t st);
+                                 cudaStream_t st);
 // small_grid: the result is not needed at once (key compression: its rows enter M only l_L tokens later, and callers
 // run it on a side stream), so the grid is kept to an eighth of the SMs instead of as many CTAs as shorten the call.
 cudaError_t launch_compress_tc(esa_ctx* ctx, const __nv_bfloat16* X, int B, int rows_per_seq, int d_in,

@@ -187,24 +187,20 @@ score_pass_kernel(ScoreParams p) {
 // proximity pooling of Eq. 8 commutes with subtracting r (x -> fl(x - r) is monotone), so the
 // kernel pools the raw scores: P_j = max of S over [j - eps, j + eps] clipped to M.  It leaves
 //   * pkey[m]  = order-preserving key of P_m,
-//   * ghist0   = per-sequence histogram of the keys' top 11 bits (first radix digit of Eq. 2),
 //   * rkey[b]  = key of r (atomic max),
-// and the selection kernel finds the k-th largest P, maps the threshold through fl(. - r) and
-// compacts on fl(P_m - r): exactly the set that selecting on s' would give, ties included.
+// and the selection kernel subtracts r from the scores as it reads them.
 // A CTA owns up to SD_TOKENS consecutive middle tokens (plus eps recomputed neighbours on each side),
-// so the window maxima come from shared memory and the histogram is flushed once per CTA.
+// so the window maxima come from shared memory.
 // ---------------------------------------------------------------------------
 constexpr int SD_TOKENS = 2048;
 constexpr int SD_HALO = 16;          // largest eps
 constexpr int SD_THREADS = 256;
-constexpr int SD_BINS = 2048;
 
 struct ScoreDecodeParams {
     const __nv_bfloat16* kc;
     const __nv_bfloat16* qc;    // [B, DC]
     uint32_t* rkey;             // [B]
     uint32_t* pkey;             // [B, max_tokens] keys of the pooled raw scores
-    uint32_t* ghist0;           // [B, SD_BINS], zero on entry
     int64_t max_tokens;
     int eps;
     int chunk;                  // middle tokens per CTA: a multiple of SD_THREADS, at most SD_TOKENS
@@ -218,7 +214,6 @@ score_decode_kernel(ScoreDecodeParams p) {
     constexpr int RPW = 32 / LPR;       // rows per warp access
     constexpr int UNROLL = 4;
     __shared__ float sS[SD_TOKENS + 2 * SD_HALO];
-    __shared__ uint32_t shist[SD_BINS];
     __shared__ float smax[SD_THREADS / 32];
     pdl_wait();
     pdl_launch_dependents();
@@ -231,7 +226,6 @@ score_decode_kernel(ScoreDecodeParams p) {
     const int nb = min(p.chunk, l_M - a);
     const int eps = p.eps;
     const uint4* kc = reinterpret_cast<const uint4*>(p.kc + ((int64_t)b * p.max_tokens + i_end) * DC);
-    for (int i = tid; i < SD_BINS; i += SD_THREADS) shist[i] = 0u;
 
     float q[8];
     {
@@ -288,7 +282,7 @@ score_decode_kernel(ScoreDecodeParams p) {
         for (int w = 1; w < SD_THREADS / 32; ++w) v = fmaxf(v, smax[w]);
         if (v > -INFINITY) atomicMax(p.rkey + b, f32_to_key(v));
     }
-    // Eq. 8 on the raw scores, keys, first radix digit
+    // Eq. 8 on the raw scores, keys
     uint32_t* pk = p.pkey + (int64_t)b * p.max_tokens + a;
     float best[SD_TOKENS / SD_THREADS];
 #pragma unroll
@@ -303,24 +297,13 @@ score_decode_kernel(ScoreDecodeParams p) {
 #pragma unroll
     for (int qd = 0; qd < SD_TOKENS / SD_THREADS; ++qd) {
         const int i = qd * SD_THREADS + tid;
-        const bool valid = i < nb;
-        const uint32_t key = f32_to_key(best[qd]);
-        if (valid) pk[i] = key;
-        // aggregated over the warp: neighbouring tokens crowd into a few bins
-        const uint32_t peers = __match_any_sync(0xffffffffu, valid ? (key >> 21) : 0xffffffffu);
-        if (valid && lane == __ffs(peers) - 1) atomicAdd(&shist[key >> 21], (uint32_t)__popc(peers));
-    }
-    __syncthreads();
-    uint32_t* gh = p.ghist0 + (int64_t)b * SD_BINS;
-    for (int i = tid; i < SD_BINS; i += SD_THREADS) {
-        const uint32_t c = shist[i];
-        if (c) atomicAdd(gh + i, c);
+        if (i < nb) pk[i] = f32_to_key(best[qd]);
     }
 }
 
 template <int DC>
 static cudaError_t launch_score_t(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache,
-                                  const SeqMeta& meta, int max_lM, bool rkey_cleared, bool ghist_cleared, cudaStream_t st,
+                                  const SeqMeta& meta, int max_lM, bool rkey_cleared, cudaStream_t st,
                                   bool* pooled_ready) {
     cudaError_t e = cudaSuccess;
     *pooled_ready = false;
@@ -329,12 +312,8 @@ static cudaError_t launch_score_t(esa_ctx* ctx, int B, int l_C, const __nv_bfloa
     if (l_C == 1) {
         ScoreDecodeParams p;
         p.kc = kc_cache; p.qc = ctx->Qc; p.rkey = ctx->rkey;
-        p.pkey = ctx->pkey; p.ghist0 = ctx->ghist0;
+        p.pkey = ctx->pkey;
         p.max_tokens = ctx->cfg.max_tokens; p.eps = ctx->cfg.eps; p.meta = meta;
-        if (!ghist_cleared) {
-            e = cudaMemsetAsync(ctx->ghist0, 0, sizeof(uint32_t) * (size_t)B * SD_BINS, st);
-            if (e != cudaSuccess) return e;
-        }
         // Tokens per CTA.  All CTAs are resident at once and the kernel ends with the SM that got the most work,
         // so the choice minimises (CTAs on the fullest SM) x (tokens per CTA + the CTA's serial start and tail:
         // clear, pooling, flush, worth about 256 tokens of loads).  Measured with 8 x 129k tokens: 2048 tokens
@@ -362,9 +341,6 @@ static cudaError_t launch_score_t(esa_ctx* ctx, int B, int l_C, const __nv_bfloa
         if (e != cudaErrorNotSupported) return e;
         cudaGetLastError();
     }
-    // the pooling kernel that follows adds to the first-digit histograms
-    e = cudaMemsetAsync(ctx->ghist0, 0, sizeof(uint32_t) * (size_t)B * SD_BINS, st);
-    if (e != cudaSuccess) return e;
     e = cudaMemset2DAsync(ctx->skey, sizeof(uint32_t) * ctx->cfg.max_tokens, 0,
                           sizeof(uint32_t) * (size_t)max_lM, B, st);
     if (e != cudaSuccess) return e;
@@ -391,11 +367,11 @@ static cudaError_t launch_score_t(esa_ctx* ctx, int B, int l_C, const __nv_bfloa
 }
 
 cudaError_t launch_score(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache, const SeqMeta& meta,
-                         int max_lM, bool rkey_cleared, bool ghist_cleared, cudaStream_t st, bool* pooled_ready) {
+                         int max_lM, bool rkey_cleared, cudaStream_t st, bool* pooled_ready) {
     switch (ctx->dc) {
-        case 32: return launch_score_t<32>(ctx, B, l_C, kc_cache, meta, max_lM, rkey_cleared, ghist_cleared, st, pooled_ready);
-        case 64: return launch_score_t<64>(ctx, B, l_C, kc_cache, meta, max_lM, rkey_cleared, ghist_cleared, st, pooled_ready);
-        case 128: return launch_score_t<128>(ctx, B, l_C, kc_cache, meta, max_lM, rkey_cleared, ghist_cleared, st, pooled_ready);
+        case 32: return launch_score_t<32>(ctx, B, l_C, kc_cache, meta, max_lM, rkey_cleared, st, pooled_ready);
+        case 64: return launch_score_t<64>(ctx, B, l_C, kc_cache, meta, max_lM, rkey_cleared, st, pooled_ready);
+        case 128: return launch_score_t<128>(ctx, B, l_C, kc_cache, meta, max_lM, rkey_cleared, st, pooled_ready);
     }
     return cudaErrorInvalidValue;
 }

@@ -224,12 +224,11 @@ score_full_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
 __global__ void __launch_bounds__(256)
 full_prepare_kernel(const __nv_bfloat16* __restrict__ Q, __nv_bfloat16* __restrict__ Qf, int64_t rows, int dG, int d, int G, int fold,
                     uint32_t* __restrict__ rkey, int64_t n_rkey, uint32_t* __restrict__ skey, int64_t max_tokens, int clear_keys,
-                    int B, uint32_t* __restrict__ ghist0, int n_hist) {
+                    int B) {
     pdl_wait();
     pdl_launch_dependents();
     const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = i0; i < n_rkey; i += step) rkey[i] = 0u;
-    for (int64_t i = i0; i < n_hist; i += step) ghist0[i] = 0u;
     for (int64_t i = i0; i < (int64_t)B * clear_keys; i += step) skey[i / clear_keys * max_tokens + i % clear_keys] = 0u;
     if (!fold) return;
     const int per_row = dG / 2;
@@ -295,7 +294,7 @@ cudaError_t launch_pass(esa_ctx* ctx, FullTcParams p, const FullTile& t, const C
 
 }  // namespace
 
-// Fills ctx->skey with the unpooled full-dimension scores (ordered keys); ctx->ghist0 is zero afterwards.
+// Fills ctx->skey with the unpooled full-dimension scores (ordered keys).
 // The keys of M may be loaded ahead of a pass's wait for the kernel before it: everything enqueued ahead of the call
 // has completed when the first launch below lets its dependents start, and M ends before the current chunk.
 cudaError_t launch_score_full(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* K, const SeqMeta& meta,
@@ -311,7 +310,7 @@ cudaError_t launch_score_full(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16*
     if (gx < 1) gx = 1;
     ProfScope prof(ctx, KC_SCORE_FULL, st);
     cudaError_t e = launch_pdl(full_prepare_kernel, dim3(gx), dim3(256), 0, st, Q, Qf, rows, ctx->dG, ctx->d, ctx->G, fold ? 1 : 0,
-                               ctx->rkey_heads, n_rkey, ctx->skey, ctx->cfg.max_tokens, per_head ? 0 : max_lM, B, ctx->ghist0, B * 2048);
+                               ctx->rkey_heads, n_rkey, ctx->skey, ctx->cfg.max_tokens, per_head ? 0 : max_lM, B);
     if (e != cudaSuccess) return e;
     ctx->launches += 1;
     if (per_head) return launch_score_tc_heads(ctx, B, l_C, Q, K, meta, max_lM, st);

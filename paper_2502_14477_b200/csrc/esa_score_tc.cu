@@ -24,8 +24,7 @@
 //           A CTA owns a contiguous range of keys and also computes the eps keys on either side
 //           of it (its tiles start eps keys early and the ranges are 128 n - 2 eps long), so the
 //           proximity pooling of Eq. 8 needs no other CTA: pooled scores leave as order-preserving
-//           keys, together with the histogram of their top 11 bits (the first radix digit of the
-//           selection, Eq. 2).
+//           keys.
 // Swapping the operands keeps both reductions inside a thread.  Every S[c, m] is the same
 // sum of the same exact bf16 products taken in the same order over d' in both passes, so
 // pass 2 reproduces pass 1's value and S - r_c is exactly 0 at each query's arg-max.
@@ -51,7 +50,6 @@ constexpr int ST_THREADS = 352;
 constexpr int ST_EPI_WARP0 = 3;    // first epilogue warp
 constexpr int ST_EPI = 256;        // epilogue threads
 constexpr int ST_QCAP = 512;       // compressed queries resident per CTA
-constexpr int ST_BINS = 2048;      // first radix digit: top 11 bits of a key
 constexpr int ST_RING = 256;       // pooled-score ring: two tiles of aggregated scores
 constexpr int ST_ONES_BYTES = ST_KEYS * 32;    // ninth k-step, key side: 128 rows x 16 bf16
 constexpr int ST_RT_BYTES = ST_QCAP * 32;      // ninth k-step, query side: 512 rows x 16 bf16
@@ -60,7 +58,6 @@ struct ScoreTcParams {
     uint32_t* rkey;     // [B, heads, l_C] ordered keys of r_c
     uint32_t* skey;     // [B, max_tokens] ordered keys of s_m (index = m - i_end); used when !pool
     uint32_t* pkey;     // [B, max_tokens] ordered keys of s'_m; written when pool
-    uint32_t* ghist0;   // [B, ST_BINS] histogram of the top 11 bits of pkey; zeroed by pass 1
     int* status;
     int64_t max_tokens;
     int l_C;
@@ -68,7 +65,7 @@ struct ScoreTcParams {
     int groups;         // gridDim.y: heads x groups of up to ST_QCAP queries
     int heads;          // 1 (compressed scores), or H: every head scores by itself (Section 4.3's vote)
     int G;              // heads > 1: query heads per key/value head
-    int pool;           // pass 2 pools and writes pkey and ghist0 (one group per sequence), else skey
+    int pool;           // pass 2 pools and writes pkey (one group per sequence), else skey
     SeqMeta meta;
 };
 
@@ -97,7 +94,7 @@ struct ScoreCfg {
     static constexpr int NMW = PASS == 1 ? 2 : 1;              // warps that issue MMAs
     static constexpr int TILE_BYTES = ST_KEYS * DC * 2;
     static constexpr int Q_BYTES = ST_QCAP * DC * 2;
-    static constexpr int EXTRA = PASS == 1 ? 0 : (ST_ONES_BYTES + ST_RT_BYTES + ST_RING * 4 + 2 * ST_KEYS * 4 + ST_BINS * 4);
+    static constexpr int EXTRA = PASS == 1 ? 0 : (ST_ONES_BYTES + ST_RT_BYTES + ST_RING * 4 + 2 * ST_KEYS * 4);
     static constexpr int SMEM = Q_BYTES + STAGES * TILE_BYTES + EXTRA + 1024;
     static constexpr int MAX_UNITS = ST_QCAP / UNIT;
     // barrier slots
@@ -125,7 +122,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
     uint8_t* sRt = sOnes + ST_ONES_BYTES;                          // pass 2: query side of the ninth k-step (pieces of -r_c)
     float* sS = reinterpret_cast<float*>(sRt + ST_RT_BYTES);       // [ST_RING] aggregated scores of the last two tiles
     float* sX = sS + ST_RING;                                      // [2][ST_KEYS] partial maxima of the second column half
-    uint32_t* sHist = reinterpret_cast<uint32_t*>(sX + 2 * ST_KEYS);   // [ST_BINS]
     __shared__ uint64_t bars[C::B_COUNT];
     __shared__ uint32_t tmem_slot;
     __shared__ int abort_flag;
@@ -292,7 +288,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
                 *reinterpret_cast<uint4*>(sOnes + plain_tile_offset(et, 1)) = make_uint4(0u, 0u, 0u, 0u);
             }
             if (fused) {
-                for (int i = e256; i < ST_BINS; i += ST_EPI) sHist[i] = 0u;
                 for (int i = e256; i < ST_RING; i += ST_EPI) sS[i] = -INFINITY;
             }
         }
@@ -301,11 +296,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
         // before it wrote is final (which is what lets a kernel load such data ahead of its own wait).
         pdl_wait();
         pdl_launch_dependents();
-        if (PASS == 1) {
-            // first CTA of a sequence: the histogram that pass 2 (or the pooling kernel) adds to
-            if (blockIdx.x == 0 && blockIdx.y == 0)
-                for (int i = e256; i < ST_BINS; i += ST_EPI) p.ghist0[(int64_t)b * ST_BINS + i] = 0u;
-        } else {
+        if (PASS == 2) {
             // query side of the ninth k-step: the three bf16 pieces of -r_c (exact: r_c = r1 + r2 + r3);
             // columns past the chunk get -inf, which no maximum picks
             for (int i = e256; i < ST_QCAP; i += ST_EPI) {
@@ -405,11 +396,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
                             float best = -INFINITY;
                             if (valid)
                                 for (int dlt = -eps; dlt <= eps; ++dlt) best = fmaxf(best, sS[(ul + dlt) & (ST_RING - 1)]);
-                            const uint32_t key = f32_to_key(best);
-                            if (valid) p.pkey[(int64_t)b * p.max_tokens + mo] = key;
-                            // histogram of the first radix digit, aggregated over the warp (neighbouring keys crowd into few bins)
-                            const uint32_t peers = __match_any_sync(0xffffffffu, valid ? (key >> 21) : 0xffffffffu);
-                            if (valid && lane == __ffs(peers) - 1) atomicAdd(&sHist[key >> 21], (uint32_t)__popc(peers));
+                            if (valid) p.pkey[(int64_t)b * p.max_tokens + mo] = f32_to_key(best);
                             asm volatile("bar.sync 1, 128;\n" ::: "memory");      // the ring slot of tile lt - 1 may be overwritten next
                         }
                     }
@@ -423,13 +410,6 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
             if (qb + 128 < p.l_C && rm1 > -INFINITY) atomicMax(rk + qb + 128, f32_to_key(rm1));
             if (qb + 256 < p.l_C && rm2 > -INFINITY) atomicMax(rk + qb + 256, f32_to_key(rm2));
             if (qb + 384 < p.l_C && rm3 > -INFINITY) atomicMax(rk + qb + 384, f32_to_key(rm3));
-        } else if (fused && n_items > 0) {
-            asm volatile("bar.sync 2, 256;\n" ::: "memory");
-            uint32_t* gh = p.ghist0 + (int64_t)b * ST_BINS;
-            for (int i = e256; i < ST_BINS; i += ST_EPI) {
-                const uint32_t c = sHist[i];
-                if (c) atomicAdd(gh + i, c);
-            }
         }
     }
     // (every thread passes the wait for the preceding kernel before the CTA ends: a CTA's exit also
@@ -445,7 +425,7 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
 template <int DC>
 cudaError_t launch_t(esa_ctx* ctx, int B, int l_C, const CUtensorMap& kmap, const CUtensorMap& qmap, ScoreTcParams& p, const SeqMeta& meta,
                      int max_lM, cudaStream_t st) {
-    p.skey = ctx->skey; p.pkey = ctx->pkey; p.ghist0 = ctx->ghist0; p.status = ctx->status;
+    p.skey = ctx->skey; p.pkey = ctx->pkey; p.status = ctx->status;
     p.max_tokens = ctx->cfg.max_tokens; p.l_C = l_C; p.eps = ctx->cfg.eps; p.meta = meta;
     using C1 = ScoreCfg<DC, 1>;
     using C2 = ScoreCfg<DC, 2>;
@@ -484,8 +464,7 @@ cudaError_t launch_t(esa_ctx* ctx, int B, int l_C, const CUtensorMap& kmap, cons
 }  // namespace
 
 // Both scoring passes; rkey must be zeroed.  d' = 32 runs as 64 with the upper half of every row read as zeros.
-// *pooled_ready: ctx->pkey and ctx->ghist0 hold the pooled keys and their first-digit histogram
-// (else ctx->skey holds the unpooled keys and ghist0 is zero).
+// *pooled_ready: ctx->pkey holds the pooled keys (else ctx->skey holds the unpooled ones).
 // Returns cudaErrorNotSupported when this path does not cover the shape.
 cudaError_t launch_score_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache, const SeqMeta& meta,
                             int max_lM, cudaStream_t st, bool* pooled_ready) {
@@ -502,7 +481,7 @@ cudaError_t launch_score_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* k
 }
 
 // The per-head vote: every head's own scores (uncompressed queries and keys), the maximum over the heads in ctx->skey,
-// unpooled.  ctx->rkey_heads must be zeroed; ctx->ghist0 is zero afterwards.
+// unpooled.  ctx->rkey_heads must be zeroed.
 cudaError_t launch_score_tc_heads(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* K, const SeqMeta& meta,
                                   int max_lM, cudaStream_t st) {
     CUtensorMap kmap, qmap;
