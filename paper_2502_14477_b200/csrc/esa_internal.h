@@ -38,10 +38,13 @@ struct KernelMemo {
     std::atomic<int> per_sm[64] = {};       // resident CTAs per SM, 0 = not asked yet
 };
 template <typename F>
-cudaError_t allow_smem(F* kernel, int device, int bytes, KernelMemo& memo) {
+cudaError_t allow_smem(F* kernel, int device, int bytes, KernelMemo& memo, bool carve_out = false) {
+    // carve_out: an SM is set up with all of its memory as shared memory for this kernel, not just what it needs
     const uint64_t bit = device >= 0 && device < 64 ? uint64_t(1) << device : 0;
     if (memo.smem_set.load(std::memory_order_acquire) & bit) return cudaSuccess;
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess && carve_out)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     if (e == cudaSuccess) memo.smem_set.fetch_or(bit, std::memory_order_release);
     return e;
 }

@@ -355,10 +355,13 @@ __global__ void read_pooled_kernel(const uint32_t* __restrict__ pkey, const uint
 
 // n_ranks = 0: asks whether the device can place clusters of more than the portable eight CTAs.
 template <int KPT>
-static cudaError_t launch_topk(const SelectParams& p, int n_ranks, int B, cudaStream_t st) {
+static cudaError_t launch_topk(int device, const SelectParams& p, int n_ranks, int B, cudaStream_t st) {
     const bool probe = n_ranks == 0;
+    static KernelMemo memo;                  // (the attention's CTAs are to start beside this kernel's: same split of the SM's memory)
+    cudaError_t e = allow_smem(select_topk_kernel<KPT>, device, 0, memo, true);
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(probe ? SEL_CLUSTER : n_ranks, B);
+    cfg.gridDim = dim3(probe ? SEL_CLUSTER : n_ranks, probe ? 1 : B);
     cfg.blockDim = dim3(SEL_THREADS);
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -371,7 +374,7 @@ static cudaError_t launch_topk(const SelectParams& p, int n_ranks, int B, cudaSt
     cfg.attrs = attr;
     cfg.numAttrs = probe ? 1 : 2;
     if (!probe) return cudaLaunchKernelEx(&cfg, select_topk_kernel<KPT>, p);
-    cudaError_t e = cudaFuncSetAttribute(select_topk_kernel<KPT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    e = cudaFuncSetAttribute(select_topk_kernel<KPT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     int n = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, select_topk_kernel<KPT>, &cfg);
     return e == cudaSuccess && n == 0 ? cudaErrorNotSupported : e;
@@ -393,20 +396,22 @@ cudaError_t launch_select(esa_ctx* ctx, int B, bool mapped, const SeqMeta& meta,
     p.idx_out = idx_out; p.n_sel_out = n_sel_out;
     p.max_tokens = ctx->cfg.max_tokens; p.top_k = ctx->cfg.top_k;
     p.mapped = mapped ? 1 : 0; p.meta = meta;                // (mapped mode reads rkey[b]: one query per sequence)
-    // CTAs of 4096 tokens (8 keys a thread), up to 8 of them; then 16 keys a thread and, where the device places them,
-    // clusters of 16
+    // CTAs of 4096 tokens (8 keys a thread), as many as it takes up to 16 (8 where the device does not place such clusters, or
+    // where all sequences' CTAs would outnumber the SMs); then 16 keys a thread.  63k tokens, select: 36.3 us with 16 CTAs,
+    // 37.6 with 8.
     static std::atomic<int> wide[64];
     std::atomic<int>& w = wide[ctx->device & 63];
     if (w.load(std::memory_order_relaxed) == 0) {
-        const bool ok = launch_topk<16>(p, 0, 1, st) == cudaSuccess;
+        const bool ok = launch_topk<8>(ctx->device, p, 0, 1, st) == cudaSuccess && launch_topk<16>(ctx->device, p, 0, 1, st) == cudaSuccess;
         if (!ok) cudaGetLastError();
         w.store(ok ? SEL_CLUSTER : 8, std::memory_order_relaxed);
     }
+    const int widest = w.load(std::memory_order_relaxed), most = SEL_CLUSTER * B <= ctx->num_sms ? widest : 8;
     int n_ranks = 1;
-    while (n_ranks < 8 && n_ranks * 8 * SEL_THREADS < max_lM) n_ranks *= 2;
-    if (n_ranks * 16 * SEL_THREADS < max_lM) n_ranks = w.load(std::memory_order_relaxed);
+    while (n_ranks < most && n_ranks * 8 * SEL_THREADS < max_lM) n_ranks *= 2;
+    if (n_ranks * 16 * SEL_THREADS < max_lM) n_ranks = widest;
     ProfScope prof(ctx, KC_SELECT_TOPK, st);
-    e = n_ranks * 8 * SEL_THREADS >= max_lM ? launch_topk<8>(p, n_ranks, B, st) : launch_topk<16>(p, n_ranks, B, st);
+    e = n_ranks * 8 * SEL_THREADS >= max_lM ? launch_topk<8>(ctx->device, p, n_ranks, B, st) : launch_topk<16>(ctx->device, p, n_ranks, B, st);
     if (e != cudaSuccess) return e;
     ctx->launches += 1;
     return cudaGetLastError();
