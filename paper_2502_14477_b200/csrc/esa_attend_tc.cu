@@ -866,11 +866,12 @@ static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_m
     const int R = p.l_C * p.G;
     const int row_tiles = (R + TC_ROWS - 1) / TC_ROWS;
     p.Rp = (R + 1) & ~1;
-    // Split the key list when that fills the machine better.  Cost in us, fitted to measured sweeps: 1.55 per 128-key tile
-    // of the longest CTA and 7 for its start and end, per wave (one CTA per SM); 7.5 for a pair's exchange or a merge
-    // launch, whose traffic (4 TB/s) counts; and 6 when the grid leaves the merge launch no SMs to start on meanwhile
-    // (37 queries, 8 units over 6300 keys: 41 us with 3 parts, 23 with 9, 21 with 14, 32 with 18).  Two-position
-    // attention needs an even number of splits (one group per part); its longer part sets the tiles per CTA.
+    // Split the key list when that fills the machine better.  Cost in us, fitted to measured sweeps: 1.85 per 128-key tile
+    // (1.55 with one Q tile) of the longest CTA, one CTA per SM, 7 for its start and end and 3 more for every wave after
+    // the first; 7.5 for a pair's exchange or a merge launch, whose traffic (4 TB/s) counts; and 6 when the last wave
+    // leaves the merge launch no SMs to start on meanwhile (37 queries, 8 units over 6300 keys: 41 us with 3 parts, 23
+    // with 9, 21 with 14, 32 with 18).  Two-position attention needs an even number of splits (one group per part); its
+    // longer part sets the tiles per CTA.
     const int ctas = row_tiles * p.HG * B;
     const int n_tiles = (n_att_max + TC_BN - 1) / TC_BN;
     int i_end_max = 0;
@@ -886,8 +887,9 @@ static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_m
         const int longest = p.two ? max(far_tiles, n_tiles - far_tiles + 1) : n_tiles;
         const int per = (longest + grp - 1) / grp;
         const int waves = (ctas * ns + ctx->num_sms - 1) / ctx->num_sms;
-        const double join = ns == 1 ? 0.0 : ns == 2 ? 7.5 : 7.5 + ns * merge_bytes / 4e6 + (ctas * ns * 8 > ctx->num_sms * 7 ? 6.0 : 0.0);
-        const double cost = waves * (1.55 * per + 7.0) + join;
+        const int last_wave = ctas * ns - (waves - 1) * ctx->num_sms;
+        const double join = ns == 1 ? 0.0 : ns == 2 ? 7.5 : 7.5 + ns * merge_bytes / 4e6 + (last_wave * 8 > ctx->num_sms * 7 ? 6.0 : 0.0);
+        const double cost = waves * ((NQT == 2 ? 1.85 : 1.55) * per + 3.0) + 4.0 + join;
         if (cost < best_cost - 1e-9) { best_cost = cost; best = ns; }
     }
     if (best == 0) return cudaErrorNotSupported;

@@ -120,9 +120,9 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // formed with one part per lane and the rows are read sixteen parts at a time, so that a merge is a few round trips to L2
 // however many parts there are (with four at a time, and the maximum searched part by part, 37 parts took 9 us).
 // Loads bypass L1: the parts may have been written by other SMs a moment ago.
-template <int D>
-__device__ __forceinline__ void merge_row(const float* o, const float* ml, int64_t stride, int nsplit, int lane, __nv_bfloat16* dst_row) {
-    constexpr int PER = D / 32, BATCH = 16;
+template <int D, int BATCH>
+__device__ __forceinline__ void merge_row_batched(const float* o, const float* ml, int64_t stride, int nsplit, int lane, __nv_bfloat16* dst_row) {
+    constexpr int PER = D / 32;
     float2 v[BATCH][PER / 2];
     auto load = [&](int s0) {
 #pragma unroll
@@ -167,6 +167,12 @@ __device__ __forceinline__ void merge_row(const float* o, const float* ml, int64
 #pragma unroll
     for (int i = 0; i < PER; i += 2)
         *reinterpret_cast<uint32_t*>(dst_row + lane * PER + i) = pack_bf16(acc[i] * inv, acc[i + 1] * inv);
+}
+
+template <int D>
+__device__ __forceinline__ void merge_row(const float* o, const float* ml, int64_t stride, int nsplit, int lane, __nv_bfloat16* dst_row) {
+    if (nsplit <= 4) merge_row_batched<D, 4>(o, ml, stride, nsplit, lane, dst_row);
+    else merge_row_batched<D, 16>(o, ml, stride, nsplit, lane, dst_row);
 }
 
 // A-operand fragment (16 rows x 16 k) of a K-major tile: row0 = first row, kc = first
