@@ -202,6 +202,70 @@ def test_all_equal_scores_take_lowest_indices():
     assert idx[0].cpu().tolist() == list(range(cfg.l_I, cfg.l_I + cfg.k))
 
 
+# (positions of the sequences, chunk, d', eps, k, runs of equal keys).  l_I + l_L = 80, so |M| = t - 80.
+_SELECTION_EDGES = [
+    # selection clusters of 1, 2, 4, 8 and 16 CTAs at, below and above their 4096 tokens a CTA; decode, then chunks
+    ([80 + 4095], 1, 32, 0, 300, 0), ([80 + 4097], 1, 64, 3, 4096, 0), ([80 + 8193], 1, 128, 3, 1, 0), ([80 + 32768], 1, 128, 15, 2048, 0),
+    ([80 + 32769], 3, 64, 3, 2048, 0), ([80 + 65536], 2, 32, 1, 4096, 0),
+    # 16 keys a thread, then more tokens than a cluster's registers hold (batches)
+    ([80 + 65537], 1, 64, 3, 5000, 0), ([80 + 131073], 1, 32, 3, 4096, 0), ([80 + 131073], 5, 32, 3, 4096, 0),
+    # more sequences than SMs / 16: clusters of 8; lengths from "everything is selected" to two batches; the shares of the
+    # decode scoring's warps cross the sequences' ends
+    ([80 + 70001, 80 + 33, 80 + 300, 80 + 301, 80 + 12345, 80 + 8191, 80 + 33001, 80, 40, 80 + 5], 1, 128, 3, 300, 0),
+    ([80 + 9001, 80 + 200], 7, 128, 5, 300, 0),
+    # shares of a few tokens, fewer than the pooling window
+    ([80 + 301], 1, 32, 15, 300, 0), ([80 + 17, 80 + 18], 1, 128, 15, 4, 0),
+    # long runs of equal scores over several CTAs: more ties at the threshold than are sent one by one
+    ([80 + 40000], 1, 64, 0, 3333, 700), ([80 + 40000], 2, 128, 3, 9999, 5000), ([80 + 140000], 1, 32, 3, 8000, 3000),
+]
+
+
+@pytest.mark.parametrize("t_list,l_C,d_c,eps,k,run", _SELECTION_EDGES)
+def test_selection_at_cluster_and_share_edges(t_list, l_C, d_c, eps, k, run):
+    """Pooled scores within the accumulation bound, and the selection EXACTLY the k best of the kernel's own pooled scores
+    with the lowest index first among equals."""
+    cfg = syn.get_config("c1").with_(d_c=d_c, l_I=16, l_L=64, eps=eps, k=k)
+    B, n = len(t_list), max(t_list) + l_C
+    ctx = hp.make_esa(cfg, max_tokens=n, max_chunk=l_C, max_batch=B)
+    gen = torch.Generator(device="cuda").manual_seed(d_c + k)
+    kc = torch.randn(B, n, d_c, device="cuda", generator=gen).bfloat16()
+    if run:
+        kc = kc[:, :7][:, (torch.arange(n, device="cuda") // run) % 7].contiguous()
+    Q = torch.randn(B, l_C, cfg.H, cfg.d, device="cuda", generator=gen).bfloat16()
+    idx = torch.full((B, k), -1, dtype=torch.int32, device="cuda")
+    n_sel = torch.full((B,), -1, dtype=torch.int32, device="cuda")
+    ctx.select(Q, kc, t_list, idx, n_sel, sync=True)
+    assert ctx.last_device_status() == 0
+    got, counts = idx.cpu().numpy().astype(np.int64), n_sel.cpu().tolist()
+    scored = any(orc.partition(t, cfg.l_I, cfg.l_L)[1] - orc.partition(t, cfg.l_I, cfg.l_L)[0] > k for t in t_list)
+    qc = syn.bf16_bits_to_f64(ctx.read_compressed_queries(B * l_C)).reshape(B, l_C, d_c) if scored else None
+    for b, t in enumerate(t_list):
+        i_end, m_end = orc.partition(t, cfg.l_I, cfg.l_L)
+        l_M = m_end - i_end
+        assert counts[b] == min(k, l_M)
+        if l_M <= k:
+            assert got[b, :l_M].tolist() == list(range(i_end, m_end))
+            continue
+        sp = ctx.read_pooled_scores(b, l_M)
+        hp.check_pooled_scores(sp, qc[b], hp.torch_to_f64(kc[b, i_end:m_end]), k, eps, what=f"seq {b} |M|={l_M}")
+        want = np.sort(np.argsort(-sp, kind="stable")[:k]) + i_end
+        assert np.array_equal(got[b], want), f"seq {b} |M|={l_M}: {int((got[b] != want).sum())} positions differ"
+
+
+@pytest.mark.parametrize("H,H_G,d,d_c,t,l_C,two", [
+    (4, 4, 64, 64, 2500, 127, False), (4, 4, 64, 64, 2500, 128, False), (4, 4, 64, 64, 2500, 129, False),   # one or two Q tiles
+    (8, 2, 64, 32, 2000, 2, False), (8, 2, 64, 32, 129, 2, False), (28, 4, 128, 128, 6001, 19, False),       # 2 rows; no M; 133 rows
+    (8, 1, 128, 128, 7000, 3, False), (8, 1, 128, 64, 7000, 64, False),                                     # one head: most splits
+    (8, 1, 128, 128, 7000, 2, True), (8, 8, 64, 64, 3001, 33, True), (16, 2, 128, 128, 5000, 17, True)])
+def test_small_chunks_at_tile_and_split_edges(H, H_G, d, d_c, t, l_C, two):
+    """Chunks of a few queries on the tensor-memory kernels: ragged row tiles, key lists split many ways, few and many heads."""
+    cfg = syn.get_config("c1").with_(H=H, H_G=H_G, d=d, d_c=d_c, l_I=16, l_L=700, k=1000)
+    if two:
+        _two_position_case(cfg, t, l_C)
+    else:
+        _stage_isolated(cfg, t, l_C)
+
+
 # ------------------------------------------------------ end to end, config 1
 def test_c1_end_to_end_prefill_and_decode():
     cfg = syn.get_config("c1")
