@@ -33,7 +33,8 @@
 //   * A long key list can be split across CTAs (blockIdx.z); a two-way split runs as CTA pairs that exchange
 //     halves of their partial (O, m, l) through distributed shared memory (PAIR, below); otherwise the partials
 //     go to the context's scratch through coalesced stores and a second launch merges them, a warp per row (on all
-//     SMs: the last CTA of a unit merging four parts by itself took 15 us).
+//     SMs: the last CTA of a unit merging four parts by itself took 15 us).  Where units are too many for two CTAs each
+//     and too few to fill the SMs, the second parts are short and run one after another on the SMs left over (TC_UNEVEN).
 //   * A call that follows the selection of its step (p.early) takes the attended set as two lists: I then L,
 //     whose rows are older than the chunk and do not depend on the selection, before the kernel's wait for the
 //     preceding kernel, and M_k then C after it.  Every role runs the two phases in turn; the selection kernel
@@ -70,6 +71,9 @@ constexpr int TC_REGS_SOFTMAX = 168;
 constexpr int TC_REGS_OTHER = 88;
 static_assert(8 * TC_REGS_SOFTMAX + 8 * TC_REGS_OTHER <= 16 * TC_REGS_LAUNCH,
               "register split exceeds the CTA's launch allocation: setmaxnreg.inc would never return");
+// what the CTAs of a unit do with their results (launch_tc): separate parts (merged by a second launch), pairs that
+// exchange halves, or separate parts of which the first is much the longer
+enum { TC_PARTS = 0, TC_PAIR = 1, TC_UNEVEN = 2 };
 constexpr float kSumLimit = 1.8446744e19f;   // 2^64: a tile whose sum of 2^(score - m) reaches this has its maximum looked up
 
 struct TcAttendParams {
@@ -86,6 +90,9 @@ struct TcAttendParams {
     int64_t max_tokens;
     int l_C, H, HG, G, top_k;
     int nsplit;
+    int main_tiles;     // TC_UNEVEN: tiles of the first part (see launch_tc)
+    int early_units;    // the second part of the first so many units takes up to this many tiles of the early list
+    int early_second;
     int Rp;             // rows of a scratch part (R rounded up to even: 16-byte aligned parts)
     int q_tma;          // Q tiles arrive by TMA (one arrival) instead of cp.async (one per producer thread)
     int staged;         // the caches hold the attended list itself: row j = list entry j
@@ -201,9 +208,10 @@ __device__ __forceinline__ void store_half_rows(const float* acc, float4* stage,
 // its copies have landed.
 // NQT: Q tiles of a CTA that hold rows.  One for chunks of at most 128 rows per key/value head: the second tile's
 // products and softmax would only be in the way.
-template <int D, bool PAIR, int NQT>
+template <int D, int MODE, int NQT>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap qgmap, TcAttendParams p) {
+    constexpr bool PAIR = MODE == TC_PAIR, UNEVEN = MODE == TC_UNEVEN;
     constexpr int STAGES = TC_STAGES;
     constexpr int CH = D / 8;                   // 16-byte chunks per row
     constexpr int Q_TILE_BYTES = 128 * D * 2;   // one 128-row Q tile
@@ -224,8 +232,10 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
     const int warp_u = __shfl_sync(0xffffffffu, warp, 0);     // provably warp-uniform copy
     const int row0 = blockIdx.x * TC_ROWS;
     const int kvh = blockIdx.y;
-    const int b = blockIdx.z / p.nsplit;
-    const int split = blockIdx.z % p.nsplit;
+    // (uneven splits: the long ones first, so that one wave holds them all and the SMs left over take the short ones)
+    const int n_seq = gridDim.z >> 1;
+    const int b = UNEVEN ? blockIdx.z % n_seq : blockIdx.z / p.nsplit;
+    const int split = UNEVEN ? blockIdx.z / n_seq : blockIdx.z % p.nsplit;
     const int G = p.G;
     const int R = p.l_C * G;
 
@@ -269,9 +279,12 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
     const int r_last = min(R, row0 + TC_ROWS) - 1;
     const int e_len = p.early ? i_end + (t - m_end) : 0;                 // entries of the early list
     const int early_all = (e_len + TC_BN - 1) / TC_BN;
-    const int early_per = (early_all + p.nsplit - 1) / p.nsplit;
+    const bool second_early = UNEVEN && (int)((b * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) < p.early_units;
+    const int early_per = UNEVEN ? early_all - (second_early ? min(early_all / 2, p.early_second) : 0)
+                                           : (early_all + p.nsplit - 1) / p.nsplit;
     const int early_begin = min(early_all, split * early_per);
-    const int n_early = min(early_all, early_begin + early_per) - early_begin;      // this CTA's early tiles
+    const int early_end = UNEVEN && split == 1 ? early_all : min(early_all, early_begin + early_per);
+    const int n_early = early_end - early_begin;                                    // this CTA's early tiles
     const KeyList list_early = {i_end, i_end, m_end, e_len};
     // set after the wait: the late (or only) list, this CTA's part of it, and the tile count of both phases
     KeyList list_late = {0, 0, 0, 0};
@@ -296,11 +309,12 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
         // (with an early list the shares run the other way round: the split with the short early share comes first)
         const int s_in = (p.two && !far) ? split - grp : (p.early ? grp - 1 - split : split);
         const int late_all = max(0, (part_hi - part_lo + TC_BN - 1) / TC_BN);
-        if (p.early && grp == 2 && late_all >= 2) {
+        if (UNEVEN || (p.early && grp == 2 && late_all >= 2)) {
             // Two splits: the late list is cut where the first split's early and late tiles together make half of
             // all tiles (rounded up).  The second split, which holds the masked tiles of C (the dearer ones), is then
             // never the one with a tile more.
-            const int cut = min(late_all, max(0, ((early_all + late_all + 1) >> 1) - min(early_all, early_per)));
+            const int first = UNEVEN ? p.main_tiles : (early_all + late_all + 1) >> 1;
+            const int cut = min(late_all, max(0, first - min(early_all, early_per)));
             tile_begin = split == 0 ? 0 : cut;
             n_tiles = n_early + (split == 0 ? cut : late_all - cut);
         } else {
@@ -807,18 +821,18 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
 
 }  // namespace
 
-template <int D, bool PAIR, int NQT>
+template <int D, int MODE, int NQT>
 static cudaError_t launch_tc_kernel(esa_ctx* ctx, const CUtensorMap& qmap, const CUtensorMap& qgmap, const TcAttendParams& p,
                                     dim3 grid, cudaStream_t st, bool probe_only) {
     constexpr int smem = 2 * 128 * D * 2 + 2 * TC_STAGES * TC_BN * D * 2 + 1024;
     static KernelMemo memo;
-    cudaError_t e = allow_smem(attend_tc_kernel<D, PAIR, NQT>, ctx->device, smem, memo);
+    cudaError_t e = allow_smem(attend_tc_kernel<D, MODE, NQT>, ctx->device, smem, memo);
     if (e != cudaSuccess) return e;
     // the in-kernel register split assumes the launch allocation it was sized for
     static int regs_checked = 0;
     if (!regs_checked) {
         cudaFuncAttributes fa;
-        e = cudaFuncGetAttributes(&fa, attend_tc_kernel<D, PAIR, NQT>);
+        e = cudaFuncGetAttributes(&fa, attend_tc_kernel<D, MODE, NQT>);
         if (e != cudaSuccess) return e;
         if (fa.numRegs != TC_REGS_LAUNCH) return cudaErrorInvalidConfiguration;
         regs_checked = 1;
@@ -836,15 +850,15 @@ static cudaError_t launch_tc_kernel(esa_ctx* ctx, const CUtensorMap& qmap, const
     attr[1].val.clusterDim.y = 1;
     attr[1].val.clusterDim.z = 2;
     cfg.attrs = attr;
-    cfg.numAttrs = PAIR ? 2 : 1;
+    cfg.numAttrs = MODE == TC_PAIR ? 2 : 1;
     if (probe_only) {
         // can the device place a pair of these CTAs at all?
         int n_clusters = 0;
-        e = cudaOccupancyMaxActiveClusters(&n_clusters, attend_tc_kernel<D, PAIR, NQT>, &cfg);
+        e = cudaOccupancyMaxActiveClusters(&n_clusters, attend_tc_kernel<D, MODE, NQT>, &cfg);
         if (e != cudaSuccess) return e;
         return n_clusters > 0 ? cudaSuccess : cudaErrorNotSupported;
     }
-    return cudaLaunchKernelEx(&cfg, attend_tc_kernel<D, PAIR, NQT>, qmap, qgmap, p);
+    return cudaLaunchKernelEx(&cfg, attend_tc_kernel<D, MODE, NQT>, qmap, qgmap, p);
 }
 
 // Merge of a key list split more than two ways: a warp per row.
@@ -892,6 +906,26 @@ static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_m
         const double cost = waves * ((NQT == 2 ? 1.85 : 1.55) * per + 3.0) + 4.0 + join;
         if (cost < best_cost - 1e-9) { best_cost = cost; best = ns; }
     }
+    // Two uneven parts (TC_UNEVEN), where one CTA per unit leaves SMs idle and a second one each would more than fill them:
+    // the first parts of all units run in one wave, and the idle SMs take the second parts, `rounds` one after another.
+    // The shortest first part that keeps the second ones from taking longer (start and end: 5 us each).  1024 queries of
+    // the 28/4-head shape, 112 units of 105 tiles: 210 us unsplit, 190 so; the whole step 307 and 292 us.  Units whose
+    // second parts are in the first wave give them up to half of the early list, so that every CTA of that wave has
+    // work while the selection runs (without: 295; all of the early list, which leaves the first parts idle: other sizes up
+    // to 8 us slower).  Estimated gains below 3 us are left: the estimate is no better than that.
+    p.main_tiles = p.early_units = p.early_second = 0;
+    const int idle = ctas < ctx->num_sms ? ctx->num_sms - ctas : 0;
+    if (NQT == 2 && !p.two && idle > 0 && ctas > idle && (size_t)B * p.HG * 2 * p.Rp * (D + 2) <= ctx->att_part_elems) {
+        const int rounds = (ctas + idle - 1) / idle;
+        const int second = max(0, (int)((n_tiles * 1.85 + 3.0 - 5.0 * rounds) / (1.85 * (rounds + 1))));
+        const double cost = 1.85 * (n_tiles - second) + 3.0 + 4.0 + 7.5 + 2 * merge_bytes / 4e6;
+        if (second > 0 && cost < best_cost - 3.0) {
+            best = 2;
+            p.main_tiles = n_tiles - second;
+            p.early_units = p.early ? idle : 0;      // (they start beside the selection kernel, like the first parts)
+            p.early_second = second;
+        }
+    }
     if (best == 0) return cudaErrorNotSupported;
     p.nsplit = best;
     CUtensorMap qmap, qgmap;
@@ -902,14 +936,17 @@ static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_m
     const dim3 grid(row_tiles, p.HG, B * best);
     // a two-way split runs as CTA pairs that merge through distributed shared memory, where the device can place pairs
     static int pair_ok = -1;                                 // per instantiation; probed once
-    if (best == 2 && pair_ok < 0) pair_ok = launch_tc_kernel<D, true, NQT>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess ? 1 : 0;
-    const bool pair = best == 2 && pair_ok == 1;
+    const bool uneven = p.main_tiles > 0;
+    if (best == 2 && !uneven && pair_ok < 0)
+        pair_ok = launch_tc_kernel<D, TC_PAIR, NQT>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess ? 1 : 0;
+    const bool pair = best == 2 && !uneven && pair_ok == 1;
     if (best == 2 && !pair && (size_t)B * p.HG * 2 * p.Rp * (D + 2) > ctx->att_part_elems) return cudaErrorNotSupported;
     cudaError_t e;
     {
         ProfScope prof(ctx, KC_ATTEND_TC, st);
-        e = pair ? launch_tc_kernel<D, true, NQT>(ctx, qmap, qgmap, p, grid, st, false)
-                 : launch_tc_kernel<D, false, NQT>(ctx, qmap, qgmap, p, grid, st, false);
+        if (pair) e = launch_tc_kernel<D, TC_PAIR, NQT>(ctx, qmap, qgmap, p, grid, st, false);
+        else if (uneven) e = launch_tc_kernel<D, TC_UNEVEN, 2>(ctx, qmap, qgmap, p, grid, st, false);
+        else e = launch_tc_kernel<D, TC_PARTS, NQT>(ctx, qmap, qgmap, p, grid, st, false);
     }
     ctx->launches += 1;
     if (e != cudaSuccess || best == 1 || pair) return e;

@@ -266,6 +266,26 @@ def test_small_chunks_at_tile_and_split_edges(H, H_G, d, d_c, t, l_C, two):
         _stage_isolated(cfg, t, l_C)
 
 
+@pytest.mark.parametrize("H_G,B,t,l_C", [(28, 1, 3000, 1000), (28, 1, 900, 1024), (11, 1, 4001, 2047), (25, 2, 2500, 300), (38, 1, 150, 700), (45, 1, 2600, 500)])
+def test_uneven_key_list_split(H_G, B, t, l_C):
+    """75 to 114 units of 256 rows: the idle SMs attend the ends of the units' key lists (nothing selected, ragged row tiles,
+    two sequences of different lengths among them)."""
+    cfg = syn.get_config("c1").with_(H=H_G, H_G=H_G, d=64, d_c=64, l_I=16, l_L=700, k=1000, B=B)
+    p, n, t_list = hp.oracle_params(cfg), t + l_C, [t - 900 * b for b in range(B)]
+    _, _, Wq, Wk = hp.oracle_weights(cfg)
+    heads = [0, H_G // 2, H_G - 1]
+    ctx = hp.make_esa(cfg, max_tokens=n, max_chunk=l_C, max_batch=B)
+    seq = hp.DeviceSeq(cfg, max_tokens=n, B=B)
+    seq.fill_kv(0, n)
+    fill_kc_gpu(ctx, seq, n, step=l_C)
+    Q = torch.stack([hp.bits_to_torch(syn.qkv_rows(cfg, "q", t_list[b], t_list[b] + l_C, 0, b)) for b in range(B)]).contiguous()
+    sel, O = run_step_gpu(ctx, seq, Q, t_list, do_compress=False)
+    for b, tb in enumerate(t_list):
+        K64, V64 = hp.torch_to_f64(seq.K[b, : tb + l_C]), hp.torch_to_f64(seq.V[b, : tb + l_C])
+        want = orc.attend(hp.torch_to_f64(Q[b]), K64, V64, sel[b], tb, p, heads=heads)
+        hp.check_attention(O[b], want, what=f"uneven split H_G={H_G} seq {b}", heads=heads)
+
+
 # ------------------------------------------------------ end to end, config 1
 def test_c1_end_to_end_prefill_and_decode():
     cfg = syn.get_config("c1")
