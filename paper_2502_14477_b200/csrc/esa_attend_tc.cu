@@ -44,7 +44,10 @@
 //   * Two-position attention (Section 3.2) is a split by construction: the first half of the splits
 //     covers the list entries of I and M_k with the second encoding (Qg, Kg), the other half covers
 //     L and C with (Q, K), so a CTA holds one pair of Q tiles whichever part it works on, and the
-//     merge that joins key-list splits also joins the two parts (Algorithm 1's merge of (O, m, l)).
+//     merge that joins key-list splits also joins the two parts (Algorithm 1's merge of (O, m, l)).  As a
+//     pair (TC_TWO_PAIR) the CTA with the shorter list goes on with the end of the other's: new Q tiles, the same
+//     running sums and accumulator (33 tiles against 20, 512 queries of the 32/8-head shape: 72 -> 64 us; 64
+//     against 12: 126 -> 87).
 #include <cstring>
 
 #include "esa_internal.h"
@@ -72,8 +75,8 @@ constexpr int TC_REGS_OTHER = 88;
 static_assert(8 * TC_REGS_SOFTMAX + 8 * TC_REGS_OTHER <= 16 * TC_REGS_LAUNCH,
               "register split exceeds the CTA's launch allocation: setmaxnreg.inc would never return");
 // what the CTAs of a unit do with their results (launch_tc): separate parts (merged by a second launch), pairs that
-// exchange halves, or separate parts of which the first is much the longer
-enum { TC_PARTS = 0, TC_PAIR = 1, TC_UNEVEN = 2 };
+// exchange halves, separate parts of which the first is much the longer, or pairs for the two lists of two-position attention
+enum { TC_PARTS = 0, TC_PAIR = 1, TC_UNEVEN = 2, TC_TWO_PAIR = 3 };
 constexpr float kSumLimit = 1.8446744e19f;   // 2^64: a tile whose sum of 2^(score - m) reaches this has its maximum looked up
 
 struct TcAttendParams {
@@ -211,7 +214,7 @@ __device__ __forceinline__ void store_half_rows(const float* acc, float4* stage,
 template <int D, int MODE, int NQT>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap qgmap, TcAttendParams p) {
-    constexpr bool PAIR = MODE == TC_PAIR, UNEVEN = MODE == TC_UNEVEN;
+    constexpr bool TWO = MODE == TC_TWO_PAIR, PAIR = MODE == TC_PAIR || TWO, UNEVEN = MODE == TC_UNEVEN;
     constexpr int STAGES = TC_STAGES;
     constexpr int CH = D / 8;                   // 16-byte chunks per row
     constexpr int Q_TILE_BYTES = 128 * D * 2;   // one 128-row Q tile
@@ -284,7 +287,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
                                            : (early_all + p.nsplit - 1) / p.nsplit;
     const int early_begin = min(early_all, split * early_per);
     const int early_end = UNEVEN && split == 1 ? early_all : min(early_all, early_begin + early_per);
-    const int n_early = early_end - early_begin;                                    // this CTA's early tiles
+    int n_early = early_end - early_begin;                   // this CTA's early tiles (TWO: of its own list, set by `plan`)
     const KeyList list_early = {i_end, i_end, m_end, e_len};
     // set after the wait: the late (or only) list, this CTA's part of it, and the tile count of both phases
     KeyList list_late = {0, 0, 0, 0};
@@ -301,6 +304,20 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
         const int j_end = c_first + r_last / G + 1;           // keys visible to the last row of the CTA
         // The part of the key list this CTA's group of splits covers: all of it, or (two-position attention)
         // the entries of I and M_k for the first half of the splits and those of L and C for the second.
+        if (TWO) {
+            // Pair: CTA 0 has the list of I and M_k, CTA 1 that of L and C, and the one with the shorter list goes on with
+            // the end of the other's, for which its Q tiles are loaded anew (about a tile's time).  Its sums and its
+            // accumulator go on: whatever is accumulated, the softmax is one over both lists.
+            const int far_all = (list_late.ng + TC_BN - 1) / TC_BN, near_all = (j_end - list_late.ng + TC_BN - 1) / TC_BN;
+            const int own = split == 0 ? far_all : near_all, other = split == 0 ? near_all : far_all;
+            const int moved = max(0, abs(own - other) - 1) >> 1;
+            n_early = own - (own > other ? moved : 0);
+            n_tiles = n_early + (own > other ? 0 : moved);
+            tile_begin = other - moved;
+            part_hi = j_end;
+            planned = true;
+            return;
+        }
         const int grp = p.two ? p.nsplit / 2 : p.nsplit;       // splits that share a part
         far = p.two && split < grp;                            // this CTA works with (Qg, Kg)
         part_lo = (p.two && !far) ? list_late.ng : 0;
@@ -328,6 +345,13 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
     // Every role takes its tiles in two phases, the early ones and, after `plan`, the late ones; tile j of the CTA
     // starts at entry key_first + (j - j_first) * TC_BN of the phase's list.
     const bool has_work = n_early > 0 || n_tiles > 0;
+    // TWO: phase 0 is the CTA's own list, phase 1 the end of the other's
+    auto phase_far = [&](int phase) { return TWO ? (phase == 0) == (split == 0) : far; };
+    auto phase_key = [&](int phase) {
+        if (TWO) return (phase_far(phase) ? 0 : list_late.ng) + (phase == 0 ? 0 : tile_begin * TC_BN);
+        return phase == 0 ? early_begin * TC_BN : part_lo + tile_begin * TC_BN;
+    };
+    const bool q_swap = TWO && n_early > 0 && n_tiles > n_early;     // the Q tiles change with the phase
 
     if (warp_u < TC_SOFTMAX_WARPS) reg_alloc<TC_REGS_SOFTMAX>();
     else reg_dealloc<TC_REGS_OTHER>();
@@ -347,11 +371,13 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
         for (int phase = 0; phase < 2; ++phase) {
         if (phase == 1 && !planned) plan();
         const int j_first = phase == 0 ? 0 : 2 * n_early, j_last = phase == 0 ? 2 * n_early : 2 * n_tiles;
-        const int key_first = phase == 0 ? early_begin * TC_BN : part_lo + tile_begin * TC_BN;
+        const int key_first = phase_key(phase);
         // first invisible entry of this row, and the smallest such limit of the Q tile (every row sees all of the
         // early list)
-        const int lim = phase == 0 ? e_len : min(part_hi, c_first + min(row / G, p.l_C - 1) + 1);
-        const int lim_min = phase == 0 ? e_len : min(part_hi, c_first + min((row0 + qt * 128) / G, p.l_C - 1) + 1);
+        const int hi = TWO && phase_far(phase) ? list_late.ng : part_hi;
+        const bool all_early = !TWO && phase == 0;
+        const int lim = all_early ? e_len : min(hi, c_first + min(row / G, p.l_C - 1) + 1);
+        const int lim_min = all_early ? e_len : min(hi, c_first + min((row0 + qt * 128) / G, p.l_C - 1) + 1);
         for (int j = j_first; active && j < j_last; ++j) {  // j counts halves: tile j >> 1, half j & 1
             const int T = j >> 1, u = j & 1;
             const int key0 = key_first + (j - j_first) * TC_HALF;
@@ -626,23 +652,25 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
     } else if (warp_u < TC_MMA_WARP) {
         // ------------------------------------------------------------ producers: Q, then K/V tiles
         const int ptid = tid - TC_SOFTMAX_WARPS * 32;      // 0..127
-        if (has_work && p.q_tma) {
-            // two boxes per 64-column block: rows (query, head-in-group) of one key/value head
-            if (ptid == 0) {
-                mbar_arrive_expect_tx(bar(BAR_Q_FULL), 2 * Q_TILE_BYTES);
-                const CUtensorMap* qm = far ? &qgmap : &qmap;
+        auto load_q = [&](bool q_far) {
+            if (p.q_tma) {
+                // two boxes per 64-column block: rows (query, head-in-group) of one key/value head
+                if (ptid == 0) {
+                    mbar_arrive_expect_tx(bar(BAR_Q_FULL), 2 * Q_TILE_BYTES);
+                    const CUtensorMap* qm = q_far ? &qgmap : &qmap;
 #pragma unroll
-                for (int qt = 0; qt < 2; ++qt)
+                    for (int qt = 0; qt < 2; ++qt)
 #pragma unroll
-                    for (int blk = 0; blk < D / 64; ++blk)
-                        tma_load_3d(smem_u32(sQ + qt * Q_TILE_BYTES + blk * Q_BLK_BYTES), qm, blk * 64, kvh * G,
-                                    b * p.l_C + (row0 + qt * 128) / G, bar(BAR_Q_FULL));
+                        for (int blk = 0; blk < D / 64; ++blk)
+                            tma_load_3d(smem_u32(sQ + qt * Q_TILE_BYTES + blk * Q_BLK_BYTES), qm, blk * 64, kvh * G,
+                                        b * p.l_C + (row0 + qt * 128) / G, bar(BAR_Q_FULL));
+                }
+                return;
             }
-        } else if (has_work) {
             // group sizes that do not divide 128: 16-byte copies, row by row
             const int chunk = ptid % CH, rsub = ptid / CH, cin = chunk & 7;
             constexpr int RSTEP = TC_PRODUCERS / CH;
-            const __nv_bfloat16* Qsrc = far ? p.Qg : p.Q;
+            const __nv_bfloat16* Qsrc = q_far ? p.Qg : p.Q;
             for (int r = rsub; r < TC_ROWS; r += RSTEP) {
                 const int row = row0 + r;
                 const bool ok = row < R;
@@ -653,7 +681,8 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
                 cp_async16(sQ + doff, Qsrc + qoff, ok ? 16 : 0);
             }
             cp_async_arrive_noinc(bar(BAR_Q_FULL));
-        }
+        };
+        if (has_work) load_q(phase_far(TWO && n_early == 0 ? 1 : 0));
         // K/V tiles: four threads share a row (one instruction of the four covers 64 contiguous bytes of it: whole
         // sectors), so a thread works out the cache position of four rows per 128-key tile, not of sixteen, and
         // copies CH / 4 chunks of each; the loop is sensitive to the instructions the CTA's warps issue, these included.
@@ -678,9 +707,11 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
 #pragma unroll 1
         for (int phase = 0; phase < 2; ++phase) {
         if (phase == 1 && !planned) plan();
-        const KeyList kl = phase == 0 ? list_early : list_late;
+        const bool k_far = phase_far(phase);
+        KeyList kl = !TWO && phase == 0 ? list_early : list_late;
+        if (TWO && k_far) kl.row_lim = kl.ng;
         const int j_first = phase == 0 ? 0 : n_early, j_last = phase == 0 ? n_early : n_tiles;
-        const int key_first = phase == 0 ? early_begin * TC_BN : part_lo + tile_begin * TC_BN;
+        const int key_first = phase_key(phase);
         for (int j = j_first; j < j_last; ++j) {
             const int s = j % STAGES;
             const uint32_t ph = ((j / STAGES) & 1) ^ 1;
@@ -707,7 +738,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
                 if ((from_idx >> it) & 1u) pos[it] = clamp_selected(pos[it], i_end, m_end, bad_idx);
 #pragma unroll
             for (int it = 0; it < NPASS; ++it) {
-                const __nv_bfloat16* src = (far ? Kb1 : Kb0) + (pos[it] < 0 ? 0 : pos[it]) * tok_stride;
+                const __nv_bfloat16* src = (k_far ? Kb1 : Kb0) + (pos[it] < 0 ? 0 : pos[it]) * tok_stride;
                 const int nbytes = pos[it] < 0 ? 0 : 16;
                 uint8_t* tile = sK + s * KV_TILE_BYTES;
 #pragma unroll
@@ -717,6 +748,11 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
                 }
             }
             cp_async_arrive_noinc(bar(BAR_K_FULL + s));
+            if (TWO && q_swap && j == n_early) {
+                // every product with the old Q tiles has run (the release of the last tile's keys says so)
+                mbar_wait(bar(BAR_K_EMPTY + (j - 1) % STAGES), ((j - 1) / STAGES) & 1, wc);
+                load_q(k_far);
+            }
             mbar_wait(bar(BAR_V_EMPTY + s), ph, wc);
 #pragma unroll
             for (int it = 0; it < NPASS; ++it) {
@@ -790,6 +826,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
                 umma_commit(bar(BAR_PV_DONE + qt), lead);
                 if (more && qt == 0) {
                     mbar_wait(bar(BAR_K_FULL + sn), (Tn / STAGES) & 1, wc);
+                    if (TWO && q_swap && Tn == n_early) mbar_wait(bar(BAR_Q_FULL), 1, wc);
                     fence_async_smem();
                 }
                 mbar_wait(bar(BAR_P_READY + qt * 2 + 1), T & 1, wc);
@@ -850,7 +887,7 @@ static cudaError_t launch_tc_kernel(esa_ctx* ctx, const CUtensorMap& qmap, const
     attr[1].val.clusterDim.y = 1;
     attr[1].val.clusterDim.z = 2;
     cfg.attrs = attr;
-    cfg.numAttrs = MODE == TC_PAIR ? 2 : 1;
+    cfg.numAttrs = MODE == TC_PAIR || MODE == TC_TWO_PAIR ? 2 : 1;
     if (probe_only) {
         // can the device place a pair of these CTAs at all?
         int n_clusters = 0;
@@ -891,6 +928,7 @@ static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_m
     int i_end_max = 0;
     for (int b = 0; b < B; ++b) i_end_max = max(i_end_max, p.meta.i_end[b]);
     const int far_tiles = min(n_tiles, (i_end_max + p.top_k + TC_BN - 1) / TC_BN);
+    const bool even_out = abs(2 * far_tiles - n_tiles) > 5;       // (a pair moves tiles between its lists)
     const int step = p.two ? 2 : 1;
     const double merge_bytes = (double)B * p.HG * p.Rp * (D + 2) * 4;      // per part
     int best = 0;
@@ -899,11 +937,14 @@ static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_m
         if (ns > 2 && (size_t)B * p.HG * ns * p.Rp * (D + 2) > ctx->att_part_elems) break;      // (pairs use no scratch)
         const int grp = p.two ? ns / 2 : ns;
         const int longest = p.two ? max(far_tiles, n_tiles - far_tiles + 1) : n_tiles;
-        const int per = (longest + grp - 1) / grp;
+        const int per = p.two && ns == 2 && even_out ? (n_tiles + 4) / 2 : (longest + grp - 1) / grp;
         const int waves = (ctas * ns + ctx->num_sms - 1) / ctx->num_sms;
         const int last_wave = ctas * ns - (waves - 1) * ctx->num_sms;
         const double join = ns == 1 ? 0.0 : ns == 2 ? 7.5 : 7.5 + ns * merge_bytes / 4e6 + (last_wave * 8 > ctx->num_sms * 7 ? 6.0 : 0.0);
-        const double cost = waves * ((NQT == 2 ? 1.85 : 1.55) * per + 3.0) + 4.0 + join;
+        const double tile = NQT == 2 ? 1.85 : 1.55;
+        double cost = waves * (tile * per + 3.0) + 4.0 + join;
+        // CTAs of unlike lengths (the two lists) fill each other's gaps: SM time over SMs, and half a CTA for the end
+        if (p.two && ns > 2 && waves > 1) cost = ctas * (tile * n_tiles + 3.0 * ns) / ctx->num_sms + (tile * per + 3.0) / 2 + 4.0 + join;
         if (cost < best_cost - 1e-9) { best_cost = cost; best = ns; }
     }
     // Two uneven parts (TC_UNEVEN), where one CTA per unit leaves SMs idle and a second one each would more than fill them:
@@ -938,13 +979,15 @@ static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_m
     static int pair_ok = -1;                                 // per instantiation; probed once
     const bool uneven = p.main_tiles > 0;
     if (best == 2 && !uneven && pair_ok < 0)
-        pair_ok = launch_tc_kernel<D, TC_PAIR, NQT>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess ? 1 : 0;
+        pair_ok = launch_tc_kernel<D, TC_PAIR, NQT>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess &&
+                  launch_tc_kernel<D, TC_TWO_PAIR, NQT>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess ? 1 : 0;
     const bool pair = best == 2 && !uneven && pair_ok == 1;
     if (best == 2 && !pair && (size_t)B * p.HG * 2 * p.Rp * (D + 2) > ctx->att_part_elems) return cudaErrorNotSupported;
     cudaError_t e;
     {
         ProfScope prof(ctx, KC_ATTEND_TC, st);
-        if (pair) e = launch_tc_kernel<D, TC_PAIR, NQT>(ctx, qmap, qgmap, p, grid, st, false);
+        if (pair && p.two && even_out) e = launch_tc_kernel<D, TC_TWO_PAIR, NQT>(ctx, qmap, qgmap, p, grid, st, false);
+        else if (pair) e = launch_tc_kernel<D, TC_PAIR, NQT>(ctx, qmap, qgmap, p, grid, st, false);
         else if (uneven) e = launch_tc_kernel<D, TC_UNEVEN, 2>(ctx, qmap, qgmap, p, grid, st, false);
         else e = launch_tc_kernel<D, TC_PARTS, NQT>(ctx, qmap, qgmap, p, grid, st, false);
     }

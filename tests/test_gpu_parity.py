@@ -628,6 +628,17 @@ def test_two_position_attention_llama_shape_and_group_of_seven():
 
 
 # ------------------------------------------------ host-resident K/V (appendix "Model Loading")
+@pytest.mark.parametrize("H,H_G,d,t,l_C,l_L,k,n_sel", [
+    (32, 8, 64, 4000, 512, 200, 2000, None), (32, 8, 64, 4000, 512, 200, 2000, 1),     # the selected part longer; the local part longer
+    (32, 8, 64, 4000, 500, 2500, 500, 0), (32, 8, 128, 120, 400, 600, 500, None),      # nothing selected; I and C only
+    (28, 4, 128, 3500, 300, 1800, 400, 77), (28, 4, 128, 3500, 301, 100, 2900, None),  # Q tiles by plain copies, both ways
+    (8, 2, 64, 3000, 257, 700, 1100, None), (4, 4, 128, 2500, 30, 64, 1500, None)])
+def test_two_position_pairs_even_their_lists_out(H, H_G, d, t, l_C, l_L, k, n_sel):
+    """Lists of unlike lengths: one CTA of a pair goes on with the end of the other's list, with the other pair of encodings."""
+    cfg = syn.get_config("c1").with_(H=H, H_G=H_G, d=d, l_I=16, l_L=l_L, k=k)
+    _two_position_case(cfg, t, l_C, heads=[0, H // 2, H - 1], n_sel=n_sel)
+
+
 @pytest.mark.parametrize("name,t,l_C,n_sel", [("c1", 3968, 128, None), ("c1", 4100, 1, None), ("c1", 2000, 5, 100),
                                                ("c1", 300, 128, None), ("c2", 8192, 512, None), ("c2", 9000, 1, None)])
 def test_attention_with_host_resident_kv(name, t, l_C, n_sel):
