@@ -943,8 +943,8 @@ static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_m
         const double join = ns == 1 ? 0.0 : ns == 2 ? 7.5 : 7.5 + ns * merge_bytes / 4e6 + (last_wave * 8 > ctx->num_sms * 7 ? 6.0 : 0.0);
         const double tile = NQT == 2 ? 1.85 : 1.55;
         double cost = waves * (tile * per + 3.0) + 4.0 + join;
-        // CTAs of unlike lengths (the two lists) fill each other's gaps: SM time over SMs, and half a CTA for the end
-        if (p.two && ns > 2 && waves > 1) cost = ctas * (tile * n_tiles + 3.0 * ns) / ctx->num_sms + (tile * per + 3.0) / 2 + 4.0 + join;
+        // CTAs of unlike lengths (the two lists) fill each other's gaps over three waves and more: SM time over SMs, and half a CTA for the end
+        if (p.two && ns > 2 && waves > 2) cost = ctas * (tile * n_tiles + 3.0 * ns) / ctx->num_sms + (tile * per + 3.0) / 2 + 4.0 + join;
         if (cost < best_cost - 1e-9) { best_cost = cost; best = ns; }
     }
     // Two uneven parts (TC_UNEVEN), where one CTA per unit leaves SMs idle and a second one each would more than fill them:

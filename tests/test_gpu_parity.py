@@ -83,6 +83,19 @@ def test_compress_keys_parity(name, n_new, with_bias):
         assert float(kc[b, n_prev[b] + n_new:].abs().sum()) == 0.0
 
 
+@pytest.mark.parametrize("H_G,d_c,n_new", [(8, 128, 17), (8, 128, 100), (8, 128, 129), (32, 128, 37), (32, 128, 127), (4, 64, 31), (28, 64, 255)])
+def test_compress_keys_ragged_row_tiles(H_G, d_c, n_new):
+    """Row tiles with few rows: a cluster's CTAs share them out, whatever the number of splits (4 to 16 here)."""
+    cfg = syn.get_config("c2").with_(H=32 if H_G != 28 else 28, H_G=H_G, d_c=d_c, S=1024, n_decode=0)
+    ctx = hp.make_esa(cfg, max_tokens=1024, max_chunk=512, max_batch=1)
+    _, _, _, Wk = hp.oracle_weights(cfg)
+    Kb = syn.qkv_rows(cfg, "k", 0, n_new)
+    kc = torch.zeros(1, 1024, d_c, dtype=torch.bfloat16, device="cuda")
+    ctx.compress_keys(hp.bits_to_torch(Kb)[None].contiguous(), kc, [300], sync=True)
+    hp.check_compressed(kc[0, 300: 300 + n_new], syn.bf16_bits_to_f64(Kb).reshape(n_new, -1), Wk, what=f"{n_new} rows")
+    assert float(kc[0, :300].abs().sum()) == 0.0 and float(kc[0, 300 + n_new:].abs().sum()) == 0.0
+
+
 def test_query_sized_compression_through_compress_keys():
     """Eq. 5 at the query compressor's shape (d_in = H d = 4096, 512 rows) through the public key
     entry point: with H_G = H the key compressor has the query compressor's shape, and the
