@@ -41,7 +41,7 @@ N_LAYERS_STACK = 32
 # dram__bytes_read.sum + dram__bytes_write.sum from the ncu captures summarised in
 # profiles/dram_bytes_per_kernel.txt (same kernels, same launch shapes as the timed workloads).
 ATTEND_TC_DRAM_BYTES = 32087552 + 1280
-DECODE_STEP_DRAM_BYTES = (205836544 + 79360) + 39168 + 300288 + 1133312 + (264913408 + 626688) + 4355328
+DECODE_STEP_DRAM_BYTES = (205835776 + 820992) + 39168 + 300032 + 1132800 + (265845504 + 2993408) + 4208128
 
 
 # ----------------------------------------------------------------------------
@@ -722,7 +722,7 @@ def run_esa(args, cfg):
     n_chunks = (cfg.S + cfg.l_C - 1) // cfg.l_C
     att = by_kernel.get("attend_tc_kernel", {"achieved": 0.0, "frac_sustained": 0.0, "frac_burst": 0.0, "launches": 0})
     att_ms = prof.get("attend_tc_kernel", (0, 0.0))[1]
-    roofline = {"bound": "tensor", "kernel": "attend_tc_kernel (key-list splits merged inside the kernel)",
+    roofline = {"bound": "tensor", "kernel": "attend_tc_kernel (two-way key-list splits merged inside the kernel)",
                 "achieved": att["achieved"], "peak": peaks["tflops_sustained"],
                 "unit": "TFLOP/s", "frac": att["frac_sustained"], "frac_sustained": att["frac_sustained"],
                 "frac_burst": att["frac_burst"], "peak_burst": peaks["tflops_burst"],

@@ -254,7 +254,7 @@ cudaError_t launch_compress_tc(esa_ctx* ctx, const __nv_bfloat16* X, int B, int 
 
 // True when launch_score takes the tcgen05 path for this call: every chunk (row numbers are 32-bit TMA coordinates).
 // For a handful of queries most of a 128-row tile is padding, but the passes are bound by the stream of keys and their
-// own latency, and pooling and the first radix digit come with the second pass: 37 queries after 50021 tokens, select
+// own latency, and pooling comes with the second pass: 37 queries after 50021 tokens, select
 // 51 -> 32 us against the mma.sync kernels with their memsets and pooling launch.
 inline bool score_uses_tc(const esa_ctx* ctx, int B) { return (int64_t)B * ctx->cfg.max_tokens < (int64_t(1) << 31); }
 
