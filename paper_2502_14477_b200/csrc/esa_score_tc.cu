@@ -219,8 +219,11 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
             const int first = min(n_ltiles, STAGES);
             for (int lt = 0; lt < first; ++lt) load_tile(lt);
             if (PASS == 1) pdl_wait();
-            for (int uu = 0; uu < NU; ++uu) {
-                const int u = (uu + woff) % NU;              // in the order the items use them
+            // in the order the items use them, and only those that are used: in a short context a CTA may have a
+            // single item, and a load that nobody waits for could land after the CTA has ended
+            const int n_units = min(NU, n_items);
+            for (int uu = 0; uu < n_units; ++uu) {
+                const int u = (uu + woff) % NU;
                 mbar_arrive_expect_tx(bar(C::B_QFULL + u), UNIT * DC * 2);
 #pragma unroll
                 for (int blk = 0; blk < NBLK; ++blk)

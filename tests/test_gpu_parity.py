@@ -265,6 +265,16 @@ def test_selection_at_cluster_and_share_edges(t_list, l_C, d_c, eps, k, run):
         assert np.array_equal(got[b], want), f"seq {b} |M|={l_M}: {int((got[b] != want).sum())} positions differ"
 
 
+@pytest.mark.parametrize("t_list,l_C,d_c,k", [
+    ([80 + 301], 512, 128, 300), ([80 + 1000], 385, 64, 300), ([80 + 4700], 512, 128, 4096),       # one item a CTA, four blocks
+    ([80 + 129, 80 + 9000], 300, 32, 100), ([80 + 2500, 80 + 130], 1100, 64, 100)])                # ragged; three groups of queries
+def test_scoring_with_fewer_items_than_query_blocks(t_list, l_C, d_c, k):
+    """Chunks of several 128-query blocks over a short middle part: a CTA of the first pass has fewer (tile, block) items than
+    there are blocks and loads only the blocks that it uses."""
+    for _ in range(3):
+        test_selection_at_cluster_and_share_edges(t_list, l_C, d_c, 3, k, 0)
+
+
 @pytest.mark.parametrize("H,H_G,d,d_c,t,l_C,two", [
     (4, 4, 64, 64, 2500, 127, False), (4, 4, 64, 64, 2500, 128, False), (4, 4, 64, 64, 2500, 129, False),   # one or two Q tiles
     (8, 2, 64, 32, 2000, 2, False), (8, 2, 64, 32, 129, 2, False), (28, 4, 128, 128, 6001, 19, False),       # 2 rows; no M; 133 rows
