@@ -233,6 +233,9 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
                                     b * p.l_C + q0 + u * UNIT + r0, bar(C::B_QFULL + u));
             }
             for (int lt = first; lt < n_ltiles; ++lt) load_tile(lt);
+            // The issuing warps release the last tiles after their last accumulator: these arrivals are seen here, so
+            // that none is still on its way to this CTA's shared memory when the CTA ends.
+            for (int lt = n_ltiles - first; lt < n_ltiles; ++lt) mbar_wait(bar(C::B_EMPTY + lt % STAGES), (lt / STAGES) & 1, wc);
         }
     } else if (warp <= 2) {
         // ------------------------------------------------------------ MMA issue (converged warps, lane 0 leads)

@@ -861,6 +861,31 @@ def test_bounded_wait_gives_up_and_the_context_stays_usable():
     hp.check_attention(Ob, res.O, what="after a timed-out wait")
 
 
+def test_steps_back_to_back_repeat_bit_for_bit():
+    """Steps of unlike kernels enqueued without a pause between them (short and longer contexts, chunks of one to four query
+    blocks): every kernel's CTAs follow the previous kernel's on an SM, and a second run of the sequence gives the same bits."""
+    cfg = syn.get_config("c2").with_(H=8, H_G=2, d_c=64, l_I=16, l_L=256, k=200, S=9000)
+    n = 9600
+    ctx = hp.make_esa(cfg, max_tokens=n, max_chunk=512, max_batch=1)
+    seq = hp.DeviceSeq(cfg, max_tokens=n, B=1)
+    seq.fill_kv(0, n)
+    fill_kc_gpu(ctx, seq, n)
+    Q = hp.bits_to_torch(syn.qkv_rows(cfg, "q", 0, 512))[None].contiguous()
+    runs = []
+    for _ in range(2):
+        outs = []
+        for t in (480, 600, 1100, 5000, 9000):
+            for l_C in (512, 385, 100, 37, 2, 1, 256):
+                q = Q[:, :l_C].contiguous()
+                idx, n_sel = torch.zeros_like(seq.idx), torch.zeros_like(seq.n_sel)
+                ctx.select(q, seq.Kc, [t], idx, n_sel)
+                outs += [idx, n_sel]
+        torch.cuda.synchronize()
+        assert ctx.last_device_status() == 0
+        runs.append(outs)
+    assert all(torch.equal(a, b) for a, b in zip(*runs))
+
+
 # ----------------------------------------------------------------- error paths
 def test_argument_errors_leave_outputs_untouched():
     import paper_2502_14477_b200 as esa
