@@ -842,6 +842,9 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
                 }
             }
         }
+        // The release of the last V tile comes after the last O_READY and nobody fetches another tile: seen here, so that no
+        // arrival is still on its way to this CTA's shared memory when the CTA ends.
+        mbar_wait(bar(BAR_V_EMPTY + (n_tiles - 1) % STAGES), ((n_tiles - 1) / STAGES) & 1, wc);
     }
 
     if (PAIR && warp_u >= TC_SOFTMAX_WARPS) {

@@ -877,9 +877,10 @@ def test_steps_back_to_back_repeat_bit_for_bit():
         for t in (480, 600, 1100, 5000, 9000):
             for l_C in (512, 385, 100, 37, 2, 1, 256):
                 q = Q[:, :l_C].contiguous()
-                idx, n_sel = torch.zeros_like(seq.idx), torch.zeros_like(seq.n_sel)
+                O, idx, n_sel = torch.empty_like(q), torch.zeros_like(seq.idx), torch.zeros_like(seq.n_sel)
                 ctx.select(q, seq.Kc, [t], idx, n_sel)
-                outs += [idx, n_sel]
+                ctx.attend(q, seq.K, seq.V, [t], idx, n_sel, O)
+                outs += [O, idx, n_sel]
         torch.cuda.synchronize()
         assert ctx.last_device_status() == 0
         runs.append(outs)
