@@ -275,6 +275,35 @@ def test_scoring_with_fewer_items_than_query_blocks(t_list, l_C, d_c, k):
         test_selection_at_cluster_and_share_edges(t_list, l_C, d_c, 3, k, 0)
 
 
+@pytest.mark.parametrize("d_c,l_C", [(32, 1), (32, 2), (32, 64), (64, 37), (128, 5), (128, 64)])
+def test_scores_of_few_queries_are_rounded_to_nearest(d_c, l_C):
+    """S and r_c are exact here (small integers times a power of two), S - r_c is not (29 significant bits): the scores must be the
+    fp32 difference rounded to nearest, bit for bit."""
+    cfg = syn.get_config("c1").with_(H=8, H_G=2, d=128, d_c=d_c, l_I=16, l_L=64, eps=0, k=100)
+    t = 1500
+    ctx = hp.make_esa(cfg, max_tokens=t + l_C, max_chunk=l_C, max_batch=1)
+    wq, wk = np.zeros((d_c, 8 * 128), np.float32), np.zeros((d_c, 2 * 128), np.float32)
+    wq[np.arange(d_c), np.arange(d_c)] = 1.0                      # q' = the first d_c values of head 0
+    ctx.set_compressors(wq, None, wk, None)
+    g = np.random.default_rng(d_c + l_C)
+    q = g.integers(1, 8, (l_C, d_c)).astype(np.float64)
+    k = g.integers(-7, 8, (t, d_c)).astype(np.float64) * 2.0 ** -14
+    k[700] = 32.0 * g.integers(1, 4, d_c)                          # every query's arg-max: r_c of up to 15 bits
+    Q = torch.zeros(1, l_C, 8, 128, dtype=torch.bfloat16, device="cuda")
+    Q[0, :, 0, :d_c] = torch.from_numpy(q).cuda().bfloat16()
+    kc = torch.zeros(1, t + l_C, d_c, dtype=torch.bfloat16, device="cuda")
+    kc[0, :t] = torch.from_numpy(k).cuda().bfloat16()
+    idx, n_sel = torch.zeros(1, cfg.k, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    ctx.select(Q, kc, [t], idx, n_sel, sync=True)
+    S = q @ k[16:t - 64].T
+    r = S.max(axis=1, keepdims=True)
+    assert np.array_equal(S.astype(np.float32).astype(np.float64), S)
+    want = (S.astype(np.float32) - r.astype(np.float32)).max(axis=0)
+    assert (want.astype(np.float64) != (S - r).max(axis=0)).mean() > 0.5          # the rounding matters
+    got = ctx.read_pooled_scores(0, t - 80)
+    assert np.array_equal(got, want)
+
+
 @pytest.mark.parametrize("H,H_G,d,d_c,t,l_C,two", [
     (4, 4, 64, 64, 2500, 127, False), (4, 4, 64, 64, 2500, 128, False), (4, 4, 64, 64, 2500, 129, False),   # one or two Q tiles
     (8, 2, 64, 32, 2000, 2, False), (8, 2, 64, 32, 129, 2, False), (28, 4, 128, 128, 6001, 19, False),       # 2 rows; no M; 133 rows
