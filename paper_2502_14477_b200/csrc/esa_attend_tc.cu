@@ -49,6 +49,7 @@
 //     running sums and accumulator (33 tiles against 20, 512 queries of the 32/8-head shape: 72 -> 64 us; 64
 //     against 12: 126 -> 87).
 #include <cstring>
+#include <type_traits>
 
 #include "esa_internal.h"
 #include "esa_umma.cuh"
@@ -211,7 +212,13 @@ __device__ __forceinline__ void store_half_rows(const float* acc, float4* stage,
 // its copies have landed.
 // NQT: Q tiles of a CTA that hold rows.  One for chunks of at most 128 rows per key/value head: the second tile's
 // products and softmax would only be in the way.
-template <int D, int MODE, int NQT>
+// FINE: P in two bf16 pieces; the second one overwrites the other 32 columns of the half, and the products of P with V
+// double.  Against a standing maximum the weight of a row's dominant key is an arbitrary number, and its rounding to 8 bits puts
+// 1.9e-3 to 3.0e-3 of error into the result (2-norm, against 64 bits, 2 to 16 queries), where rounding against the row's own maximum,
+// an exact 1, gives 1.7e-3.  The pieces leave the rounding of the result itself, 1.6e-3.  For chunks of at most 64 rows per
+// key/value head, as exact as the decode kernel beside them: a step of them takes 0.5 to 1.5 us longer for it (8 queries
+// 29.6 -> 30.2 us, 9 queries of the 28/4-head shape after 100k tokens 50.4 -> 51.7).
+template <int D, int MODE, int NQT, bool FINE>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap qgmap, TcAttendParams p) {
     constexpr bool TWO = MODE == TC_TWO_PAIR, PAIR = MODE == TC_PAIR || TWO, UNEVEN = MODE == TC_UNEVEN;
@@ -398,7 +405,8 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
             }
             // P = 2^(S * scale - m) as packed bf16 (it will overwrite the first 32 columns of this half); returns the
             // sum of the half.  A row without a visible key so far has m = -inf: its P must be 0, not 2^(+inf).
-            uint32_t pk[TC_HALF / 2];
+            // FINE: the second piece of P.
+            uint32_t pk[TC_HALF / 2], lo[FINE ? TC_HALF / 2 : 1];
             auto exps = [&](float m) {
                 const float neg_m = (m == -INFINITY) ? 0.f : -m;
                 const float2 sl2v = make_float2(sl2, sl2), nm = make_float2(neg_m, neg_m);
@@ -411,6 +419,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
                     e.y = fast_exp2(x.y);
                     sum4[i & 3] = fadd2(sum4[i & 3], e);
                     pk[i] = pack_bf16(e.x, e.y);
+                    if (FINE) lo[i] = pack_bf16(e.x - __uint_as_float(pk[i] << 16), e.y - __uint_as_float(pk[i] & 0xffff0000u));
                 }
                 const float2 a = fadd2(sum4[0], sum4[1]), c = fadd2(sum4[2], sum4[3]);
                 return (a.x + a.y) + (c.x + c.y);
@@ -458,6 +467,7 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
                 part_sum = exps(m_run);
             }
             tmem_st32(tS + u * 64, pk);
+            if (FINE) tmem_st32(tS + u * 64 + 32, lo);
             l_run += part_sum;
             tmem_wait_st();
             tc_fence_before_sync();
@@ -796,6 +806,11 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
 #pragma unroll
             for (int ks = 0; ks < TC_HALF / 16; ++ks)
                 umma_ts(tmem + 256 + qt * D, tmem + qt * 128 + u * 64 + ks * 8, b0 + ks * (2048 >> 4), hi, ID_PV, acc | ks, lead);
+            if (FINE) {
+#pragma unroll
+                for (int ks = 0; ks < TC_HALF / 16; ++ks)
+                    umma_ts(tmem + 256 + qt * D, tmem + qt * 128 + u * 64 + 32 + ks * 8, b0 + ks * (2048 >> 4), hi, ID_PV, 1, lead);
+            }
         };
         mbar_wait(bar(BAR_Q_FULL), 0, wc);
         mbar_wait(bar(BAR_K_FULL + 0), 0, wc);
@@ -861,18 +876,18 @@ attend_tc_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant
 
 }  // namespace
 
-template <int D, int MODE, int NQT>
+template <int D, int MODE, int NQT, bool FINE>
 static cudaError_t launch_tc_kernel(esa_ctx* ctx, const CUtensorMap& qmap, const CUtensorMap& qgmap, const TcAttendParams& p,
                                     dim3 grid, cudaStream_t st, bool probe_only) {
     constexpr int smem = 2 * 128 * D * 2 + 2 * TC_STAGES * TC_BN * D * 2 + 1024;
     static KernelMemo memo;
-    cudaError_t e = allow_smem(attend_tc_kernel<D, MODE, NQT>, ctx->device, smem, memo);
+    cudaError_t e = allow_smem(attend_tc_kernel<D, MODE, NQT, FINE>, ctx->device, smem, memo);
     if (e != cudaSuccess) return e;
     // the in-kernel register split assumes the launch allocation it was sized for
     static int regs_checked = 0;
     if (!regs_checked) {
         cudaFuncAttributes fa;
-        e = cudaFuncGetAttributes(&fa, attend_tc_kernel<D, MODE, NQT>);
+        e = cudaFuncGetAttributes(&fa, attend_tc_kernel<D, MODE, NQT, FINE>);
         if (e != cudaSuccess) return e;
         if (fa.numRegs != TC_REGS_LAUNCH) return cudaErrorInvalidConfiguration;
         regs_checked = 1;
@@ -894,11 +909,11 @@ static cudaError_t launch_tc_kernel(esa_ctx* ctx, const CUtensorMap& qmap, const
     if (probe_only) {
         // can the device place a pair of these CTAs at all?
         int n_clusters = 0;
-        e = cudaOccupancyMaxActiveClusters(&n_clusters, attend_tc_kernel<D, MODE, NQT>, &cfg);
+        e = cudaOccupancyMaxActiveClusters(&n_clusters, attend_tc_kernel<D, MODE, NQT, FINE>, &cfg);
         if (e != cudaSuccess) return e;
         return n_clusters > 0 ? cudaSuccess : cudaErrorNotSupported;
     }
-    return cudaLaunchKernelEx(&cfg, attend_tc_kernel<D, MODE, NQT>, qmap, qgmap, p);
+    return cudaLaunchKernelEx(&cfg, attend_tc_kernel<D, MODE, NQT, FINE>, qmap, qgmap, p);
 }
 
 // Merge of a key list split more than two ways: a warp per row.
@@ -915,7 +930,7 @@ __global__ void __launch_bounds__(256) attend_tc_merge_kernel(const float* part,
                  O + (((int64_t)b * l_C + row / G) * H + kvh * G + row % G) * D);
 }
 
-template <int D, int NQT>
+template <int D, int NQT, bool FINE>
 static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_max, cudaStream_t st) {
     const int R = p.l_C * p.G;
     const int row_tiles = (R + TC_ROWS - 1) / TC_ROWS;
@@ -982,17 +997,17 @@ static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_m
     static int pair_ok = -1;                                 // per instantiation; probed once
     const bool uneven = p.main_tiles > 0;
     if (best == 2 && !uneven && pair_ok < 0)
-        pair_ok = launch_tc_kernel<D, TC_PAIR, NQT>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess &&
-                  launch_tc_kernel<D, TC_TWO_PAIR, NQT>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess ? 1 : 0;
+        pair_ok = launch_tc_kernel<D, TC_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess &&
+                  launch_tc_kernel<D, TC_TWO_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess ? 1 : 0;
     const bool pair = best == 2 && !uneven && pair_ok == 1;
     if (best == 2 && !pair && (size_t)B * p.HG * 2 * p.Rp * (D + 2) > ctx->att_part_elems) return cudaErrorNotSupported;
     cudaError_t e;
     {
         ProfScope prof(ctx, KC_ATTEND_TC, st);
-        if (pair && p.two && even_out) e = launch_tc_kernel<D, TC_TWO_PAIR, NQT>(ctx, qmap, qgmap, p, grid, st, false);
-        else if (pair) e = launch_tc_kernel<D, TC_PAIR, NQT>(ctx, qmap, qgmap, p, grid, st, false);
-        else if (uneven) e = launch_tc_kernel<D, TC_UNEVEN, 2>(ctx, qmap, qgmap, p, grid, st, false);
-        else e = launch_tc_kernel<D, TC_PARTS, NQT>(ctx, qmap, qgmap, p, grid, st, false);
+        if (pair && p.two && even_out) e = launch_tc_kernel<D, TC_TWO_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, false);
+        else if (pair) e = launch_tc_kernel<D, TC_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, false);
+        else if (uneven) e = launch_tc_kernel<D, TC_UNEVEN, 2, false>(ctx, qmap, qgmap, p, grid, st, false);
+        else e = launch_tc_kernel<D, TC_PARTS, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, false);
     }
     ctx->launches += 1;
     if (e != cudaSuccess || best == 1 || pair) return e;
@@ -1018,9 +1033,14 @@ cudaError_t launch_attend_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* 
     p.top_k = ctx->cfg.top_k; p.nsplit = 1;
     p.scale_log2 = ctx->scale * 1.4426950408889634f;
     p.meta = meta;
-    const bool one = l_C * ctx->G <= 128;
-    if (ctx->d == 128) return one ? launch_tc<128, 1>(ctx, p, B, n_att_max, st) : launch_tc<128, 2>(ctx, p, B, n_att_max, st);
-    if (ctx->d == 64) return one ? launch_tc<64, 1>(ctx, p, B, n_att_max, st) : launch_tc<64, 2>(ctx, p, B, n_att_max, st);
+    const int rows = l_C * ctx->G;
+    auto run = [&](auto dim) {
+        constexpr int D = decltype(dim)::value;
+        if (rows <= kAttSplitRows) return launch_tc<D, 1, true>(ctx, p, B, n_att_max, st);
+        return rows <= 128 ? launch_tc<D, 1, false>(ctx, p, B, n_att_max, st) : launch_tc<D, 2, false>(ctx, p, B, n_att_max, st);
+    };
+    if (ctx->d == 128) return run(std::integral_constant<int, 128>());
+    if (ctx->d == 64) return run(std::integral_constant<int, 64>());
     return cudaErrorNotSupported;
 }
 

@@ -318,6 +318,38 @@ def test_small_chunks_at_tile_and_split_edges(H, H_G, d, d_c, t, l_C, two):
         _stage_isolated(cfg, t, l_C)
 
 
+@pytest.mark.parametrize("H,H_G,d,t,l_C,l_L,k", [
+    (32, 8, 128, 20000, 2, 2048, 4096), (32, 8, 128, 9000, 16, 1024, 1024), (28, 4, 128, 12000, 9, 1024, 2048),
+    (8, 2, 64, 4000, 7, 512, 256), (4, 4, 64, 3000, 64, 700, 1000), (4, 4, 64, 3000, 61, 700, 1000), (32, 2, 128, 9000, 1, 1024, 1024), (6, 2, 128, 700, 21, 128, 100)])
+def test_small_chunk_attention_is_the_rounding_of_the_exact_result(H, H_G, d, t, l_C, l_L, k):
+    """Chunks of at most 64 rows per key/value head keep the probabilities to 16 bits, so the result is the bf16 rounding of the
+    exact one unless that lies within the kernel's own error of a rounding boundary.  That error is at most 2^-16 max|V| (two
+    bf16 pieces of every weight: 2^-17 of a weighted mean of V; sums and exponentials in fp32), against a rounding step of
+    2^-8 to 2^-7 of the value: at most 2 % of the elements may round the other way (measured: 0.3 %; with
+    weights of 8 bits 34 to 40 %), and none may be off by more than one rounding and that error."""
+    cfg = syn.get_config("c1").with_(H=H, H_G=H_G, d=d, d_c=64, l_I=16, l_L=l_L, k=k)
+    p, n = hp.oracle_params(cfg), t + l_C
+    g = torch.Generator(device="cuda").manual_seed(t + l_C)
+    scale = lambda x: x.mul_((0.5 + 1.5 * torch.rand(x.shape[2], 1, device="cuda", generator=g)).bfloat16())
+    draw = lambda *s: scale(torch.randn(*s, device="cuda", dtype=torch.bfloat16, generator=g))
+    Q, K, V, Qf, Kf = draw(1, l_C, H, d), draw(1, n, H_G, d), draw(1, n, H_G, d), draw(1, l_C, H, d), draw(1, n, H_G, d)
+    sel = torch.sort(torch.randperm(t - l_L - 16, device="cuda", generator=g)[:k])[0] + 16
+    idx, n_sel = sel.int()[None].contiguous(), torch.tensor([k], dtype=torch.int32, device="cuda")
+    ctx = hp.make_esa(cfg, max_tokens=n, max_chunk=l_C, max_batch=1)
+    O, O2 = torch.empty_like(Q), torch.empty_like(Q)
+    ctx.attend(Q, K, V, [t], idx, n_sel, O, sync=True)
+    ctx.attend_two_position(Q, Qf, K, Kf, V, [t], idx, n_sel, O2, sync=True)
+    assert ctx.last_device_status() == 0
+    f64 = lambda x: hp.torch_to_f64(x[0])
+    for what, got, kw in (("one position", O, {}), ("two positions", O2, dict(Q_global=f64(Qf), K_global=f64(Kf)))):
+        want = orc.attend(f64(Q), f64(K), f64(V), sel.cpu().numpy(), t, p, **kw)
+        got = f64(got)
+        other = got != orc.bf16_round(want)
+        assert other.mean() <= 0.02, (what, float(other.mean()))
+        slack = 2.0 ** -8 * np.abs(want) + 2.0 ** -16 * float(V.float().abs().max())
+        assert (np.abs(got - want) <= slack).all(), what
+
+
 @pytest.mark.parametrize("H_G,B,t,l_C", [(28, 1, 3000, 1000), (28, 1, 900, 1024), (11, 1, 4001, 2047), (25, 2, 2500, 300), (38, 1, 150, 700), (45, 1, 2600, 500)])
 def test_uneven_key_list_split(H_G, B, t, l_C):
     """75 to 114 units of 256 rows: the idle SMs attend the ends of the units' key lists (nothing selected, ragged row tiles,
