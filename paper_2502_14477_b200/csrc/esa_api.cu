@@ -100,10 +100,14 @@ esa_status build_meta(const esa_ctx* ctx, int B, const int64_t* n_prev, int64_t 
 
 esa_status from_cuda(cudaError_t e) { return e == cudaSuccess ? ESA_OK : ESA_ERR_CUDA; }
 
-// The selection of a step has been enqueued on `st`: the attention call that follows it there may start early.
-void arm_attention(esa_ctx* ctx, cudaStream_t st) {
+// The selection of a step has been enqueued on `st`: the attention call that follows it there with the same queries may
+// start early.
+void arm_attention(esa_ctx* ctx, cudaStream_t st, const void* Q, int B, int l_C) {
     ctx->sel_armed = true;
     ctx->sel_stream = st;
+    ctx->sel_Q = Q;
+    ctx->sel_B = B;
+    ctx->sel_l_C = l_C;
 }
 
 }  // namespace
@@ -173,6 +177,8 @@ esa_status esa_create(const esa_config* cfg, esa_ctx** out) {
     c->last_decode = false;
     c->sel_armed = false;
     c->sel_stream = nullptr;
+    c->sel_Q = nullptr;
+    c->sel_B = c->sel_l_C = 0;
     c->attend_early = false;
     c->att_part = reinterpret_cast<float*>(base + L.att);
     c->att_part_elems = L.att_elems;
@@ -315,7 +321,7 @@ esa_status esa_select_async(esa_ctx* ctx, int32_t B, const void* Q_cur, int32_t 
         if (e != cudaSuccess) return ESA_ERR_CUDA;
     }
     if (!any_large) {
-        arm_attention(ctx, st);
+        arm_attention(ctx, st, Q_cur, B, l_C);
         return ESA_OK;
     }
     // q' = f_q(q) (Eq. 5)
@@ -349,7 +355,7 @@ esa_status esa_select_async(esa_ctx* ctx, int32_t B, const void* Q_cur, int32_t 
     e = launch_score(ctx, B, l_C, (const __nv_bfloat16*)kc_cache, smeta, max_lM, rkey_cleared, st, &pooled_ready);
     if (e != cudaSuccess) return ESA_ERR_CUDA;
     e = launch_select(ctx, B, l_C == 1, smeta, max_lM, pooled_ready, idx_out, n_sel_out, st);
-    if (e == cudaSuccess) arm_attention(ctx, st);
+    if (e == cudaSuccess) arm_attention(ctx, st, Q_cur, B, l_C);
     return from_cuda(e);
 }
 
@@ -375,7 +381,7 @@ esa_status esa_select_full_async(esa_ctx* ctx, int32_t B, const void* Q_cur, int
     ctx->last_q_rows = 0;
     if (any_small && launch_select_all(ctx, B, meta, idx_out, n_sel_out, st) != cudaSuccess) return ESA_ERR_CUDA;
     if (!any_large) {
-        arm_attention(ctx, st);
+        arm_attention(ctx, st, Q_cur, B, l_C);
         return ESA_OK;
     }
     SeqMeta smeta = meta;
@@ -386,7 +392,7 @@ esa_status esa_select_full_async(esa_ctx* ctx, int32_t B, const void* Q_cur, int
                                       mode == ESA_SCORE_PER_HEAD, st);
     if (e != cudaSuccess) return ESA_ERR_CUDA;
     e = launch_select(ctx, B, false, smeta, max_lM, false, idx_out, n_sel_out, st);
-    if (e == cudaSuccess) arm_attention(ctx, st);
+    if (e == cudaSuccess) arm_attention(ctx, st, Q_cur, B, l_C);
     return from_cuda(e);
 }
 
@@ -416,8 +422,10 @@ esa_status esa_attend_two_position_async(esa_ctx* ctx, int32_t B, const void* Q_
     SeqMeta meta;
     s = build_meta(ctx, B, n_prev, l_C, &meta, nullptr);
     if (s != ESA_OK) return s;
-    // a call that follows the selection of its step on the same stream may attend the older rows early
-    ctx->attend_early = ctx->sel_armed && ctx->sel_stream == (cudaStream_t)stream;
+    // A call that follows the selection of its step on the same stream may attend the older rows early, with the queries
+    // that the selection has read: others may be what the preceding kernel is writing.
+    ctx->attend_early = ctx->sel_armed && ctx->sel_stream == (cudaStream_t)stream && ctx->sel_Q == Q_cur && ctx->sel_B == B &&
+                        ctx->sel_l_C == l_C;
     ctx->sel_armed = false;
     cudaError_t e = launch_attend(ctx, B, l_C, (const __nv_bfloat16*)Q_cur, (const __nv_bfloat16*)Q_far,
                                   (const __nv_bfloat16*)K_cache, (const __nv_bfloat16*)K_far_cache,

@@ -140,7 +140,10 @@ attend_decode_kernel(AttendParams p) {
         }
     };
 
-    // B fragments of Q^T for every 16-wide slice of D: element (k = d, n = head); heads >= G are zero
+    // B fragments of Q^T for every 16-wide slice of D: element (k = d, n = head); heads >= G are zero.  An early call's
+    // queries are the selection's, read by a kernel before the preceding one; any other call's may be what the preceding
+    // kernel writes.
+    if (!early) pdl_wait();
     uint32_t qb[D / 16][2];
     uint32_t qbg[TWO ? D / 16 : 1][2];      // the same for the queries used against I and M_k
     {

@@ -124,12 +124,14 @@ struct esa_ctx {
     uint32_t* skey;      // [max_batch, max_tokens] unpooled aggregated scores (ordered keys) of the scoring paths that do not pool
     uint32_t* pkey;      // [max_batch, max_tokens] pooled scores s' as ordered keys (l_C = 1: of the pooled raw scores, r not yet subtracted)
     bool last_decode;    // the last selection ran with l_C = 1 (pkey holds raw pooled scores)
-    // The attention kernels may read cache rows older than the chunk ahead of their wait for the preceding kernel
-    // only when the work ahead of them in the stream is known not to write such rows: a selection enqueued through
-    // this context arms the next attention call on the same stream (the caller's side of it: nothing enqueued
-    // between the two calls writes cache rows older than the chunk).
+    // The attention kernels may read the queries and cache rows older than the chunk ahead of their wait for the preceding
+    // kernel only when the work ahead of them in the stream is known not to write either: a selection enqueued through
+    // this context arms the next attention call on the same stream with the same queries (the caller's side of it: nothing
+    // enqueued between the two calls writes those queries or cache rows older than the chunk).
     bool sel_armed;
     cudaStream_t sel_stream;
+    const void* sel_Q;   // queries of that selection, compared with the attention call's, never read
+    int sel_B, sel_l_C;
     bool attend_early;   // set around the launch of an armed attention call
     float* att_part;     // split-KV partial outputs + (m, l)
     size_t att_part_elems;

@@ -817,6 +817,52 @@ def test_attention_that_follows_its_selection_attends_the_older_rows_early(name,
     hp.check_attention(O_plain[0], want, what=f"plain {name} t={t} l_C={l_C}", heads=[0, cfg.H - 1])
 
 
+@pytest.mark.parametrize("call", ["attend", "two_position", "noalloc", "armed_by_other_queries", "chunk_armed_by_other_queries"])
+def test_attention_reads_queries_that_the_preceding_kernel_writes(call):
+    """The kernel just ahead of the attention writes its queries and lets its dependents start before it has written them (as a
+    rotary encoding with programmatic dependent launch would; here another context's append copies 128 MB whose last rows are
+    the queries).  Every attention call but the one that follows a selection made with the same queries must wait for it."""
+    import paper_2502_14477_b200 as esa
+    cfg = syn.get_config("c2")
+    t, l_C, rows = 9000, 37 if call.startswith("chunk") else 1, 16384
+    n = t + l_C
+    ctx = hp.make_esa(cfg, max_tokens=n, max_chunk=l_C, max_batch=1)
+    writer = esa.Esa(esa.EsaConfig(cfg.H, cfg.H, cfg.d, cfg.d_c, 4, 64, 64, 3, 1, 1, rows))
+    g = torch.Generator(device="cuda").manual_seed(9)
+    draw = lambda *s: torch.randn(*s, device="cuda", dtype=torch.bfloat16, generator=g)
+    K, V, Kf = (draw(1, n, cfg.H_G, cfg.d) for _ in range(3))
+    kc, Q_sel, src = draw(1, n, cfg.d_c), draw(1, l_C, cfg.H, cfg.d), draw(1, rows, cfg.H, cfg.d)
+    dst = torch.zeros_like(src)
+    Q, other = dst[:, rows - l_C:], torch.empty_like(dst)
+    idx, n_sel = torch.zeros(1, cfg.k, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    O = torch.empty(1, l_C, cfg.H, cfg.d, dtype=torch.bfloat16, device="cuda")
+
+    def attend():
+        if call == "two_position":
+            ctx.attend_two_position(Q_sel, Q, K, Kf, V, [t], idx, n_sel, O)
+        elif call == "noalloc":
+            esa.attend_noalloc(ctx.cfg, Q, K, V, [t], idx, n_sel, O)
+        else:
+            ctx.attend(Q, K, V, [t], idx, n_sel, O)
+
+    ctx.select(Q_sel, kc, [t], idx, n_sel, sync=True)
+    ctx.attend(Q_sel, K, V, [t], idx, n_sel, O, sync=True)               # (takes the selection's arming)
+    for _ in range(5):
+        dst.zero_()
+        torch.cuda.synchronize()
+        if call.endswith("armed_by_other_queries"):
+            ctx.select(Q_sel, kc, [t], idx, n_sel)
+        writer.append_kv(src, src, dst, other, [0])
+        attend()
+        torch.cuda.synchronize()
+        got = O.clone()
+        assert torch.equal(Q, src[:, rows - l_C:])
+        attend()
+        torch.cuda.synchronize()
+        assert ctx.last_device_status() == 0
+        assert torch.equal(got, O)
+
+
 @pytest.mark.parametrize("t,l_C", [(3000, 1), (3000, 5), (2944, 128)])
 def test_selected_position_outside_M_is_clamped_and_reported(t, l_C):
     """A stale index buffer must not become a read outside the caches: the position is replaced
