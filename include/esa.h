@@ -231,9 +231,10 @@ esa_status esa_attend_host_kv_async(esa_ctx* ctx, int32_t B, const void* Q_cur, 
  * The partial results of the key-list splits go to a fixed 8 MiB array inside the library
  * image (held on every GPU that loads the library, until the process exits).  A call is
  * refused with ESA_ERR_CAPACITY when the chunk has more than 64 rows per key/value head,
- * or when B * H_G * rows * (head_dim + 2) * 4 floats exceed the array (four splits is the
- * least it will run with); e.g. B = 8, H_G = 8, l_C = 1, H / H_G = 4, head_dim = 128 uses
- * 0.13 MiB per split.  Used fields of cfg: n_q_heads, n_kv_heads, head_dim, l_init,
+ * or when the array has no room for four parts of every row (B * H_G * rows * (head_dim + 2) * 4
+ * floats), whatever the call would use; e.g. B = 8, H_G = 8, l_C = 1, H / H_G = 4, head_dim = 128 uses
+ * 0.13 MiB per split.  (A short key list is split less far; the parts of a split list are joined by
+ * a second launch.)  Used fields of cfg: n_q_heads, n_kv_heads, head_dim, l_init,
  * l_local, top_k, max_tokens, softmax_scale.  All other arguments are as for
  * esa_attend_async; work is only enqueued on `stream`.
  *
@@ -241,11 +242,17 @@ esa_status esa_attend_host_kv_async(esa_ctx* ctx, int32_t B, const void* Q_cur, 
  * the device current and before any stream capture is started on that device.  Host threads
  * may make that first call at the same time (the look-up is serialised inside the library).  Every call
  * on a device shares the one array: calls that may overlap on the GPU (different streams,
- * no ordering between them) race on it and give wrong results; order them.  Nothing in the
- * array has to be cleared between calls -- each call writes every slot it later reads. */
+ * no ordering between them) race on it and give wrong results; order them.  Nothing has to be
+ * cleared between calls -- each call writes every slot it later reads, and keeps nothing else, so
+ * that calls which did overlap leave nothing behind for later ones. */
 esa_status esa_attend_noalloc(const esa_config* cfg, int32_t B, const void* Q_cur, int32_t l_C,
                               const void* K_cache, const void* V_cache, const int64_t* n_prev,
                               const int32_t* idx, const int32_t* n_sel, void* O, void* stream);
+
+/* The counterpart of esa_last_device_status for the calls of esa_attend_noalloc on the current
+ * device, which share one status word: synchronises the stream, then returns ESA_OK or the error that
+ * a kernel recorded since the last read (and clears the record).  ESA_OK before the first call. */
+esa_status esa_attend_noalloc_status(void* stream);
 
 /* Eq. 7: fitting the two compressors.  A trainer holds W_q [d_c, H*d], b_q, W_k [d_c, H_G*d], b_k
  * and their Adam moments on the device (fp32).  One step takes a batch of n query-key pairs

@@ -13,7 +13,9 @@ from .binding import (  # noqa: F401
     library_path,
     STATUS_NAMES,
     attend_noalloc,
+    attend_noalloc_status,
 )
 from .build import build_library  # noqa: F401
 
-__all__ = ["EsaError", "EsaConfig", "Esa", "EsaFit", "load_library", "library_path", "build_library", "STATUS_NAMES", "attend_noalloc"]
+__all__ = ["EsaError", "EsaConfig", "Esa", "EsaFit", "load_library", "library_path", "build_library", "STATUS_NAMES", "attend_noalloc",
+           "attend_noalloc_status"]

@@ -101,6 +101,7 @@ _PROTOS = {
                                            C.c_void_p]),
     "esa_attend_noalloc": (C.c_int, [C.POINTER(_CConfig), C.c_int32, C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p,
                                      C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]),
+    "esa_attend_noalloc_status": (C.c_int, [C.c_void_p]),
     "esa_fit_create": (C.c_int, [C.POINTER(_CConfig), C.c_int32, C.c_float, C.POINTER(C.c_void_p)]),
     "esa_fit_destroy": (C.c_int, [C.c_void_p]),
     "esa_fit_set_weights": (C.c_int, [C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p]),
@@ -351,3 +352,9 @@ def attend_noalloc(cfg: EsaConfig, Q_cur, K_cache, V_cache, n_prev, idx, n_sel, 
     callers that must not allocate once running (see ``include/esa.h``).  Calls on one device
     share that array and must be ordered with respect to each other."""
     load_native().attend_noalloc(cfg, Q_cur, K_cache, V_cache, n_prev, idx, n_sel, O, stream)
+
+
+def attend_noalloc_status(stream=None) -> int:
+    """``esa_attend_noalloc_status``: what the kernels of ``attend_noalloc`` on the current device recorded since
+    the last read (0: nothing)."""
+    return int(load_library().esa_attend_noalloc_status(_stream_ptr(stream)))

@@ -90,3 +90,53 @@ def test_noalloc_rejects_what_does_not_fit():
     with pytest.raises(esa.EsaError) as e:
         esa.attend_noalloc(ec, Q, K, V, [8193], idx, n_sel, torch.empty_like(Q))
     assert e.value.status == 3
+
+
+def test_noalloc_is_independent_of_what_overlapping_calls_left():
+    """Calls that overlap on two streams race on the shared array (their results are not looked at); ordered calls after
+    them, on other inputs, give the bits of the same calls before them."""
+    import paper_2502_14477_b200 as esa
+    cfg = syn.get_config("c4").with_(l_I=16, l_L=1024, k=1024)
+    # a long call that leaves a few SMs to short ones, with unlike numbers of parts
+    shapes = [(32, 6000), (1, 1200)]
+    checks = [_case(cfg, B, t, seed=20 + B) for B, t in shapes]
+
+    def run(case, stream=None):
+        ec, Q, K, V, idx, n_sel, ts = case
+        O = torch.full_like(Q, float("nan"))
+        esa.attend_noalloc(ec, Q, K, V, ts, idx, n_sel, O, stream=stream)
+        return O
+
+    before = []
+    for c in checks:
+        before.append(run(c))
+        torch.cuda.synchronize()
+    long_call, short_call = (_case(cfg, B, t, seed=40 + B) for B, t in shapes)
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    torch.cuda.synchronize()
+    keep = []
+    for _ in range(300):
+        keep.append(run(long_call, streams[0]))
+        for _ in range(8):
+            keep.append(run(short_call, streams[1]))
+    torch.cuda.synchronize()
+    for c, want in zip(checks, before):
+        got = run(c)
+        torch.cuda.synchronize()
+        assert torch.isfinite(want.float()).all() and torch.equal(got, want)
+
+
+@pytest.mark.parametrize("l_C", [1, 8])
+def test_noalloc_status_word(l_C):
+    """A selected position outside M is clamped, recorded, and the record is cleared by reading it."""
+    import paper_2502_14477_b200 as esa
+    cfg = syn.get_config("c3")
+    ec, Q, K, V, idx, n_sel, ts = _case(cfg, 1, 9000, seed=4, l_C=l_C)
+    esa.attend_noalloc(ec, Q, K, V, ts, idx, n_sel, torch.empty_like(Q))
+    assert esa.attend_noalloc_status() == 0
+    idx[0, 7] = 2 ** 30
+    O = torch.full_like(Q, float("nan"))
+    esa.attend_noalloc(ec, Q, K, V, ts, idx, n_sel, O)
+    assert esa.attend_noalloc_status() == 8
+    assert torch.isfinite(O.float()).all()
+    assert esa.attend_noalloc_status() == 0
