@@ -22,7 +22,9 @@
  *     found on the host before anything is launched and leave all outputs untouched.
  *   - "device" pointers are CUDA device memory owned by the caller; "host" pointers are
  *     ordinary host memory read before the call returns.  The library never frees or
- *     reallocates caller memory.  Tensors are dense, row-major, bf16 unless noted.
+ *     reallocates caller memory.  Tensors are dense, row-major, bf16 unless noted, and start on a
+ *     16-byte boundary.  (Some calls read or write a tensor in smaller pieces and take less; a pointer
+ *     that the kernels of a call could not access is refused with ESA_ERR_INVALID_ARG.)
  *   - *_async variants only enqueue work on the given CUDA stream (a cudaStream_t passed
  *     as void*) and return without synchronising.  The plain variants run on the legacy
  *     default stream and return after the work has finished.

@@ -98,7 +98,7 @@ esa_status build_meta(const esa_ctx* ctx, int B, const int64_t* n_prev, int64_t 
     return ESA_OK;
 }
 
-esa_status from_cuda(cudaError_t e) { return e == cudaSuccess ? ESA_OK : ESA_ERR_CUDA; }
+esa_status from_cuda(cudaError_t e) { return e == cudaSuccess ? ESA_OK : e == kErrAlign ? ESA_ERR_INVALID_ARG : ESA_ERR_CUDA; }
 
 // The selection of a step has been enqueued on `st`: the attention call that follows it there with the same queries may
 // start early.
@@ -240,6 +240,7 @@ esa_status esa_append_kv_async(esa_ctx* ctx, int32_t B, const void* K_new, const
         map.row0[b] = (int)n_prev[b];
     }
     if (n_new == 0) return ESA_OK;
+    if (!aligned(K_new, 16) || !aligned(V_new, 16) || !aligned(K_cache, 16) || !aligned(V_cache, 16)) return ESA_ERR_INVALID_ARG;
     return from_cuda(launch_append_kv(ctx, B, (const __nv_bfloat16*)K_new, (const __nv_bfloat16*)V_new, n_new,
                                       (__nv_bfloat16*)K_cache, (__nv_bfloat16*)V_cache, map,
                                       (cudaStream_t)stream));
@@ -268,6 +269,8 @@ esa_status esa_compress_keys_async(esa_ctx* ctx, int32_t B, const void* K_new, i
         map.row0[b] = (int)n_prev[b];
     }
     if (n_new == 0) return ESA_OK;
+    // (a few rows are written value by value, more in groups of four)
+    if (!aligned(K_new, 16) || !aligned(kc_cache, B * n_new <= kCompressGemvRows ? 2 : 8)) return ESA_ERR_INVALID_ARG;
     if (B * n_new <= kCompressGemvRows) {
         cudaError_t e = launch_compress_gemv(ctx, (const __nv_bfloat16*)K_new, B, n_new, ctx->dG, ctx->Wk,
                                              ctx->has_bk ? ctx->bk : nullptr, (__nv_bfloat16*)kc_cache,
@@ -308,11 +311,11 @@ esa_status esa_select_async(esa_ctx* ctx, int32_t B, const void* Q_cur, int32_t 
     if (s != ESA_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
     bool any_small = false, any_large = false;
-    for (int b = 0; b < B; ++b) {
-        int lM = meta.m_end[b] - meta.i_end[b];
-        ctx->last_lM[b] = lM;
-        if (lM > ctx->cfg.top_k) any_large = true; else any_small = true;
-    }
+    for (int b = 0; b < B; ++b)
+        if (meta.m_end[b] - meta.i_end[b] > ctx->cfg.top_k) any_large = true; else any_small = true;
+    if (!aligned(idx_out, 4) || !aligned(n_sel_out, 4)) return ESA_ERR_INVALID_ARG;
+    if (any_large && (!aligned(Q_cur, 16) || !aligned(kc_cache, 16))) return ESA_ERR_INVALID_ARG;
+    for (int b = 0; b < B; ++b) ctx->last_lM[b] = meta.m_end[b] - meta.i_end[b];
     ctx->last_scored = any_large;
     ctx->last_q_rows = any_large ? (int64_t)B * l_C : 0;
     cudaError_t e = cudaSuccess;
@@ -372,11 +375,14 @@ esa_status esa_select_full_async(esa_ctx* ctx, int32_t B, const void* Q_cur, int
     if (s != ESA_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
     bool any_small = false, any_large = false;
-    for (int b = 0; b < B; ++b) {
-        int lM = meta.m_end[b] - meta.i_end[b];
-        ctx->last_lM[b] = lM;
-        if (lM > ctx->cfg.top_k) any_large = true; else any_small = true;
-    }
+    for (int b = 0; b < B; ++b)
+        if (meta.m_end[b] - meta.i_end[b] > ctx->cfg.top_k) any_large = true; else any_small = true;
+    if (!aligned(idx_out, 4) || !aligned(n_sel_out, 4)) return ESA_ERR_INVALID_ARG;
+    // (folded queries are read in words of two values, others by TMA)
+    const bool per_head = mode == ESA_SCORE_PER_HEAD;
+    if (any_large && (!aligned(Q_cur, score_full_folds(ctx, (int64_t)B * l_C, per_head) ? 4 : 16) || !aligned(K_cache, 16)))
+        return ESA_ERR_INVALID_ARG;
+    for (int b = 0; b < B; ++b) ctx->last_lM[b] = meta.m_end[b] - meta.i_end[b];
     ctx->last_scored = any_large;
     ctx->last_q_rows = 0;
     if (any_small && launch_select_all(ctx, B, meta, idx_out, n_sel_out, st) != cudaSuccess) return ESA_ERR_CUDA;
@@ -389,7 +395,7 @@ esa_status esa_select_full_async(esa_ctx* ctx, int32_t B, const void* Q_cur, int
         if (meta.m_end[b] - meta.i_end[b] <= ctx->cfg.top_k) smeta.m_end[b] = smeta.i_end[b];
     ctx->last_decode = false;
     cudaError_t e = launch_score_full(ctx, B, l_C, (const __nv_bfloat16*)Q_cur, (const __nv_bfloat16*)K_cache, smeta, max_lM,
-                                      mode == ESA_SCORE_PER_HEAD, st);
+                                      per_head, st);
     if (e != cudaSuccess) return ESA_ERR_CUDA;
     e = launch_select(ctx, B, false, smeta, max_lM, false, idx_out, n_sel_out, st);
     if (e == cudaSuccess) arm_attention(ctx, st, Q_cur, B, l_C);
@@ -478,6 +484,7 @@ esa_status esa_attend_host_kv_async(esa_ctx* ctx, int32_t B, const void* Q_cur, 
         if (n_att > stage_rows) return ESA_ERR_CAPACITY;
     }
     if (stage_rows >= (int64_t(1) << 31)) return ESA_ERR_CAPACITY;
+    if (!aligned(K_host, 16) || !aligned(V_host, 16) || !aligned(K_stage, 16) || !aligned(V_stage, 16)) return ESA_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     ctx->sel_armed = false;       // (the staged list is written by the gather kernel just ahead: never attended early)
     if (launch_gather_kv(ctx, B, l_C, K_host, V_host, meta, idx, n_sel, K_stage, V_stage, stage_rows, st) != cudaSuccess)

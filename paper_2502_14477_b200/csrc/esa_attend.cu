@@ -391,6 +391,8 @@ static cudaError_t launch_decode_t(esa_ctx* ctx, AttendParams& p, int B, int n_a
     while (nsplit > 1 && (size_t)B * p.HG * nsplit * G * (D + 2) > ctx->att_part_elems) --nsplit;
     if (nsplit < 1) nsplit = 1;
     p.nsplit = nsplit;
+    // the queries are read, and merged rows written, in words of two values
+    if (!aligned(p.Q, 4) || !aligned(p.Qg, 4) || !aligned(p.O, nsplit == 1 ? 2 : 4)) return kErrAlign;
     if (ctx->att_count && (size_t)B * p.HG > ctx->att_count_elems) return cudaErrorInvalidConfiguration;
     p.unit_count = ctx->att_count;
     ProfScope prof(ctx, KC_ATTEND_DECODE, st);
@@ -431,6 +433,7 @@ cudaError_t launch_attend(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, 
     p.top_k = ctx->cfg.top_k; p.nsplit = 1;
     p.scale_log2 = ctx->scale * 1.4426950408889634f;
     p.meta = meta;
+    if (!aligned(p.K, 16) || !aligned(p.Kg, 16) || !aligned(p.V, 16) || !aligned(idx, 4) || !aligned(n_sel, 4)) return kErrAlign;
     int n_att_max = 0;
     for (int b = 0; b < B; ++b) {
         int lM = meta.m_end[b] - meta.i_end[b];
@@ -489,6 +492,7 @@ extern "C" esa_status esa_attend_noalloc(const esa_config* cfg, int32_t B, const
     using namespace esa;
     if (!cfg || !Q_cur || !K_cache || !V_cache || !n_prev || !idx || !n_sel || !O || B <= 0 || l_C <= 0)
         return ESA_ERR_INVALID_ARG;
+    if (!aligned(K_cache, 16) || !aligned(V_cache, 16) || !aligned(idx, 4) || !aligned(n_sel, 4)) return ESA_ERR_INVALID_ARG;
     if (cfg->n_q_heads <= 0 || cfg->n_kv_heads <= 0 || cfg->n_q_heads % cfg->n_kv_heads ||
         (cfg->head_dim != 64 && cfg->head_dim != 128) || cfg->l_init < 0 || cfg->l_local < 0 || cfg->top_k <= 0 ||
         cfg->max_tokens <= 0 || cfg->max_tokens >= (int64_t(1) << 31) || !(cfg->softmax_scale >= 0.f))
@@ -547,7 +551,7 @@ extern "C" esa_status esa_attend_noalloc(const esa_config* cfg, int32_t B, const
     c.status = dev.status;                 // (no arrival counters)
     const cudaError_t e = launch_attend(&c, B, l_C, (const __nv_bfloat16*)Q_cur, nullptr, (const __nv_bfloat16*)K_cache, nullptr,
                                         (const __nv_bfloat16*)V_cache, meta, idx, n_sel, (__nv_bfloat16*)O, (cudaStream_t)stream);
-    return e == cudaSuccess ? ESA_OK : ESA_ERR_CUDA;
+    return e == cudaSuccess ? ESA_OK : e == kErrAlign ? ESA_ERR_INVALID_ARG : ESA_ERR_CUDA;
 }
 
 extern "C" esa_status esa_attend_noalloc_status(void* stream) {

@@ -986,6 +986,11 @@ static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_m
         }
     }
     if (best == 0) return cudaErrorNotSupported;
+    // Finished rows are stored 16 bytes at a time, merged ones four: an O that is not 16-byte aligned is written by the merge
+    // launch, where the scratch holds two parts (always for the small chunks).
+    const bool wide_O = aligned(p.O, 16);
+    if (!aligned(p.Q, 16) || !aligned(p.Qg, 16) || !aligned(p.O, 4)) return kErrAlign;
+    if (!wide_O && best == 1) best = 2;
     p.nsplit = best;
     CUtensorMap qmap, qgmap;
     p.q_tma = make_tensor_map_q(&qmap, p.Q, (uint64_t)B * p.l_C, p.H, D, p.G) ? 1 : 0;
@@ -999,8 +1004,9 @@ static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_m
     if (best == 2 && !uneven && pair_ok < 0)
         pair_ok = launch_tc_kernel<D, TC_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess &&
                   launch_tc_kernel<D, TC_TWO_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess ? 1 : 0;
-    const bool pair = best == 2 && !uneven && pair_ok == 1;
-    if (best == 2 && !pair && (size_t)B * p.HG * 2 * p.Rp * (D + 2) > ctx->att_part_elems) return cudaErrorNotSupported;
+    const bool pair = best == 2 && !uneven && wide_O && pair_ok == 1;
+    if (best == 2 && !pair && (size_t)B * p.HG * 2 * p.Rp * (D + 2) > ctx->att_part_elems)
+        return wide_O ? cudaErrorNotSupported : kErrAlign;
     cudaError_t e;
     {
         ProfScope prof(ctx, KC_ATTEND_TC, st);

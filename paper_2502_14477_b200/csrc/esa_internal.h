@@ -76,6 +76,11 @@ enum KernelClass {
     KC_SCORE_DECODE, KC_SCORE_FULL, KC_POOL, KC_SELECT_TOPK, KC_SELECT_ALL, KC_ATTEND_TC, KC_ATTEND_DECODE,
     KC_ATTEND_MERGE, KC_GATHER_KV, KC_COUNT
 };
+// Alignment of a caller's pointer.  Kernels load and store up to 16 bytes at once; a launch that needs more alignment than
+// its tensors have returns kErrAlign before anything is enqueued (ESA_ERR_INVALID_ARG at the boundary).
+inline bool aligned(const void* p, unsigned bytes) { return (reinterpret_cast<uintptr_t>(p) & (bytes - 1)) == 0; }
+constexpr cudaError_t kErrAlign = cudaErrorInvalidDevicePointer;      // (no longer returned by the runtime itself)
+
 struct ProfRec {
     int cls;
     cudaEvent_t a, b;
@@ -213,6 +218,9 @@ cudaError_t launch_score_full(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16*
 // (only_small = 1) or all sequences (only_small = 0).
 cudaError_t launch_select_all(esa_ctx* ctx, int B, const SeqMeta& meta, int32_t* idx_out,
                               int32_t* n_sel_out, cudaStream_t st);
+
+// True when the full-dimension scoring adds the queries of a group up first (see esa_score_full.cu).
+bool score_full_folds(const esa_ctx* ctx, int64_t rows, bool per_head);
 
 // Qg / Kg: queries and key cache used against I and M_k (two-position attention, Section 3.2); null = Q / K.
 // cache_rows: rows per sequence of the K/V caches handed in (0 = the configuration's max_tokens).

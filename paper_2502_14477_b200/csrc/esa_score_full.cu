@@ -294,15 +294,19 @@ cudaError_t launch_pass(esa_ctx* ctx, FullTcParams p, const FullTile& t, const C
 
 }  // namespace
 
+// The folded queries go to the attention's scratch (written and read within the attention kernel, idle here).
+// Three pieces beat the heads of a group from four heads on.
+bool score_full_folds(const esa_ctx* ctx, int64_t rows, bool per_head) {
+    return !per_head && ctx->G > 3 && (size_t)rows * 3 * ctx->dG * 2 <= ctx->att_part_elems * sizeof(float);
+}
+
 // Fills ctx->skey with the unpooled full-dimension scores (ordered keys).
 // The keys of M may be loaded ahead of a pass's wait for the kernel before it: everything enqueued ahead of the call
 // has completed when the first launch below lets its dependents start, and M ends before the current chunk.
 cudaError_t launch_score_full(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* K, const SeqMeta& meta,
                               int max_lM, bool per_head, cudaStream_t st) {
     const int64_t rows = (int64_t)B * l_C;
-    // The folded queries go to the attention's scratch (written and read within the attention kernel, idle here).
-    // Three pieces beat the heads of a group from four heads on.
-    const bool fold = !per_head && ctx->G > 3 && (size_t)rows * 3 * ctx->dG * 2 <= ctx->att_part_elems * sizeof(float);
+    const bool fold = score_full_folds(ctx, rows, per_head);
     __nv_bfloat16* Qf = reinterpret_cast<__nv_bfloat16*>(ctx->att_part);
     const int64_t n_rkey = rows * (per_head ? ctx->H : 1);
     int gx = (int)((rows * (fold ? ctx->dG / 2 : 0) + (int64_t)B * max_lM + 511) / 512);

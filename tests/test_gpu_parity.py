@@ -1021,3 +1021,87 @@ def test_argument_errors_leave_outputs_untouched():
         esa.Esa(esa.EsaConfig(cfg.H, cfg.H_G, cfg.d, cfg.d_c, 4, 512, 256, 16, 128, 1, 1024))
     assert e.value.status == 2
     esa.Esa(esa.EsaConfig(cfg.H, cfg.H_G, cfg.d, cfg.d_c, 4, 512, 256, 15, 128, 1, 1024))
+
+
+def _offset(t, elements):
+    """A contiguous copy of t that starts `elements` values behind an allocation's (aligned) start."""
+    flat = torch.empty(t.numel() + elements, dtype=t.dtype, device=t.device)
+    out = flat[elements:].view(t.shape)
+    out.copy_(t)
+    return out
+
+
+def test_misaligned_tensors_are_refused_or_handled():
+    """Contiguous views that do not start on a 16-byte boundary: refused with an error, outputs untouched, where the kernels of the
+    call could not access them; the same results as from aligned tensors where they can."""
+    import paper_2502_14477_b200 as esa
+    cfg = syn.get_config("c1")
+    t, n = 3000, 3200
+    ctx = hp.make_esa(cfg, max_tokens=n, max_chunk=1000, max_batch=1)
+    seq = hp.DeviceSeq(cfg, max_tokens=n, B=1)
+    seq.fill_kv(0, n)
+    fill_kc_gpu(ctx, seq, t, step=1000)
+    Q = hp.bits_to_torch(syn.qkv_rows(cfg, "q", t, t + 128))[None].contiguous()
+    q1, q5, q3 = (Q[:, :m].contiguous() for m in (1, 5, 3))
+    k5, k40 = seq.K[:, t:t + 5].contiguous(), seq.K[:, t:t + 40].contiguous()
+    idx, n_sel = seq.idx, seq.n_sel
+
+    def refused(f, *outs):
+        held = [o.clone() for o in outs]
+        with pytest.raises(esa.EsaError) as e:
+            f()
+        assert e.value.status == 1
+        torch.cuda.synchronize()
+        for a, b in zip(held, outs):
+            assert torch.equal(a, b)
+
+    K, V = seq.K.clone(), seq.V.clone()
+    refused(lambda: ctx.append_kv(_offset(k5, 1), k5, K, V, [t]), K, V)
+    refused(lambda: ctx.append_kv(k5, _offset(k5, 4), K, V, [t]), K, V)
+    refused(lambda: ctx.append_kv(k5, k5, _offset(K, 2), V, [t]), V)
+    refused(lambda: ctx.compress_keys(_offset(k5, 2), seq.Kc, [t]), seq.Kc)
+    refused(lambda: ctx.compress_keys(k40, _offset(seq.Kc, 2), [t]))
+    for q in (q1, q5, Q):
+        refused(lambda: ctx.select(_offset(q, 4), seq.Kc, [t], idx, n_sel), idx, n_sel)
+        refused(lambda: ctx.select(q, _offset(seq.Kc, 4), [t], idx, n_sel), idx, n_sel)
+        refused(lambda: ctx.select_full(q, _offset(seq.K, 4), [t], idx, n_sel), idx, n_sel)
+        refused(lambda: ctx.select_full(_offset(q, 1), seq.K, [t], idx, n_sel), idx, n_sel)
+        refused(lambda: ctx.select_full(_offset(q, 2), seq.K, [t], idx, n_sel, per_head=True), idx, n_sel)
+    ctx.select(Q, seq.Kc, [t], idx, n_sel, sync=True)
+    for q in (q1, q5, Q):
+        O = torch.zeros_like(q)
+        refused(lambda: ctx.attend(q, _offset(seq.K, 4), seq.V, [t], idx, n_sel, O), O)
+        refused(lambda: ctx.attend(q, seq.K, _offset(seq.V, 2), [t], idx, n_sel, O), O)
+        refused(lambda: ctx.attend(_offset(q, 1), seq.K, seq.V, [t], idx, n_sel, O), O)
+        refused(lambda: ctx.attend_two_position(q, _offset(q, 1), seq.K, seq.K, seq.V, [t], idx, n_sel, O), O)
+        odd = _offset(O, 1)
+        refused(lambda: ctx.attend(q, seq.K, seq.V, [t], idx, n_sel, odd), odd)
+        if q is not q1:
+            refused(lambda: ctx.attend(_offset(q, 4), seq.K, seq.V, [t], idx, n_sel, O), O)
+    stage = torch.zeros(1, cfg.l_I + cfg.k + cfg.l_L + 1, cfg.H_G, cfg.d, dtype=torch.bfloat16, device="cuda")
+    Kh, Vh = seq.K.cpu().pin_memory(), seq.V.cpu().pin_memory()
+    O = torch.zeros_like(q1)
+    refused(lambda: ctx.attend_host_kv(q1, Kh, Vh, [t], idx, n_sel, _offset(stage, 2), stage, O), O)
+
+    # accepted: queries of a single-query call in words of two values, merged rows on such boundaries (lists of any length), a
+    # few compressed rows anywhere, queries that are folded
+    none = torch.zeros_like(n_sel)
+    for q, off_q, off_o in ((q1, 2, 2), (q3, 0, 2), (q5, 0, 4), (q5, 0, 6), (Q, 0, 2)):
+        want, got = torch.empty_like(q), _offset(torch.zeros_like(q), off_o)
+        for tt, ns in ((t, n_sel), (20, none)):
+            ctx.attend(q, seq.K, seq.V, [tt], idx, ns, want, sync=True)
+            ctx.attend(_offset(q, off_q), seq.K, seq.V, [tt], idx, ns, got, sync=True)
+            hp.check_attention(got[0], hp.torch_to_f64(want[0]), what=f"{q.shape[1]} queries after {tt}, output {2 * off_o} bytes off")
+    want, got = torch.empty_like(q1), _offset(torch.zeros_like(q1), 1)
+    ctx.attend(q1, seq.K, seq.V, [20], idx, none, want, sync=True)
+    ctx.attend(q1, seq.K, seq.V, [20], idx, none, got, sync=True)
+    assert torch.equal(got, want)
+    kc = _offset(torch.zeros_like(seq.Kc), 1)
+    ctx.compress_keys(k5, kc, [t], sync=True)
+    ctx.compress_keys(k5, seq.Kc, [t], sync=True)
+    assert torch.equal(kc[:, t:t + 5], seq.Kc[:, t:t + 5])
+    full, folded = torch.zeros_like(idx), torch.zeros_like(idx)
+    ctx.select_full(Q, seq.K, [t], full, n_sel, sync=True)
+    ctx.select_full(_offset(Q, 2), seq.K, [t], folded, n_sel, sync=True)
+    assert torch.equal(full, folded)
+    assert ctx.last_device_status() == 0

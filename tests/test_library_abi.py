@@ -67,6 +67,16 @@ def test_null_handles_are_rejected(lib):
     assert lib.esa_create(C.byref(bad), C.byref(h)) == 2 and not h.value
 
 
+def test_misaligned_caches_are_refused_before_the_device_is_asked(lib):
+    import paper_2502_14477_b200 as esa
+    cfg = esa.EsaConfig(8, 2, 64, 32, 4, 512, 256, 3, 8, 1, 4096).to_c()
+    n_prev = (C.c_int64 * 1)(3000)
+    good = 1 << 20                                     # (addresses are only looked at)
+    for K, V, idx, n_sel in ((good + 2, good, good, good), (good, good + 8, good, good), (good, good, good + 2, good),
+                             (good, good, good, good + 1)):
+        assert lib.esa_attend_noalloc(C.byref(cfg), 1, good, 1, K, V, n_prev, idx, n_sel, good, None) == 1
+
+
 @pytest.mark.skipif(torch.cuda.is_available(), reason="checks the no-device error path")
 def test_create_without_a_device_reports_cuda_error(lib):
     import paper_2502_14477_b200 as esa
