@@ -539,7 +539,7 @@ int32_t esa_kernel_class_count(void) { return KC_COUNT; }
 const char* esa_kernel_class_name(int32_t cls) {
     static const char* names[KC_COUNT] = {
         "compress_tc_kernel", "compress_gemv_kernel", "compress_kernel", "append_kv_kernel", "score_tc_kernel<.,1>",
-        "score_tc_kernel<.,2>", "score_pass_kernel<.,1>+<.,2>", "score_decode_kernel", "score_full_kernel<.,1>+<.,2>",
+        "score_tc_kernel<.,2>", "score_decode_kernel", "score_full_kernel<.,1>+<.,2>",
         "pool_kernel",
         "select_topk_kernel", "select_all_kernel", "attend_tc_kernel", "attend_decode_kernel",
         "attend_tc_merge_kernel", "gather_kv_kernel"};

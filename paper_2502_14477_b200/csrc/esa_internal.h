@@ -72,7 +72,7 @@ struct RowMap {
 
 // Kernel classes of the per-kernel timing facility (esa_set_profiling / esa_read_profile).
 enum KernelClass {
-    KC_COMPRESS_TC = 0, KC_COMPRESS_GEMV, KC_COMPRESS_MMA, KC_APPEND_KV, KC_SCORE_PASS1, KC_SCORE_PASS2, KC_SCORE_MMA,
+    KC_COMPRESS_TC = 0, KC_COMPRESS_GEMV, KC_COMPRESS_MMA, KC_APPEND_KV, KC_SCORE_PASS1, KC_SCORE_PASS2,
     KC_SCORE_DECODE, KC_SCORE_FULL, KC_POOL, KC_SELECT_TOPK, KC_SELECT_ALL, KC_ATTEND_TC, KC_ATTEND_DECODE,
     KC_ATTEND_MERGE, KC_GATHER_KV, KC_COUNT
 };
@@ -91,18 +91,20 @@ struct ProfRec {
 // or refuses the shape.
 bool make_tensor_map_bf16(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
 
-// A descriptor kept with the matrix it was made for (column count and box never change for one user of it).
+// The same for a cache [B, rows, cols] with the sequence as third coordinate: a coordinate stays within a sequence (rows of
+// all sequences together may be too many for one), and rows past a sequence's end read as zeros.
+bool make_tensor_map_cache(CUtensorMap* map, const void* base, uint64_t B, uint64_t rows, uint64_t cols, uint32_t box_rows);
+
+// A descriptor kept with the matrix it was made for (all but base and outer extent never change for one user of it).
 struct CachedMap {
     CUtensorMap map;
     const void* base = nullptr;
-    uint64_t rows = 0;
-    bool matches(const void* b, uint64_t r) const { return base == b && rows == r; }
-    bool encode(const void* b, uint64_t r, uint64_t cols, uint32_t box_rows) {
-        base = nullptr;
-        if (!make_tensor_map_bf16(&map, b, r, cols, box_rows)) return false;
-        base = b;
-        rows = r;
-        return true;
+    uint64_t extent = 0;
+    bool matches(const void* b, uint64_t n) const { return base == b && extent == n; }
+    bool keep(const void* b, uint64_t n, bool encoded) {
+        base = encoded ? b : nullptr;
+        extent = n;
+        return encoded;
     }
 };
 
@@ -196,8 +198,10 @@ cudaError_t launch_compress(esa_ctx* ctx, const __nv_bfloat16* X, int B, int row
 cudaError_t launch_score(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache,
                          const SeqMeta& meta, int max_lM, bool rkey_cleared, cudaStream_t st, bool* pooled_ready);
 
-// The same on tcgen05 with TMA-fed tiles; expects
-// ctx->rkey zeroed (pass 1 clears what pass 2 accumulates into).  cudaErrorNotSupported when the shape is not covered.
+// Two queries and more, on tcgen05 with TMA-fed tiles; expects ctx->rkey zeroed (pass 1 clears what pass 2 accumulates into).
+// For a handful of queries most of a 128-row tile is padding, but the passes are bound by the stream of keys and their own
+// latency, and pooling comes with the second pass: 37 queries after 50021 tokens, select 51 -> 27.4 us against mma.sync
+// kernels with their memsets and pooling launch.
 cudaError_t launch_score_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache,
                             const SeqMeta& meta, int max_lM, cudaStream_t st, bool* pooled_ready);
 
@@ -261,12 +265,6 @@ cudaError_t launch_compress_tc(esa_ctx* ctx, const __nv_bfloat16* X, int B, int 
                                const CUtensorMap* wmap, const float* bias, __nv_bfloat16* dst,
                                int64_t dst_seq_stride, const RowMap& map, uint32_t* zero_words, int zero_count,
                                cudaStream_t st, bool small_grid = false);
-
-// True when launch_score takes the tcgen05 path for this call: every chunk (row numbers are 32-bit TMA coordinates).
-// For a handful of queries most of a 128-row tile is padding, but the passes are bound by the stream of keys and their
-// own latency, and pooling comes with the second pass: 37 queries after 50021 tokens, select
-// 51 -> 32 us against the mma.sync kernels with their memsets and pooling launch.
-inline bool score_uses_tc(const esa_ctx* ctx, int B) { return (int64_t)B * ctx->cfg.max_tokens < (int64_t(1) << 31); }
 
 cudaError_t launch_append_kv(esa_ctx* ctx, int B, const __nv_bfloat16* K_new,
                              const __nv_bfloat16* V_new, int n_new, __nv_bfloat16* K_cache,

@@ -100,7 +100,7 @@ score_full_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
         if (lane == 0 && work) {
             tma_prefetch_desc(&kmap);
             tma_prefetch_desc(&qmap);
-            const int krow = (int)((int64_t)b * p.max_tokens + i_end) + key0, qrow = b * p.l_C + q0;
+            const int krow = i_end + key0, qrow = b * p.l_C + q0;
             const int k_box = min(128, key_rows), q_box = min(128, q_rows);
             int qi = 0;
             // the queries may come from the preceding kernel; the keys are older (see launch_score_full)
@@ -110,7 +110,7 @@ score_full_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_cons
                 mbar_wait(bar(FB_K_EMPTY + s), ((i / p.k_slots) & 1) ^ 1, wc);
                 mbar_arrive_expect_tx(bar(FB_K_FULL + s), k_bytes);
                 for (int r = 0; r < key_rows; r += k_box)
-                    tma_load_2d(smem_u32(sK + s * k_bytes + r * 128), &kmap, i * 64, krow + r, bar(FB_K_FULL + s));
+                    tma_load_3d(smem_u32(sK + s * k_bytes + r * 128), &kmap, i * 64, krow + r, b, bar(FB_K_FULL + s));
                 if (!waited) {
                     pdl_wait();
                     waited = true;
@@ -327,11 +327,11 @@ cudaError_t launch_score_full(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16*
     const FullTile t1 = pick_tile(1, l_C, max_lM, B, p.k_chunks, p.pieces, ctx->num_sms);
     const FullTile t2 = pick_tile(2, l_C, max_lM, B, p.k_chunks, p.pieces, ctx->num_sms);
     const __nv_bfloat16* qbase = fold ? Qf : Q;
-    const uint64_t qcols = fold ? 3 * (uint64_t)ctx->dG : (uint64_t)ctx->dH, krows = (uint64_t)B * ctx->cfg.max_tokens;
+    const uint64_t qcols = fold ? 3 * (uint64_t)ctx->dG : (uint64_t)ctx->dH, krows = ctx->cfg.max_tokens;
     CUtensorMap k1, q1, k2, q2;
     auto box = [](int r) { return (uint32_t)(r < 128 ? r : 128); };
-    if (!make_tensor_map_bf16(&k1, K, krows, ctx->dG, box(t1.key_rows)) || !make_tensor_map_bf16(&q1, qbase, rows, qcols, box(t1.q_rows)) ||
-        !make_tensor_map_bf16(&k2, K, krows, ctx->dG, box(t2.key_rows)) || !make_tensor_map_bf16(&q2, qbase, rows, qcols, box(t2.q_rows)))
+    if (!make_tensor_map_cache(&k1, K, B, krows, ctx->dG, box(t1.key_rows)) || !make_tensor_map_bf16(&q1, qbase, rows, qcols, box(t1.q_rows)) ||
+        !make_tensor_map_cache(&k2, K, B, krows, ctx->dG, box(t2.key_rows)) || !make_tensor_map_bf16(&q2, qbase, rows, qcols, box(t2.q_rows)))
         return cudaErrorInvalidValue;
     e = launch_pass<1>(ctx, p, t1, k1, q1, B, max_lM, st);
     if (e == cudaSuccess) e = launch_pass<2>(ctx, p, t2, k2, q2, B, max_lM, st);

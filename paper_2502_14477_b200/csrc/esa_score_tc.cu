@@ -213,15 +213,14 @@ score_tc_kernel(const __grid_constant__ CUtensorMap kmap, const __grid_constant_
         if (lane == 0 && n_items > 0) {
             tma_prefetch_desc(&kmap);
             tma_prefetch_desc(&qmap);
-            const int64_t row_base = (int64_t)b * p.max_tokens + i_end;
             auto load_tile = [&](int lt) {
                 const int s = lt % STAGES;
                 mbar_wait(bar(C::B_EMPTY + s), ((lt / STAGES) & 1) ^ 1, wc);
                 mbar_arrive_expect_tx(bar(C::B_FULL + s), TILE_BYTES);
 #pragma unroll
                 for (int blk = 0; blk < NBLK; ++blk)
-                    tma_load_2d(smem_u32(sK + s * TILE_BYTES + blk * (ST_KEYS * 128)), &kmap, kx + blk * 64,
-                                (int)(row_base + key_first + (int64_t)lt * ST_KEYS), bar(C::B_FULL + s));
+                    tma_load_3d(smem_u32(sK + s * TILE_BYTES + blk * (ST_KEYS * 128)), &kmap, kx + blk * 64,
+                                i_end + key_first + lt * ST_KEYS, b, bar(C::B_FULL + s));
             };
             const int first = min(n_ltiles, STAGES);
             for (int lt = 0; lt < first; ++lt) load_tile(lt);
@@ -503,19 +502,21 @@ cudaError_t launch_t(esa_ctx* ctx, int B, int l_C, const CUtensorMap& kmap, cons
 
 // Both scoring passes; rkey must be zeroed.  d' = 32 runs as 64 with the upper half of every row read as zeros.
 // *pooled_ready: ctx->pkey holds the pooled keys (else ctx->skey holds the unpooled ones).
-// Returns cudaErrorNotSupported when this path does not cover the shape.
 cudaError_t launch_score_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* kc_cache, const SeqMeta& meta,
                             int max_lM, cudaStream_t st, bool* pooled_ready) {
     // the descriptors of the last call serve again while the caller keeps its cache and chunk size
-    const uint64_t k_rows = (uint64_t)B * ctx->cfg.max_tokens, q_rows = (uint64_t)B * l_C;
-    if (!ctx->kc_map.matches(kc_cache, k_rows) && !ctx->kc_map.encode(kc_cache, k_rows, ctx->dc, ST_KEYS)) return cudaErrorNotSupported;
-    if (!ctx->qc_map.matches(ctx->Qc, q_rows) && !ctx->qc_map.encode(ctx->Qc, q_rows, ctx->dc, 128)) return cudaErrorNotSupported;
+    const uint64_t q_rows = (uint64_t)B * l_C;
+    CachedMap &k = ctx->kc_map, &q = ctx->qc_map;
+    if (!k.matches(kc_cache, B) && !k.keep(kc_cache, B, make_tensor_map_cache(&k.map, kc_cache, B, ctx->cfg.max_tokens, ctx->dc, ST_KEYS)))
+        return cudaErrorInvalidValue;
+    if (!q.matches(ctx->Qc, q_rows) && !q.keep(ctx->Qc, q_rows, make_tensor_map_bf16(&q.map, ctx->Qc, q_rows, ctx->dc, 128)))
+        return cudaErrorInvalidValue;
     ScoreTcParams p;
     p.rkey = ctx->rkey;
     p.groups = (l_C + ST_QCAP - 1) / ST_QCAP; p.heads = 1; p.G = 1; p.pool = p.groups == 1 ? 1 : 0;
     *pooled_ready = p.pool != 0;
-    return ctx->dc == 128 ? launch_t<128>(ctx, B, l_C, ctx->kc_map.map, ctx->qc_map.map, p, meta, max_lM, st)
-                          : launch_t<64>(ctx, B, l_C, ctx->kc_map.map, ctx->qc_map.map, p, meta, max_lM, st);
+    return ctx->dc == 128 ? launch_t<128>(ctx, B, l_C, k.map, q.map, p, meta, max_lM, st)
+                          : launch_t<64>(ctx, B, l_C, k.map, q.map, p, meta, max_lM, st);
 }
 
 // The per-head vote: every head's own scores (uncompressed queries and keys), the maximum over the heads in ctx->skey,
@@ -523,7 +524,7 @@ cudaError_t launch_score_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* k
 cudaError_t launch_score_tc_heads(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* K, const SeqMeta& meta,
                                   int max_lM, cudaStream_t st) {
     CUtensorMap kmap, qmap;
-    if (!make_tensor_map_bf16(&kmap, K, (uint64_t)B * ctx->cfg.max_tokens, ctx->dG, ST_KEYS) ||
+    if (!make_tensor_map_cache(&kmap, K, B, ctx->cfg.max_tokens, ctx->dG, ST_KEYS) ||
         !make_tensor_map_bf16(&qmap, Q, (uint64_t)B * l_C, ctx->dH, 128))
         return cudaErrorInvalidValue;
     ScoreTcParams p;
