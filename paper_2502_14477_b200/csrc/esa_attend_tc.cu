@@ -884,13 +884,13 @@ static cudaError_t launch_tc_kernel(esa_ctx* ctx, const CUtensorMap& qmap, const
     cudaError_t e = allow_smem(attend_tc_kernel<D, MODE, NQT, FINE>, ctx->device, smem, memo);
     if (e != cudaSuccess) return e;
     // the in-kernel register split assumes the launch allocation it was sized for
-    static int regs_checked = 0;
-    if (!regs_checked) {
+    static std::atomic<bool> regs_checked{false};
+    if (!regs_checked.load(std::memory_order_relaxed)) {
         cudaFuncAttributes fa;
         e = cudaFuncGetAttributes(&fa, attend_tc_kernel<D, MODE, NQT, FINE>);
         if (e != cudaSuccess) return e;
         if (fa.numRegs != TC_REGS_LAUNCH) return cudaErrorInvalidConfiguration;
-        regs_checked = 1;
+        regs_checked.store(true, std::memory_order_relaxed);
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -999,12 +999,16 @@ static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_m
     if (!p.q_tma || !p.two) memset(&qgmap, 0, sizeof(qgmap));
     const dim3 grid(row_tiles, p.HG, B * best);
     // a two-way split runs as CTA pairs that merge through distributed shared memory, where the device can place pairs
-    static int pair_ok = -1;                                 // per instantiation; probed once
+    static std::atomic<int> pair_ok[64];                     // per instantiation and device: 0 not asked yet, 1 yes, 2 no
+    std::atomic<int>& ok = pair_ok[ctx->device & 63];
     const bool uneven = p.main_tiles > 0;
-    if (best == 2 && !uneven && pair_ok < 0)
-        pair_ok = launch_tc_kernel<D, TC_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess &&
-                  launch_tc_kernel<D, TC_TWO_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess ? 1 : 0;
-    const bool pair = best == 2 && !uneven && wide_O && pair_ok == 1;
+    if (best == 2 && !uneven && ok.load(std::memory_order_relaxed) == 0) {
+        const bool yes = launch_tc_kernel<D, TC_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess &&
+                         launch_tc_kernel<D, TC_TWO_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess;
+        if (!yes) cudaGetLastError();
+        ok.store(yes ? 1 : 2, std::memory_order_relaxed);
+    }
+    const bool pair = best == 2 && !uneven && wide_O && ok.load(std::memory_order_relaxed) == 1;
     if (best == 2 && !pair && (size_t)B * p.HG * 2 * p.Rp * (D + 2) > ctx->att_part_elems)
         return wide_O ? cudaErrorNotSupported : kErrAlign;
     cudaError_t e;

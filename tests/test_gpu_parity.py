@@ -1023,6 +1023,48 @@ def test_argument_errors_leave_outputs_untouched():
     esa.Esa(esa.EsaConfig(cfg.H, cfg.H_G, cfg.d, cfg.d_c, 4, 512, 256, 15, 128, 1, 1024))
 
 
+_THREADS = """
+import threading, torch
+import paper_2502_14477_b200 as esa
+H, HG, d, dc, t, l_C, k = 32, 8, 128, 128, 6000, 300, 1024
+g = torch.Generator(device="cuda").manual_seed(1)
+draw = lambda *s: torch.randn(*s, device="cuda", dtype=torch.bfloat16, generator=g)
+Q, K, V, Kc = draw(1, l_C, H, d), draw(1, t + l_C, HG, d), draw(1, t + l_C, HG, d), draw(1, t + l_C, dc)
+wq, wk = torch.randn(dc, H * d).numpy() / 64, torch.randn(dc, HG * d).numpy() / 32
+torch.cuda.synchronize()
+n, outs, gate = 8, [None] * 8, threading.Barrier(8)
+def work(i):
+    ctx, stream = esa.Esa(esa.EsaConfig(H, HG, d, dc, 16, 512, k, 3, l_C, 1, t + l_C)), torch.cuda.Stream()
+    ctx.set_compressors(wq, None, wk, None)
+    idx, n_sel = torch.zeros(1, k, dtype=torch.int32, device="cuda"), torch.zeros(1, dtype=torch.int32, device="cuda")
+    O = torch.zeros_like(Q)
+    torch.cuda.synchronize()
+    gate.wait()
+    ctx.select(Q, Kc, [t], idx, n_sel, stream=stream)
+    ctx.attend(Q, K, V, [t], idx, n_sel, O, stream=stream)
+    stream.synchronize()
+    assert ctx.last_device_status(stream) == 0
+    outs[i] = (O, idx)
+threads = [threading.Thread(target=work, args=(i,)) for i in range(n)]
+for x in threads: x.start()
+for x in threads: x.join()
+assert all(torch.equal(outs[0][0], o) and torch.equal(outs[0][1], i) for o, i in outs)
+print("threads agree")
+"""
+
+
+def test_first_calls_of_several_threads_together():
+    """Host threads with a context and a stream each make the first calls of a process at the same time: what the library asks of
+    the driver once per process or device is asked once, and every thread gets the same results."""
+    import os
+    import subprocess
+    import sys
+    for _ in range(2):
+        res = subprocess.run([sys.executable, "-c", _THREADS], cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                             capture_output=True, text=True, timeout=300)
+        assert res.returncode == 0 and "threads agree" in res.stdout, res.stderr[-2000:]
+
+
 def _offset(t, elements):
     """A contiguous copy of t that starts `elements` values behind an allocation's (aligned) start."""
     flat = torch.empty(t.numel() + elements, dtype=t.dtype, device=t.device)
