@@ -9,7 +9,10 @@
 #include <Python.h>
 
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
+
+#include <new>
 
 #include "../../include/esa.h"
 
@@ -140,12 +143,7 @@ bool read_n_prev(PyObject* o, int64_t B, NPrev* out) {
 // stream: None (torch's current stream), an integer handle, or an object with a cuda_stream attribute
 bool read_stream(PyObject* o, void** out) {
     if (o == Py_None) {
-        try {
-            *out = (void*)c10::cuda::getCurrentCUDAStream().stream();
-        } catch (const std::exception& e) {
-            PyErr_SetString(PyExc_RuntimeError, e.what());
-            return false;
-        }
+        *out = (void*)c10::cuda::getCurrentCUDAStream().stream();
         return true;
     }
     PyObject* v = PyLong_Check(o) ? Py_NewRef(o) : PyObject_GetAttrString(o, "cuda_stream");
@@ -179,10 +177,16 @@ bool want_args(Py_ssize_t got, Py_ssize_t want, const char* name) {
 // Runs a library call without the interpreter lock (it may wait for the device, or for room in the launch queue).
 template <typename F>
 PyObject* finish(const char* name, F call) {
-    esa_status st;
+    esa_status st = ESA_OK;
+    bool threw = false;
     Py_BEGIN_ALLOW_THREADS
-    st = call();
+    try {
+        st = call();
+    } catch (...) {                 // (the library throws nothing but what its allocations on the host throw)
+        threw = true;
+    }
     Py_END_ALLOW_THREADS
+    if (threw) return PyErr_NoMemory();
     if (st != ESA_OK) {
         raise_status(st, name);
         return nullptr;
@@ -314,14 +318,7 @@ PyObject* ctx_attend_two_position(CtxObject* self, PyObject* const* a, Py_ssize_
 bool pinned_ptr(PyObject* o, const char* name, std::initializer_list<int64_t> shape, void** out) {
     const at::Tensor* t = as_tensor(o, name);
     if (!t) return false;
-    bool pinned = false;
-    try {
-        pinned = !t->is_cuda() && t->is_pinned();
-    } catch (const std::exception& e) {
-        PyErr_SetString(PyExc_RuntimeError, e.what());
-        return false;
-    }
-    if (!pinned) {
+    if (t->is_cuda() || !t->is_pinned()) {
         PyErr_Format(PyExc_TypeError, "%s must be a pinned host tensor", name);
         return false;
     }
@@ -440,21 +437,42 @@ PyObject* obj_drop(PyObject* self, PyObject*) {
     Py_RETURN_NONE;
 }
 
-#define ESA_FAST(f) reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(f))
+// A C++ exception must not leave a function that the interpreter has called (it would end the process).  torch throws where
+// a tensor has no plain storage, sizes or layout to ask for -- sparse, fake, or wrapped by a transformation: these become the
+// errors that its own Python methods raise.
+template <typename Self, PyObject* (*F)(Self*, PyObject* const*, Py_ssize_t)>
+PyObject* entry(PyObject* self, PyObject* const* a, Py_ssize_t n) {
+    try {
+        return F(reinterpret_cast<Self*>(self), a, n);
+    } catch (python_error& e) {
+        e.restore();
+    } catch (const c10::NotImplementedError& e) {
+        PyErr_SetString(PyExc_NotImplementedError, e.what_without_backtrace());
+    } catch (const c10::Error& e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what_without_backtrace());
+    } catch (const std::bad_alloc&) {
+        PyErr_NoMemory();
+    } catch (const std::exception& e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what());
+    }
+    return nullptr;
+}
+
+#define ESA_FAST(...) reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)(void)>(entry<__VA_ARGS__>))
 
 PyMethodDef ctx_methods[] = {
-    {"append_kv", ESA_FAST(ctx_append_kv), METH_FASTCALL, nullptr},
-    {"compress_keys", ESA_FAST(ctx_compress_keys), METH_FASTCALL, nullptr},
-    {"select", ESA_FAST(ctx_select), METH_FASTCALL, nullptr},
-    {"select_full", ESA_FAST(ctx_select_full), METH_FASTCALL, nullptr},
-    {"attend", ESA_FAST(ctx_attend), METH_FASTCALL, nullptr},
-    {"attend_two_position", ESA_FAST(ctx_attend_two_position), METH_FASTCALL, nullptr},
-    {"attend_host_kv", ESA_FAST(ctx_attend_host_kv), METH_FASTCALL, nullptr},
+    {"append_kv", ESA_FAST(CtxObject, ctx_append_kv), METH_FASTCALL, nullptr},
+    {"compress_keys", ESA_FAST(CtxObject, ctx_compress_keys), METH_FASTCALL, nullptr},
+    {"select", ESA_FAST(CtxObject, ctx_select), METH_FASTCALL, nullptr},
+    {"select_full", ESA_FAST(CtxObject, ctx_select_full), METH_FASTCALL, nullptr},
+    {"attend", ESA_FAST(CtxObject, ctx_attend), METH_FASTCALL, nullptr},
+    {"attend_two_position", ESA_FAST(CtxObject, ctx_attend_two_position), METH_FASTCALL, nullptr},
+    {"attend_host_kv", ESA_FAST(CtxObject, ctx_attend_host_kv), METH_FASTCALL, nullptr},
     {"drop", obj_drop<CtxObject>, METH_NOARGS, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 
 PyMethodDef fit_methods[] = {
-    {"step", ESA_FAST(fit_step), METH_FASTCALL, nullptr},
+    {"step", ESA_FAST(FitObject, fit_step), METH_FASTCALL, nullptr},
     {"drop", obj_drop<FitObject>, METH_NOARGS, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 
@@ -471,7 +489,7 @@ PyObject* mod_set_error(PyObject*, PyObject* cls) {
 }
 
 PyMethodDef mod_methods[] = {
-    {"attend_noalloc", ESA_FAST(mod_attend_noalloc), METH_FASTCALL, nullptr},
+    {"attend_noalloc", ESA_FAST(PyObject, mod_attend_noalloc), METH_FASTCALL, nullptr},
     {"set_error", mod_set_error, METH_O, nullptr},
     {nullptr, nullptr, 0, nullptr}};
 

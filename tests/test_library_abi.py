@@ -91,3 +91,48 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(binding, "LIB_PATH", str(tmp_path / "nope.so"))
     with pytest.raises(RuntimeError, match="no CPU or PyTorch fallback"):
         binding.load_library()
+
+
+_WRAPPERS = """
+import torch
+import paper_2502_14477_b200 as esa
+from paper_2502_14477_b200 import binding
+
+class Wrapper(torch.Tensor):
+    @classmethod
+    def __torch_dispatch__(cls, func, types, args=(), kwargs=None):
+        raise ValueError("asked " + str(func))
+
+def z(*shape, dtype=torch.bfloat16):
+    # a CUDA tensor without storage whose sizes are asked of its class, which refuses
+    return torch.Tensor._make_wrapper_subclass(Wrapper, shape, dtype=dtype, device="cuda", dispatch_sizes_strides_policy="sizes")
+
+cfg = esa.EsaConfig(8, 2, 64, 32, 4, 512, 256, 3, 128, 1, 1024)
+native = binding.load_native()
+ctx, fit = native.Ctx(0, cfg), native.Fit(0, cfg)
+k, K, kc, q = z(1, 5, 2, 64), z(1, 1024, 2, 64), z(1, 1024, 32), z(1, 5, 8, 64)
+idx, n_sel = z(1, 256, dtype=torch.int32), z(1, dtype=torch.int32)
+calls = [lambda: ctx.append_kv(k, k, K, K, [0], 0, False), lambda: ctx.compress_keys(k, kc, [0], 0, False),
+         lambda: ctx.select(q, kc, [0], idx, n_sel, 0, False), lambda: ctx.select_full(q, K, [0], False, idx, n_sel, 0, False),
+         lambda: ctx.attend(q, K, K, [0], idx, n_sel, q, 0, False),
+         lambda: ctx.attend_two_position(q, q, K, K, K, [0], idx, n_sel, q, 0, False),
+         lambda: ctx.attend_host_kv(q, K, K, [0], idx, n_sel, K, K, q, 0, False),
+         lambda: native.attend_noalloc(cfg, q, K, K, [0], idx, n_sel, q, 0),
+         lambda: fit.step(z(5, 8, 64), z(5, 2, 64), None, 0)]
+for f in calls:
+    try:
+        f()
+    except ValueError as e:
+        assert str(e).startswith("asked"), e
+    else:
+        raise SystemExit("accepted")
+print("all refused")
+"""
+
+
+def test_tensors_that_torch_throws_about_raise_python_errors(lib):
+    """The native half of the binding asks torch about its arguments; what torch throws must not end the process."""
+    import subprocess
+    import sys
+    res = subprocess.run([sys.executable, "-c", _WRAPPERS], cwd=ROOT, capture_output=True, text=True, timeout=300)
+    assert res.returncode == 0 and "all refused" in res.stdout, (res.returncode, res.stderr[-2000:])
