@@ -118,6 +118,7 @@ struct NPrev {
 };
 
 bool read_n_prev(PyObject* o, int64_t B, NPrev* out) {
+    if (PyObject_Size(o) < 0) return false;         // (something with a length: a call would use an iterator up)
     PyObject* seq = PySequence_Fast(o, "n_prev must be a sequence of integers");
     if (!seq) return false;
     const Py_ssize_t n = PySequence_Fast_GET_SIZE(seq);

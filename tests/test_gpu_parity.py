@@ -1065,6 +1065,22 @@ def test_first_calls_of_several_threads_together():
         assert res.returncode == 0 and "threads agree" in res.stdout, res.stderr[-2000:]
 
 
+def test_positions_are_given_by_anything_with_a_length():
+    """n_prev: lists, tuples, ranges, arrays and tensors of integers; not iterators, which the call would use up."""
+    cfg = syn.get_config("c1")
+    ctx = hp.make_esa(cfg, max_tokens=512, max_batch=2)
+    k = torch.randn(2, 3, cfg.H_G, cfg.d, device="cuda").bfloat16()
+    want = torch.zeros(2, 512, cfg.d_c, dtype=torch.bfloat16, device="cuda")
+    ctx.compress_keys(k, want, [7, 8], sync=True)
+    for good in ((7, 8), range(7, 9), np.array([7, 8]), np.array([7, 8], np.int32), torch.tensor([7, 8]), [np.int64(7), 8.0]):
+        kc = torch.zeros_like(want)
+        ctx.compress_keys(k, kc, good, sync=True)
+        assert torch.equal(kc, want)
+    for bad, error in (((x for x in (7, 8)), TypeError), (iter([7, 8]), TypeError), (7, TypeError), ([7], ValueError), ([7, 8, 9], ValueError)):
+        with pytest.raises(error):
+            ctx.compress_keys(k, want, bad, sync=True)
+
+
 def _offset(t, elements):
     """A contiguous copy of t that starts `elements` values behind an allocation's (aligned) start."""
     flat = torch.empty(t.numel() + elements, dtype=t.dtype, device=t.device)
