@@ -4,16 +4,28 @@ from __future__ import annotations
 
 import glob
 import os
+import re
 import shutil
 import subprocess
+import sys
 import sysconfig
+
+import torch
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libesa_b200.so")
 NATIVE_SRC = os.path.join(CSRC, "esa_native.cpp")
-NATIVE_PATH = os.path.join(PKG_DIR, "_esa_native.so")
 INCLUDE_DIR = os.path.join(os.path.dirname(PKG_DIR), "include")
+
+
+def native_path(python: str = sys.implementation.cache_tag, torch_version: str = torch.__version__) -> str:
+    """File of the native module.  It is compiled against one torch and one Python, whose internals it reads, so both are
+    part of its name: a module built against others is not found (and rebuilt), never loaded."""
+    return os.path.join(PKG_DIR, "_esa_native.%s-torch%s.so" % (python, re.sub(r"[^0-9A-Za-z.]+", "_", torch_version)))
+
+
+NATIVE_PATH = native_path()
 
 
 def _nvcc() -> str:
@@ -51,7 +63,6 @@ def _run(cmd) -> str:
 
 
 def _build_native() -> None:
-    import torch
     tdir = os.path.dirname(torch.__file__)
     cuda_inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_nvcc()))), "include")
     _run([

@@ -136,3 +136,16 @@ def test_tensors_that_torch_throws_about_raise_python_errors(lib):
     import sys
     res = subprocess.run([sys.executable, "-c", _WRAPPERS], cwd=ROOT, capture_output=True, text=True, timeout=300)
     assert res.returncode == 0 and "all refused" in res.stdout, (res.returncode, res.stderr[-2000:])
+
+
+def test_a_native_module_of_another_torch_or_python_is_stale(lib, monkeypatch):
+    from paper_2502_14477_b200 import binding, build
+    assert os.path.exists(build.NATIVE_PATH) and not build.is_stale()
+    for other in (build.native_path(torch_version="9.9.0+cu999"), build.native_path(python="cpython-399")):
+        assert other != build.NATIVE_PATH
+        monkeypatch.setattr(build, "NATIVE_PATH", other)
+        assert build.is_stale()
+        monkeypatch.setattr(binding, "NATIVE_PATH", other)
+        monkeypatch.setattr(binding, "_native", None)
+        with pytest.raises(RuntimeError, match="missing"):
+            binding.load_native()
