@@ -287,6 +287,21 @@ esa_status esa_read_pooled_scores(esa_ctx* ctx, int32_t b, float* dst_host, int6
  * ESA_ERR_STATE if that call did no scoring, ESA_ERR_CAPACITY if n_rows exceeds its rows. */
 esa_status esa_read_compressed_queries(esa_ctx* ctx, void* dst_host, int64_t n_rows, void* stream);
 
+/* Diagnostic (host only, no device needed): the form in which esa_attend -- or, two_position != 0, a call of
+ * esa_attend_two_position with a second encoding -- deals out its key lists on a GPU of num_sms SMs: the streaming
+ * kernel for single queries (its parts depend on the device: *parts = 0), or the tensor-memory kernel with the key list
+ * of every 256 rows in *parts parts that a second launch merges (1: unsplit), as a pair of CTAs that exchange their halves,
+ * as a long and a short part, or as a pair for the two lists of two encodings.  Tensors aligned as the conventions say. */
+typedef enum {
+    ESA_ATTEND_DECODE = 0,
+    ESA_ATTEND_PARTS = 1,
+    ESA_ATTEND_PAIR = 2,
+    ESA_ATTEND_UNEVEN = 3,
+    ESA_ATTEND_TWO_PAIR = 4
+} esa_attend_form;
+esa_status esa_attend_plan(const esa_config* cfg, int32_t num_sms, int32_t B, int32_t l_C, const int64_t* n_prev,
+                           int32_t two_position, int32_t* kernel, int32_t* parts);
+
 /* Diagnostic of the bounded device-side waits: enqueues a one-thread kernel that waits, for
  * at most limit_cycles SM clock cycles (1 <= limit_cycles <= 2e9, about a second), on a
  * barrier that nothing ever completes.  The wait gives up, ESA_ERR_TIMEOUT is recorded in the

@@ -110,6 +110,7 @@ _PROTOS = {
     "esa_fit_launch_count": (C.c_int64, [C.c_void_p]),
     "esa_read_pooled_scores": (C.c_int, [C.c_void_p, C.c_int32, C.c_void_p, C.c_int64, C.c_void_p]),
     "esa_read_compressed_queries": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p]),
+    "esa_attend_plan": (C.c_int, [C.POINTER(_CConfig), C.c_int32, C.c_int32, C.c_int32, C.c_void_p, C.c_int32, C.c_void_p, C.c_void_p]),
     "esa_debug_wait_timeout": (C.c_int, [C.c_void_p, C.c_int64, C.c_void_p]),
     "esa_kernel_class_count": (C.c_int32, []),
     "esa_kernel_class_name": (C.c_char_p, [C.c_int32]),
@@ -358,3 +359,16 @@ def attend_noalloc_status(stream=None) -> int:
     """``esa_attend_noalloc_status``: what the kernels of ``attend_noalloc`` on the current device recorded since
     the last read (0: nothing)."""
     return int(load_library().esa_attend_noalloc_status(_stream_ptr(stream)))
+
+
+ATTEND_FORMS = ("decode", "parts", "pair", "uneven", "two_pair")
+
+
+def attend_plan(cfg: EsaConfig, num_sms: int, l_C: int, n_prev, two_position: bool = False):
+    """``esa_attend_plan``: (form, parts) in which an attention call deals out its key lists; needs no device."""
+    kernel, parts = C.c_int32(), C.c_int32()
+    c, n = cfg.to_c(), (C.c_int64 * len(n_prev))(*[int(x) for x in n_prev])
+    st = load_library().esa_attend_plan(C.byref(c), num_sms, len(n_prev), l_C, n, 1 if two_position else 0, C.byref(kernel), C.byref(parts))
+    if st != 0:
+        raise EsaError(st, "esa_attend_plan")
+    return ATTEND_FORMS[kernel.value], parts.value

@@ -78,15 +78,15 @@ esa_status check_common(esa_ctx* ctx, int32_t B) {
 }
 
 // Section 3.1 partition for every sequence of the call.
-esa_status build_meta(const esa_ctx* ctx, int B, const int64_t* n_prev, int64_t n_cur, SeqMeta* m,
+esa_status build_meta(const esa_config& cfg, int B, const int64_t* n_prev, int64_t n_cur, SeqMeta* m,
                       int* max_lM) {
     int mx = 0;
     for (int b = 0; b < B; ++b) {
         const int64_t t = n_prev[b];
         if (t < 0) return ESA_ERR_INVALID_ARG;
-        if (t + n_cur > ctx->cfg.max_tokens) return ESA_ERR_CAPACITY;
-        const int64_t i_end = t < ctx->cfg.l_init ? t : ctx->cfg.l_init;
-        int64_t m_end = t - ctx->cfg.l_local;
+        if (t + n_cur > cfg.max_tokens) return ESA_ERR_CAPACITY;
+        const int64_t i_end = t < cfg.l_init ? t : cfg.l_init;
+        int64_t m_end = t - cfg.l_local;
         if (m_end < i_end) m_end = i_end;
         m->t[b] = (int)t;
         m->i_end[b] = (int)i_end;
@@ -307,7 +307,7 @@ esa_status esa_select_async(esa_ctx* ctx, int32_t B, const void* Q_cur, int32_t 
     if (!ctx->has_w) return ESA_ERR_STATE;
     SeqMeta meta;
     int max_lM = 0;
-    s = build_meta(ctx, B, n_prev, l_C, &meta, &max_lM);
+    s = build_meta(ctx->cfg, B, n_prev, l_C, &meta, &max_lM);
     if (s != ESA_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
     bool any_small = false, any_large = false;
@@ -371,7 +371,7 @@ esa_status esa_select_full_async(esa_ctx* ctx, int32_t B, const void* Q_cur, int
     if (l_C > ctx->cfg.max_chunk) return ESA_ERR_CAPACITY;
     SeqMeta meta;
     int max_lM = 0;
-    s = build_meta(ctx, B, n_prev, l_C, &meta, &max_lM);
+    s = build_meta(ctx->cfg, B, n_prev, l_C, &meta, &max_lM);
     if (s != ESA_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
     bool any_small = false, any_large = false;
@@ -426,7 +426,7 @@ esa_status esa_attend_two_position_async(esa_ctx* ctx, int32_t B, const void* Q_
     if (!Q_cur || !K_cache || !V_cache || !n_prev || !idx || !n_sel || !O || l_C <= 0) return ESA_ERR_INVALID_ARG;
     if (l_C > ctx->cfg.max_chunk) return ESA_ERR_CAPACITY;
     SeqMeta meta;
-    s = build_meta(ctx, B, n_prev, l_C, &meta, nullptr);
+    s = build_meta(ctx->cfg, B, n_prev, l_C, &meta, nullptr);
     if (s != ESA_OK) return s;
     // A call that follows the selection of its step on the same stream may attend the older rows early, with the queries
     // that the selection has read: others may be what the preceding kernel is writing.
@@ -475,7 +475,7 @@ esa_status esa_attend_host_kv_async(esa_ctx* ctx, int32_t B, const void* Q_cur, 
         return ESA_ERR_INVALID_ARG;
     if (l_C > ctx->cfg.max_chunk) return ESA_ERR_CAPACITY;
     SeqMeta meta;
-    s = build_meta(ctx, B, n_prev, l_C, &meta, nullptr);
+    s = build_meta(ctx->cfg, B, n_prev, l_C, &meta, nullptr);
     if (s != ESA_OK) return s;
     // rows of the attended list per sequence (the selection may hold fewer than top_k: the upper bound sizes the stage)
     for (int b = 0; b < B; ++b) {
@@ -527,6 +527,31 @@ esa_status esa_read_compressed_queries(esa_ctx* ctx, void* dst_host, int64_t n_r
     if (cudaMemcpyAsync(dst_host, ctx->Qc, 2 * (size_t)n_rows * ctx->dc, cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return ESA_ERR_CUDA;
     return from_cuda(cudaStreamSynchronize(st));
+}
+
+esa_status esa_attend_plan(const esa_config* cfg, int32_t num_sms, int32_t B, int32_t l_C, const int64_t* n_prev,
+                           int32_t two_position, int32_t* kernel, int32_t* parts) {
+    if (!cfg || !n_prev || !kernel || !parts || num_sms <= 0 || B <= 0 || l_C <= 0) return ESA_ERR_INVALID_ARG;
+    if (!config_ok(cfg)) return ESA_ERR_SHAPE;
+    if (B > cfg->max_batch || l_C > cfg->max_chunk) return ESA_ERR_CAPACITY;
+    SeqMeta meta;
+    const esa_status s = build_meta(*cfg, B, n_prev, l_C, &meta, nullptr);
+    if (s != ESA_OK) return s;
+    const int G = cfg->n_q_heads / cfg->n_kv_heads;
+    if (attend_decode_covers(l_C, G)) {
+        *kernel = ESA_ATTEND_DECODE;
+        *parts = 0;
+        return ESA_OK;
+    }
+    const TcPlan p = plan_attend_tc(num_sms, make_layout(cfg).att_elems, cfg->head_dim, G, cfg->n_kv_heads, cfg->top_k, B, l_C, meta,
+                                    two_position != 0, false);
+    if (p.nsplit == 0) return ESA_ERR_UNSUPPORTED;
+    *kernel = p.mode == TC_PAIR       ? ESA_ATTEND_PAIR
+              : p.mode == TC_UNEVEN   ? ESA_ATTEND_UNEVEN
+              : p.mode == TC_TWO_PAIR ? ESA_ATTEND_TWO_PAIR
+                                      : ESA_ATTEND_PARTS;
+    *parts = p.nsplit;
+    return ESA_OK;
 }
 
 esa_status esa_debug_wait_timeout(esa_ctx* ctx, int64_t limit_cycles, void* stream) {

@@ -405,6 +405,9 @@ static cudaError_t launch_decode_t(esa_ctx* ctx, AttendParams& p, int B, int n_a
     return e;
 }
 
+// Decode: the streaming kernel for the usual group sizes.
+bool attend_decode_covers(int l_C, int G) { return l_C == 1 && (G == 1 || G == 2 || G == 4 || G == 7 || G == 8); }
+
 template <int D, bool TWO>
 static cudaError_t launch_decode(esa_ctx* ctx, AttendParams& p, int B, int n_att_max, cudaStream_t st) {
     switch (p.G) {
@@ -440,18 +443,15 @@ cudaError_t launch_attend(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, 
         int n = meta.i_end[b] + (lM < ctx->cfg.top_k ? lM : ctx->cfg.top_k) + (meta.t[b] - meta.m_end[b]) + l_C;
         if (n > n_att_max) n_att_max = n;
     }
-    if (l_C == 1) {
-        // decode: streaming kernel for the usual group sizes
-        cudaError_t e;
-        if (ctx->d == 128) e = two ? launch_decode<128, true>(ctx, p, B, n_att_max, st) : launch_decode<128, false>(ctx, p, B, n_att_max, st);
-        else e = two ? launch_decode<64, true>(ctx, p, B, n_att_max, st) : launch_decode<64, false>(ctx, p, B, n_att_max, st);
-        if (e != cudaErrorNotSupported) return e;
+    if (attend_decode_covers(l_C, ctx->G)) {
+        if (ctx->d == 128) return two ? launch_decode<128, true>(ctx, p, B, n_att_max, st) : launch_decode<128, false>(ctx, p, B, n_att_max, st);
+        return two ? launch_decode<64, true>(ctx, p, B, n_att_max, st) : launch_decode<64, false>(ctx, p, B, n_att_max, st);
     }
     // Any other chunk: tcgen05 kernel.  Few rows leave most of its 128-row tile empty, but the key list is then split far
     // enough that the products do not matter: 3 queries (12 rows a head) over 7400 keys 39 -> 22 us, 8 queries 32 -> 21 us
     // against a split mma.sync kernel.
-    return launch_attend_tc(ctx, B, l_C, Q, two ? p.Qg : nullptr, K, two ? p.Kg : nullptr, V, meta, idx, n_sel, O, n_att_max, st,
-                            cache_rows, staged);
+    return launch_attend_tc(ctx, B, l_C, Q, two ? p.Qg : nullptr, K, two ? p.Kg : nullptr, V, meta, idx, n_sel, O, st, cache_rows,
+                            staged);
 }
 
 // ---------------------------------------------------------------------------

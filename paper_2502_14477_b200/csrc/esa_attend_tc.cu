@@ -48,6 +48,8 @@
 //     pair (TC_TWO_PAIR) the CTA with the shorter list goes on with the end of the other's: new Q tiles, the same
 //     running sums and accumulator (33 tiles against 20, 512 queries of the 32/8-head shape: 72 -> 64 us; 64
 //     against 12: 126 -> 87).
+#include <algorithm>
+#include <cstdlib>
 #include <cstring>
 #include <type_traits>
 
@@ -75,9 +77,6 @@ constexpr int TC_REGS_SOFTMAX = 168;
 constexpr int TC_REGS_OTHER = 88;
 static_assert(8 * TC_REGS_SOFTMAX + 8 * TC_REGS_OTHER <= 16 * TC_REGS_LAUNCH,
               "register split exceeds the CTA's launch allocation: setmaxnreg.inc would never return");
-// what the CTAs of a unit do with their results (launch_tc): separate parts (merged by a second launch), pairs that
-// exchange halves, separate parts of which the first is much the longer, or pairs for the two lists of two-position attention
-enum { TC_PARTS = 0, TC_PAIR = 1, TC_UNEVEN = 2, TC_TWO_PAIR = 3 };
 constexpr float kSumLimit = 1.8446744e19f;   // 2^64: a tile whose sum of 2^(score - m) reaches this has its maximum looked up
 
 struct TcAttendParams {
@@ -94,9 +93,7 @@ struct TcAttendParams {
     int64_t max_tokens;
     int l_C, H, HG, G, top_k;
     int nsplit;
-    int main_tiles;     // TC_UNEVEN: tiles of the first part (see launch_tc)
-    int early_units;    // the second part of the first so many units takes up to this many tiles of the early list
-    int early_second;
+    int main_tiles, early_units, early_second;     // TC_UNEVEN: see TcPlan
     int Rp;             // rows of a scratch part (R rounded up to even: 16-byte aligned parts)
     int q_tma;          // Q tiles arrive by TMA (one arrival) instead of cp.async (one per producer thread)
     int staged;         // the caches hold the attended list itself: row j = list entry j
@@ -930,41 +927,47 @@ __global__ void __launch_bounds__(256) attend_tc_merge_kernel(const float* part,
                  O + (((int64_t)b * l_C + row / G) * H + kvh * G + row % G) * D);
 }
 
-template <int D, int NQT, bool FINE>
-static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_max, cudaStream_t st) {
-    const int R = p.l_C * p.G;
+TcPlan plan_attend_tc(int num_sms, size_t part_elems, int D, int G, int HG, int top_k, int B, int l_C, const SeqMeta& meta, bool two,
+                      bool early) {
+    const int R = l_C * G, Rp = (R + 1) & ~1;
     const int row_tiles = (R + TC_ROWS - 1) / TC_ROWS;
-    p.Rp = (R + 1) & ~1;
+    const bool one_tile = R <= 128;                                // (NQT = 1)
     // Split the key list when that fills the machine better.  Cost in us, fitted to measured sweeps: 1.85 per 128-key tile
     // (1.55 with one Q tile) of the longest CTA, one CTA per SM, 7 for its start and end and 3 more for every wave after
     // the first; 7.5 for a pair's exchange or a merge launch, whose traffic (4 TB/s) counts; and 6 when the last wave
     // leaves the merge launch no SMs to start on meanwhile (37 queries, 8 units over 6300 keys: 41 us with 3 parts, 23
     // with 9, 21 with 14, 32 with 18).  Two-position attention needs an even number of splits (one group per part); its
     // longer part sets the tiles per CTA.
-    const int ctas = row_tiles * p.HG * B;
+    const int ctas = row_tiles * HG * B;
+    int n_att_max = 0, far_max = 0;
+    for (int b = 0; b < B; ++b) {
+        const int far = meta.i_end[b] + std::min(meta.m_end[b] - meta.i_end[b], top_k);      // entries of I and M_k
+        n_att_max = std::max(n_att_max, far + (meta.t[b] - meta.m_end[b]) + l_C);
+        far_max = std::max(far_max, far);
+    }
     const int n_tiles = (n_att_max + TC_BN - 1) / TC_BN;
-    int i_end_max = 0;
-    for (int b = 0; b < B; ++b) i_end_max = max(i_end_max, p.meta.i_end[b]);
-    const int far_tiles = min(n_tiles, (i_end_max + p.top_k + TC_BN - 1) / TC_BN);
-    const bool even_out = abs(2 * far_tiles - n_tiles) > 5;       // (a pair moves tiles between its lists)
-    const int step = p.two ? 2 : 1;
-    const double merge_bytes = (double)B * p.HG * p.Rp * (D + 2) * 4;      // per part
+    const int far_tiles = std::min(n_tiles, (far_max + TC_BN - 1) / TC_BN);
+    const bool even_out = std::abs(2 * far_tiles - n_tiles) > 5;       // (a pair moves tiles between its lists)
+    const int step = two ? 2 : 1;
+    const size_t part = (size_t)B * HG * Rp * (D + 2);                 // floats of the scratch per part
+    const double merge_bytes = (double)part * 4;
     int best = 0;
     double best_cost = 1e30;
     for (int ns = step; ns <= kAttPrefillSplits && (ns <= n_tiles || best == 0); ns += step) {
-        if (ns > 2 && (size_t)B * p.HG * ns * p.Rp * (D + 2) > ctx->att_part_elems) break;      // (pairs use no scratch)
-        const int grp = p.two ? ns / 2 : ns;
-        const int longest = p.two ? max(far_tiles, n_tiles - far_tiles + 1) : n_tiles;
-        const int per = p.two && ns == 2 && even_out ? (n_tiles + 4) / 2 : (longest + grp - 1) / grp;
-        const int waves = (ctas * ns + ctx->num_sms - 1) / ctx->num_sms;
-        const int last_wave = ctas * ns - (waves - 1) * ctx->num_sms;
-        const double join = ns == 1 ? 0.0 : ns == 2 ? 7.5 : 7.5 + ns * merge_bytes / 4e6 + (last_wave * 8 > ctx->num_sms * 7 ? 6.0 : 0.0);
-        const double tile = NQT == 2 ? 1.85 : 1.55;
+        if (ns > 2 && part * ns > part_elems) break;                    // (pairs use no scratch)
+        const int grp = two ? ns / 2 : ns;
+        const int longest = two ? std::max(far_tiles, n_tiles - far_tiles + 1) : n_tiles;
+        const int per = two && ns == 2 && even_out ? (n_tiles + 4) / 2 : (longest + grp - 1) / grp;
+        const int waves = (ctas * ns + num_sms - 1) / num_sms;
+        const int last_wave = ctas * ns - (waves - 1) * num_sms;
+        const double join = ns == 1 ? 0.0 : ns == 2 ? 7.5 : 7.5 + ns * merge_bytes / 4e6 + (last_wave * 8 > num_sms * 7 ? 6.0 : 0.0);
+        const double tile = one_tile ? 1.55 : 1.85;
         double cost = waves * (tile * per + 3.0) + 4.0 + join;
         // CTAs of unlike lengths (the two lists) fill each other's gaps over three waves and more: SM time over SMs, and half a CTA for the end
-        if (p.two && ns > 2 && waves > 2) cost = ctas * (tile * n_tiles + 3.0 * ns) / ctx->num_sms + (tile * per + 3.0) / 2 + 4.0 + join;
+        if (two && ns > 2 && waves > 2) cost = ctas * (tile * n_tiles + 3.0 * ns) / num_sms + (tile * per + 3.0) / 2 + 4.0 + join;
         if (cost < best_cost - 1e-9) { best_cost = cost; best = ns; }
     }
+    TcPlan plan = {best, best != 2 ? TC_PARTS : two && even_out ? TC_TWO_PAIR : TC_PAIR, 0, 0, 0};
     // Two uneven parts (TC_UNEVEN), where one CTA per unit leaves SMs idle and a second one each would more than fill them:
     // the first parts of all units run in one wave, and the idle SMs take the second parts, `rounds` one after another.
     // The shortest first part that keeps the second ones from taking longer (start and end: 5 us each).  1024 queries of
@@ -972,55 +975,64 @@ static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_m
     // second parts are in the first wave give them up to half of the early list, so that every CTA of that wave has
     // work while the selection runs (without: 295; all of the early list, which leaves the first parts idle: other sizes up
     // to 8 us slower).  Estimated gains below 3 us are left: the estimate is no better than that.
-    p.main_tiles = p.early_units = p.early_second = 0;
-    const int idle = ctas < ctx->num_sms ? ctx->num_sms - ctas : 0;
-    if (NQT == 2 && !p.two && idle > 0 && ctas > idle && (size_t)B * p.HG * 2 * p.Rp * (D + 2) <= ctx->att_part_elems) {
+    const int idle = ctas < num_sms ? num_sms - ctas : 0;
+    if (!one_tile && !two && idle > 0 && ctas > idle && part * 2 <= part_elems) {
         const int rounds = (ctas + idle - 1) / idle;
-        const int second = max(0, (int)((n_tiles * 1.85 + 3.0 - 5.0 * rounds) / (1.85 * (rounds + 1))));
+        const int second = std::max(0, (int)((n_tiles * 1.85 + 3.0 - 5.0 * rounds) / (1.85 * (rounds + 1))));
         const double cost = 1.85 * (n_tiles - second) + 3.0 + 4.0 + 7.5 + 2 * merge_bytes / 4e6;
-        if (second > 0 && cost < best_cost - 3.0) {
-            best = 2;
-            p.main_tiles = n_tiles - second;
-            p.early_units = p.early ? idle : 0;      // (they start beside the selection kernel, like the first parts)
-            p.early_second = second;
-        }
+        if (second > 0 && cost < best_cost - 3.0)      // (early: the second parts start beside the selection kernel, like the first)
+            plan = {2, TC_UNEVEN, n_tiles - second, early ? idle : 0, second};
     }
-    if (best == 0) return cudaErrorNotSupported;
+    return plan;
+}
+
+template <int D, int NQT, bool FINE>
+static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, cudaStream_t st) {
+    const int R = p.l_C * p.G;
+    const int row_tiles = (R + TC_ROWS - 1) / TC_ROWS;
+    p.Rp = (R + 1) & ~1;
+    TcPlan plan = plan_attend_tc(ctx->num_sms, ctx->att_part_elems, D, p.G, p.HG, p.top_k, B, p.l_C, p.meta, p.two != 0, p.early != 0);
+    if (plan.nsplit == 0) return cudaErrorNotSupported;
     // Finished rows are stored 16 bytes at a time, merged ones four: an O that is not 16-byte aligned is written by the merge
     // launch, where the scratch holds two parts (always for the small chunks).
     const bool wide_O = aligned(p.O, 16);
     if (!aligned(p.Q, 16) || !aligned(p.Qg, 16) || !aligned(p.O, 4)) return kErrAlign;
-    if (!wide_O && best == 1) best = 2;
-    p.nsplit = best;
+    if (!wide_O) {
+        if (plan.nsplit == 1) plan.nsplit = 2;
+        if (plan.mode != TC_UNEVEN) plan.mode = TC_PARTS;
+    }
+    p.nsplit = plan.nsplit;
+    p.main_tiles = plan.main_tiles; p.early_units = plan.early_units; p.early_second = plan.early_second;
     CUtensorMap qmap, qgmap;
     p.q_tma = make_tensor_map_q(&qmap, p.Q, (uint64_t)B * p.l_C, p.H, D, p.G) ? 1 : 0;
     if (p.q_tma && p.two) p.q_tma = make_tensor_map_q(&qgmap, p.Qg, (uint64_t)B * p.l_C, p.H, D, p.G) ? 1 : 0;
     if (!p.q_tma) memset(&qmap, 0, sizeof(qmap));
     if (!p.q_tma || !p.two) memset(&qgmap, 0, sizeof(qgmap));
-    const dim3 grid(row_tiles, p.HG, B * best);
-    // a two-way split runs as CTA pairs that merge through distributed shared memory, where the device can place pairs
-    static std::atomic<int> pair_ok[64];                     // per instantiation and device: 0 not asked yet, 1 yes, 2 no
-    std::atomic<int>& ok = pair_ok[ctx->device & 63];
-    const bool uneven = p.main_tiles > 0;
-    if (best == 2 && !uneven && ok.load(std::memory_order_relaxed) == 0) {
-        const bool yes = launch_tc_kernel<D, TC_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess &&
-                         launch_tc_kernel<D, TC_TWO_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess;
-        if (!yes) cudaGetLastError();
-        ok.store(yes ? 1 : 2, std::memory_order_relaxed);
+    const dim3 grid(row_tiles, p.HG, B * p.nsplit);
+    // pairs, which merge through distributed shared memory, where the device can place them
+    if (plan.mode == TC_PAIR || plan.mode == TC_TWO_PAIR) {
+        static std::atomic<int> pair_ok[64];                 // per instantiation and device: 0 not asked yet, 1 yes, 2 no
+        std::atomic<int>& ok = pair_ok[ctx->device & 63];
+        if (ok.load(std::memory_order_relaxed) == 0) {
+            const bool yes = launch_tc_kernel<D, TC_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess &&
+                             launch_tc_kernel<D, TC_TWO_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, true) == cudaSuccess;
+            if (!yes) cudaGetLastError();
+            ok.store(yes ? 1 : 2, std::memory_order_relaxed);
+        }
+        if (ok.load(std::memory_order_relaxed) != 1) plan.mode = TC_PARTS;
     }
-    const bool pair = best == 2 && !uneven && wide_O && ok.load(std::memory_order_relaxed) == 1;
-    if (best == 2 && !pair && (size_t)B * p.HG * 2 * p.Rp * (D + 2) > ctx->att_part_elems)
+    if (plan.mode == TC_PARTS && p.nsplit == 2 && (size_t)B * p.HG * 2 * p.Rp * (D + 2) > ctx->att_part_elems)
         return wide_O ? cudaErrorNotSupported : kErrAlign;
     cudaError_t e;
     {
         ProfScope prof(ctx, KC_ATTEND_TC, st);
-        if (pair && p.two && even_out) e = launch_tc_kernel<D, TC_TWO_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, false);
-        else if (pair) e = launch_tc_kernel<D, TC_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, false);
-        else if (uneven) e = launch_tc_kernel<D, TC_UNEVEN, 2, false>(ctx, qmap, qgmap, p, grid, st, false);
+        if (plan.mode == TC_TWO_PAIR) e = launch_tc_kernel<D, TC_TWO_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, false);
+        else if (plan.mode == TC_PAIR) e = launch_tc_kernel<D, TC_PAIR, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, false);
+        else if (plan.mode == TC_UNEVEN) e = launch_tc_kernel<D, TC_UNEVEN, 2, false>(ctx, qmap, qgmap, p, grid, st, false);
         else e = launch_tc_kernel<D, TC_PARTS, NQT, FINE>(ctx, qmap, qgmap, p, grid, st, false);
     }
     ctx->launches += 1;
-    if (e != cudaSuccess || best == 1 || pair) return e;
+    if (e != cudaSuccess || p.nsplit == 1 || plan.mode == TC_PAIR || plan.mode == TC_TWO_PAIR) return e;
     ProfScope prof(ctx, KC_ATTEND_MERGE, st);
     e = launch_pdl(attend_tc_merge_kernel<D>, dim3((R + 7) / 8, p.HG, B), dim3(256), 0, st, (const float*)p.part, p.nsplit, p.Rp, R, p.G,
                    p.HG, p.H, p.l_C, p.O);
@@ -1030,8 +1042,8 @@ static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, int n_att_m
 
 cudaError_t launch_attend_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* Qg,
                              const __nv_bfloat16* K, const __nv_bfloat16* Kg, const __nv_bfloat16* V, const SeqMeta& meta,
-                             const int32_t* idx, const int32_t* n_sel, __nv_bfloat16* O, int n_att_max, cudaStream_t st,
-                             int64_t cache_rows, bool staged) {
+                             const int32_t* idx, const int32_t* n_sel, __nv_bfloat16* O, cudaStream_t st, int64_t cache_rows,
+                             bool staged) {
     const bool two = Qg != nullptr || Kg != nullptr;
     TcAttendParams p;
     p.Q = Q; p.K = K; p.Qg = Qg ? Qg : Q; p.Kg = Kg ? Kg : K;
@@ -1046,8 +1058,8 @@ cudaError_t launch_attend_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* 
     const int rows = l_C * ctx->G;
     auto run = [&](auto dim) {
         constexpr int D = decltype(dim)::value;
-        if (rows <= kAttSplitRows) return launch_tc<D, 1, true>(ctx, p, B, n_att_max, st);
-        return rows <= 128 ? launch_tc<D, 1, false>(ctx, p, B, n_att_max, st) : launch_tc<D, 2, false>(ctx, p, B, n_att_max, st);
+        if (rows <= kAttSplitRows) return launch_tc<D, 1, true>(ctx, p, B, st);
+        return rows <= 128 ? launch_tc<D, 1, false>(ctx, p, B, st) : launch_tc<D, 2, false>(ctx, p, B, st);
     };
     if (ctx->d == 128) return run(std::integral_constant<int, 128>());
     if (ctx->d == 64) return run(std::integral_constant<int, 64>());

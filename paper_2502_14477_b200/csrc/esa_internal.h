@@ -244,8 +244,23 @@ cudaError_t launch_gather_kv(esa_ctx* ctx, int B, int l_C, const void* K_host, c
 // Qg / Kg non-null: two-position attention (both given then).
 cudaError_t launch_attend_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* Qg,
                              const __nv_bfloat16* K, const __nv_bfloat16* Kg, const __nv_bfloat16* V, const SeqMeta& meta,
-                             const int32_t* idx, const int32_t* n_sel, __nv_bfloat16* O,
-                             int n_att_max, cudaStream_t st, int64_t cache_rows = 0, bool staged = false);
+                             const int32_t* idx, const int32_t* n_sel, __nv_bfloat16* O, cudaStream_t st,
+                             int64_t cache_rows = 0, bool staged = false);
+
+// What the CTAs of a unit (256 rows of a key/value head) of the tcgen05 attention do with their results: separate parts
+// (merged by a second launch), pairs that exchange halves, separate parts of which the first is much the longer, or pairs for
+// the two lists of two-position attention.
+enum { TC_PARTS = 0, TC_PAIR = 1, TC_UNEVEN = 2, TC_TWO_PAIR = 3 };
+struct TcPlan {
+    int nsplit;         // parts of the key list; 0: no form fits the scratch
+    int mode;
+    int main_tiles;     // TC_UNEVEN: tiles of the first part
+    int early_units;    // the second part of the first so many units takes up to early_second tiles of the early list
+    int early_second;
+};
+TcPlan plan_attend_tc(int num_sms, size_t part_elems, int D, int G, int HG, int top_k, int B, int l_C, const SeqMeta& meta, bool two,
+                      bool early);
+bool attend_decode_covers(int l_C, int G);
 
 // TMA descriptor of the query tensor [n_queries, H, D] for the attention kernel (group size G must
 // divide 128).

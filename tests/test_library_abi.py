@@ -149,3 +149,26 @@ def test_a_native_module_of_another_torch_or_python_is_stale(lib, monkeypatch):
         monkeypatch.setattr(binding, "_native", None)
         with pytest.raises(RuntimeError, match="missing"):
             binding.load_native()
+
+
+def test_attention_plan_counts_the_tokens_that_exist(lib):
+    """Where there are fewer middle tokens than k, the form of a call is that of the same lists with k = |M|."""
+    import paper_2502_14477_b200 as esa
+    from paper_2502_14477_b200.binding import attend_plan
+    seen = set()
+    for H, H_G, d in ((32, 8, 128), (28, 4, 128), (8, 2, 64), (16, 16, 64)):
+        for l_C in (2, 37, 130, 512, 1000):
+            for l_L in (300, 2048, 4000):
+                for l_M in (1, 100, 900, 3000):
+                    for two in (False, True):
+                        t = 128 + l_M + l_L
+                        plans = [attend_plan(esa.EsaConfig(H, H_G, d, 64, 128, l_L, k, 3, l_C, 1, t + l_C), 148, l_C, [t], two)
+                                 for k in (l_M, l_M + 700, 2 * l_M + 2500, 20000)]
+                        assert all(p == plans[0] for p in plans), (H, H_G, l_C, l_L, l_M, two, plans)
+                        seen.add(plans[0][0])
+    assert {"parts", "pair", "two_pair"} <= seen
+    cfg = esa.EsaConfig(32, 8, 128, 128, 128, 2048, 4096, 3, 512, 1, 131072)
+    assert attend_plan(cfg, 148, 1, [65536]) == ("decode", 0) and attend_plan(cfg, 148, 512, [65536]) == ("pair", 2)
+    with pytest.raises(esa.EsaError) as e:
+        attend_plan(cfg, 148, 512, [131072])
+    assert e.value.status == 3
