@@ -583,9 +583,13 @@ def time_extensions(peaks):
     for per_head, key in ((False, "select_full_uniform"), (True, "select_full_per_head")):
         pr = timed(lambda: ctx.select_full(Q, K, [t], idx, n_sel, per_head=per_head), key)
         us = pr["score_full_kernel<.,1>+<.,2>"]
+        # the queries of a group are added up first and cut into three pieces where that is fewer products than the heads
+        made = fl_full if per_head else fl_full * min(1.0, 3.0 / (cfg.H // cfg.H_G))
         out[key] = {"score_us_per_call": us, "achieved_tflops": fl_full / us * 1e-6, "frac_burst": fl_full / us * 1e-6 / peaks["tflops_burst"],
+                    "products_made_frac_burst": made / us * 1e-6 / peaks["tflops_burst"],
                     "pool_us": pr.get("pool_kernel"), "select_topk_us": pr.get("select_topk_kernel"),
-                    "note": "mma.sync kernels (both passes timed together); flops = 2 passes x 2 d_H l_C l_M"}
+                    "note": "tcgen05 kernels (both passes timed together); flops = 2 passes x 2 d_H l_C l_M as the method counts them"
+                            + ("" if per_head else "; with folded queries 3 products are made in place of H / H_G")}
     idx[0] = (torch.sort(torch.randperm(l_M, device="cuda", generator=g)[: cfg.k])[0] + i_end).to(torch.int32)
     n_sel[0] = cfg.k
     K_host, V_host = K.cpu().pin_memory(), V.cpu().pin_memory()
@@ -615,8 +619,8 @@ def time_extensions(peaks):
     us = 1e3 * e0.elapsed_time(e1) / steps
     fl = 4.0 * nb * cfg.d_c * (cfg.d_H + cfg.d_G) + 2.0 * nb * nb * (cfg.d_G + 3 * cfg.d_c)
     out["compressor_fitting"] = {"us_per_step": us, "steps_per_s": 1e6 / us, "achieved_tflops_fp32": fl / us * 1e-6,
-                                 "launches_per_step": fit.launch_count / (steps + 5), "bound": "launch latency / fp32 ALU",
-                                 "note": "batch of 128 pairs, fp32 kernels; the paper's 10 epochs over 50k pairs are 3900 such steps"}
+                                 "launches_per_step": fit.launch_count / (steps + 5), "bound": "latency of three dependent launches",
+                                 "note": "batch of 128 pairs; long products on mma.sync, fp32 operands in three bf16 pieces; the paper's 10 epochs over 50k pairs are 3900 such steps"}
     fit.close()
     del K, V, Kf, K_host, V_host
     torch.cuda.empty_cache()

@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(FP_THREADS) fit_pairs_kernel(FitParams p) {
 // Launch 3: gradients and Adam.  A CTA owns a FU_J x FU_N tile of W_q or W_k: its gradient, reduced over the pairs,
 // stays in the accumulators and the update is applied from there, so gradients never go to memory.  Tiles of 32 x 128
 // read the least (6 bytes per feature and pair in pieces, 2 per column and pair: 56 KB a CTA for 128 pairs, against
-// 104 KB for 128 x 32, which took 10 us where this takes 6) and update whole 512-byte row segments.  The parameters
+// 104 KB for 128 x 32, which took 10 us where this takes 8) and update whole 512-byte row segments.  The parameters
 // and moments of the tile are requested first: they were last written by the launch before the last but one.  The
 // last two CTAs do the biases, and add up the loss.
 // ---------------------------------------------------------------------------

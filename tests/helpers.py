@@ -191,6 +191,16 @@ def check_compressed(kc_gpu: torch.Tensor, X: np.ndarray, W: np.ndarray, b=None,
     return int(neq.sum())
 
 
+# (H, H_G, d, positions, l_C, l_L, k, n_sel): calls that the split rule deals out unevenly on 148 SMs (more units than half of
+# the SMs, long lists): ragged last row tiles, Q tiles by plain copies (group of seven), a second sequence shorter than the
+# first part of the other's list, one row tile a head, nothing selected, a short and an empty list of older rows.
+UNEVEN_CASES = [
+    (28, 28, 64, (9000,), 1000, 3000, 5000, None), (28, 4, 128, (12000,), 1000, 4000, 6000, None),
+    (25, 25, 64, (9000, 3000), 400, 3000, 4000, None), (14, 2, 128, (9000, 2500), 1000, 3000, 5000, None),
+    (114, 114, 64, (9000,), 130, 3000, 4000, None), (20, 20, 64, (6500,), 1200, 6000, 100, 0),
+    (45, 45, 64, (10000,), 500, 200, 7000, None), (24, 24, 128, (9000,), 1000, 0, 7000, 6999)]
+
+
 class DeviceSeq:
     """Device caches for B sequences of a workload, filled from the seeded generators."""
 

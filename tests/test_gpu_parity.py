@@ -351,9 +351,9 @@ def test_small_chunk_attention_is_the_rounding_of_the_exact_result(H, H_G, d, t,
 
 
 @pytest.mark.parametrize("H_G,B,t,l_C", [(28, 1, 3000, 1000), (28, 1, 900, 1024), (11, 1, 4001, 2047), (25, 2, 2500, 300), (38, 1, 150, 700), (45, 1, 2600, 500)])
-def test_uneven_key_list_split(H_G, B, t, l_C):
-    """75 to 114 units of 256 rows: the idle SMs attend the ends of the units' key lists (nothing selected, ragged row tiles,
-    two sequences of different lengths among them)."""
+def test_units_that_fill_most_of_the_sms(H_G, B, t, l_C):
+    """75 to 114 units of 256 rows over short lists: one part each, or three (ragged row tiles, two sequences of different lengths
+    among them)."""
     cfg = syn.get_config("c1").with_(H=H_G, H_G=H_G, d=64, d_c=64, l_I=16, l_L=700, k=1000, B=B)
     p, n, t_list = hp.oracle_params(cfg), t + l_C, [t - 900 * b for b in range(B)]
     _, _, Wq, Wk = hp.oracle_weights(cfg)
@@ -367,7 +367,38 @@ def test_uneven_key_list_split(H_G, B, t, l_C):
     for b, tb in enumerate(t_list):
         K64, V64 = hp.torch_to_f64(seq.K[b, : tb + l_C]), hp.torch_to_f64(seq.V[b, : tb + l_C])
         want = orc.attend(hp.torch_to_f64(Q[b]), K64, V64, sel[b], tb, p, heads=heads)
-        hp.check_attention(O[b], want, what=f"uneven split H_G={H_G} seq {b}", heads=heads)
+        hp.check_attention(O[b], want, what=f"H_G={H_G} seq {b}", heads=heads)
+
+
+@pytest.mark.parametrize("case", hp.UNEVEN_CASES, ids=lambda c: f"{c[0]}-{c[1]}-{c[2]}-{len(c[3])}x{c[4]}")
+def test_uneven_key_list_split(case):
+    """Units that fill most of the SMs, with long lists: the idle SMs attend the ends of the units' lists.  The call that follows
+    its selection (older rows early) and the one that follows none, against the oracle on the same selection."""
+    from paper_2502_14477_b200.binding import attend_plan
+    H, H_G, d, t_list, l_C, l_L, k, n_sel = case
+    B, n = len(t_list), max(t_list) + l_C
+    cfg = syn.get_config("c1").with_(H=H, H_G=H_G, d=d, d_c=64, l_I=16, l_L=l_L, k=k)
+    p, heads = hp.oracle_params(cfg), [0, H // 2, H - 1]
+    ctx = hp.make_esa(cfg, max_tokens=n, max_chunk=l_C, max_batch=B)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert sms != 148 or attend_plan(ctx.cfg, sms, l_C, t_list) == ("uneven", 2)
+    g = torch.Generator(device="cuda").manual_seed(H + l_C)
+    draw = lambda *s: torch.randn(*s, device="cuda", dtype=torch.bfloat16, generator=g)
+    Q, K, V, kc = draw(B, l_C, H, d), draw(B, n, H_G, d), draw(B, n, H_G, d), draw(B, n, 64)
+    idx, counts = torch.zeros(B, k, dtype=torch.int32, device="cuda"), torch.zeros(B, dtype=torch.int32, device="cuda")
+    O_early, O = torch.full_like(Q, float("nan")), torch.full_like(Q, float("nan"))
+    torch.cuda.synchronize()
+    ctx.select(Q, kc, t_list, idx, counts)
+    if n_sel is not None:
+        counts.fill_(n_sel)
+    ctx.attend(Q, K, V, t_list, idx, counts, O_early)
+    ctx.attend(Q, K, V, t_list, idx, counts, O, sync=True)
+    assert ctx.last_device_status() == 0
+    for b, t in enumerate(t_list):
+        sel = idx[b, : int(counts[b])].cpu().numpy().astype(np.int64)
+        want = orc.attend(hp.torch_to_f64(Q[b]), hp.torch_to_f64(K[b, : t + l_C]), hp.torch_to_f64(V[b, : t + l_C]), sel, t, p, heads=heads)
+        for what, got in (("early", O_early), ("plain", O)):
+            hp.check_attention(got[b], want, what=f"{what} seq {b}", heads=heads)
 
 
 # ------------------------------------------------------ end to end, config 1
@@ -711,7 +742,6 @@ def test_two_position_attention_llama_shape_and_group_of_seven():
     _two_position_case(cfg, 10000, 1)
 
 
-# ------------------------------------------------ host-resident K/V (appendix "Model Loading")
 @pytest.mark.parametrize("H,H_G,d,t,l_C,l_L,k,n_sel", [
     (32, 8, 64, 4000, 512, 200, 2000, None), (32, 8, 64, 4000, 512, 200, 2000, 1),     # the selected part longer; the local part longer
     (32, 8, 64, 4000, 500, 2500, 500, 0), (32, 8, 128, 120, 400, 600, 500, None),      # nothing selected; I and C only
@@ -723,6 +753,7 @@ def test_two_position_pairs_even_their_lists_out(H, H_G, d, t, l_C, l_L, k, n_se
     _two_position_case(cfg, t, l_C, heads=[0, H // 2, H - 1], n_sel=n_sel)
 
 
+# ------------------------------------------------ host-resident K/V (appendix "Model Loading")
 @pytest.mark.parametrize("name,t,l_C,n_sel", [("c1", 3968, 128, None), ("c1", 4100, 1, None), ("c1", 2000, 5, 100),
                                                ("c1", 300, 128, None), ("c2", 8192, 512, None), ("c2", 9000, 1, None)])
 def test_attention_with_host_resident_kv(name, t, l_C, n_sel):

@@ -172,3 +172,12 @@ def test_attention_plan_counts_the_tokens_that_exist(lib):
     with pytest.raises(esa.EsaError) as e:
         attend_plan(cfg, 148, 512, [131072])
     assert e.value.status == 3
+
+
+def test_the_uneven_cases_of_the_gpu_tests_are_dealt_out_unevenly(lib):
+    import paper_2502_14477_b200 as esa
+    from paper_2502_14477_b200.binding import attend_plan
+    from tests import helpers as hp
+    for H, H_G, d, ts, l_C, l_L, k, _ in hp.UNEVEN_CASES:
+        cfg = esa.EsaConfig(H, H_G, d, 64, 16, l_L, k, 3, l_C, len(ts), max(ts) + l_C)
+        assert attend_plan(cfg, 148, l_C, ts) == ("uneven", 2), (H, H_G, d, ts, l_C)
