@@ -20,10 +20,16 @@
 // the first (k - #greater) in index order: exactly "lowest index wins", output ascending.
 // With one query per sequence (decode) the scoring kernel pooled the raw scores P; Eq. 4's s' = fl(P - r) is a monotone
 // map of P, taken when the keys are loaded.
+// A sequence longer than a cluster deals with well is selected in two levels (LEVEL): a cluster per segment of it leaves the
+// segment's k best as candidates, keys and positions, in index order; one cluster then selects among the candidates, whose
+// order is the tokens' order, so the same tie rule gives the same selection.
 // Bound: latency (a read of 4 l_M bytes that sit in L2).  An older form wrote candidate lists to memory that the last
 // CTA of a sequence gathered and finished by itself.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+#include <cmath>
+#include <type_traits>
 #include <utility>
 
 #include "esa_internal.h"
@@ -40,6 +46,8 @@ constexpr int SEL_WARPS = SEL_THREADS / 32;
 constexpr int SEL_BINS = 2048;
 constexpr int SEL_CLUSTER = 16;       // largest cluster (8 where the device does not place 16)
 constexpr int SEL_EQ_CAP = 32;        // keys sharing T's top 22 bits that a CTA sends one by one
+constexpr int SEL_SEGMENT = SEL_CLUSTER * 8 * SEL_THREADS;           // two levels: tokens of a segment, the least
+constexpr int SEL_TWO_LEVELS = 2 * SEL_CLUSTER * 16 * SEL_THREADS;   // longest middle part of one level
 constexpr int POOL_THREADS = 256;
 constexpr int POOL_TOKENS = 2048;     // tokens per CTA of the pooling kernel
 
@@ -51,8 +59,12 @@ struct SelectParams {
     int64_t max_tokens;
     int top_k;
     int mapped;
+    uint32_t* cand;         // [B, max_tokens] two levels: candidates of a sequence, keys then positions
+    int seg_tokens;         // two levels: tokens of a segment, at most
     SeqMeta meta;
 };
+// Segments of a sequence's middle tokens (one: no two levels); every segment holds more than k of them.
+__host__ __device__ __forceinline__ int select_segments(int l_M, int seg_tokens) { return (l_M - 1) / seg_tokens + 1; }
 
 // Finds, in the histogram `g` of one digit (nb <= SEL_BINS bins, larger bin = larger key), the bin
 // holding the krem-th largest remaining key.  Returns through sh_out[0] (bin) and sh_out[1] (keys
@@ -86,14 +98,16 @@ __device__ __forceinline__ void find_bin(const uint32_t* g, int nb, uint32_t kre
     __syncthreads();
 }
 
-// grid (cluster size, B).  CTA `rank` owns the middle tokens [rank * per, rank * per + per), in batches of
+// LEVEL 0: a sequence's tokens -> its selection; grid (cluster size, B).  LEVEL 1: a segment's tokens -> candidates; grid
+// (cluster size, segments, B).  LEVEL 2: the candidates (tokens, for a sequence of one segment) -> the selection.
+// CTA `rank` owns the middle tokens [rank * per, rank * per + per), in batches of
 // KPT * SEL_THREADS (one batch unless the sequence is longer than the cluster's registers hold: then the keys are read
 // again from L2 in every step); warp w holds 32 KPT consecutive tokens of a batch.
-template <int KPT>
+template <int KPT, int LEVEL>
 __global__ void __launch_bounds__(SEL_THREADS, 3)
 select_topk_kernel(SelectParams p) {
     constexpr int BATCH = KPT * SEL_THREADS;
-    const int b = blockIdx.y, rank = blockIdx.x, n_ranks = gridDim.x;
+    const int b = LEVEL == 1 ? blockIdx.z : blockIdx.y, rank = blockIdx.x, n_ranks = gridDim.x;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     __shared__ __align__(16) uint32_t part[SEL_BINS];    // this CTA's counts of a digit
@@ -113,21 +127,28 @@ select_topk_kernel(SelectParams p) {
     const int k = p.top_k;
     // sequences whose middle part fits in k are emitted whole by another kernel
     if (l_M <= k) return;
+    const int segs = LEVEL == 0 ? 1 : select_segments(l_M, p.seg_tokens);
+    if (LEVEL == 1 && (segs == 1 || (int)blockIdx.y >= segs)) return;
+    const bool second = LEVEL == 2 && segs > 1;          // the keys are the candidates'
+    uint32_t* cand_key = LEVEL == 0 ? nullptr : p.cand + (int64_t)b * p.max_tokens;
+    uint32_t* cand_pos = LEVEL == 0 ? nullptr : cand_key + (int64_t)segs * k;
+    const int seg_len = (l_M + segs - 1) / segs, seg_lo = LEVEL == 1 ? blockIdx.y * seg_len : 0;
+    const int n_keys = LEVEL == 1 ? min(seg_len, l_M - seg_lo) : second ? segs * k : l_M;
     cg::cluster_group cluster = cg::this_cluster();
     for (int i = tid; i < SEL_BINS; i += SEL_THREADS) part[i] = allA[i] = allB[i] = 0u;
     if (tid == 0) mine_gt = mine_eq = 0;
     __syncthreads();
     auto token = cluster.barrier_arrive();               // (nothing is sent to a CTA before its copies are clear)
 
-    const int per = ((l_M + n_ranks - 1) / n_ranks + 31) & ~31;
-    const int base = min(l_M, rank * per), n_mine = min(l_M, base + per) - base;
+    const int per = ((n_keys + n_ranks - 1) / n_ranks + 31) & ~31;
+    const int base = min(n_keys, rank * per), n_mine = min(n_keys, base + per) - base;
     const int n_batches = max(1, (n_mine + BATCH - 1) / BATCH);
     const int t0 = warp * 32 * KPT + lane;               // this thread's first token of a batch; the others 32 apart
 
     pdl_wait();         // the keys come from the preceding kernel
     pdl_launch_dependents();
-    const bool mapped = p.mapped != 0;
-    const uint32_t* pk = p.pkey + (int64_t)b * p.max_tokens + base;
+    const bool mapped = p.mapped != 0 && !second;
+    const uint32_t* pk = (second ? cand_key : p.pkey + (int64_t)b * p.max_tokens + seg_lo) + base;
     const float r0 = mapped ? key_to_f32(__ldcg(p.rkey + b)) : 0.f;
     uint32_t key[KPT];
     auto load_batch = [&](int bt) {
@@ -273,6 +294,10 @@ select_topk_kernel(SelectParams p) {
 
     // ---- ordered compaction
     int32_t* out = p.idx_out + (int64_t)b * p.top_k;
+    if (LEVEL == 1) {
+        cand_key += (int64_t)blockIdx.y * k;
+        cand_pos += (int64_t)blockIdx.y * k;
+    }
     for (int bt = 0; bt < n_batches; ++bt) {
         if (n_batches > 1) load_batch(bt);
         int g = 0, e = 0;
@@ -288,13 +313,21 @@ select_topk_kernel(SelectParams p) {
         const int before = __reduce_add_sync(0xffffffffu, lane < warp ? wt : 0), total = __reduce_add_sync(0xffffffffu, wt);
         int my_gt = gt_before + (before & 0xffff), my_eq = eq_before + (before >> 16);
         const uint32_t lt_mask = (1u << lane) - 1u;
-        const int tok = i_end + base + bt * BATCH + t0;
+        const int tok = (second ? 0 : i_end + seg_lo) + base + bt * BATCH + t0;
 #pragma unroll
         for (int j = 0; j < KPT; ++j) {
             const bool gt = key[j] > T, eq = key[j] == T;
             const uint32_t bg = __ballot_sync(0xffffffffu, gt), be = __ballot_sync(0xffffffffu, eq);
             const int eq_at = my_eq + __popc(be & lt_mask);
-            if (gt || (eq && eq_at < take_eq)) out[my_gt + __popc(bg & lt_mask) + min(eq_at, take_eq)] = tok + j * 32;
+            if (gt || (eq && eq_at < take_eq)) {
+                const int at = my_gt + __popc(bg & lt_mask) + min(eq_at, take_eq);
+                if (LEVEL == 1) {
+                    cand_key[at] = key[j];
+                    cand_pos[at] = (uint32_t)(tok + j * 32);
+                } else {
+                    out[at] = second ? (int)__ldcg(cand_pos + tok + j * 32) : tok + j * 32;
+                }
+            }
             my_gt += __popc(bg);
             my_eq += __popc(be);
         }
@@ -302,7 +335,7 @@ select_topk_kernel(SelectParams p) {
         eq_before += total >> 16;
         __syncthreads();
     }
-    if (rank == 0 && tid == 0) p.n_sel_out[b] = k;
+    if (LEVEL != 1 && rank == 0 && tid == 0) p.n_sel_out[b] = k;
 }
 
 // Eq. 8 for the scoring paths that leave unpooled keys: pools skey into pkey.  A CTA owns POOL_TOKENS consecutive
@@ -354,14 +387,14 @@ __global__ void read_pooled_kernel(const uint32_t* __restrict__ pkey, const uint
 }
 
 // n_ranks = 0: asks whether the device can place clusters of more than the portable eight CTAs.
-template <int KPT>
-static cudaError_t launch_topk(int device, const SelectParams& p, int n_ranks, int B, cudaStream_t st) {
+template <int KPT, int LEVEL>
+static cudaError_t launch_topk(int device, const SelectParams& p, int n_ranks, int segs, int B, cudaStream_t st) {
     const bool probe = n_ranks == 0;
     static KernelMemo memo;                  // (the attention's CTAs are to start beside this kernel's: same split of the SM's memory)
-    cudaError_t e = allow_smem(select_topk_kernel<KPT>, device, 0, memo, true);
+    cudaError_t e = allow_smem(select_topk_kernel<KPT, LEVEL>, device, 0, memo, true);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(probe ? SEL_CLUSTER : n_ranks, probe ? 1 : B);
+    cfg.gridDim = probe ? dim3(SEL_CLUSTER) : LEVEL == 1 ? dim3(n_ranks, segs, B) : dim3(n_ranks, B);
     cfg.blockDim = dim3(SEL_THREADS);
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
@@ -373,10 +406,10 @@ static cudaError_t launch_topk(int device, const SelectParams& p, int n_ranks, i
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = probe ? 1 : 2;
-    if (!probe) return cudaLaunchKernelEx(&cfg, select_topk_kernel<KPT>, p);
-    e = cudaFuncSetAttribute(select_topk_kernel<KPT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (!probe) return cudaLaunchKernelEx(&cfg, select_topk_kernel<KPT, LEVEL>, p);
+    e = cudaFuncSetAttribute(select_topk_kernel<KPT, LEVEL>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     int n = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, select_topk_kernel<KPT>, &cfg);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, select_topk_kernel<KPT, LEVEL>, &cfg);
     return e == cudaSuccess && n == 0 ? cudaErrorNotSupported : e;
 }
 
@@ -395,6 +428,7 @@ cudaError_t launch_select(esa_ctx* ctx, int B, bool mapped, const SeqMeta& meta,
     p.pkey = ctx->pkey; p.rkey = ctx->rkey;
     p.idx_out = idx_out; p.n_sel_out = n_sel_out;
     p.max_tokens = ctx->cfg.max_tokens; p.top_k = ctx->cfg.top_k;
+    p.cand = nullptr; p.seg_tokens = 0;
     p.mapped = mapped ? 1 : 0; p.meta = meta;                // (mapped mode reads rkey[b]: one query per sequence)
     // CTAs of 4096 tokens (8 keys a thread), as many as it takes up to 16 (8 where the device does not place such clusters, or
     // where all sequences' CTAs would outnumber the SMs); then 16 keys a thread.  63k tokens, select: 36.3 us with 16 CTAs,
@@ -402,18 +436,48 @@ cudaError_t launch_select(esa_ctx* ctx, int B, bool mapped, const SeqMeta& meta,
     static std::atomic<int> wide[64];
     std::atomic<int>& w = wide[ctx->device & 63];
     if (w.load(std::memory_order_relaxed) == 0) {
-        const bool ok = launch_topk<8>(ctx->device, p, 0, 1, st) == cudaSuccess && launch_topk<16>(ctx->device, p, 0, 1, st) == cudaSuccess;
+        auto places = [&](auto probe) { return probe(ctx->device, p, 0, 1, 1, st) == cudaSuccess; };
+        const bool ok = places(launch_topk<8, 0>) && places(launch_topk<16, 0>) && places(launch_topk<8, 1>) && places(launch_topk<16, 1>) &&
+                        places(launch_topk<8, 2>) && places(launch_topk<16, 2>);
         if (!ok) cudaGetLastError();
         w.store(ok ? SEL_CLUSTER : 8, std::memory_order_relaxed);
     }
-    const int widest = w.load(std::memory_order_relaxed), most = SEL_CLUSTER * B <= ctx->num_sms ? widest : 8;
-    int n_ranks = 1;
-    while (n_ranks < most && n_ranks * 8 * SEL_THREADS < max_lM) n_ranks *= 2;
-    if (n_ranks * 16 * SEL_THREADS < max_lM) n_ranks = widest;
+    const int widest = w.load(std::memory_order_relaxed);
+    auto topk = [&](auto level, int n_keys, int segs) {
+        constexpr int LEVEL = decltype(level)::value;
+        const int most = SEL_CLUSTER * B * segs <= ctx->num_sms ? widest : 8;
+        int n_ranks = 1;
+        while (n_ranks < most && n_ranks * 8 * SEL_THREADS < n_keys) n_ranks *= 2;
+        if (n_ranks * 16 * SEL_THREADS < n_keys) n_ranks = widest;
+        ctx->launches += 1;
+        return n_ranks * 8 * SEL_THREADS >= n_keys ? launch_topk<8, LEVEL>(ctx->device, p, n_ranks, segs, B, st)
+                                                   : launch_topk<16, LEVEL>(ctx->device, p, n_ranks, segs, B, st);
+    };
     ProfScope prof(ctx, KC_SELECT_TOPK, st);
-    e = n_ranks * 8 * SEL_THREADS >= max_lM ? launch_topk<8>(ctx->device, p, n_ranks, B, st) : launch_topk<16>(ctx->device, p, n_ranks, B, st);
+    // Two levels from twice the tokens that a cluster's registers hold on: there every step reads the keys from L2 again (one
+    // sequence: 200k tokens 27 us in one level, 400k 42 and 26 in two, 700k 57 and 30, 2M 128 and 41).  Segments of 65536 tokens
+    // (a cluster's registers; of sqrt(|M| k) tokens they take 26, 30 and 57), of 4 k at least, so that a segment has more than k and
+    // the candidates (keys and positions) fit a row of the unpooled keys' buffer, and of sqrt(|M| k) where the candidates would be
+    // too many for the second level.
+    if (max_lM <= SEL_TWO_LEVELS) {
+        e = topk(std::integral_constant<int, 0>(), max_lM, 1);
+    } else {
+        const int k = ctx->cfg.top_k;
+        p.cand = ctx->skey;                                  // (unpooled keys are not needed any more)
+        double seg = std::max((double)SEL_SEGMENT, 4.0 * k);
+        if (max_lM / seg * k > SEL_TWO_LEVELS) seg = std::max(seg, std::sqrt((double)max_lM * k));
+        p.seg_tokens = (int)std::min(2147483647.0, seg);
+        const int segs = select_segments(max_lM, p.seg_tokens);
+        int seg_len = 0, n_cand = 0;                         // most tokens of a segment, most keys of the second level
+        for (int b = 0; b < B; ++b) {
+            const int lM = meta.m_end[b] - meta.i_end[b], n = lM > k ? select_segments(lM, p.seg_tokens) : 1;
+            if (n > 1) seg_len = std::max(seg_len, (lM + n - 1) / n);
+            n_cand = std::max(n_cand, n > 1 ? n * k : lM);
+        }
+        e = segs > 1 ? topk(std::integral_constant<int, 1>(), seg_len, segs) : cudaSuccess;
+        if (e == cudaSuccess) e = topk(std::integral_constant<int, 2>(), n_cand, 1);
+    }
     if (e != cudaSuccess) return e;
-    ctx->launches += 1;
     return cudaGetLastError();
 }
 

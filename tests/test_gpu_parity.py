@@ -230,6 +230,12 @@ _SELECTION_EDGES = [
     ([80 + 301], 1, 32, 15, 300, 0), ([80 + 17, 80 + 18], 1, 128, 15, 4, 0),
     # long runs of equal scores over several CTAs: more ties at the threshold than are sent one by one
     ([80 + 40000], 1, 64, 0, 3333, 700), ([80 + 40000], 2, 128, 3, 9999, 5000), ([80 + 140000], 1, 32, 3, 8000, 3000),
+    # two levels: from 262145 tokens on; a few and many candidates, ties within and across segments, sequences of both kinds and
+    # one that is selected whole, chunks, a k that leaves two segments and one that leaves one
+    ([80 + 262144], 1, 32, 3, 4096, 0), ([80 + 262145], 1, 32, 3, 4096, 0), ([80 + 300000], 3, 64, 0, 1, 0),
+    ([80 + 400000], 1, 32, 3, 8000, 3000), ([80 + 900000], 1, 32, 3, 300, 100000), ([80 + 500001], 2, 32, 5, 16000, 0),
+    ([80 + 270001, 80 + 300, 80 + 70001, 80 + 131073, 80 + 65537], 1, 32, 3, 300, 0),
+    ([80 + 300000], 1, 32, 3, 70000, 0), ([80 + 280000], 1, 32, 1, 100000, 0),
 ]
 
 
