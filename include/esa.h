@@ -289,7 +289,8 @@ esa_status esa_read_compressed_queries(esa_ctx* ctx, void* dst_host, int64_t n_r
 
 /* Diagnostic (host only, no device needed): the form in which esa_attend -- or, two_position != 0, a call of
  * esa_attend_two_position with a second encoding -- deals out its key lists on a GPU of num_sms SMs: the streaming
- * kernel for single queries (its parts depend on the device: *parts = 0), or the tensor-memory kernel with the key list
+ * kernel for single queries or the one for small chunks in large batches (their parts depend on the
+ * device: *parts = 0), or the tensor-memory kernel with the key list
  * of every 256 rows in *parts parts that a second launch merges (1: unsplit), as a pair of CTAs that exchange their halves,
  * as a long and a short part, or as a pair for the two lists of two encodings.  Tensors aligned as the conventions say. */
 typedef enum {
@@ -297,7 +298,8 @@ typedef enum {
     ESA_ATTEND_PARTS = 1,
     ESA_ATTEND_PAIR = 2,
     ESA_ATTEND_UNEVEN = 3,
-    ESA_ATTEND_TWO_PAIR = 4
+    ESA_ATTEND_TWO_PAIR = 4,
+    ESA_ATTEND_SMALL = 5
 } esa_attend_form;
 esa_status esa_attend_plan(const esa_config* cfg, int32_t num_sms, int32_t B, int32_t l_C, const int64_t* n_prev,
                            int32_t two_position, int32_t* kernel, int32_t* parts);

@@ -361,7 +361,7 @@ def attend_noalloc_status(stream=None) -> int:
     return int(load_library().esa_attend_noalloc_status(_stream_ptr(stream)))
 
 
-ATTEND_FORMS = ("decode", "parts", "pair", "uneven", "two_pair")
+ATTEND_FORMS = ("decode", "parts", "pair", "uneven", "two_pair", "small")
 
 
 def attend_plan(cfg: EsaConfig, num_sms: int, l_C: int, n_prev, two_position: bool = False):

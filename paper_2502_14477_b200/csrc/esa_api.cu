@@ -545,6 +545,17 @@ esa_status esa_attend_plan(const esa_config* cfg, int32_t num_sms, int32_t B, in
     }
     const TcPlan p = plan_attend_tc(num_sms, make_layout(cfg).att_elems, cfg->head_dim, G, cfg->n_kv_heads, cfg->top_k, B, l_C, meta,
                                     two_position != 0, false);
+    int n_att_max = 0;
+    for (int b = 0; b < B; ++b) {
+        const int lM = meta.m_end[b] - meta.i_end[b], far = meta.i_end[b] + (lM < cfg->top_k ? lM : cfg->top_k);
+        const int n = far + (meta.t[b] - meta.m_end[b]) + l_C;
+        if (n > n_att_max) n_att_max = n;
+    }
+    if (attend_small_wins(num_sms, cfg->head_dim, G, cfg->n_kv_heads, B, l_C, n_att_max, two_position != 0, p.cost)) {
+        *kernel = ESA_ATTEND_SMALL;
+        *parts = 0;
+        return ESA_OK;
+    }
     if (p.nsplit == 0) return ESA_ERR_UNSUPPORTED;
     *kernel = p.mode == TC_PAIR       ? ESA_ATTEND_PAIR
               : p.mode == TC_UNEVEN   ? ESA_ATTEND_UNEVEN
@@ -566,7 +577,7 @@ const char* esa_kernel_class_name(int32_t cls) {
         "compress_tc_kernel", "compress_gemv_kernel", "compress_kernel", "append_kv_kernel", "score_tc_kernel<.,1>",
         "score_tc_kernel<.,2>", "score_decode_kernel", "score_full_kernel<.,1>+<.,2>",
         "pool_kernel",
-        "select_topk_kernel", "select_all_kernel", "attend_tc_kernel", "attend_decode_kernel",
+        "select_topk_kernel", "select_all_kernel", "attend_tc_kernel", "attend_decode_kernel", "attend_small_kernel",
         "attend_tc_merge_kernel", "gather_kv_kernel"};
     return cls >= 0 && cls < KC_COUNT ? names[cls] : "";
 }

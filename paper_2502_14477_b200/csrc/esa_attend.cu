@@ -15,8 +15,9 @@
 // that share it.  Flash-style online softmax in the exp2 domain, bf16 operands, fp32
 // scores and accumulators.
 //
-// This file holds the streaming kernel for decode (one query per sequence), the choice between it and the tcgen05
-// kernel of esa_attend_tc.cu (every other chunk), and the entry point that needs no allocation.
+// This file holds the streaming kernel for decode (one query per sequence), the kernel for small chunks in large batches, the
+// choice between them and the tcgen05 kernel of esa_attend_tc.cu (every other chunk), and the entry point that needs no allocation.
+#include <algorithm>
 #include <mutex>
 
 #include "esa_internal.h"
@@ -362,15 +363,27 @@ attend_decode_kernel(AttendParams p) {
     }
 }
 
-// The same merge as a launch of its own, a warp per row of O: for callers without arrival counters.
+// The merge as a launch of its own, a warp per row of O: for callers without arrival counters, and for small chunks.  R = l_C G
+// rows a unit.
 template <int D>
-__global__ void __launch_bounds__(256) attend_decode_merge_kernel(const float* part, int nsplit, int rows, int G, __nv_bfloat16* O) {
+__global__ void __launch_bounds__(256) attend_merge_kernel(const float* part, int nsplit, int rows, int R, int l_C, int HG, int G,
+                                                           __nv_bfloat16* O) {
     pdl_wait();
     pdl_launch_dependents();
     const int lane = threadIdx.x & 31, row = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (row >= rows) return;
-    const float* base = part + ((int64_t)(row / G) * nsplit * G + row % G) * (D + 2);
-    merge_row<D>(base, base + D, (int64_t)G * (D + 2), nsplit, lane, O + (int64_t)row * D);
+    const int unit = row / R, r = row % R;
+    const float* base = part + ((int64_t)unit * nsplit * R + r) * (D + 2);
+    const int64_t out = ((int64_t)(unit / HG) * l_C + r / G) * HG * G + unit % HG * G + r % G;
+    merge_row<D>(base, base + D, (int64_t)R * (D + 2), nsplit, lane, O + out * D);
+}
+
+template <int D>
+static cudaError_t launch_merge(esa_ctx* ctx, const AttendParams& p, int B, cudaStream_t st) {
+    const int R = p.l_C * p.G, rows = B * p.HG * R;
+    ctx->launches += 1;
+    return launch_pdl(attend_merge_kernel<D>, dim3((rows + 7) / 8), dim3(256), 0, st, (const float*)p.part, p.nsplit, rows, R, p.l_C, p.HG,
+                      p.G, p.O);
 }
 
 template <int D, int G, bool TWO>
@@ -399,10 +412,328 @@ static cudaError_t launch_decode_t(esa_ctx* ctx, AttendParams& p, int B, int n_a
     e = launch_pdl(attend_decode_kernel<D, G, TWO>, dim3(nsplit, p.HG, B), dim3(DEC_WARPS * 32), smem, st, p);
     ctx->launches += 1;
     if (e != cudaSuccess || nsplit == 1 || ctx->att_count) return e;
-    const int rows = B * p.H;
-    e = launch_pdl(attend_decode_merge_kernel<D>, dim3((rows + 7) / 8), dim3(256), 0, st, (const float*)p.part, nsplit, rows, G, p.O);
+    return launch_merge<D>(ctx, p, B, st);
+}
+
+// ---------------------------------------------------------------------------
+// Small chunks (at most 64 rows per key/value head) in large batches: a CTA of one or four warps per unit and part, flash-style
+// on mma.sync with double-buffered K/V tiles of BN rows, several CTAs an SM.  Where the units are many the tensor-memory kernel,
+// one CTA of 256 rows an SM, is bound by its chain per tile while nearly all of its rows are padding; here the SM's CTAs hide
+// each other's latency (see attend_small_wins for the line and both sides).
+// Parts of a split list, per (b, kvh, split): R rows x (D + 2) floats (unnormalised O row, running max m in the exp2 domain,
+// running sum l).
+// ---------------------------------------------------------------------------
+// TWO: the list entries of I and M_k (the first n_glob) take their logits from Qg and Kg, the entries
+// of L and C from Q and K; both score tiles are formed and each key column keeps the one that applies.
+template <int D, int NW, int BN, bool TWO>
+__global__ void __launch_bounds__(NW * 32)
+attend_small_kernel(AttendParams p) {
+    constexpr int CH = D / 8;
+    constexpr int BM = NW * 16;
+    constexpr int NT = NW * 32;
+    extern __shared__ uint4 smem[];
+    uint4* sQ = smem;                         // [BM][CH]
+    uint4* sK = sQ + BM * CH;                 // 2 x [BN][CH]
+    uint4* sV = sK + 2 * BN * CH;             // 2 x [BN][CH]
+    uint4* sQg = sV + 2 * BN * CH;            // [BM][CH] (TWO)
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int row0 = blockIdx.x * BM;
+    const int kvh = blockIdx.y;
+    const int b = blockIdx.z / p.nsplit;
+    const int split = blockIdx.z % p.nsplit;
+    const int G = p.G;
+    const int R = p.l_C * G;
+
+    pdl_wait();
+    pdl_launch_dependents();
+    const int t = p.meta.t[b], i_end = p.meta.i_end[b], m_end = p.meta.m_end[b];
+    int n_sel = p.n_sel[b];
+    n_sel = max(0, min(n_sel, min(p.top_k, m_end - i_end)));
+    const int n_glob = i_end + n_sel;                  // entries before L
+    const int n_att = n_glob + (t - m_end) + p.l_C;
+    const int c_first = n_att - p.l_C;                 // list position of the chunk's first key
+
+    // keys this row tile can see: up to the chunk key of its last query
+    const int r_last = min(R, row0 + BM) - 1;
+    const int j_end = c_first + r_last / G + 1;
+    const int n_tiles = (j_end + BN - 1) / BN;
+    const int per = (n_tiles + p.nsplit - 1) / p.nsplit;
+    const int tile_begin = split * per;
+    const int tile_end = min(n_tiles, tile_begin + per);
+
+    const __nv_bfloat16* Kb = p.K + ((int64_t)b * p.max_tokens * p.HG + kvh) * D;
+    const __nv_bfloat16* Kgb = p.Kg + ((int64_t)b * p.max_tokens * p.HG + kvh) * D;
+    const __nv_bfloat16* Vb = p.V + ((int64_t)b * p.max_tokens * p.HG + kvh) * D;
+    const int32_t* idx = p.idx + (int64_t)b * p.top_k;
+    const int64_t tok_stride = (int64_t)p.HG * D;
+
+    int bad_idx = 0;
+    auto load_kv = [&](int st, int tile) {
+        uint4* dk = sK + st * BN * CH;
+        uint4* dv = sV + st * BN * CH;
+        for (int i = tid; i < BN * CH; i += NT) {
+            int r = i / CH, c = i % CH;
+            int j = tile * BN + r;
+            bool ok = j < n_att;
+            int pos = 0;
+            if (ok) {
+                if (p.staged) pos = j;
+                else if (j < i_end) pos = j;
+                else if (j < n_glob) pos = clamp_selected(__ldg(idx + (j - i_end)), i_end, m_end, bad_idx);
+                else pos = m_end + (j - n_glob);
+            }
+            const int64_t off = (int64_t)pos * tok_stride + c * 8;
+            cp_async16(&dk[swz<CH>(r, c)], ((TWO && j < n_glob) ? Kgb : Kb) + off, ok ? 16 : 0);
+            cp_async16(&dv[swz<CH>(r, c)], Vb + off, ok ? 16 : 0);
+        }
+    };
+
+    // Q tile -> smem (rows past R are zero)
+    for (int i = tid; i < BM * CH; i += NT) {
+        int r = i / CH, c = i % CH;
+        int row = row0 + r;
+        bool ok = row < R;
+        int cq = ok ? row / G : 0, g = ok ? row % G : 0;
+        const int64_t qoff = (((int64_t)b * p.l_C + cq) * p.H + kvh * G + g) * D + c * 8;
+        cp_async16(&sQ[swz<CH>(r, c)], p.Q + qoff, ok ? 16 : 0);
+        if (TWO) cp_async16(&sQg[swz<CH>(r, c)], p.Qg + qoff, ok ? 16 : 0);
+    }
+    if (tile_begin < tile_end) load_kv(0, tile_begin);
+    cp_async_commit();
+
+    float o_acc[D / 8][4];
+#pragma unroll
+    for (int i = 0; i < D / 8; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) o_acc[i][j] = 0.f;
+    float m_run[2] = {-INFINITY, -INFINITY};
+    float l_run[2] = {0.f, 0.f};
+
+    // this thread's two rows and their causal limits (first invisible list position)
+    const int r_lo = row0 + warp * 16 + (lane >> 2);
+    const int lim_lo = c_first + min(r_lo / G, p.l_C - 1) + 1;
+    const int lim_hi = c_first + min((r_lo + 8) / G, p.l_C - 1) + 1;
+    const int warp_min_lim = c_first + min((row0 + warp * 16) / G, p.l_C - 1) + 1;
+
+    uint32_t qf[D / 16][4];
+    uint32_t qfg[TWO ? D / 16 : 1][4];
+    bool q_loaded = false;
+
+    for (int tile = tile_begin; tile < tile_end; ++tile) {
+        const int st = (tile - tile_begin) & 1;
+        if (tile + 1 < tile_end) {
+            load_kv(st ^ 1, tile + 1);
+            cp_async_commit();
+            cp_async_wait<1>();
+        } else {
+            cp_async_wait<0>();
+        }
+        __syncthreads();
+        if (!q_loaded) {
+#pragma unroll
+            for (int ks = 0; ks < D / 16; ++ks) load_a_frag<CH>(qf[ks], sQ, warp * 16, ks * 2, lane);
+            if (TWO) {
+#pragma unroll
+                for (int ks = 0; ks < D / 16; ++ks) load_a_frag<CH>(qfg[ks], sQg, warp * 16, ks * 2, lane);
+            }
+            q_loaded = true;
+        }
+        const uint4* tk = sK + st * BN * CH;
+        const uint4* tv = sV + st * BN * CH;
+
+        // S = Q K^T
+        float s[BN / 8][4];
+#pragma unroll
+        for (int i = 0; i < BN / 8; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < D / 16; ++ks) {
+#pragma unroll
+            for (int nb = 0; nb < BN / 16; ++nb) {
+                uint32_t kb[4];
+                load_b_frag_nk<CH>(kb, tk, nb * 16, ks * 2, lane);
+                mma_bf16_16816(s[2 * nb], qf[ks], kb[0], kb[1]);
+                mma_bf16_16816(s[2 * nb + 1], qf[ks], kb[2], kb[3]);
+            }
+        }
+        const int j0 = tile * BN;
+        if (TWO && j0 < n_glob) {
+            // some key columns of this tile belong to I or M_k: their logits come from Qg (the tile holds Kg rows there)
+            float sg[BN / 8][4];
+#pragma unroll
+            for (int i = 0; i < BN / 8; ++i)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) sg[i][j] = 0.f;
+#pragma unroll
+            for (int ks = 0; ks < D / 16; ++ks) {
+#pragma unroll
+                for (int nb = 0; nb < BN / 16; ++nb) {
+                    uint32_t kb[4];
+                    load_b_frag_nk<CH>(kb, tk, nb * 16, ks * 2, lane);
+                    mma_bf16_16816(sg[2 * nb], qfg[ks], kb[0], kb[1]);
+                    mma_bf16_16816(sg[2 * nb + 1], qfg[ks], kb[2], kb[3]);
+                }
+            }
+#pragma unroll
+            for (int nb = 0; nb < BN / 8; ++nb)
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+                    if (j0 + nb * 8 + (lane & 3) * 2 + e < n_glob) {
+                        s[nb][e] = sg[nb][e];
+                        s[nb][2 + e] = sg[nb][2 + e];
+                    }
+        }
+
+        // scale, mask (causal inside C and the ragged tail), online softmax
+        const bool need_mask = j0 + BN > warp_min_lim;
+        float mx_lo = -INFINITY, mx_hi = -INFINITY;
+#pragma unroll
+        for (int nb = 0; nb < BN / 8; ++nb) {
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float a = s[nb][e] * p.scale_log2, c2 = s[nb][2 + e] * p.scale_log2;
+                if (need_mask) {
+                    int j = j0 + nb * 8 + (lane & 3) * 2 + e;
+                    if (j >= lim_lo) a = -INFINITY;
+                    if (j >= lim_hi) c2 = -INFINITY;
+                }
+                s[nb][e] = a;
+                s[nb][2 + e] = c2;
+                mx_lo = fmaxf(mx_lo, a);
+                mx_hi = fmaxf(mx_hi, c2);
+            }
+        }
+        mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 1));
+        mx_lo = fmaxf(mx_lo, __shfl_xor_sync(0xffffffffu, mx_lo, 2));
+        mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 1));
+        mx_hi = fmaxf(mx_hi, __shfl_xor_sync(0xffffffffu, mx_hi, 2));
+        const float mn_lo = fmaxf(m_run[0], mx_lo), mn_hi = fmaxf(m_run[1], mx_hi);
+        const float ms_lo = (mn_lo == -INFINITY) ? 0.f : mn_lo;   // a fully masked row stays empty
+        const float ms_hi = (mn_hi == -INFINITY) ? 0.f : mn_hi;
+        const float al_lo = fast_exp2(m_run[0] - ms_lo), al_hi = fast_exp2(m_run[1] - ms_hi);
+        m_run[0] = mn_lo;
+        m_run[1] = mn_hi;
+        float sum_lo = 0.f, sum_hi = 0.f;
+        uint32_t pf[BN / 16][4];
+#pragma unroll
+        for (int nb = 0; nb < BN / 8; ++nb) {
+            float p0 = fast_exp2(s[nb][0] - ms_lo), p1 = fast_exp2(s[nb][1] - ms_lo);
+            float p2 = fast_exp2(s[nb][2] - ms_hi), p3 = fast_exp2(s[nb][3] - ms_hi);
+            sum_lo += p0 + p1;
+            sum_hi += p2 + p3;
+            pf[nb >> 1][(nb & 1) * 2] = pack_bf16(p0, p1);
+            pf[nb >> 1][(nb & 1) * 2 + 1] = pack_bf16(p2, p3);
+        }
+        l_run[0] = l_run[0] * al_lo + sum_lo;
+        l_run[1] = l_run[1] * al_hi + sum_hi;
+#pragma unroll
+        for (int nb = 0; nb < D / 8; ++nb) {
+            o_acc[nb][0] *= al_lo;
+            o_acc[nb][1] *= al_lo;
+            o_acc[nb][2] *= al_hi;
+            o_acc[nb][3] *= al_hi;
+        }
+        // O += P V
+#pragma unroll
+        for (int kk = 0; kk < BN / 16; ++kk) {
+#pragma unroll
+            for (int dp = 0; dp < D / 16; ++dp) {
+                uint32_t vb[4];
+                load_b_frag_kn<CH>(vb, tv, kk * 16, dp * 2, lane);
+                mma_bf16_16816(o_acc[2 * dp], pf[kk], vb[0], vb[1]);
+                mma_bf16_16816(o_acc[2 * dp + 1], pf[kk], vb[2], vb[3]);
+            }
+        }
+        __syncthreads();
+    }
+    cp_async_wait<0>();
+    if (bad_idx) atomicExch(p.status, kStatusBadIndex);
+
+    l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 1);
+    l_run[0] += __shfl_xor_sync(0xffffffffu, l_run[0], 2);
+    l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], 1);
+    l_run[1] += __shfl_xor_sync(0xffffffffu, l_run[1], 2);
+
+#pragma unroll
+    for (int half = 0; half < 2; ++half) {
+        const int row = r_lo + half * 8;
+        if (row >= R) continue;
+        if (p.nsplit == 1) {
+            const float inv = 1.f / l_run[half];
+            const int cq = row / G, g = row % G;
+            __nv_bfloat16* dst = p.O + (((int64_t)b * p.l_C + cq) * p.H + kvh * G + g) * D;
+#pragma unroll
+            for (int nb = 0; nb < D / 8; ++nb) {
+                int col = nb * 8 + (lane & 3) * 2;
+                *reinterpret_cast<uint32_t*>(dst + col) =
+                    pack_bf16(o_acc[nb][half * 2] * inv, o_acc[nb][half * 2 + 1] * inv);
+            }
+        } else {
+            float* dst = p.part + ((((int64_t)b * p.HG + kvh) * p.nsplit + split) * R + row) * (D + 2);
+#pragma unroll
+            for (int nb = 0; nb < D / 8; ++nb) {
+                int col = nb * 8 + (lane & 3) * 2;
+                *reinterpret_cast<float2*>(dst + col) = make_float2(o_acc[nb][half * 2], o_acc[nb][half * 2 + 1]);
+            }
+            if ((lane & 3) == 0) {
+                dst[D] = m_run[half];
+                dst[D + 1] = l_run[half];
+            }
+        }
+    }
+}
+
+template <int D, int NW, int BN, bool TWO>
+static cudaError_t launch_small_t(esa_ctx* ctx, AttendParams& p, int B, int n_att_max, cudaStream_t st) {
+    constexpr int smem = ((TWO ? 2 : 1) * NW * 16 + 4 * BN) * (D / 8) * 16;
+    static KernelMemo memo;
+    cudaError_t e = allow_smem(attend_small_kernel<D, NW, BN, TWO>, ctx->device, smem, memo);
+    if (e != cudaSuccess) return e;
+    // split the key list so that one wave of CTAs fills the machine (never a second, short wave)
+    int per_sm = 1;
+    e = resident_per_sm(attend_small_kernel<D, NW, BN, TWO>, ctx->device, NW * 32, smem, memo, &per_sm);
+    if (e != cudaSuccess) return e;
+    const int R = p.l_C * p.G, n_tiles = (n_att_max + BN - 1) / BN;
+    int nsplit = (per_sm * ctx->num_sms) / (p.HG * B);
+    if (nsplit > kAttMaxSplits) nsplit = kAttMaxSplits;
+    if (nsplit > n_tiles) nsplit = n_tiles;
+    while (nsplit > 1 && (size_t)B * p.HG * nsplit * R * (D + 2) > ctx->att_part_elems) --nsplit;
+    if (nsplit < 1) nsplit = 1;
+    p.nsplit = nsplit;
+    if (!aligned(p.Q, 16) || !aligned(p.Qg, 16) || !aligned(p.O, 4)) return kErrAlign;
+    {
+        ProfScope prof(ctx, KC_ATTEND_SMALL, st);
+        e = launch_pdl(attend_small_kernel<D, NW, BN, TWO>, dim3(1, p.HG, B * nsplit), dim3(NW * 32), smem, st, p);
+    }
     ctx->launches += 1;
-    return e;
+    if (e != cudaSuccess || nsplit == 1) return e;
+    ProfScope prof(ctx, KC_ATTEND_MERGE, st);
+    return launch_merge<D>(ctx, p, B, st);
+}
+
+template <bool TWO>
+static cudaError_t launch_small(esa_ctx* ctx, AttendParams& p, int B, int n_att_max, cudaStream_t st) {
+    const int R = p.l_C * p.G;
+    if (ctx->d == 128) return R <= 16 ? launch_small_t<128, 1, 32, TWO>(ctx, p, B, n_att_max, st) : launch_small_t<128, 4, 64, TWO>(ctx, p, B, n_att_max, st);
+    return R <= 16 ? launch_small_t<64, 1, 32, TWO>(ctx, p, B, n_att_max, st) : launch_small_t<64, 4, 64, TWO>(ctx, p, B, n_att_max, st);
+}
+
+// Units enough for most of the SMs, and an estimate below the tensor-memory kernel's (`tc_cost`, of its split rule; heads of 128
+// with two encodings: times 1.3, which measurements bear out and that rule does not need).  The estimate, fitted to 128 to 2048 units
+// over 640 to 6300 keys: 13 us and so many ns per unit and 128 keys, and no less than one CTA takes for an unsplit list.
+// 512 units of 2 rows, heads of 64, 2178 keys: 138 us on the tensor-memory kernel, 82 here; with two encodings 157 and 121;
+// 1024 units of 32 rows, 2208 keys, 244 and 201.  128 units of 8 rows, heads of 128, 6274 keys: 99 and 168.
+bool attend_small_wins(int num_sms, int D, int G, int HG, int B, int l_C, int n_att_max, bool two, double tc_cost) {
+    const int R = l_C * G, units = HG * B;
+    if (R > kAttSplitRows || units * 4 < num_sms * 3) return false;
+    const bool one_warp = R <= 16;
+    const double ns = D == 64 ? (one_warp ? 10.0 : two ? 17.0 : 11.0) : (one_warp ? (two ? 21.0 : 25.0) : two ? 29.5 : 40.0);
+    const double tiles = n_att_max / 128.0;
+    double cost = 13.0 + units * tiles * ns * 1e-3;
+    if (units > num_sms) cost = std::max(cost, 13.0 + tiles * (one_warp ? 2.6 : D == 64 ? 4.0 : 6.0));
+    return cost < tc_cost * (two && D == 128 ? 1.3 : 1.0);
 }
 
 // Decode: the streaming kernel for the usual group sizes.
@@ -447,11 +778,14 @@ cudaError_t launch_attend(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, 
         if (ctx->d == 128) return two ? launch_decode<128, true>(ctx, p, B, n_att_max, st) : launch_decode<128, false>(ctx, p, B, n_att_max, st);
         return two ? launch_decode<64, true>(ctx, p, B, n_att_max, st) : launch_decode<64, false>(ctx, p, B, n_att_max, st);
     }
+    const TcPlan plan = plan_attend_tc(ctx->num_sms, ctx->att_part_elems, ctx->d, ctx->G, ctx->HG, p.top_k, B, l_C, meta, two, p.early != 0);
+    if (attend_small_wins(ctx->num_sms, ctx->d, ctx->G, ctx->HG, B, l_C, n_att_max, two, plan.cost))
+        return two ? launch_small<true>(ctx, p, B, n_att_max, st) : launch_small<false>(ctx, p, B, n_att_max, st);
     // Any other chunk: tcgen05 kernel.  Few rows leave most of its 128-row tile empty, but the key list is then split far
     // enough that the products do not matter: 3 queries (12 rows a head) over 7400 keys 39 -> 22 us, 8 queries 32 -> 21 us
     // against a split mma.sync kernel.
-    return launch_attend_tc(ctx, B, l_C, Q, two ? p.Qg : nullptr, K, two ? p.Kg : nullptr, V, meta, idx, n_sel, O, st, cache_rows,
-                            staged);
+    return launch_attend_tc(ctx, B, l_C, Q, two ? p.Qg : nullptr, K, two ? p.Kg : nullptr, V, meta, idx, n_sel, O, plan, st,
+                            cache_rows, staged);
 }
 
 // ---------------------------------------------------------------------------

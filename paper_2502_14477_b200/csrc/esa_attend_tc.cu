@@ -967,7 +967,7 @@ TcPlan plan_attend_tc(int num_sms, size_t part_elems, int D, int G, int HG, int 
         if (two && ns > 2 && waves > 2) cost = ctas * (tile * n_tiles + 3.0 * ns) / num_sms + (tile * per + 3.0) / 2 + 4.0 + join;
         if (cost < best_cost - 1e-9) { best_cost = cost; best = ns; }
     }
-    TcPlan plan = {best, best != 2 ? TC_PARTS : two && even_out ? TC_TWO_PAIR : TC_PAIR, 0, 0, 0};
+    TcPlan plan = {best, best != 2 ? TC_PARTS : two && even_out ? TC_TWO_PAIR : TC_PAIR, 0, 0, 0, best_cost};
     // Two uneven parts (TC_UNEVEN), where one CTA per unit leaves SMs idle and a second one each would more than fill them:
     // the first parts of all units run in one wave, and the idle SMs take the second parts, `rounds` one after another.
     // The shortest first part that keeps the second ones from taking longer (start and end: 5 us each).  1024 queries of
@@ -981,17 +981,16 @@ TcPlan plan_attend_tc(int num_sms, size_t part_elems, int D, int G, int HG, int 
         const int second = std::max(0, (int)((n_tiles * 1.85 + 3.0 - 5.0 * rounds) / (1.85 * (rounds + 1))));
         const double cost = 1.85 * (n_tiles - second) + 3.0 + 4.0 + 7.5 + 2 * merge_bytes / 4e6;
         if (second > 0 && cost < best_cost - 3.0)      // (early: the second parts start beside the selection kernel, like the first)
-            plan = {2, TC_UNEVEN, n_tiles - second, early ? idle : 0, second};
+            plan = {2, TC_UNEVEN, n_tiles - second, early ? idle : 0, second, cost};
     }
     return plan;
 }
 
 template <int D, int NQT, bool FINE>
-static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, cudaStream_t st) {
+static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, TcPlan plan, int B, cudaStream_t st) {
     const int R = p.l_C * p.G;
     const int row_tiles = (R + TC_ROWS - 1) / TC_ROWS;
     p.Rp = (R + 1) & ~1;
-    TcPlan plan = plan_attend_tc(ctx->num_sms, ctx->att_part_elems, D, p.G, p.HG, p.top_k, B, p.l_C, p.meta, p.two != 0, p.early != 0);
     if (plan.nsplit == 0) return cudaErrorNotSupported;
     // Finished rows are stored 16 bytes at a time, merged ones four: an O that is not 16-byte aligned is written by the merge
     // launch, where the scratch holds two parts (always for the small chunks).
@@ -1042,8 +1041,8 @@ static cudaError_t launch_tc(esa_ctx* ctx, TcAttendParams& p, int B, cudaStream_
 
 cudaError_t launch_attend_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* Qg,
                              const __nv_bfloat16* K, const __nv_bfloat16* Kg, const __nv_bfloat16* V, const SeqMeta& meta,
-                             const int32_t* idx, const int32_t* n_sel, __nv_bfloat16* O, cudaStream_t st, int64_t cache_rows,
-                             bool staged) {
+                             const int32_t* idx, const int32_t* n_sel, __nv_bfloat16* O, const TcPlan& plan, cudaStream_t st,
+                             int64_t cache_rows, bool staged) {
     const bool two = Qg != nullptr || Kg != nullptr;
     TcAttendParams p;
     p.Q = Q; p.K = K; p.Qg = Qg ? Qg : Q; p.Kg = Kg ? Kg : K;
@@ -1058,8 +1057,8 @@ cudaError_t launch_attend_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* 
     const int rows = l_C * ctx->G;
     auto run = [&](auto dim) {
         constexpr int D = decltype(dim)::value;
-        if (rows <= kAttSplitRows) return launch_tc<D, 1, true>(ctx, p, B, st);
-        return rows <= 128 ? launch_tc<D, 1, false>(ctx, p, B, st) : launch_tc<D, 2, false>(ctx, p, B, st);
+        if (rows <= kAttSplitRows) return launch_tc<D, 1, true>(ctx, p, plan, B, st);
+        return rows <= 128 ? launch_tc<D, 1, false>(ctx, p, plan, B, st) : launch_tc<D, 2, false>(ctx, p, plan, B, st);
     };
     if (ctx->d == 128) return run(std::integral_constant<int, 128>());
     if (ctx->d == 64) return run(std::integral_constant<int, 64>());

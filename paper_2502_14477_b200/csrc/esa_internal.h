@@ -73,7 +73,7 @@ struct RowMap {
 // Kernel classes of the per-kernel timing facility (esa_set_profiling / esa_read_profile).
 enum KernelClass {
     KC_COMPRESS_TC = 0, KC_COMPRESS_GEMV, KC_COMPRESS_MMA, KC_APPEND_KV, KC_SCORE_PASS1, KC_SCORE_PASS2,
-    KC_SCORE_DECODE, KC_SCORE_FULL, KC_POOL, KC_SELECT_TOPK, KC_SELECT_ALL, KC_ATTEND_TC, KC_ATTEND_DECODE,
+    KC_SCORE_DECODE, KC_SCORE_FULL, KC_POOL, KC_SELECT_TOPK, KC_SELECT_ALL, KC_ATTEND_TC, KC_ATTEND_DECODE, KC_ATTEND_SMALL,
     KC_ATTEND_MERGE, KC_GATHER_KV, KC_COUNT
 };
 // Alignment of a caller's pointer.  Kernels load and store up to 16 bytes at once; a launch that needs more alignment than
@@ -239,14 +239,6 @@ cudaError_t launch_gather_kv(esa_ctx* ctx, int B, int l_C, const void* K_host, c
                              const int32_t* idx, const int32_t* n_sel, void* K_stage, void* V_stage, int64_t stage_rows,
                              cudaStream_t st);
 
-// Chunks on tcgen05 (the partials of a key list split more than two ways
-// pass through ctx->att_part and are merged by a second launch).
-// Qg / Kg non-null: two-position attention (both given then).
-cudaError_t launch_attend_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* Qg,
-                             const __nv_bfloat16* K, const __nv_bfloat16* Kg, const __nv_bfloat16* V, const SeqMeta& meta,
-                             const int32_t* idx, const int32_t* n_sel, __nv_bfloat16* O, cudaStream_t st,
-                             int64_t cache_rows = 0, bool staged = false);
-
 // What the CTAs of a unit (256 rows of a key/value head) of the tcgen05 attention do with their results: separate parts
 // (merged by a second launch), pairs that exchange halves, separate parts of which the first is much the longer, or pairs for
 // the two lists of two-position attention.
@@ -257,10 +249,21 @@ struct TcPlan {
     int main_tiles;     // TC_UNEVEN: tiles of the first part
     int early_units;    // the second part of the first so many units takes up to early_second tiles of the early list
     int early_second;
+    double cost;        // estimated us
 };
 TcPlan plan_attend_tc(int num_sms, size_t part_elems, int D, int G, int HG, int top_k, int B, int l_C, const SeqMeta& meta, bool two,
                       bool early);
 bool attend_decode_covers(int l_C, int G);
+// Small chunks: whether the mma.sync kernel of esa_attend.cu is taken, the plan above costing tc_cost.
+bool attend_small_wins(int num_sms, int D, int G, int HG, int B, int l_C, int n_att_max, bool two, double tc_cost);
+
+// Chunks on tcgen05 (the partials of a key list split more than two ways
+// pass through ctx->att_part and are merged by a second launch).
+// Qg / Kg non-null: two-position attention (both given then).
+cudaError_t launch_attend_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* Qg,
+                             const __nv_bfloat16* K, const __nv_bfloat16* Kg, const __nv_bfloat16* V, const SeqMeta& meta,
+                             const int32_t* idx, const int32_t* n_sel, __nv_bfloat16* O, const TcPlan& plan, cudaStream_t st,
+                             int64_t cache_rows = 0, bool staged = false);
 
 // TMA descriptor of the query tensor [n_queries, H, D] for the attention kernel (group size G must
 // divide 128).

@@ -201,6 +201,16 @@ UNEVEN_CASES = [
     (45, 45, 64, (10000,), 500, 200, 7000, None), (24, 24, 128, (9000,), 1000, 0, 7000, 6999)]
 
 
+# (H, H_G, d, B, t, step, l_C, l_L, k, two): batches of small chunks that the rule gives to the mma.sync kernel on 148 SMs; sequence b
+# holds t - step b tokens.  One and four warps a CTA, full and ragged row tiles, groups of 1, 3, 4, both head dimensions, lists
+# split (few units) and not, everything selected in the shorter sequences.
+SMALL_BATCH_CASES = [
+    (8, 8, 64, 32, 3000, 60, 2, 700, 1000, False), (8, 8, 64, 32, 3000, 60, 2, 700, 1000, True), (32, 8, 64, 32, 3000, 60, 4, 700, 1000, False),
+    (16, 16, 64, 32, 2000, 20, 17, 500, 600, False), (8, 2, 64, 64, 2000, 20, 16, 256, 300, True), (16, 16, 128, 16, 2000, 60, 3, 256, 300, True),
+    (32, 32, 64, 16, 3000, 100, 64, 400, 300, False), (32, 8, 128, 32, 2000, 30, 4, 200, 100, True), (24, 8, 64, 32, 2500, 60, 1, 700, 900, False),
+    (64, 64, 64, 4, 900, 200, 5, 300, 200, False)]
+
+
 class DeviceSeq:
     """Device caches for B sequences of a workload, filled from the seeded generators."""
 

@@ -407,6 +407,44 @@ def test_uneven_key_list_split(case):
             hp.check_attention(got[b], want, what=f"{what} seq {b}", heads=heads)
 
 
+@pytest.mark.parametrize("case", hp.SMALL_BATCH_CASES, ids=lambda c: f"{c[0]}-{c[1]}-{c[2]}-{c[3]}x{c[6]}-{c[9]}")
+def test_small_chunks_in_large_batches(case):
+    """More units of a few rows than SMs, against the oracle on sampled sequences and heads, and with the output off its boundary."""
+    from paper_2502_14477_b200.binding import attend_plan
+    H, H_G, d, B, t, step, l_C, l_L, k, two = case
+    t_list, n = [t - step * b for b in range(B)], t + l_C
+    cfg = syn.get_config("c1").with_(H=H, H_G=H_G, d=d, d_c=64, l_I=16, l_L=l_L, k=k)
+    p, heads = hp.oracle_params(cfg), sorted({0, H // 2, H - 1})
+    ctx = hp.make_esa(cfg, max_tokens=n, max_chunk=l_C, max_batch=B)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert sms != 148 or attend_plan(ctx.cfg, sms, l_C, t_list, two) == ("small", 0)
+    g = torch.Generator(device="cuda").manual_seed(H + B)
+    draw = lambda *s: torch.randn(*s, device="cuda", dtype=torch.bfloat16, generator=g)
+    Q, Qf, K, Kf, V = draw(B, l_C, H, d), draw(B, l_C, H, d), draw(B, n, H_G, d), draw(B, n, H_G, d), draw(B, n, H_G, d)
+    idx, counts = torch.zeros(B, k, dtype=torch.int32, device="cuda"), torch.zeros(B, dtype=torch.int32, device="cuda")
+    for b, tb in enumerate(t_list):
+        l_M = max(0, tb - l_L - 16)
+        c = min(k, l_M) if b % 5 else min(3, l_M)
+        idx[b, :c] = torch.sort(torch.randperm(l_M, device="cuda", generator=g)[:c])[0].int() + 16
+        counts[b] = c
+    O = torch.full_like(Q, float("nan"))
+    odd = _offset(O, 2)
+    for out in (O, odd):
+        if two:
+            ctx.attend_two_position(Q, Qf, K, Kf, V, t_list, idx, counts, out, sync=True)
+        else:
+            ctx.attend(Q, K, V, t_list, idx, counts, out, sync=True)
+    assert ctx.last_device_status() == 0
+    assert torch.equal(O, odd)
+    for b in sorted({0, 1, B // 2, B - 1}):
+        tb, m = t_list[b], t_list[b] + l_C
+        f64 = lambda x: hp.torch_to_f64(x)
+        kw = dict(Q_global=f64(Qf[b]), K_global=f64(Kf[b, :m])) if two else {}
+        sel = idx[b, : int(counts[b])].cpu().numpy().astype(np.int64)
+        want = orc.attend(f64(Q[b]), f64(K[b, :m]), f64(V[b, :m]), sel, tb, p, heads=heads, **kw)
+        hp.check_attention(O[b], want, what=f"seq {b}", heads=heads)
+
+
 # ------------------------------------------------------ end to end, config 1
 def test_c1_end_to_end_prefill_and_decode():
     cfg = syn.get_config("c1")

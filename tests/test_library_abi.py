@@ -181,3 +181,17 @@ def test_the_uneven_cases_of_the_gpu_tests_are_dealt_out_unevenly(lib):
     for H, H_G, d, ts, l_C, l_L, k, _ in hp.UNEVEN_CASES:
         cfg = esa.EsaConfig(H, H_G, d, 64, 16, l_L, k, 3, l_C, len(ts), max(ts) + l_C)
         assert attend_plan(cfg, 148, l_C, ts) == ("uneven", 2), (H, H_G, d, ts, l_C)
+
+
+def test_small_chunks_go_to_the_small_kernel_in_large_batches_only(lib):
+    import paper_2502_14477_b200 as esa
+    from paper_2502_14477_b200.binding import attend_plan
+    from tests import helpers as hp
+    for H, H_G, d, B, t, step, l_C, l_L, k, two in hp.SMALL_BATCH_CASES:
+        cfg = esa.EsaConfig(H, H_G, d, 64, 16, l_L, k, 3, l_C, B, t + l_C)
+        assert attend_plan(cfg, 148, l_C, [t - step * b for b in range(B)], two) == ("small", 0), (H, H_G, d, B, l_C)
+    # few units, or heads of 128 with long lists: the tensor-memory kernel
+    for H, H_G, d, B, l_C in ((32, 8, 128, 1, 2), (32, 8, 128, 16, 4), (8, 2, 64, 16, 8), (32, 8, 128, 8, 16)):
+        cfg = esa.EsaConfig(H, H_G, d, 64, 128, 2048, 4096, 3, l_C, B, 20000)
+        for two in (False, True):
+            assert attend_plan(cfg, 148, l_C, [16000] * B, two)[0] != "small", (H, H_G, d, B, l_C, two)
