@@ -445,8 +445,8 @@ attend_small_kernel(AttendParams p) {
     const int G = p.G;
     const int R = p.l_C * G;
 
+    // (its dependents start when its CTAs end: let in early, they take places from CTAs that are still to come, 171 us for 158)
     pdl_wait();
-    pdl_launch_dependents();
     const int t = p.meta.t[b], i_end = p.meta.i_end[b], m_end = p.meta.m_end[b];
     int n_sel = p.n_sel[b];
     n_sel = max(0, min(n_sel, min(p.top_k, m_end - i_end)));
