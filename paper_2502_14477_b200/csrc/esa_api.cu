@@ -485,6 +485,9 @@ esa_status esa_attend_host_kv_async(esa_ctx* ctx, int32_t B, const void* Q_cur, 
     }
     if (stage_rows >= (int64_t(1) << 31)) return ESA_ERR_CAPACITY;
     if (!aligned(K_host, 16) || !aligned(V_host, 16) || !aligned(K_stage, 16) || !aligned(V_stage, 16)) return ESA_ERR_INVALID_ARG;
+    // (what the attention launch will ask for, ahead of the gather; merged rows of a single query are the one case left to it)
+    const bool decode = attend_decode_covers(l_C, ctx->G);
+    if (!aligned(Q_cur, decode ? 4 : 16) || !aligned(O, decode ? 2 : 4) || !aligned(idx, 4) || !aligned(n_sel, 4)) return ESA_ERR_INVALID_ARG;
     cudaStream_t st = (cudaStream_t)stream;
     ctx->sel_armed = false;       // (the staged list is written by the gather kernel just ahead: never attended early)
     if (launch_gather_kv(ctx, B, l_C, K_host, V_host, meta, idx, n_sel, K_stage, V_stage, stage_rows, st) != cudaSuccess)

@@ -1215,6 +1215,7 @@ def test_misaligned_tensors_are_refused_or_handled():
     Kh, Vh = seq.K.cpu().pin_memory(), seq.V.cpu().pin_memory()
     O = torch.zeros_like(q1)
     refused(lambda: ctx.attend_host_kv(q1, Kh, Vh, [t], idx, n_sel, _offset(stage, 2), stage, O), O)
+    refused(lambda: ctx.attend_host_kv(_offset(q1, 1), Kh, Vh, [t], idx, n_sel, stage, stage.clone(), O), O, stage)
 
     # accepted: queries of a single-query call in words of two values, merged rows on such boundaries (lists of any length), a
     # few compressed rows anywhere, queries that are folded
