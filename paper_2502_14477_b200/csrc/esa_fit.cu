@@ -13,12 +13,13 @@
 //
 // The work of a batch of 128 pairs is 0.4 GFLOP and the 16 MB of parameters and moments live in L2, so a step is
 // bound by its chain of dependent launches and by the latency inside each.  It is three launches
-// (fit_forward_kernel, fit_pairs_kernel, fit_update_kernel) chained with programmatic dependent launch; 28 us on the
-// Llama-3-8B shape (forward 10, pairs 5, update 8, the rest boundaries), where 17 launches of generic fp32 product
-// kernels took 202 us.
+// (fit_forward_kernel, fit_pairs_kernel, fit_update_kernel) chained with programmatic dependent launch; 26 us on the
+// Llama-3-8B shape, where 17 launches of generic fp32 product kernels took 202 us.
 // The long products have one bf16 operand (the batch), so they run on mma.sync with the fp32 operand cut into three
 // bf16 pieces (w = w1 + w2 + w3, 24 significant bits): every product is exact and the sums are fp32, as with fp32
-// multiply-adds.  The tensor core truncates when it adds, so its sums are kept short (64 terms) and added up in fp32
+// multiply-adds.  The weights' pieces are kept beside the weights: the update writes both, and the forward launch copies the
+// pieces as they are (64 steps of 128 pairs and the weights read back 2035 -> 1925 us, together with the update's reads of
+// the batch ahead of its wait; cut anew by every warp of the forward launch, the pieces were two thirds of its instructions).  The tensor core truncates when it adds, so its sums are kept short (64 terms) and added up in fp32
 // registers, smallest pieces first.
 #include <cooperative_groups.h>
 
@@ -40,6 +41,8 @@ struct esa_fit {
     float* m2;                    // Adam second moments
     float *Qf, *T, *A, *Bm, *dP, *dA, *dBm;
     __nv_bfloat16 *dA3, *dBm3;    // [3][n, dc]: gradients of A and Bm as bf16 pieces
+    __nv_bfloat16 *Wq3, *Wk3;     // [3][dc, dH], [3][dc, dG]: the weights as bf16 pieces
+    bool pieces_old;              // the pieces are not those of the weights (set, or updated by the generic kernels)
     float* loss_part;             // per-band partial losses
     float* part;                  // partial sums of split reductions (generic kernels)
     float* loss_acc;              // one float
@@ -69,14 +72,14 @@ __device__ __forceinline__ void split3(float lo, float hi, uint32_t (&w)[3]) {
 // ---------------------------------------------------------------------------
 constexpr int FF_M = 32, FF_N = 32, FF_K = 64, FF_STAGES = 4, FF_CLUSTER = 8, FF_THREADS = 256;
 constexpr int FF_XBYTES = FF_M * FF_K * 2;
-constexpr int FF_YROW = (FF_K + 8) * 4;          // fp32 row stride: 8 rows x 4 column pairs of 8 bytes hit all banks
-constexpr int FF_YROW16 = (FF_K + 8) * 2;        // the same for bf16 rows
-constexpr int FF_YBYTES = FF_N * FF_YROW;
+constexpr int FF_YPIECE = FF_N * FF_K * 2;       // one bf16 piece of the fp32 operand
+constexpr int FF_YBYTES = 3 * FF_YPIECE;
 constexpr int FF_SMEM = FF_STAGES * (FF_XBYTES + FF_YBYTES);
 
 struct FitParams {
     const __nv_bfloat16 *Q, *K;
     float *Wq, *bq, *Wk, *bk;
+    __nv_bfloat16 *Wq3, *Wk3;    // [3][dc, dH], [3][dc, dG]: the weights' bf16 pieces
     float *m1, *m2;              // moments, laid out like [Wq | bq | Wk | bk]
     float *A, *Bm, *T;           // [n, dc], [n, dc], [n, n]
     __nv_bfloat16 *dA, *dBm;     // [3][n, dc]: the pieces of the gradients of A and Bm
@@ -105,7 +108,7 @@ __global__ void __launch_bounds__(FF_THREADS, 3) fit_forward_kernel(FitParams p)
     const int r0 = (job / cols) * FF_M, c0 = (job % cols) * FF_N;
     const __nv_bfloat16* X = kind == 1 ? p.K : p.Q;
     const int kdim = kind == 1 ? p.dG : p.dH;                // columns of X, all reduced over
-    const float* Y = kind == 0 ? p.Wq : p.Wk;                // fp32 operand of A and Bm
+    const __nv_bfloat16* Y = kind == 0 ? p.Wq3 : p.Wk3;      // fp32 operand of A and Bm, in pieces
     const int n_cols = kind == 2 ? p.n : p.dc;
     const int chunks = (kdim + FF_K - 1) / FF_K;
     const int per = (chunks + FF_CLUSTER - 1) / FF_CLUSTER;
@@ -124,19 +127,18 @@ __global__ void __launch_bounds__(FF_THREADS, 3) fit_forward_kernel(FitParams p)
                 const bool ok = r0 + r < p.n && k < kdim;
                 cp_async16(reinterpret_cast<uint4*>(sx) + swz<FF_K / 8>(r, c), X + (ok ? (int64_t)(r0 + r) * kdim + k : 0), ok ? 16 : 0);
             }
+            const int r = tid / (FF_K / 8), c = tid % (FF_K / 8), k = k0 + c * 8;
             if (kind == 2) {
                 // row m of K, the column of the head's group (a 16-byte chunk stays inside a head)
-                const int r = tid / (FF_K / 8), c = tid % (FF_K / 8), k = k0 + c * 8;
                 const bool ok = c0 + r < p.n && k < kdim;
                 const int g = k / p.d / p.G;
-                cp_async16(sy + r * FF_YROW16 + c * 16, p.K + (ok ? (int64_t)(c0 + r) * p.dG + g * p.d + k % p.d : 0), ok ? 16 : 0);
+                cp_async16(reinterpret_cast<uint4*>(sy) + swz<FF_K / 8>(r, c), p.K + (ok ? (int64_t)(c0 + r) * p.dG + g * p.d + k % p.d : 0), ok ? 16 : 0);
             } else {
+                const bool ok = c0 + r < p.dc && k < kdim;
 #pragma unroll
-                for (int i = tid; i < FF_N * (FF_K / 4); i += FF_THREADS) {
-                    const int r = i / (FF_K / 4), c = i % (FF_K / 4), k = k0 + c * 4;
-                    const bool ok = c0 + r < p.dc && k < kdim;
-                    cp_async16(sy + r * FF_YROW + c * 16, Y + (ok ? (int64_t)(c0 + r) * kdim + k : 0), ok ? 16 : 0);
-                }
+                for (int q = 0; q < 3; ++q)
+                    cp_async16(reinterpret_cast<uint4*>(sy + q * FF_YPIECE) + swz<FF_K / 8>(r, c),
+                               Y + (ok ? ((int64_t)q * p.dc + c0 + r) * kdim + k : 0), ok ? 16 : 0);
             }
         }
         cp_async_commit();
@@ -165,29 +167,21 @@ __global__ void __launch_bounds__(FF_THREADS, 3) fit_forward_kernel(FitParams p)
             for (int m = 0; m < FF_M / 16; ++m)
 #pragma unroll
                 for (int e = 0; e < 4; ++e) acc[q][m][e] = 0.f;
+        static_assert(FF_K / 16 / KQ == 2, "one ldmatrix holds a warp's two k-steps of a piece");
+        uint32_t a[2][FF_M / 16][4];
 #pragma unroll
-        for (int kk = 0; kk < FF_K / 16 / KQ; ++kk) {
-            const int ks = kh + kk;
-            uint32_t a[FF_M / 16][4];
+        for (int kk = 0; kk < 2; ++kk)
 #pragma unroll
-            for (int m = 0; m < FF_M / 16; ++m) load_a_frag<FF_K / 8>(a[m], reinterpret_cast<const uint4*>(sx), m * 16, ks * 2, lane);
-            const int row = wn + (lane >> 2), k = ks * 16 + (lane & 3) * 2;
-            if (kind == 2) {
-                const uint32_t b0 = *reinterpret_cast<const uint32_t*>(sy + row * FF_YROW16 + k * 2);
-                const uint32_t b1 = *reinterpret_cast<const uint32_t*>(sy + row * FF_YROW16 + (k + 8) * 2);
+            for (int m = 0; m < FF_M / 16; ++m) load_a_frag<FF_K / 8>(a[kk][m], reinterpret_cast<const uint4*>(sx), m * 16, (kh + kk) * 2, lane);
 #pragma unroll
-                for (int m = 0; m < FF_M / 16; ++m) mma_bf16_16816(acc[0][m], a[m], b0, b1);
-            } else {
-                const float2 f0 = *reinterpret_cast<const float2*>(sy + row * FF_YROW + k * 4);
-                const float2 f1 = *reinterpret_cast<const float2*>(sy + row * FF_YROW + (k + 8) * 4);
-                uint32_t b0[3], b1[3];
-                split3(f0.x, f0.y, b0);
-                split3(f1.x, f1.y, b1);
+        for (int q = 0; q < 3; ++q) {
+            if (q > 0 && kind == 2) break;                   // (bf16 as it is)
+            uint32_t b[4];
+            ldmatrix_x4(b, reinterpret_cast<const uint4*>(sy + q * FF_YPIECE) + swz<FF_K / 8>(wn + (lane & 7), kh * 2 + (lane >> 3)));
 #pragma unroll
-                for (int q = 0; q < 3; ++q)
+            for (int kk = 0; kk < 2; ++kk)
 #pragma unroll
-                    for (int m = 0; m < FF_M / 16; ++m) mma_bf16_16816(acc[q][m], a[m], b0[q], b1[q]);
-            }
+                for (int m = 0; m < FF_M / 16; ++m) mma_bf16_16816(acc[q][m], a[kk][m], b[2 * kk], b[2 * kk + 1]);
         }
 #pragma unroll
         for (int m = 0; m < FF_M / 16; ++m)
@@ -340,6 +334,17 @@ __global__ void __launch_bounds__(FP_THREADS) fit_pairs_kernel(FitParams p) {
 }
 
 // ---------------------------------------------------------------------------
+// The pieces of weights that were set, or updated by the generic kernels.
+__global__ void fit_pieces_kernel(const float* __restrict__ W, __nv_bfloat16* __restrict__ W3, int64_t count) {
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x) {
+        uint32_t w[3];
+        split3(W[e], 0.f, w);
+#pragma unroll
+        for (int q = 0; q < 3; ++q) W3[q * count + e] = __ushort_as_bfloat16((unsigned short)(w[q] & 0xffffu));
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Launch 3: gradients and Adam.  A CTA owns a FU_J x FU_N tile of W_q or W_k: its gradient, reduced over the pairs,
 // stays in the accumulators and the update is applied from there, so gradients never go to memory.  Tiles of 32 x 128
 // read the least (6 bytes per feature and pair in pieces, 2 per column and pair: 56 KB a CTA for 128 pairs, against
@@ -418,6 +423,7 @@ __global__ void __launch_bounds__(FU_THREADS, 2) fit_update_kernel(FitParams p) 
     const __nv_bfloat16* X = qs ? p.Q : p.K;
     const __nv_bfloat16* D = qs ? p.dA : p.dBm;
     float* W = qs ? p.Wq : p.Wk;
+    __nv_bfloat16* W3 = qs ? p.Wq3 : p.Wk3;
     const int64_t base = W - p.Wq;
 
     // this thread's elements of the tile: rows jb + warp + 16 u, four columns
@@ -432,11 +438,9 @@ __global__ void __launch_bounds__(FU_THREADS, 2) fit_update_kernel(FitParams p) 
         a1[u] = __ldcg(reinterpret_cast<const float4*>(p.m1 + off));
         a2[u] = __ldcg(reinterpret_cast<const float4*>(p.m2 + off));
     }
-    pdl_wait();
-    pdl_launch_dependents();
-    auto load = [&](int c0) {
+    auto load_d = [&](int c0) {
+        uint8_t* st = fu_smem + ((c0 / FU_C) % FU_STAGES) * FU_STAGE;
         if (c0 < n) {
-            uint8_t* st = fu_smem + ((c0 / FU_C) % FU_STAGES) * FU_STAGE;
 #pragma unroll
             for (int i = tid; i < 3 * FU_C * (FU_J / 8); i += FU_THREADS) {
                 const int q = i / (FU_C * (FU_J / 8)), r = i / (FU_J / 8) % FU_C, c = i % (FU_J / 8);
@@ -444,6 +448,11 @@ __global__ void __launch_bounds__(FU_THREADS, 2) fit_update_kernel(FitParams p) 
                 cp_async16(reinterpret_cast<uint4*>(st + q * FU_PBYTES) + swz<FU_J / 8>(r, c),
                            D + (ok ? ((int64_t)q * n + c0 + r) * dc + jb + c * 8 : 0), ok ? 16 : 0);
             }
+        }
+    };
+    auto load_x = [&](int c0) {
+        uint8_t* st = fu_smem + ((c0 / FU_C) % FU_STAGES) * FU_STAGE;
+        if (c0 < n) {
 #pragma unroll
             for (int i = tid; i < FU_C * (FU_N / 8); i += FU_THREADS) {
                 const int r = i / (FU_N / 8), c = i % (FU_N / 8);
@@ -452,8 +461,12 @@ __global__ void __launch_bounds__(FU_THREADS, 2) fit_update_kernel(FitParams p) 
                            X + (ok ? (int64_t)(c0 + r) * ld + i0 + c * 8 : 0), ok ? 16 : 0);
             }
         }
-        cp_async_commit();
     };
+    // the batch was read by the launch before the last as well: the first two chunks of it come ahead of the wait, too
+    load_x(0);
+    load_x(FU_C);
+    pdl_wait();
+    pdl_launch_dependents();
     // warps: 2 groups of 16 features x 8 of 16 columns
     const int wj = (warp & 1) * 16, wi = (warp >> 1) * 16;
     float g[2][4];
@@ -461,10 +474,12 @@ __global__ void __launch_bounds__(FU_THREADS, 2) fit_update_kernel(FitParams p) 
     for (int nb = 0; nb < 2; ++nb)
 #pragma unroll
         for (int e = 0; e < 4; ++e) g[nb][e] = 0.f;
-    load(0);
+    load_d(0);
+    cp_async_commit();
+    load_d(FU_C);
+    cp_async_commit();
     for (int c0 = 0; c0 < n; c0 += FU_C) {
-        load(c0 + FU_C);
-        cp_async_wait<1>();
+        cp_async_wait<FU_STAGES - 1>();
         __syncthreads();
         const uint8_t* st = fu_smem + ((c0 / FU_C) % FU_STAGES) * FU_STAGE;
         {
@@ -494,6 +509,9 @@ __global__ void __launch_bounds__(FU_THREADS, 2) fit_update_kernel(FitParams p) 
             }
         }
         __syncthreads();
+        load_d(c0 + FU_STAGES * FU_C);
+        load_x(c0 + FU_STAGES * FU_C);
+        cp_async_commit();
     }
     cp_async_wait<0>();
     // gradient tile -> shared memory (the stages are idle), row stride FU_N + 4
@@ -517,6 +535,12 @@ __global__ void __launch_bounds__(FU_THREADS, 2) fit_update_kernel(FitParams p) 
         adam(w[u].z, a1[u].z, a2[u].z, gr.z, p);
         adam(w[u].w, a1[u].w, a2[u].w, gr.w, p);
         *reinterpret_cast<float4*>(p.Wq + off) = w[u];
+        uint32_t lo[3], hi[3];
+        split3(w[u].x, w[u].y, lo);
+        split3(w[u].z, w[u].w, hi);
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+            *reinterpret_cast<uint2*>(W3 + ((int64_t)q * dc + jr + 16 * u) * ld + i0 + ic) = make_uint2(lo[q], hi[q]);
         *reinterpret_cast<float4*>(p.m1 + off) = a1[u];
         *reinterpret_cast<float4*>(p.m2 + off) = a2[u];
     }
@@ -737,7 +761,8 @@ esa_status esa_fit_create(const esa_config* cfg, int32_t batch, float lr, esa_fi
     const size_t n = batch, dc = f->dc;
     const size_t part_floats = 32 * (n * n > n * dc ? n * n : n * dc);
     const size_t piece_floats = (3 * n * dc + 1) / 2 + 4;      // 3 n dc bf16 values, rounded up
-    const size_t floats = 4 * f->n_params + n * f->dG + 2 * n * n + 4 * n * dc + part_floats + 2 * piece_floats + n + 128;
+    const size_t weight_floats = (3 * f->n_params + 1) / 2 + 8;  // 3 bf16 values a weight
+    const size_t floats = 4 * f->n_params + weight_floats + n * f->dG + 2 * n * n + 4 * n * dc + part_floats + 2 * piece_floats + n + 128;
     if (cudaGetDevice(&f->device) != cudaSuccess || cudaMalloc(&f->base, floats * sizeof(float)) != cudaSuccess) {
         cudaGetLastError();
         delete f;
@@ -754,6 +779,11 @@ esa_status esa_fit_create(const esa_config* cfg, int32_t batch, float lr, esa_fi
     f->dA3 = reinterpret_cast<__nv_bfloat16*>(p); p += piece_floats;
     p = align16(p);
     f->dBm3 = reinterpret_cast<__nv_bfloat16*>(p); p += piece_floats;
+    p = align16(p);
+    f->Wq3 = reinterpret_cast<__nv_bfloat16*>(p);
+    f->Wk3 = f->Wq3 + 3 * dc * f->dH;
+    p += weight_floats;
+    f->pieces_old = true;
     f->loss_part = p; p += n;
     f->grads = p; p += f->n_params;
     f->Qf = p; p += n * f->dG;
@@ -797,6 +827,7 @@ esa_status esa_fit_set_weights(esa_fit* f, const float* Wq, const float* bq, con
     if (bq && cudaMemcpy(f->params + obq, bq, sizeof(float) * f->dc, cudaMemcpyHostToDevice) != cudaSuccess) return ESA_ERR_CUDA;
     if (bk && cudaMemcpy(f->params + obk, bk, sizeof(float) * f->dc, cudaMemcpyHostToDevice) != cudaSuccess) return ESA_ERR_CUDA;
     f->step = 0;
+    f->pieces_old = true;
     return ESA_OK;
 }
 
@@ -831,9 +862,21 @@ esa_status esa_fit_step_async(esa_fit* f, const void* Q_batch, const void* K_bat
         f->step += 1;
         p.ic1 = 1.f / (1.f - std::pow(f->beta1, (float)f->step));
         p.ic2 = 1.f / (1.f - std::pow(f->beta2, (float)f->step));
+        p.Wq3 = f->Wq3; p.Wk3 = f->Wk3;
         f->launches += 3;
+        if (f->pieces_old) {
+            // (a step that is being captured does not run now: the pieces stay old for the one after it)
+            cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+            if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) return ESA_ERR_CUDA;
+            fit_pieces_kernel<<<256, 256, 0, st>>>(Wq, f->Wq3, (int64_t)dc * dH);
+            fit_pieces_kernel<<<256, 256, 0, st>>>(Wk, f->Wk3, (int64_t)dc * dG);
+            if (cudaGetLastError() != cudaSuccess) return ESA_ERR_CUDA;
+            f->launches += 2;
+            f->pieces_old = capture != cudaStreamCaptureStatusNone;
+        }
         return launch_fit_step(f->device, p, st) == cudaSuccess ? ESA_OK : ESA_ERR_CUDA;
     }
+    f->pieces_old = true;
     // targets (Eq. 3 for every pair)
     fit_fold_kernel<<<(unsigned)(((int64_t)n * dG + 255) / 256), 256, 0, st>>>(Q, f->Qf, n, f->H, f->HG, f->d);
     int launches = 5;                                  // fold, loss, two column sums, Adam

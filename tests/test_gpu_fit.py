@@ -71,6 +71,37 @@ def test_fit_steps_at_tile_edges(kw, n, steps):
         assert d.max() <= 2.5 * 5e-4, key
 
 
+def test_fit_steps_on_the_two_routes_in_turn():
+    """Batches on a 16-byte boundary and off it (the generic kernels) in turn, and weights set anew in between: every step starts from
+    the weights of the step before it, whichever kernels made them.  Oracle and tolerance of the tests above."""
+    import paper_2502_14477_b200 as esa
+    cfg, n, lr = syn.get_config("c1"), 48, 5e-4
+    fit = esa.EsaFit(esa.EsaConfig(cfg.H, cfg.H_G, cfg.d, cfg.d_c, cfg.l_I, cfg.l_L, cfg.k, cfg.eps, 1, 1, 16), n, lr)
+    wq, wk = syn.compressor_weights(cfg)
+    loss = torch.zeros(1, dtype=torch.float32, device="cuda")
+
+    def off(x):
+        flat = torch.empty(x.numel() + 1, dtype=x.dtype, device="cuda")[1:]
+        flat.copy_(x.flatten())
+        return flat.view(x.shape)
+
+    for scale in (1.0, 0.5):
+        fit.set_weights(scale * wq, None, scale * wk, None)
+        P = {"Wq": scale * wq.astype(np.float64), "bq": np.zeros(cfg.d_c), "Wk": scale * wk.astype(np.float64), "bk": np.zeros(cfg.d_c)}
+        st = fo.AdamState(lr=lr)
+        for it, odd in enumerate((False, True, False, False, True, False)):
+            Qb, Kb = syn.qkv_rows(cfg, "q", it * n, it * n + n), syn.qkv_rows(cfg, "k", it * n, it * n + n)
+            Q, K = hp.bits_to_torch(Qb).contiguous(), hp.bits_to_torch(Kb).contiguous()
+            fit.step(off(Q) if odd else Q, off(K) if odd else K, loss)
+            want = fo.fit_step(P, syn.bf16_bits_to_f64(Qb), syn.bf16_bits_to_f64(Kb), st)
+            assert abs(float(loss[0]) - want) <= 2e-4 * abs(want), (scale, it)
+        for key, got in zip(("Wq", "bq", "Wk", "bk"), fit.get_weights()):
+            d = np.abs(got.astype(np.float64) - P[key])
+            assert (d > 2e-6 + 1e-4 * np.abs(P[key])).mean() <= 2e-3, key
+            assert d.max() <= 2.5 * lr, key
+    fit.close()
+
+
 def test_fitting_lowers_the_loss_and_raises_the_recall_of_the_selection():
     """A short fit on the mixture workload: the loss falls, and the selection made with the fitted
     compressors recovers more of the full-dimension selection (Fig. 3's recall) than the one made
