@@ -109,6 +109,13 @@ __device__ __forceinline__ float fast_exp2(float x) {
     return y;
 }
 
+// Last barrier of a thread-block cluster whose CTAs read each other's shared memory: no CTA ends before the others' reads are
+// done, which they are when their values have been used.  Relaxed: an ordinary cluster barrier would first wait for this
+// CTA's stores to global memory.
+__device__ __forceinline__ void cluster_leave() {
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;\nbarrier.cluster.wait.aligned;\n" ::: "memory");
+}
+
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *reinterpret_cast<uint32_t*>(&v);

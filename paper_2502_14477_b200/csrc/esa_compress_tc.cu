@@ -170,7 +170,8 @@ compress_tc_kernel(const __grid_constant__ CUtensorMap xmap, const __grid_consta
         __nv_bfloat16* o = p.dst + ((int64_t)b * p.seq_stride + p.map.row0[b] + ii) * DC + c4;
         *reinterpret_cast<uint2*>(o) = make_uint2(pack_bf16(s.x, s.y), pack_bf16(s.z, s.w));
     }
-    cluster.sync();    // shared memory stays alive until every remote read is done
+    __syncwarp();
+    cluster_leave();   // shared memory stays alive until every remote read is done
     if (warp == 1) tmem_dealloc(tmem, DC < 32 ? 32 : DC);
 }
 

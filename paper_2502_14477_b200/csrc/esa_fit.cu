@@ -223,7 +223,8 @@ __global__ void __launch_bounds__(FF_THREADS, 3) fit_forward_kernel(FitParams p)
             else p.T[(int64_t)r * p.n + c] = s;
         }
     }
-    cluster.sync();          // shared memory stays alive until every remote read is done
+    __syncwarp();
+    cluster_leave();         // shared memory stays alive until every remote read is done
 }
 
 // ---------------------------------------------------------------------------
