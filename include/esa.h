@@ -291,8 +291,8 @@ esa_status esa_read_compressed_queries(esa_ctx* ctx, void* dst_host, int64_t n_r
  * esa_attend_two_position with a second encoding -- deals out its key lists on a GPU of num_sms SMs: the streaming
  * kernel for single queries or the one for small chunks in large batches (their parts depend on the
  * device: *parts = 0), or the tensor-memory kernel with the key list
- * of every 256 rows in *parts parts that a second launch merges (1: unsplit), as a pair of CTAs that exchange their halves,
- * as a long and a short part, or as a pair for the two lists of two encodings.  Tensors aligned as the conventions say. */
+ * of every 256 rows in *parts parts that a second launch merges (1: unsplit), for a pair of CTAs (which share it, or take
+ * half each and exchange), as a long and a short part, or for a pair with the two lists of two encodings.  Tensors aligned as the conventions say. */
 typedef enum {
     ESA_ATTEND_DECODE = 0,
     ESA_ATTEND_PARTS = 1,

@@ -559,6 +559,14 @@ esa_status esa_attend_plan(const esa_config* cfg, int32_t num_sms, int32_t B, in
         *parts = 0;
         return ESA_OK;
     }
+    if (attend_pair_covers(cfg->head_dim, l_C, G)) {
+        const PairDeal d = plan_attend_pair(num_sms, make_layout(cfg).att_elems, G, cfg->n_kv_heads, cfg->top_k, B, l_C, meta, false);
+        if (attend_pair_wins(d, p)) {
+            *kernel = d.units > d.whole * d.pairs ? ESA_ATTEND_UNEVEN : two_position ? ESA_ATTEND_TWO_PAIR : ESA_ATTEND_PAIR;
+            *parts = 2;
+            return ESA_OK;
+        }
+    }
     if (p.nsplit == 0) return ESA_ERR_UNSUPPORTED;
     *kernel = p.mode == TC_PAIR       ? ESA_ATTEND_PAIR
               : p.mode == TC_UNEVEN   ? ESA_ATTEND_UNEVEN

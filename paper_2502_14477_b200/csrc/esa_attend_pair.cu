@@ -1,0 +1,869 @@
+// Eq. 1 / Algorithm 1 for chunks of more than 128 rows per key/value head, heads of 128: CTA pairs on the
+// 5th-generation tensor cores.
+//
+//   * A unit is 256 rows (row = query c * G + head-in-group g) of one key/value head.  A pair of CTAs (a thread-block
+//     cluster) works on it: CTA r holds rows r * 128 .. + 127 as its Q tile, and every product is one tcgen05.mma of both
+//     (cta_group::2, M = 256, N = 128).  A 128-key tile crosses L2 once per pair: CTA r gathers its keys r * 64 .. + 63 of K
+//     and columns r * 64 .. + 63 of V, which is half of what a CTA with two Q tiles of its own gathers per product.
+//   * That leaves tensor memory for three score tiles per CTA (3 x 128 columns, P in bf16 over the scores it came from)
+//     beside O (128 columns): the products of a tile no longer wait for the softmax of the tile before it.  (With one score
+//     tile per Q tile the loop was a chain S -> softmax -> P V -> next S: 3900 cycles per 128 keys and 256 rows, of which
+//     the tensor core idled 1100.)
+//     512 queries of the 32/8-head shape over 6784 keys 60.4 -> 54.2 us, with two encodings 61.4 -> 54, 1024 queries of the 28/4-head
+//     shape over 13.4k keys 181 -> 168.  What bounds it now: a tile takes 1680 cycles, against 1024 of the tensor core and 1024 of the
+//     special-function unit; a warpgroup spends 2600 of its 3360 on a tile (exponentials 1800) and waits 500 for its scores.
+//   * Two softmax warpgroups take the tiles in turn, a thread per row.  They share the row's running maximum: it is set by
+//     the first half tile of a unit, handed over through shared memory, and after that only raised when a half's
+//     sum of 2^(score - m) reaches 2^64.  A raise is by a whole number, so that what the other warpgroup has
+//     formed with the old maximum is brought up to date by an exact power of two: a warpgroup looks at the maximum once
+//     more after the tile before its own is decided and before it gives its P away.
+//   * Warps of a CTA: 0-3 / 4-7 softmax of the even / odd tiles, 8-11 gather Q and K/V (index-driven 16-byte cp.async into
+//     128-byte-swizzled tiles, four stages of K and five of V), 12 and 13 issue the scores and P V (even CTA) or pass on to it which
+//     K and V tiles their CTA has loaded (odd CTA).  (One warp for both kinds of products was busy issuing all the time: beside the softmax
+//     warps of its scheduler a product costs it 137 cycles, not 64; 64.9 us.)
+//   * The other CTA is told with arrivals of CTA scope: what they announce lies in the telling CTA's own shared or tensor memory, behind
+//     the fence of the proxy that the products read through.  (An arrival that releases at cluster scope waits for all of the
+//     thread's earlier accesses: 74 us.)
+//   * Units and SMs.  Pairs are persistent: pair p takes `whole` units, p, p + pairs, ..., and then the p-th of `pairs` equal
+//     ranges of the units left over, whose parts (O, m, l) a second launch merges.  Units that fit the SMs need neither.
+//   * A call that follows the selection of its step (p.early) takes the attended set as two lists: I then L, whose rows are
+//     older than the chunk and do not depend on the selection, before the wait for the preceding kernel, and M_k then
+//     C after it.
+//   * Two-position attention (Section 3.2): the tiles of I and M_k use (Qg, Kg), those of L and C (Q, K); both Q tiles are
+//     in shared memory, and whatever is accumulated, the softmax is one over both lists.
+#include <algorithm>
+#include <cstring>
+
+#include "esa_attend_tc.cuh"
+#include "esa_internal.h"
+#include "esa_umma.cuh"
+
+namespace esa {
+
+namespace {
+
+constexpr int AP_D = 128;             // head dimension
+constexpr int AP_BN = 128;            // keys per tile
+constexpr int AP_HALF = 64;           // keys per softmax step
+constexpr int AP_ROWS = 256;          // rows per unit
+constexpr int AP_S = 3;               // score tiles in tensor memory
+constexpr int AP_KS = 4;              // K tiles in shared memory
+constexpr int AP_VS = 5;              // V tiles (used three tiles later)
+constexpr int AP_SOFTMAX_WARPS = 8;
+constexpr int AP_PRODUCER_WARPS = 4;
+constexpr int AP_MMA_WARP = AP_SOFTMAX_WARPS + AP_PRODUCER_WARPS;
+constexpr int AP_THREADS = 512;       // 13 working warps, padded to whole warpgroups for setmaxnreg
+constexpr int AP_PRODUCERS = AP_PRODUCER_WARPS * 32;
+// Register split after start-up: setmaxnreg.inc draws from the pool the CTA was launched with.
+constexpr int AP_REGS_LAUNCH = 128;
+constexpr int AP_REGS_SOFTMAX = 168;
+constexpr int AP_REGS_OTHER = 88;
+static_assert(8 * AP_REGS_SOFTMAX + 8 * AP_REGS_OTHER <= 16 * AP_REGS_LAUNCH,
+              "register split exceeds the CTA's launch allocation: setmaxnreg.inc would never return");
+constexpr int AP_Q_BYTES = 128 * AP_D * 2;       // one CTA's Q tile: two 64-column blocks
+constexpr int AP_Q_BLK = 128 * 128;
+constexpr int AP_K_BYTES = 64 * AP_D * 2;        // one CTA's half of a K tile: 64 keys, two 64-column blocks
+constexpr int AP_K_BLK = 64 * 128;
+constexpr int AP_V_BYTES = AP_BN * 128;          // one CTA's half of a V tile: 128 keys x 64 columns
+constexpr int AP_SMEM = 2 * AP_Q_BYTES + AP_KS * AP_K_BYTES + AP_VS * AP_V_BYTES + 1024;
+constexpr int AP_PART = AP_ROWS * (AP_D + 2);    // floats of a part in the scratch: O [256][128], (m, l) [256][2]
+
+struct PairParams {
+    const __nv_bfloat16* Q;
+    const __nv_bfloat16* K;
+    const __nv_bfloat16* Qg;   // two-position attention (Section 3.2): queries / keys used against I and M_k
+    const __nv_bfloat16* Kg;
+    const __nv_bfloat16* V;
+    __nv_bfloat16* O;
+    const int32_t* idx;
+    const int32_t* n_sel;
+    float* part;
+    int* status;
+    int64_t max_tokens;
+    int l_C, H, HG, G, top_k;
+    PairDeal deal;
+    int q_tma;          // Q tiles arrive by TMA (one arrival) instead of cp.async (one per producer thread)
+    int staged;         // the caches hold the attended list itself: row j = list entry j
+    int early;          // the rows of I and L are attended ahead of the wait for the preceding kernel (never with staged or two)
+    int wide_O;         // O is 16-byte aligned
+    float scale_log2;
+    SeqMeta meta;
+};
+
+// barrier slots in shared memory.  Those that the issuing warp of the even CTA waits on count arrivals of both CTAs.
+enum {
+    AB_Q_FULL = 0,                       // per Q buffer
+    AB_K_FULL = AB_Q_FULL + 2,
+    AB_V_FULL = AB_K_FULL + AP_KS,
+    AB_QK_DONE = AB_V_FULL + AP_VS,      // by tile % AP_KS: scores ready, K stage free
+    AB_PV_DONE = AB_QK_DONE + AP_KS,     // by tile % AP_VS: V stage free
+    AB_P_READY = AB_PV_DONE + AP_VS,     // by tile % AP_S: P written, maximum decided
+    AB_M_READY = AB_P_READY + AP_S,      // per unit: its first maximum is in shared memory
+    AB_O_FREE = AB_M_READY + 1,          // per unit: the accumulator has been read
+    AB_COUNT = AB_O_FREE + 1
+};
+
+// What a pair does, one after another: a unit or a range of one.
+struct Segment {
+    int b, kvh, row0;
+    int lo, hi, of;             // range of the unit's tiles, in `of`-ths
+    int part, n_parts, slot;    // n_parts > 1: part `part` goes to scratch slot `slot`
+};
+__device__ __forceinline__ bool segment(const PairDeal& d, int HG, int pair, int i, Segment& s) {
+    int u;
+    if (i < d.whole) {
+        u = pair + i * d.pairs;
+        if (u >= d.units) return false;
+        s.lo = 0;
+        s.hi = s.of = 1;
+        s.part = s.slot = 0;
+        s.n_parts = 1;
+    } else {
+        const int rest = d.units - d.whole * d.pairs;
+        if (rest <= 0) return false;
+        s.of = deal_weight(d);
+        const int x0 = deal_start(d, pair) * rest, x1 = deal_start(d, pair + 1) * rest, v = x0 / s.of + (i - d.whole);
+        s.lo = max(x0 - v * s.of, 0);
+        s.hi = min(x1 - v * s.of, s.of);
+        if (s.lo >= s.hi) return false;
+        int first;
+        deal_parts(d, v, first, s.n_parts);
+        s.part = pair - first;
+        s.slot = v * d.max_parts + s.part;
+        u = d.whole * d.pairs + v;
+    }
+    s.row0 = (u % d.row_tiles) * AP_ROWS;
+    const int h = u / d.row_tiles;
+    s.kvh = h % HG;
+    s.b = h / HG;
+    return true;
+}
+
+// An attended list: entry j is cache row j below `ie`, idx[j - ie] below `ng`, cache row me + (j - ng) from there on, and
+// nothing from `row_lim` on.
+struct KeyList { int ie, ng, me, row_lim; };
+
+struct Late {            // the late (or only) list of a unit
+    KeyList list;
+    int c_first;         // entry of the chunk's first token
+    int far_tiles;       // two encodings: tiles of I and M_k, which come first
+    int begin, end;      // tiles of the segment
+};
+
+template <bool TWO>
+__global__ void __launch_bounds__(AP_THREADS, 1)
+attend_pair_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap qgmap, const __grid_constant__ PairParams p) {
+    extern __shared__ uint8_t smem_dyn[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~uintptr_t(1023));
+    uint8_t* sQ = smem;                               // two buffers: unit after unit, or (TWO) far and near
+    uint8_t* sK = sQ + 2 * AP_Q_BYTES;
+    uint8_t* sV = sK + AP_KS * AP_K_BYTES;
+    __shared__ uint64_t bars[AB_COUNT];
+    __shared__ float m_row[2][128];                   // running maxima (log2 domain) of the units in turn
+    __shared__ float l_row[2][2][128];                // [unit][warpgroup]
+    __shared__ uint32_t tmem_slot;
+    __shared__ int abort_flag;
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int warp_u = __shfl_sync(0xffffffffu, warp, 0);     // provably warp-uniform copy
+    const int rank = blockIdx.x & 1, pair = blockIdx.x >> 1;
+    const int R = p.l_C * p.G;
+
+    WaitCtx wc{&abort_flag, p.status};
+    auto bar = [&](int i) { return smem_u32(&bars[i]); };
+
+    if (tid == 0) {
+        abort_flag = 0;
+        const int relay = rank == 0 ? 1 : 0;          // the odd CTA's loads are reported to the even one
+        for (int s = 0; s < 2; ++s) mbar_init(bar(AB_Q_FULL + s), (p.q_tma ? 1 : AP_PRODUCERS) + relay);
+        for (int s = 0; s < AP_KS; ++s) {
+            mbar_init(bar(AB_K_FULL + s), AP_PRODUCERS + relay);
+            mbar_init(bar(AB_QK_DONE + s), 1);
+        }
+        for (int s = 0; s < AP_VS; ++s) {
+            mbar_init(bar(AB_V_FULL + s), AP_PRODUCERS + relay);
+            mbar_init(bar(AB_PV_DONE + s), 1);
+        }
+        for (int s = 0; s < AP_S; ++s) mbar_init(bar(AB_P_READY + s), 128 + 4 * relay);
+        mbar_init(bar(AB_M_READY), 128);
+        mbar_init(bar(AB_O_FREE), 16);                // a warp of either CTA each
+        mbar_init_fence();
+    }
+    if (warp == 0) tmem_alloc_pair(smem_u32(&tmem_slot), 512);
+    tc_fence_before_sync();
+    __syncthreads();
+    cluster_arrive();
+    cluster_wait();
+    tc_fence_after_sync();
+    const uint32_t tmem = tmem_slot;
+    // columns: scores of tile j at (j % 3) * 128 (half u at + u * 64); O at 384
+
+    bool planned = false;
+    auto plan = [&]() {
+        if (planned) return;
+        pdl_wait();
+        pdl_launch_dependents();
+        planned = true;
+    };
+    auto early_len = [&](const Segment& s) { return p.early ? p.meta.i_end[s.b] + (p.meta.t[s.b] - p.meta.m_end[s.b]) : 0; };
+    // early tiles of a segment: rounded down at both ends, the late ones up, so that neighbours differ by a tile in all
+    auto early_range = [&](const Segment& s, int& begin, int& end) {
+        const int all = (early_len(s) + AP_BN - 1) / AP_BN;
+        begin = (int)((int64_t)all * s.lo / s.of);
+        end = (int)((int64_t)all * s.hi / s.of);
+    };
+    auto late_list = [&](const Segment& s) {          // after `plan`
+        const int t = p.meta.t[s.b], i_end = p.meta.i_end[s.b], m_end = p.meta.m_end[s.b];
+        const int n_sel = max(0, min(p.n_sel[s.b], min(p.top_k, m_end - i_end)));
+        Late l;
+        if (p.early) l.list = {0, n_sel, t, n_sel + p.l_C};
+        else l.list = {i_end, i_end + n_sel, m_end, i_end + n_sel + (t - m_end) + p.l_C};
+        l.c_first = l.list.row_lim - p.l_C;
+        const int r_last = min(R, s.row0 + AP_ROWS) - 1;
+        const int j_end = l.c_first + r_last / p.G + 1;           // keys visible to the last row of the unit
+        l.far_tiles = TWO ? (l.list.ng + AP_BN - 1) / AP_BN : 0;
+        const int all = l.far_tiles + (j_end - (TWO ? l.list.ng : 0) + AP_BN - 1) / AP_BN;
+        l.begin = all - (int)((int64_t)all * (s.of - s.lo) / s.of);
+        l.end = all - (int)((int64_t)all * (s.of - s.hi) / s.of);
+        return l;
+    };
+    // first entry of late tile i
+    auto late_key = [&](const Late& l, int i) { return TWO && i >= l.far_tiles ? l.list.ng + (i - l.far_tiles) * AP_BN : i * AP_BN; };
+
+    if (warp_u < AP_SOFTMAX_WARPS) reg_alloc<AP_REGS_SOFTMAX>();
+    else reg_dealloc<AP_REGS_OTHER>();
+
+    if (warp_u < AP_SOFTMAX_WARPS) {
+        // ------------------------------------------------------------ softmax, one row per thread
+        const int wg = warp_u >> 2;
+        const int lane_base = (warp_u & 3) * 32;         // TMEM lanes this warp may touch
+        const int wrow = lane_base + lane;               // row within the CTA
+        const uint32_t tO = tmem_addr(tmem, lane_base, AP_S * 128);
+        const uint32_t lead_bars = cluster_map(smem_u32(bars), 0);      // barriers of the even CTA
+        const float sl2 = p.scale_log2;
+        int j = 0;                                       // tiles of all segments so far
+        int n_unit = 0;                                  // segments with tiles so far
+
+        Segment s;
+#pragma unroll 1
+        for (int i = 0; segment(p.deal, p.HG, pair, i, s); ++i) {
+            const int row = s.row0 + rank * 128 + wrow;
+            const int j0 = j, buf = n_unit & 1;
+            // entries of the chunk that this row sees, and the fewest that a row of the CTA does
+            const int sees = min(row / p.G, p.l_C - 1) + 1, sees_min = min((s.row0 + rank * 128) / p.G, p.l_C - 1) + 1;
+            const int e_len = early_len(s);
+            float m_run = -INFINITY, l_run = 0.f;
+            int e_begin, e_end;
+            early_range(s, e_begin, e_end);
+            Late late;
+#pragma unroll 1
+            for (int phase = 0; phase < 2; ++phase) {
+                int begin = e_begin, end = e_end;
+                if (phase == 1) {
+                    plan();
+                    late = late_list(s);
+                    begin = late.begin;
+                    end = late.end;
+                }
+                // (the other warpgroup takes every other tile)
+                const int j_base = j;
+                j += end - begin;
+#pragma unroll 1
+                for (int jt = j_base + ((j_base ^ wg) & 1); jt < j; jt += 2) {
+                    const int T = begin + (jt - j_base);
+                    const bool first = jt == j0;
+                    const int sb = jt % AP_S, turn = jt / AP_S;
+                    const uint32_t tS = tmem_addr(tmem, lane_base, sb * 128);
+                    const bool far = TWO && phase == 1 && T < late.far_tiles;
+                    const int key_tile = phase == 0 ? T * AP_BN : late_key(late, T);
+                    // first invisible entry of this row, and the smallest such limit of the CTA's rows
+                    const int lim = phase == 0 ? e_len : far ? late.list.ng : late.c_first + sees;
+                    const int lim_min = phase == 0 ? e_len : far ? late.list.ng : late.c_first + sees_min;
+                    // the barrier of the tile before
+                    const int prev_p = AB_P_READY + (sb == 0 ? AP_S - 1 : sb - 1), prev_par = (sb == 0 ? turn - 1 : turn) & 1;
+                    if (jt == j0 + 1) {
+                        // every row has its first visible key in the unit's first half tile, if it has one at all
+                        mbar_wait(bar(AB_M_READY), n_unit & 1, wc);
+                        m_run = m_row[buf][wrow];
+                    }
+                    mbar_wait(bar(AB_QK_DONE + jt % AP_KS), (jt / AP_KS) & 1, wc);
+                    tc_fence_after_sync();
+                    // multiplies the stored P of half h by a power of two
+                    auto scale_p = [&](int h, float a) {
+                        uint32_t q[32];
+                        tmem_wait_st();
+                        tmem_ld32(tS + h * 64, q);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int c = 0; c < 32; ++c)
+                            q[c] = pack_bf16(__uint_as_float(q[c] << 16) * a, __uint_as_float(q[c] & 0xffff0000u) * a);
+                        tmem_st32(tS + h * 64, q);
+                    };
+#pragma unroll 1
+                    for (int u = 0; u < 2; ++u) {
+                        const int key0 = key_tile + u * AP_HALF;
+                        uint32_t v[AP_HALF];             // the score row of this thread
+                        tmem_ld32(tS + u * 64, v);
+                        tmem_ld32(tS + u * 64 + 32, v + 32);
+                        tmem_wait_ld();
+                        if (key0 + AP_HALF > lim_min) {
+#pragma unroll
+                            for (int c = 0; c < AP_HALF; ++c)
+                                if (key0 + c >= lim) v[c] = 0xff800000u;   // -inf
+                        }
+                        auto max_score = [&]() {
+                            float mxc[8];
+#pragma unroll
+                            for (int c = 0; c < 8; ++c) mxc[c] = fmaxf(__uint_as_float(v[2 * c]), __uint_as_float(v[2 * c + 1]));
+#pragma unroll
+                            for (int o = 16; o < AP_HALF; o += 16)
+#pragma unroll
+                                for (int c = 0; c < 8; ++c)
+                                    mxc[c] = fmax3(mxc[c], __uint_as_float(v[o + 2 * c]), __uint_as_float(v[o + 2 * c + 1]));
+                            return fmaxf(fmax3(mxc[0], mxc[1], mxc[2]), fmax3(fmax3(mxc[3], mxc[4], mxc[5]), mxc[6], mxc[7])) * sl2;
+                        };
+                        // P = 2^(S * scale - m) as packed bf16 over the first 32 columns of this half; returns the sum.
+                        // A row without a visible key has m = -inf: its P must be 0, not 2^(+inf).
+                        uint32_t pk[AP_HALF / 2];
+                        auto exps = [&](float m) {
+                            const float neg_m = (m == -INFINITY) ? 0.f : -m;
+                            const float2 sl2v = make_float2(sl2, sl2), nm = make_float2(neg_m, neg_m);
+                            float2 sum4[4] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+                            for (int c = 0; c < AP_HALF / 2; ++c) {
+                                const float2 x = ffma2(make_float2(__uint_as_float(v[2 * c]), __uint_as_float(v[2 * c + 1])), sl2v, nm);
+                                float2 e;
+                                e.x = fast_exp2(x.x);
+                                e.y = fast_exp2(x.y);
+                                sum4[c & 3] = fadd2(sum4[c & 3], e);
+                                pk[c] = pack_bf16(e.x, e.y);
+                            }
+                            const float2 a = fadd2(sum4[0], sum4[1]), c = fadd2(sum4[2], sum4[3]);
+                            return (a.x + a.y) + (c.x + c.y);
+                        };
+                        if (first && u == 0) {
+                            m_run = max_score();
+                            m_row[buf][wrow] = m_run;
+                            mbar_arrive(bar(AB_M_READY));
+                        }
+                        float sum = exps(m_run);
+                        // The decision is taken per warp: tensor-memory accesses are warp-wide.
+                        const bool raise = !(sum < kSumLimit);           // also true for inf and NaN
+                        if (__any_sync(0xffffffffu, raise)) {
+                            if (!first) mbar_wait(bar(prev_p), prev_par, wc);     // the maximum is this warpgroup's to change now
+                            const float m_cur = m_row[buf][wrow];
+                            const float by = raise ? fmaxf(ceilf(max_score() - m_cur), 0.f) : 0.f;
+                            const float m_new = m_cur + by;
+                            const float a_own = m_run == m_new ? 1.f : fast_exp2(rintf(m_run - m_new));
+                            if (u == 1) scale_p(0, a_own);
+                            if (!first) {
+                                // O must be quiescent: wait for the P V product of the previous tile
+                                mbar_wait(bar(AB_PV_DONE + (jt - 1) % AP_VS), ((jt - 1) / AP_VS) & 1, wc);
+                                tc_fence_after_sync();
+                                const float a_o = m_cur == m_new ? 1.f : fast_exp2(rintf(m_cur - m_new));
+#pragma unroll
+                                for (int c0 = 0; c0 < AP_D; c0 += 32) {
+                                    uint32_t o[32];
+                                    tmem_ld32(tO + c0, o);
+                                    tmem_wait_ld();
+#pragma unroll
+                                    for (int c = 0; c < 32; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * a_o);
+                                    tmem_st32(tO + c0, o);
+                                }
+                            }
+                            l_run *= a_own;
+                            m_run = m_new;
+                            m_row[buf][wrow] = m_new;
+                            sum = exps(m_run);
+                        }
+                        tmem_st32(tS + u * 64, pk);
+                        l_run += sum;
+                    }
+                    if (!first) {
+                        // has the other warpgroup raised the maximum in the tile before this one?
+                        mbar_wait(bar(prev_p), prev_par, wc);
+                        const float m_cur = m_row[buf][wrow];
+                        const bool raised = m_cur != m_run;
+                        if (__any_sync(0xffffffffu, raised)) {
+                            const float a = raised ? fast_exp2(rintf(m_run - m_cur)) : 1.f;
+                            scale_p(0, a);
+                            scale_p(1, a);
+                            l_run *= a;
+                            m_run = m_cur;
+                        }
+                    }
+                    tmem_wait_st();
+                    tc_fence_before_sync();
+                    mbar_arrive(bar(AB_P_READY + sb));
+                    if (rank == 1) {
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive_remote(lead_bars + 8 * (AB_P_READY + sb));
+                    }
+                }
+            }
+
+            // ---- end of the segment: O / l, or the unnormalised part for the merge
+            const bool row_ok = row < R;
+            const int cq = row_ok ? row / p.G : 0, g = row_ok ? row % p.G : 0;
+            float* part = p.part + (int64_t)s.slot * AP_PART;
+            if (j == j0) {
+                if (s.n_parts > 1 && wg == 0) __stcg(reinterpret_cast<float2*>(part + AP_ROWS * AP_D) + rank * 128 + wrow, make_float2(-INFINITY, 0.f));
+                continue;
+            }
+            mbar_wait(bar(AB_PV_DONE + (j - 1) % AP_VS), ((j - 1) / AP_VS) & 1, wc);
+            mbar_wait(bar(AB_P_READY + (j - 1) % AP_S), ((j - 1) / AP_S) & 1, wc);      // (the last maximum: m_row)
+            tc_fence_after_sync();
+            const float m_fin = m_row[buf][wrow];
+            l_row[buf][wg][wrow] = m_run == m_fin || l_run == 0.f ? l_run : l_run * fast_exp2(rintf(m_run - m_fin));
+            asm volatile("bar.sync 1, 256;\n" ::: "memory");
+            const float l = l_row[buf][0][wrow] + l_row[buf][1][wrow];
+            // warpgroup w has columns w * 64 .. + 63 of its row
+            uint32_t o[64];
+            tmem_ld32(tO + wg * 64, o);
+            tmem_ld32(tO + wg * 64 + 32, o + 32);
+            tmem_wait_ld();
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_remote(lead_bars + 8 * AB_O_FREE);
+            if (s.n_parts > 1) {
+                float4* dst = reinterpret_cast<float4*>(part + (rank * 128 + wrow) * AP_D + wg * 64);
+#pragma unroll
+                for (int c = 0; c < 16; ++c)
+                    __stcg(dst + c, make_float4(__uint_as_float(o[4 * c]), __uint_as_float(o[4 * c + 1]), __uint_as_float(o[4 * c + 2]),
+                                                __uint_as_float(o[4 * c + 3])));
+                if (wg == 0) __stcg(reinterpret_cast<float2*>(part + AP_ROWS * AP_D) + rank * 128 + wrow, make_float2(m_fin, l));
+            } else if (row_ok) {
+                const float inv = 1.f / l;
+                __nv_bfloat16* dst = p.O + (((int64_t)s.b * p.l_C + cq) * p.H + s.kvh * p.G + g) * AP_D + wg * 64;
+                uint32_t w[32];
+#pragma unroll
+                for (int c = 0; c < 32; ++c) w[c] = pack_bf16(__uint_as_float(o[2 * c]) * inv, __uint_as_float(o[2 * c + 1]) * inv);
+                if (p.wide_O) {
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) reinterpret_cast<uint4*>(dst)[c] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 32; ++c) reinterpret_cast<uint32_t*>(dst)[c] = w[c];
+                }
+            }
+            ++n_unit;
+        }
+        plan();       // (a pair without work)
+    } else if (warp_u < AP_MMA_WARP) {
+        // ------------------------------------------------------------ producers: Q, then K/V tiles
+        const int ptid = tid - AP_SOFTMAX_WARPS * 32;      // 0..127
+        auto load_q = [&](const Segment& s, bool q_far, int buf) {
+            uint8_t* dst = sQ + buf * AP_Q_BYTES;
+            const int r0 = s.row0 + rank * 128;
+            if (p.q_tma) {
+                if (ptid == 0) {
+                    mbar_arrive_expect_tx(bar(AB_Q_FULL + buf), AP_Q_BYTES);
+                    const CUtensorMap* qm = q_far ? &qgmap : &qmap;
+#pragma unroll
+                    for (int blk = 0; blk < AP_D / 64; ++blk)
+                        tma_load_3d(smem_u32(dst + blk * AP_Q_BLK), qm, blk * 64, s.kvh * p.G, s.b * p.l_C + r0 / p.G, bar(AB_Q_FULL + buf));
+                }
+                return;
+            }
+            // group sizes that do not divide 128: 16-byte copies, row by row
+            constexpr int CH = AP_D / 8;
+            const int chunk = ptid % CH, rsub = ptid / CH, cin = chunk & 7;
+            const __nv_bfloat16* Qsrc = q_far ? p.Qg : p.Q;
+            for (int r = rsub; r < 128; r += AP_PRODUCERS / CH) {
+                const bool ok = r0 + r < R;
+                const int cq = ok ? (r0 + r) / p.G : 0, g = ok ? (r0 + r) % p.G : 0;
+                const int64_t qoff = (((int64_t)s.b * p.l_C + cq) * p.H + s.kvh * p.G + g) * AP_D + chunk * 8;
+                cp_async16(dst + (chunk >> 3) * AP_Q_BLK + r * 128 + ((cin ^ (r & 7)) << 4), Qsrc + qoff, ok ? 16 : 0);
+            }
+            cp_async_arrive_noinc(bar(AB_Q_FULL + buf));
+        };
+        // Four threads share a row (one instruction of the four covers 64 contiguous bytes of it: whole sectors), so a thread
+        // works out the cache position of four keys per tile; two of them are also K rows of this CTA.
+        constexpr int RPP = AP_PRODUCERS / 4;              // rows per pass: 32
+        const int q4 = ptid % 4, rfirst = ptid / 4;
+        const int64_t tok_stride = (int64_t)p.HG * AP_D;
+        // chunk c of row r of a block goes to byte r * 128 + (((c & 7) ^ (r & 7)) << 4); rows 32 apart swizzle alike
+        const uint32_t row_off = (uint32_t)(rfirst * 128) | (uint32_t)((rfirst & 7) << 4);
+        int bad_idx = 0;
+        int j = 0, n_unit = 0;
+        int last[2] = {-1, -1};                            // last tile of the latest unit, and of the one before it
+        int ks = 0, vs = 0;                                // stages, and parities of their previous releases
+        uint32_t kph = 1, vph = 1;
+        Segment s;
+#pragma unroll 1
+        for (int i = 0; segment(p.deal, p.HG, pair, i, s); ++i) {
+            const int i_end = p.meta.i_end[s.b], m_end = p.meta.m_end[s.b];
+            const int64_t head = ((int64_t)s.b * p.max_tokens * p.HG + s.kvh) * AP_D + q4 * 8;
+            const __nv_bfloat16* Kb = p.K + head;
+            const __nv_bfloat16* Kgb = p.Kg + head;
+            const __nv_bfloat16* Vb = p.V + head + rank * 64;
+            const int32_t* idx = p.idx + (int64_t)s.b * p.top_k;
+            const int j0 = j;
+            int e_begin, e_end;
+            early_range(s, e_begin, e_end);
+#pragma unroll 1
+            for (int phase = 0; phase < 2; ++phase) {
+                int begin = e_begin, end = e_end;
+                Late late;
+                if (phase == 1) {
+                    plan();
+                    late = late_list(s);
+                    begin = late.begin;
+                    end = late.end;
+                } else {
+                    late.list = {i_end, i_end, m_end, early_len(s)};
+                    late.far_tiles = 0;
+                }
+                // cache positions of this thread's four keys of a tile; bit it of from_idx: read from the selection
+                auto positions = [&](int T, int (&pos)[4]) {
+                    const int key0 = phase == 0 ? T * AP_BN : late_key(late, T);
+                    const int row_lim = TWO && phase == 1 && T < late.far_tiles ? late.list.ng : late.list.row_lim;
+                    uint32_t from_idx = 0;
+#pragma unroll
+                    for (int it = 0; it < 4; ++it) {
+                        const int jj = key0 + rfirst + it * RPP;
+                        int q = -1;
+                        if (jj >= row_lim) q = -1;
+                        else if (p.staged || jj < late.list.ie) q = jj;
+                        else if (jj < late.list.ng) {
+                            q = __ldg(idx + (jj - late.list.ie));
+                            from_idx |= 1u << it;
+                        } else q = late.list.me + (jj - late.list.ng);
+                        pos[it] = q;
+                    }
+                    return from_idx;
+                };
+                // (a tile's index loads are in flight while the copies of the tile before it are issued)
+                int next[4] = {0, 0, 0, 0};
+                uint32_t next_idx = begin < end ? positions(begin, next) : 0u;
+                for (int T = begin; T < end; ++T, ++j) {
+                    if (j == j0) {
+                        // The Q buffers: free when the last products with what they hold have run.  (A release further back than
+                        // the stages reach has been seen already, by the wait for its stage.)
+                        const int before = TWO ? last[0] : last[1];
+                        if (before >= 0 && before >= j - AP_KS) mbar_wait(bar(AB_QK_DONE + before % AP_KS), (before / AP_KS) & 1, wc);
+                        if (TWO) {
+                            load_q(s, true, 0);
+                            load_q(s, false, 1);
+                        } else {
+                            load_q(s, false, n_unit & 1);
+                        }
+                    }
+                    const bool far = TWO && phase == 1 && T < late.far_tiles;
+                    int pos[4];
+#pragma unroll
+                    for (int it = 0; it < 4; ++it) pos[it] = next[it];
+                    const uint32_t from_idx = next_idx;
+                    if (T + 1 < end) next_idx = positions(T + 1, next);
+                    mbar_wait(bar(AB_QK_DONE + ks), kph, wc);
+#pragma unroll
+                    for (int it = 0; it < 4; ++it)
+                        if ((from_idx >> it) & 1u) pos[it] = clamp_selected(pos[it], i_end, m_end, bad_idx);
+#pragma unroll
+                    for (int it = 0; it < 2; ++it) {
+                        const int q = rank == 0 ? pos[it] : pos[2 + it];
+                        const __nv_bfloat16* src = (far ? Kgb : Kb) + (q < 0 ? 0 : q) * tok_stride;
+                        uint8_t* dst = sK + ks * AP_K_BYTES + it * RPP * 128;
+#pragma unroll
+                        for (int c = 0; c < 4; ++c)        // chunk 4 c + q4
+                            cp_async16(dst + (c >> 1) * AP_K_BLK + (row_off ^ (uint32_t)((((c & 1) << 2) + q4) << 4)), src + c * 32, q < 0 ? 0 : 16);
+                    }
+                    cp_async_arrive_noinc(bar(AB_K_FULL + ks));
+                    mbar_wait(bar(AB_PV_DONE + vs), vph, wc);
+#pragma unroll
+                    for (int it = 0; it < 4; ++it) {
+                        const int q = pos[it];
+                        const __nv_bfloat16* src = Vb + (q < 0 ? 0 : q) * tok_stride;
+                        uint8_t* dst = sV + vs * AP_V_BYTES + it * RPP * 128;
+#pragma unroll
+                        for (int c = 0; c < 2; ++c)
+                            cp_async16(dst + (row_off ^ (uint32_t)(((c << 2) + q4) << 4)), src + c * 32, q < 0 ? 0 : 16);
+                    }
+                    cp_async_arrive_noinc(bar(AB_V_FULL + vs));
+                    if (++ks == AP_KS) { ks = 0; kph ^= 1; }
+                    if (++vs == AP_VS) { vs = 0; vph ^= 1; }
+                }
+            }
+            if (j > j0) {
+                ++n_unit;
+                last[1] = last[0];
+                last[0] = j - 1;
+            }
+        }
+        plan();
+        if (bad_idx) atomicExch(p.status, kStatusBadIndex);
+        cp_async_wait<0>();
+    } else if (warp_u == AP_MMA_WARP || warp_u == AP_MMA_WARP + 1) {
+        // Walks the tiles of all segments in order.  `refill` leaves the number of tiles at hand in `rem` (those ahead of the wait
+        // for the preceding kernel first), or 0 at the end.
+        Segment s;
+        int seg = -1, stage = 1, rem = 0, tile = 0, far_tiles = 0, n_unit = -1;
+        int n_all = 0;
+        bool first = false, done = false;
+        auto refill = [&]() {
+            while (rem == 0 && !done) {
+                if (stage == 1) {
+                    if (!segment(p.deal, p.HG, pair, ++seg, s)) {
+                        done = true;
+                        break;
+                    }
+                    int begin, end;
+                    early_range(s, begin, end);
+                    stage = 0;
+                    rem = end - begin;
+                    tile = 0;
+                    far_tiles = 0;
+                    first = true;
+                } else {
+                    plan();
+                    const Late l = late_list(s);
+                    stage = 1;
+                    rem = l.end - l.begin;
+                    tile = l.begin;
+                    far_tiles = l.far_tiles;
+                }
+            }
+        };
+        const uint32_t lead = lane == 0;
+        if (rank == 0) {
+            // -------------------------------------------------------- MMA issue: one converged warp, lane 0 leads
+            constexpr uint32_t ID_QK = idesc_bf16(256, AP_BN, false, false);
+            constexpr uint32_t ID_PV = idesc_bf16(256, AP_D, false, true);
+            const uint32_t hi = desc_hi_sw128(), tm = tmem;
+            const uint32_t qlo = desc_lo_kmajor(smem_u32(sQ)), klo = desc_lo_kmajor(smem_u32(sK));
+            const uint32_t vlo = desc_lo_mnmajor(smem_u32(sV), AP_V_BYTES);
+            int j = 0;
+            if (warp_u == AP_MMA_WARP) {
+                while (refill(), !done) {
+                    const bool far = TWO && tile < far_tiles;
+                    if (first) {
+                        ++n_unit;
+                        if (TWO) {
+                            mbar_wait(bar(AB_Q_FULL + 0), n_unit & 1, wc);
+                            mbar_wait(bar(AB_Q_FULL + 1), n_unit & 1, wc);
+                        } else {
+                            mbar_wait(bar(AB_Q_FULL + (n_unit & 1)), (n_unit >> 1) & 1, wc);
+                        }
+                        first = false;
+                    }
+                    const int sk = j % AP_KS;
+                    mbar_wait(bar(AB_K_FULL + sk), (j / AP_KS) & 1, wc);
+                    if (j >= AP_S) mbar_wait(bar(AB_PV_DONE + (j - AP_S) % AP_VS), ((j - AP_S) / AP_VS) & 1, wc);
+                    fence_async_smem();
+                    tc_fence_after_sync();
+                    const uint32_t a0 = qlo + (TWO ? (far ? 0 : 1) : n_unit & 1) * (AP_Q_BYTES >> 4);
+                    const uint32_t b0 = klo + sk * (AP_K_BYTES >> 4);
+                    const uint32_t d = tm + (j % AP_S) * 128;
+#pragma unroll
+                    for (int ks = 0; ks < AP_D / 16; ++ks)
+                        umma_ss_pair(d, a0 + (((ks >> 2) * AP_Q_BLK + (ks & 3) * 32) >> 4), b0 + (((ks >> 2) * AP_K_BLK + (ks & 3) * 32) >> 4),
+                                     hi, ID_QK, ks, lead);
+                    umma_commit_pair(bar(AB_QK_DONE + sk), lead);
+                    ++j; ++tile; --rem;
+                }
+            } else {
+                while (refill(), !done) {
+                    const bool fresh = first;
+                    if (first) {
+                        ++n_unit;
+                        if (n_unit > 0) mbar_wait(bar(AB_O_FREE), (n_unit - 1) & 1, wc);
+                        first = false;
+                    }
+                    const int sv = j % AP_VS;
+                    mbar_wait(bar(AB_V_FULL + sv), (j / AP_VS) & 1, wc);
+                    mbar_wait(bar(AB_P_READY + j % AP_S), (j / AP_S) & 1, wc);
+                    fence_async_smem();
+                    tc_fence_after_sync();
+                    const uint32_t pcol = tm + (j % AP_S) * 128;
+#pragma unroll
+                    for (int ks = 0; ks < AP_BN / 16; ++ks)
+                        umma_ts_pair(tm + AP_S * 128, pcol + (ks >> 2) * 64 + (ks & 3) * 8, vlo + ((sv * AP_V_BYTES + ks * 2048) >> 4), hi, ID_PV,
+                                     ks > 0 || !fresh, lead);
+                    umma_commit_pair(bar(AB_PV_DONE + sv), lead);
+                    ++j; --rem;
+                }
+            }
+            n_all = j;
+            // (the last arrival from the odd CTA)
+            if (warp_u != AP_MMA_WARP && n_unit >= 0) mbar_wait(bar(AB_O_FREE), n_unit & 1, wc);
+        } else {
+            // -------------------------------------------------------- the odd CTA: what has been loaded here is reported to the even one
+            const uint32_t lead_bars = cluster_map(smem_u32(bars), 0);
+            int j = 0;
+            while (refill(), !done) {
+                auto pass_on = [&](int b, int parity) {
+                    mbar_wait(bar(b), parity, wc);
+                    fence_async_smem();                    // copies by the generic proxy, read by the products through the other
+                    if (lead) mbar_arrive_remote(lead_bars + 8 * b);
+                };
+                if (first && warp_u == AP_MMA_WARP) {
+                    ++n_unit;
+                    if (TWO) {
+                        pass_on(AB_Q_FULL + 0, n_unit & 1);
+                        pass_on(AB_Q_FULL + 1, n_unit & 1);
+                    } else {
+                        pass_on(AB_Q_FULL + (n_unit & 1), (n_unit >> 1) & 1);
+                    }
+                    first = false;
+                }
+                if (warp_u == AP_MMA_WARP) pass_on(AB_K_FULL + j % AP_KS, (j / AP_KS) & 1);
+                else pass_on(AB_V_FULL + j % AP_VS, (j / AP_VS) & 1);
+                ++j;
+                --rem;
+            }
+            n_all = j;
+        }
+        plan();
+        // The releases of the last V stages, which nobody fetches into again, are seen here, so that no arrival is still on its
+        // way to this CTA's shared memory when it ends.
+        for (int j = max(0, n_all - AP_VS); j < n_all; ++j) mbar_wait(bar(AB_PV_DONE + j % AP_VS), (j / AP_VS) & 1, wc);
+    } else {
+        plan();
+    }
+
+    // neither CTA leaves, or frees its tensor memory, while the other may still use it
+    tc_fence_before_sync();
+    __syncthreads();
+    cluster_leave();
+    if (warp == 0) tmem_dealloc_pair(tmem, 512);
+}
+
+// Merge of the units dealt out in ranges: a warp per row.
+__global__ void __launch_bounds__(256) attend_pair_merge_kernel(const float* part, PairDeal d, int R, int G, int HG, int H, int l_C, __nv_bfloat16* O) {
+    pdl_wait();
+    pdl_launch_dependents();
+    const int lane = threadIdx.x & 31, v = blockIdx.x / (AP_ROWS / 8), r = (blockIdx.x % (AP_ROWS / 8)) * 8 + (threadIdx.x >> 5);
+    const int u = d.whole * d.pairs + v, row = (u % d.row_tiles) * AP_ROWS + r, h = u / d.row_tiles;
+    int first, n_parts;
+    deal_parts(d, v, first, n_parts);
+    if (row >= R || n_parts == 1) return;            // (one part: written as it is)
+    const float* unit = part + (int64_t)v * d.max_parts * AP_PART;
+    merge_row<AP_D>(unit + r * AP_D, unit + AP_ROWS * AP_D + 2 * r, AP_PART, n_parts, lane,
+                    O + (((int64_t)(h / HG) * l_C + row / G) * H + (h % HG) * G + row % G) * AP_D);
+}
+
+template <bool TWO>
+cudaError_t launch_pair_kernel(esa_ctx* ctx, const CUtensorMap& qmap, const CUtensorMap& qgmap, const PairParams& p, cudaStream_t st) {
+    static KernelMemo memo;
+    cudaError_t e = allow_smem(attend_pair_kernel<TWO>, ctx->device, AP_SMEM, memo);
+    if (e != cudaSuccess) return e;
+    // the in-kernel register split assumes the launch allocation it was sized for
+    static std::atomic<bool> regs_checked{false};
+    if (!regs_checked.load(std::memory_order_relaxed)) {
+        cudaFuncAttributes fa;
+        e = cudaFuncGetAttributes(&fa, attend_pair_kernel<TWO>);
+        if (e != cudaSuccess) return e;
+        if (fa.numRegs != AP_REGS_LAUNCH) return cudaErrorInvalidConfiguration;
+        regs_checked.store(true, std::memory_order_relaxed);
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * p.deal.pairs);
+    cfg.blockDim = dim3(AP_THREADS);
+    cfg.dynamicSmemBytes = AP_SMEM;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = 2;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, attend_pair_kernel<TWO>, qmap, qgmap, p);
+}
+
+}  // namespace
+
+// (esa_attend_tc.cu's estimates lie about 4 us above what its calls take: 64.5 and 60.4 for 512 queries of the 32/8-head shape.  Lists
+// that would have to be split for the pairs to fill the SMs stay with it: 40 queries, 8 units, 19.0 us there and 20.4 in 72 pairs.)
+bool attend_pair_wins(const PairDeal& deal, const TcPlan& plan) { return plan.nsplit == 0 || deal.cost < plan.cost - 4.0; }
+bool attend_pair_covers(int D, int l_C, int G) { return D == AP_D && l_C * (int64_t)G > 128; }
+
+PairDeal plan_attend_pair(int num_sms, size_t part_elems, int G, int HG, int top_k, int B, int l_C, const SeqMeta& meta, bool early) {
+    const int R = l_C * G;
+    PairDeal d;
+    d.row_tiles = (R + AP_ROWS - 1) / AP_ROWS;
+    d.units = d.row_tiles * HG * B;
+    const int slots = std::max(1, num_sms / 2);
+    int n_att_max = 0, max_lM = 0;
+    for (int b = 0; b < B; ++b) {
+        max_lM = std::max(max_lM, meta.m_end[b] - meta.i_end[b]);
+        n_att_max = std::max(n_att_max, meta.i_end[b] + std::min(meta.m_end[b] - meta.i_end[b], top_k) + (meta.t[b] - meta.m_end[b]) + l_C);
+    }
+    const int n_tiles = (n_att_max + AP_BN - 1) / AP_BN;
+    // us, fitted to measured calls: a tile of a unit, start and end of a pair, of every further unit, and of a merge launch, whose
+    // traffic (4 TB/s) counts
+    const double tile = 0.93, ends = 5.0, more = 5.0, merge = 4.0;
+    // every unit whole, the pairs evenly loaded
+    d.whole = (d.units + slots - 1) / slots;
+    d.pairs = (d.units + d.whole - 1) / d.whole;
+    d.max_parts = 1;
+    d.late = 0;
+    d.w_early = d.w_late = 1;
+    d.cost = ends + d.whole * tile * n_tiles + (d.whole - 1) * more;
+    // or the units that do not fill a round in ranges
+    if (d.units > slots && d.units % slots) {
+        PairDeal c = d;
+        c.pairs = slots;
+        c.whole = d.units / slots;
+        const int rest = c.units - c.whole * slots;
+        // Beside the selection kernel of its step a call starts on the SMs that this one leaves free; the last pairs follow when it ends,
+        // 5 us and 0.08 us per 1000 middle tokens later (63k tokens 9.5, 202k 21), and get ranges shorter by as many tiles.
+        // (1024 queries of the 28/4-head shape after 202752 tokens: eight pairs of 74 ended 15 us after the others.)
+        if (early && max_lM > top_k) {
+            const double range = (double)n_tiles * rest / slots, behind = (5.0 + 0.08e-3 * max_lM) / tile;
+            c.late = std::min(slots - 1, (select_ctas(num_sms, B, max_lM) + 1) / 2);
+            const double on_time = range + behind * c.late / slots;
+            c.w_early = 64;
+            c.w_late = std::max(0, (int)(64.0 * (on_time - behind) / on_time));
+        }
+        for (int v = 0; v < rest; ++v) {
+            int first, n;
+            deal_parts(c, v, first, n);
+            c.max_parts = std::max(c.max_parts, n);
+        }
+        const size_t floats = (size_t)rest * c.max_parts * AP_PART;
+        c.cost = ends + tile * n_tiles * (c.whole + (double)rest / slots) + c.whole * more + merge + floats * 4 / 4e6;
+        if (floats <= part_elems && c.max_parts <= 64 && c.cost < d.cost) d = c;
+    }
+    return d;
+}
+
+cudaError_t launch_attend_pair(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* Qg, const __nv_bfloat16* K,
+                               const __nv_bfloat16* Kg, const __nv_bfloat16* V, const SeqMeta& meta, const int32_t* idx, const int32_t* n_sel,
+                               __nv_bfloat16* O, const PairDeal& deal, cudaStream_t st, int64_t cache_rows, bool staged) {
+    const bool two = Qg != nullptr || Kg != nullptr;
+    PairParams p;
+    p.Q = Q; p.K = K; p.Qg = Qg ? Qg : Q; p.Kg = Kg ? Kg : K;
+    p.V = V; p.O = O; p.idx = idx; p.n_sel = n_sel; p.part = ctx->att_part; p.status = ctx->status;
+    p.staged = staged ? 1 : 0;
+    p.early = ctx->attend_early && !two && !staged ? 1 : 0;
+    p.max_tokens = cache_rows > 0 ? cache_rows : ctx->cfg.max_tokens; p.l_C = l_C; p.H = ctx->H; p.HG = ctx->HG; p.G = ctx->G;
+    p.top_k = ctx->cfg.top_k;
+    p.deal = deal;
+    p.scale_log2 = ctx->scale * 1.4426950408889634f;
+    p.meta = meta;
+    if (!aligned(p.Q, 16) || !aligned(p.Qg, 16) || !aligned(p.O, 4)) return kErrAlign;
+    p.wide_O = aligned(p.O, 16) ? 1 : 0;
+    CUtensorMap qmap, qgmap;
+    p.q_tma = make_tensor_map_q(&qmap, p.Q, (uint64_t)B * l_C, p.H, AP_D, p.G) ? 1 : 0;
+    if (p.q_tma && two) p.q_tma = make_tensor_map_q(&qgmap, p.Qg, (uint64_t)B * l_C, p.H, AP_D, p.G) ? 1 : 0;
+    if (!p.q_tma) memset(&qmap, 0, sizeof(qmap));
+    if (!p.q_tma || !two) memset(&qgmap, 0, sizeof(qgmap));
+    cudaError_t e;
+    {
+        ProfScope prof(ctx, KC_ATTEND_TC, st);
+        e = two ? launch_pair_kernel<true>(ctx, qmap, qgmap, p, st) : launch_pair_kernel<false>(ctx, qmap, qgmap, p, st);
+    }
+    ctx->launches += 1;
+    const int rest = deal.units - deal.whole * deal.pairs;
+    if (e != cudaSuccess || rest <= 0) return e;
+    ProfScope prof(ctx, KC_ATTEND_MERGE, st);
+    e = launch_pdl(attend_pair_merge_kernel, dim3(rest * (AP_ROWS / 8)), dim3(256), 0, st, (const float*)p.part, deal, l_C * p.G, p.G, p.HG, p.H,
+                   l_C, O);
+    ctx->launches += 1;
+    return e;
+}
+
+}  // namespace esa

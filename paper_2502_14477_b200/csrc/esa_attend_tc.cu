@@ -1,4 +1,5 @@
-// Eq. 1 / Algorithm 1 for prefill-sized chunks on the 5th-generation tensor cores.
+// Eq. 1 / Algorithm 1 for prefill-sized chunks on the 5th-generation tensor cores.  (Heads of 128 and enough rows to fill the SMs:
+// esa_attend_pair.cu.)
 //
 // Same computation as the decode kernel in esa_attend.cu (one softmax over the key list
 // I u M_k u L u C, C causal), organised for tcgen05:
@@ -53,6 +54,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include "esa_attend_tc.cuh"
 #include "esa_internal.h"
 #include "esa_umma.cuh"
 
@@ -77,7 +79,6 @@ constexpr int TC_REGS_SOFTMAX = 168;
 constexpr int TC_REGS_OTHER = 88;
 static_assert(8 * TC_REGS_SOFTMAX + 8 * TC_REGS_OTHER <= 16 * TC_REGS_LAUNCH,
               "register split exceeds the CTA's launch allocation: setmaxnreg.inc would never return");
-constexpr float kSumLimit = 1.8446744e19f;   // 2^64: a tile whose sum of 2^(score - m) reaches this has its maximum looked up
 
 struct TcAttendParams {
     const __nv_bfloat16* Q;
@@ -118,55 +119,12 @@ enum {
     BAR_COUNT = BAR_PAIR + 1
 };
 
-__device__ __forceinline__ void cp_async_arrive_noinc(uint32_t bar) {
-    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];\n" ::"r"(bar) : "memory");
-}
-template <int N>
-__device__ __forceinline__ void reg_alloc() {
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;\n" ::"n"(N));
-}
-template <int N>
-__device__ __forceinline__ void reg_dealloc() {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;\n" ::"n"(N));
-}
-// Barrier over all threads of a thread-block cluster, split in two so that warps with nothing to publish
-// can arrive early.  Arrive releases this thread's shared-memory writes, wait acquires the others'.
-__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;\n" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;\n" ::: "memory"); }
-// address of the same shared-memory location in another CTA of the cluster
-__device__ __forceinline__ uint32_t cluster_map(uint32_t smem_addr, uint32_t cta_rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(smem_addr), "r"(cta_rank));
-    return r;
-}
 // Bulk copy from this CTA's shared memory into another CTA's of the cluster; the bytes are counted on the
 // destination CTA's mbarrier.  Addresses and size are multiples of 16.
 __device__ __forceinline__ void bulk_copy_to_cluster(uint32_t dst_cluster, uint32_t src_cta, uint32_t bytes, uint32_t mbar_cluster) {
     asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst_cluster),
                  "r"(src_cta), "r"(bytes), "r"(mbar_cluster)
                  : "memory");
-}
-__device__ __forceinline__ float fmax3(float a, float b, float c) {
-    float d;
-    asm("max.f32 %0, %1, %2, %3;\n" : "=f"(d) : "f"(a), "f"(b), "f"(c));
-    return d;
-}
-// two-wide fp32 arithmetic (one instruction for a pair of columns)
-__device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
-    float2 d;
-    asm("{\n.reg .b64 ra, rb, rc, rd;\nmov.b64 ra, {%2, %3};\nmov.b64 rb, {%4, %5};\nmov.b64 rc, {%6, %7};\n"
-        "fma.rn.f32x2 rd, ra, rb, rc;\nmov.b64 {%0, %1}, rd;\n}\n"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-    return d;
-}
-__device__ __forceinline__ float2 fadd2(float2 a, float2 b) {
-    float2 d;
-    asm("{\n.reg .b64 ra, rb, rd;\nmov.b64 ra, {%2, %3};\nmov.b64 rb, {%4, %5};\n"
-        "add.rn.f32x2 rd, ra, rb;\nmov.b64 {%0, %1}, rd;\n}\n"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
-    return d;
 }
 // The merged rows of one column half (DH columns) leave as bf16 through a per-warp staging buffer: 16-byte
 // stores, whole rows per instruction.  acc: this lane's row; lane rr of the warp owns row wrow0 + rr, whose

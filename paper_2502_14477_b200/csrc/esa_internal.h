@@ -218,6 +218,9 @@ cudaError_t launch_select(esa_ctx* ctx, int B, bool mapped, const SeqMeta& meta,
 cudaError_t launch_score_full(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* K, const SeqMeta& meta,
                               int max_lM, bool per_head, cudaStream_t st);
 
+// CTAs of a selection of B sequences, the longest with max_lM middle tokens (as many SMs are busy with it).
+int select_ctas(int num_sms, int B, int max_lM);
+
 // idx_out[b, 0..l_M) = i_end + 0..l_M-1, n_sel_out[b] = l_M for sequences with l_M <= top_k
 // (only_small = 1) or all sequences (only_small = 0).
 cudaError_t launch_select_all(esa_ctx* ctx, int B, const SeqMeta& meta, int32_t* idx_out,
@@ -264,6 +267,37 @@ cudaError_t launch_attend_tc(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* 
                              const __nv_bfloat16* K, const __nv_bfloat16* Kg, const __nv_bfloat16* V, const SeqMeta& meta,
                              const int32_t* idx, const int32_t* n_sel, __nv_bfloat16* O, const TcPlan& plan, cudaStream_t st,
                              int64_t cache_rows = 0, bool staged = false);
+
+// Chunks of more than 128 rows per key/value head, heads of 128, on tcgen05 with CTA pairs (esa_attend_pair.cu).  How its
+// units (256 rows of a key/value head) are dealt out: pair i of `pairs` takes the units i + w * pairs, w < whole, and then
+// range i of the rest, cut whatever units the ranges touch; parts of these are merged by a second launch.  Ranges are as long as their
+// weights: w_early, or w_late for the last `late` pairs, which start only when the selection kernel leaves their SMs.
+struct PairDeal {
+    int row_tiles, units;
+    int pairs, whole;
+    int late, w_early, w_late;
+    int max_parts;      // largest number of parts of a unit of the rest
+    double cost;        // estimated us
+};
+// Places in the rest are counted in `deal_weight`-ths of a unit: range i starts at rest * deal_start(i).
+__host__ __device__ inline int deal_start(const PairDeal& d, int i) {
+    const int n = d.pairs - d.late;
+    return i <= n ? i * d.w_early : n * d.w_early + (i - n) * d.w_late;
+}
+__host__ __device__ inline int deal_weight(const PairDeal& d) { return deal_start(d, d.pairs); }
+// Unit v of the rest is covered by n_parts ranges, those of the pairs from `first` on.
+__host__ __device__ inline void deal_parts(const PairDeal& d, int v, int& first, int& n_parts) {
+    const int rest = d.units - d.whole * d.pairs, w = deal_weight(d), n = d.pairs - d.late;
+    const int a = v * w / rest, b = ((v + 1) * w - 1) / rest;
+    first = a < n * d.w_early ? a / d.w_early : n + (a - n * d.w_early) / d.w_late;
+    n_parts = (b < n * d.w_early ? b / d.w_early : n + (b - n * d.w_early) / d.w_late) - first + 1;
+}
+bool attend_pair_covers(int D, int l_C, int G);
+bool attend_pair_wins(const PairDeal& deal, const TcPlan& plan);       // against esa_attend_tc.cu
+PairDeal plan_attend_pair(int num_sms, size_t part_elems, int G, int HG, int top_k, int B, int l_C, const SeqMeta& meta, bool early);
+cudaError_t launch_attend_pair(esa_ctx* ctx, int B, int l_C, const __nv_bfloat16* Q, const __nv_bfloat16* Qg, const __nv_bfloat16* K,
+                               const __nv_bfloat16* Kg, const __nv_bfloat16* V, const SeqMeta& meta, const int32_t* idx, const int32_t* n_sel,
+                               __nv_bfloat16* O, const PairDeal& deal, cudaStream_t st, int64_t cache_rows = 0, bool staged = false);
 
 // TMA descriptor of the query tensor [n_queries, H, D] for the attention kernel (group size G must
 // divide 128).

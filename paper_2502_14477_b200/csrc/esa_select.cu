@@ -413,6 +413,13 @@ static cudaError_t launch_topk(int device, const SelectParams& p, int n_ranks, i
     return e == cudaSuccess && n == 0 ? cudaErrorNotSupported : e;
 }
 
+int select_ctas(int num_sms, int B, int max_lM) {
+    const int most = SEL_CLUSTER * B <= num_sms ? SEL_CLUSTER : 8;
+    int n = 1;
+    while (n < most && n * 8 * SEL_THREADS < max_lM) n *= 2;
+    return n * B;
+}
+
 // pooled_ready: ctx->pkey already holds the pooled keys; otherwise ctx->skey holds unpooled ones.
 cudaError_t launch_select(esa_ctx* ctx, int B, bool mapped, const SeqMeta& meta, int max_lM, bool pooled_ready,
                           int32_t* idx_out, int32_t* n_sel_out, cudaStream_t st) {

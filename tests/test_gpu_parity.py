@@ -407,6 +407,46 @@ def test_uneven_key_list_split(case):
             hp.check_attention(got[b], want, what=f"{what} seq {b}", heads=heads)
 
 
+@pytest.mark.parametrize("H,H_G,t_list,l_C,l_L,k,form", [
+    (60, 60, (3000,), 129, 300, 1000, "pair"), (40, 40, (3000,), 255, 64, 900, "pair"), (40, 40, (3000,), 256, 0, 900, "pair"),    # one row tile, ragged and full
+    (36, 36, (3000,), 257, 300, 1000, "pair"), (28, 4, (3000, 700), 100, 300, 1000, "pair"), (8, 1, (120,), 300, 600, 500, "pair"),
+    (37, 37, (2500,), 500, 300, 1000, "pair"), (19, 19, (2500,), 1024, 300, 1000, "uneven"), (38, 38, (9000,), 512, 1000, 5000, "uneven"),  # 74, 76, 76 units
+    (20, 20, (40000,), 1024, 1000, 3000, "uneven"), (35, 35, (2500, 300, 150, 1400), 250, 500, 700, None),
+    (28, 4, (700, 6000, 30), 600, 1500, 2000, "pair"), (16, 2, (40,), 2300, 500, 700, None)])
+def test_paired_attention_at_unit_and_deal_edges(H, H_G, t_list, l_C, l_L, k, form):
+    """Chunks of more than 128 rows per key/value head, heads of 128: ragged row tiles, units dealt out whole, several to a pair of CTAs,
+    and with the rest in ranges that end inside a unit (equal ones, and shorter ones for the pairs that the selection holds up), sequences
+    of unlike lengths; one position (the call that follows its selection, and one that follows none) and two, against the oracle on
+    the same selection."""
+    from paper_2502_14477_b200.binding import attend_plan
+    B, n = len(t_list), max(t_list) + l_C
+    cfg = syn.get_config("c1").with_(H=H, H_G=H_G, d=128, d_c=64, l_I=16, l_L=l_L, k=k)
+    p, heads = hp.oracle_params(cfg), sorted({0, H // 2, H - 1})
+    ctx = hp.make_esa(cfg, max_tokens=n, max_chunk=l_C, max_batch=B)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert sms != 148 or form is None or attend_plan(ctx.cfg, sms, l_C, t_list)[0] == form
+    g = torch.Generator(device="cuda").manual_seed(H + l_C)
+    draw = lambda *s: torch.randn(*s, device="cuda", dtype=torch.bfloat16, generator=g)
+    Q, Qf, K, Kf, V, kc = draw(B, l_C, H, 128), draw(B, l_C, H, 128), draw(B, n, H_G, 128), draw(B, n, H_G, 128), draw(B, n, H_G, 128), draw(B, n, 64)
+    idx, counts = torch.zeros(B, k, dtype=torch.int32, device="cuda"), torch.zeros(B, dtype=torch.int32, device="cuda")
+    early, plain, two = (torch.full_like(Q, float("nan")) for _ in range(3))
+    torch.cuda.synchronize()
+    ctx.select(Q, kc, list(t_list), idx, counts)
+    ctx.attend(Q, K, V, list(t_list), idx, counts, early)
+    ctx.attend(Q, K, V, list(t_list), idx, counts, plain)
+    ctx.attend_two_position(Q, Qf, K, Kf, V, list(t_list), idx, counts, two, sync=True)
+    assert ctx.last_device_status() == 0
+    f64 = hp.torch_to_f64
+    for b, t in enumerate(t_list):
+        sel, m = idx[b, : int(counts[b])].cpu().numpy().astype(np.int64), t + l_C
+        args = (f64(Q[b]), f64(K[b, :m]), f64(V[b, :m]), sel, t, p)
+        want = orc.attend(*args, heads=heads)
+        hp.check_attention(early[b], want, what=f"early seq {b}", heads=heads)
+        hp.check_attention(plain[b], want, what=f"plain seq {b}", heads=heads)
+        want = orc.attend(*args, heads=heads, Q_global=f64(Qf[b]), K_global=f64(Kf[b, :m]))
+        hp.check_attention(two[b], want, what=f"two seq {b}", heads=heads)
+
+
 @pytest.mark.parametrize("case", hp.SMALL_BATCH_CASES, ids=lambda c: f"{c[0]}-{c[1]}-{c[2]}-{c[3]}x{c[6]}-{c[9]}")
 def test_small_chunks_in_large_batches(case):
     """More units of a few rows than SMs, against the oracle on sampled sequences and heads, and with the output off its boundary."""
