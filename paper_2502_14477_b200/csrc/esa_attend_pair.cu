@@ -13,10 +13,10 @@
 //     shape over 13.4k keys 181 -> 168.  What bounds it now: a tile takes 1680 cycles, against 1024 of the tensor core and 1024 of the
 //     special-function unit; a warpgroup spends 2600 of its 3360 on a tile (exponentials 1800) and waits 500 for its scores.
 //   * Two softmax warpgroups take the tiles in turn, a thread per row.  They share the row's running maximum: it is set by
-//     the first half tile of a unit, handed over through shared memory, and after that only raised when a half's
-//     sum of 2^(score - m) reaches 2^64.  A raise is by a whole number, so that what the other warpgroup has
-//     formed with the old maximum is brought up to date by an exact power of two: a warpgroup looks at the maximum once
-//     more after the tile before its own is decided and before it gives its P away.
+//     the first tile of a unit, handed over through shared memory, and after that only raised when a half tile's
+//     sum of 2^(score - m) reaches 2^64 (esa_attend_tc.cu says why that is enough).  A raise is by a whole number, so that what the
+//     other warpgroup has formed with the old maximum is brought up to date by an exact power of two: a warpgroup looks at
+//     the maximum once more after the tile before its own is decided and before it gives its P away.
 //   * Warps of a CTA: 0-3 / 4-7 softmax of the even / odd tiles, 8-11 gather Q and K/V (index-driven 16-byte cp.async into
 //     128-byte-swizzled tiles, four stages of K and five of V), 12 and 13 issue the scores and P V (even CTA) or pass on to it which
 //     K and V tiles their CTA has loaded (odd CTA).  (One warp for both kinds of products was busy issuing all the time: beside the softmax
@@ -268,24 +268,44 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_consta
                 // (the other warpgroup takes every other tile)
                 const int j_base = j;
                 j += end - begin;
+                // first invisible entry of this row in late tile T, and of the CTA's first row
+                auto visible = [&](int T, int seen) { return TWO && T < late.far_tiles ? late.list.ng : late.c_first + seen; };
+                if (j_base == j0 && begin < end) {
+                    // The unit's first tile sets the maximum, all of it: every row has its first visible key there, if it has one at
+                    // all, and its dominant key as often as with a list in two parts that look at half a tile each.  (A dominant
+                    // weight of exactly 1 is not rounded: with half a tile the 2-norm error against 64 bits was 0.7 % larger.)
+                    if ((j0 & 1) == wg) {
+                        const int key0 = phase == 0 ? begin * AP_BN : late_key(late, begin), lim = phase == 0 ? e_len : visible(begin, sees);
+                        mbar_wait(bar(AB_QK_DONE + j0 % AP_KS), (j0 / AP_KS) & 1, wc);
+                        tc_fence_after_sync();
+                        float mx = -INFINITY;
+#pragma unroll 1
+                        for (int q = 0; q < AP_BN; q += 32) {
+                            uint32_t w[32];
+                            tmem_ld32(tmem_addr(tmem, lane_base, (j0 % AP_S) * 128 + q), w);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int c = 0; c < 32; ++c)
+                                if (key0 + q + c < lim) mx = fmaxf(mx, __uint_as_float(w[c]));
+                        }
+                        m_run = mx * sl2;
+                        m_row[buf][wrow] = m_run;
+                        mbar_arrive(bar(AB_M_READY));
+                    } else {
+                        mbar_wait(bar(AB_M_READY), n_unit & 1, wc);
+                        m_run = m_row[buf][wrow];
+                    }
+                }
 #pragma unroll 1
                 for (int jt = j_base + ((j_base ^ wg) & 1); jt < j; jt += 2) {
                     const int T = begin + (jt - j_base);
                     const bool first = jt == j0;
                     const int sb = jt % AP_S, turn = jt / AP_S;
                     const uint32_t tS = tmem_addr(tmem, lane_base, sb * 128);
-                    const bool far = TWO && phase == 1 && T < late.far_tiles;
                     const int key_tile = phase == 0 ? T * AP_BN : late_key(late, T);
-                    // first invisible entry of this row, and the smallest such limit of the CTA's rows
-                    const int lim = phase == 0 ? e_len : far ? late.list.ng : late.c_first + sees;
-                    const int lim_min = phase == 0 ? e_len : far ? late.list.ng : late.c_first + sees_min;
+                    const int lim = phase == 0 ? e_len : visible(T, sees), lim_min = phase == 0 ? e_len : visible(T, sees_min);
                     // the barrier of the tile before
                     const int prev_p = AB_P_READY + (sb == 0 ? AP_S - 1 : sb - 1), prev_par = (sb == 0 ? turn - 1 : turn) & 1;
-                    if (jt == j0 + 1) {
-                        // every row has its first visible key in the unit's first half tile, if it has one at all
-                        mbar_wait(bar(AB_M_READY), n_unit & 1, wc);
-                        m_run = m_row[buf][wrow];
-                    }
                     mbar_wait(bar(AB_QK_DONE + jt % AP_KS), (jt / AP_KS) & 1, wc);
                     tc_fence_after_sync();
                     // multiplies the stored P of half h by a power of two
@@ -341,11 +361,6 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_consta
                             const float2 a = fadd2(sum4[0], sum4[1]), c = fadd2(sum4[2], sum4[3]);
                             return (a.x + a.y) + (c.x + c.y);
                         };
-                        if (first && u == 0) {
-                            m_run = max_score();
-                            m_row[buf][wrow] = m_run;
-                            mbar_arrive(bar(AB_M_READY));
-                        }
                         float sum = exps(m_run);
                         // The decision is taken per warp: tensor-memory accesses are warp-wide.
                         const bool raise = !(sum < kSumLimit);           // also true for inf and NaN
