@@ -13,7 +13,7 @@
 //     shape over 13.4k keys 181 -> 168.  What bounds it now: a tile takes 1680 cycles, against 1024 of the tensor core and 1024 of the
 //     special-function unit; a warpgroup spends 2600 of its 3360 on a tile (exponentials 1800) and waits 500 for its scores.
 //   * Two softmax warpgroups take the tiles in turn, a thread per row.  They share the row's running maximum: it is set by
-//     the first tile of a unit, handed over through shared memory, and after that only raised when a half tile's
+//     the first two tiles of a unit, exchanged through shared memory, and after that only raised when a half tile's
 //     sum of 2^(score - m) reaches 2^64 (esa_attend_tc.cu says why that is enough).  A raise is by a whole number, so that what the
 //     other warpgroup has formed with the old maximum is brought up to date by an exact power of two: a warpgroup looks at
 //     the maximum once more after the tile before its own is decided and before it gives its P away.
@@ -98,8 +98,7 @@ enum {
     AB_QK_DONE = AB_V_FULL + AP_VS,      // by tile % AP_KS: scores ready, K stage free
     AB_PV_DONE = AB_QK_DONE + AP_KS,     // by tile % AP_VS: V stage free
     AB_P_READY = AB_PV_DONE + AP_VS,     // by tile % AP_S: P written, maximum decided
-    AB_M_READY = AB_P_READY + AP_S,      // per unit: its first maximum is in shared memory
-    AB_O_FREE = AB_M_READY + 1,          // per unit: the accumulator has been read
+    AB_O_FREE = AB_P_READY + AP_S,         // per unit: the accumulator has been read
     AB_COUNT = AB_O_FREE + 1
 };
 
@@ -185,7 +184,6 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_consta
             mbar_init(bar(AB_PV_DONE + s), 1);
         }
         for (int s = 0; s < AP_S; ++s) mbar_init(bar(AB_P_READY + s), 128 + 4 * relay);
-        mbar_init(bar(AB_M_READY), 128);
         mbar_init(bar(AB_O_FREE), 16);                // a warp of either CTA each
         mbar_init_fence();
     }
@@ -271,30 +269,30 @@ attend_pair_kernel(const __grid_constant__ CUtensorMap qmap, const __grid_consta
                 // first invisible entry of this row in late tile T, and of the CTA's first row
                 auto visible = [&](int T, int seen) { return TWO && T < late.far_tiles ? late.list.ng : late.c_first + seen; };
                 if (j_base == j0 && begin < end) {
-                    // The unit's first tile sets the maximum, all of it: every row has its first visible key there, if it has one at
-                    // all, and its dominant key as often as with a list in two parts that look at half a tile each.  (A dominant
-                    // weight of exactly 1 is not rounded: with half a tile the 2-norm error against 64 bits was 0.7 % larger.)
-                    if ((j0 & 1) == wg) {
-                        const int key0 = phase == 0 ? begin * AP_BN : late_key(late, begin), lim = phase == 0 ? e_len : visible(begin, sees);
-                        mbar_wait(bar(AB_QK_DONE + j0 % AP_KS), (j0 / AP_KS) & 1, wc);
+                    // The unit's first two tiles (first, where the phase has no more) set the maximum, one looked at by each warpgroup:
+                    // every row has its first visible key in the first, if it has one at all, and its dominant key among these 256 as
+                    // often as with a list in up to four parts that look at half a tile each.  (A dominant weight of
+                    // exactly 1 is not rounded: with half a tile the 2-norm error against 64 bits was 0.7 % larger.)
+                    const int jm = j0 + ((j0 ^ wg) & 1), T = begin + (jm - j0);
+                    float mx = -INFINITY;
+                    if (T < end) {
+                        const int key0 = phase == 0 ? T * AP_BN : late_key(late, T), lim = phase == 0 ? e_len : visible(T, sees);
+                        mbar_wait(bar(AB_QK_DONE + jm % AP_KS), (jm / AP_KS) & 1, wc);
                         tc_fence_after_sync();
-                        float mx = -INFINITY;
 #pragma unroll 1
                         for (int q = 0; q < AP_BN; q += 32) {
                             uint32_t w[32];
-                            tmem_ld32(tmem_addr(tmem, lane_base, (j0 % AP_S) * 128 + q), w);
+                            tmem_ld32(tmem_addr(tmem, lane_base, (jm % AP_S) * 128 + q), w);
                             tmem_wait_ld();
 #pragma unroll
                             for (int c = 0; c < 32; ++c)
                                 if (key0 + q + c < lim) mx = fmaxf(mx, __uint_as_float(w[c]));
                         }
-                        m_run = mx * sl2;
-                        m_row[buf][wrow] = m_run;
-                        mbar_arrive(bar(AB_M_READY));
-                    } else {
-                        mbar_wait(bar(AB_M_READY), n_unit & 1, wc);
-                        m_run = m_row[buf][wrow];
                     }
+                    l_row[buf][wg][wrow] = mx * sl2;              // (the sums come at the unit's end)
+                    asm volatile("bar.sync 1, 256;\n" ::: "memory");
+                    m_run = fmaxf(mx * sl2, l_row[buf][wg ^ 1][wrow]);
+                    if (jm == j0) m_row[buf][wrow] = m_run;
                 }
 #pragma unroll 1
                 for (int jt = j_base + ((j_base ^ wg) & 1); jt < j; jt += 2) {
