@@ -726,7 +726,7 @@ def run_esa(args, cfg):
     n_chunks = (cfg.S + cfg.l_C - 1) // cfg.l_C
     att = by_kernel.get("attend_tc_kernel", {"achieved": 0.0, "frac_sustained": 0.0, "frac_burst": 0.0, "launches": 0})
     att_ms = prof.get("attend_tc_kernel", (0, 0.0))[1]
-    roofline = {"bound": "tensor", "kernel": "attend_tc_kernel (two-way key-list splits merged inside the kernel)",
+    roofline = {"bound": "tensor", "kernel": "attend_pair_kernel (CTA pairs, unsplit key lists; timed in the class attend_tc_kernel)",
                 "achieved": att["achieved"], "peak": peaks["tflops_sustained"],
                 "unit": "TFLOP/s", "frac": att["frac_sustained"], "frac_sustained": att["frac_sustained"],
                 "frac_burst": att["frac_burst"], "peak_burst": peaks["tflops_burst"],
